@@ -464,7 +464,8 @@ def _em(x, model, iters, tol, reg=REG):
         if len(trace) > 1 and abs(trace[-1] - trace[-2]) < tol:
             break
     return {"weights": w, "means": mu + off, "covs": cov, "iters_done": len(trace),
-            "trace": np.array(trace + [math.nan] * (iters - len(trace))), "final_loglik": float(_estep(x, w, mu, cov, False)[0].mean())}
+            "trace": np.array(trace + [math.nan] * (iters - len(trace))),
+            "final_loglik": float(_estep(x, w, mu, cov, False)[0].mean())}
 
 
 def _fit(x, case, k):
