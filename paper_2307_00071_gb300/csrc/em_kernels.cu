@@ -1068,22 +1068,6 @@ int estep_grad_occupancy(int k, int64_t ppc) {
     return occ;
 }
 
-constexpr int KCHUNK = 512;   // components per chunk: the 4-warp shape
-
-int chunk_components() { return KCHUNK; }
-
-int64_t chunk_param_floats() { return (int64_t)params_pairs_padded(KCHUNK) * PAIR_FLOATS; }
-
-cudaError_t launch_estep_chunks(const EStepLaunch& a, int pass, int nunits, int64_t ppc, cudaStream_t s) {
-    void* args[] = {(void*)&a};
-    const void* fn = (pass == 1) ? (const void*)estep_kernel<2, QB, 128, 3, false, false, 1>
-                                 : (const void*)estep_kernel<2, QB, 128, 3, true, false, 2>;
-    const size_t smem = estep_smem(ppc);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    return cudaLaunchKernel(fn, dim3(nunits), dim3(128), args, smem, s);
-}
-
 namespace {
 thread_local std::string t_estep_name;
 thread_local const void* t_estep_fn = nullptr;
@@ -1106,6 +1090,7 @@ void note_estep_kernel(const void* fn) {
     std::free(dem);
     size_t at = name.find("estep_kernel<");
     if (at == std::string::npos) at = name.find("estep_pt_kernel<");
+    if (at == std::string::npos) at = name.find("estep_reach_kernel<");
     if (at == std::string::npos) at = name.find("estep4_kernel<");
     if (at != std::string::npos) name = name.substr(at);
     const size_t par = name.rfind(">(");
@@ -1235,50 +1220,9 @@ cudaError_t launch_fill_padding(float* params, int k, int npairs_pad, cudaStream
 
 // ------------------------------------------------------------------ log-likelihood reduce
 namespace {
-// ------------------------------------------------------------------ large K (chunks)
-constexpr int CHUNK_K = 512;
+// ------------------------------------------------------------------ two-level log-sum-exp (4-D chunks)
 constexpr int COMBINE_BLOCKS = 608;
 constexpr int COMBINE_THREADS = 256;
-
-// component b of a chunked parameter buffer
-__device__ __forceinline__ const float* chunk_slot(const float* params, int b) {
-    const int c = b / CHUNK_K, l = b - c * CHUNK_K;
-    return params + (size_t)c * (CHUNK_K / 2) * PAIR_FLOATS + (size_t)(l >> 1) * PAIR_FLOATS + (l & 1);
-}
-
-// gref[0] = max_b c_b, gref[1] = the log-likelihood reference (cmax - log2 sum_a N_a
-// after an M-step, else cmax): the per-CTA kernel's prologue over all k components.
-__global__ void chunk_ref_kernel(const float* __restrict__ params, int k, const DeviceState* st, float* gref) {
-    __shared__ float s_m[8];
-    __shared__ double s_w[8];
-    float m = -INFINITY;
-    double w = 0.0;
-    for (int b = threadIdx.x; b < k; b += blockDim.x) {
-        const float* p = chunk_slot(params, b);
-        m = fmaxf(m, p[2 * SLOT_C]);
-        w += (double)p[2 * SLOT_W];
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-        w += __shfl_xor_sync(0xffffffffu, w, o);
-    }
-    if ((threadIdx.x & 31) == 0) {
-        s_m[threadIdx.x >> 5] = m;
-        s_w[threadIdx.x >> 5] = w;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float mm = s_m[0];
-        double ww = s_w[0];
-        for (int i = 1; i < (int)(blockDim.x >> 5); ++i) {
-            mm = fmaxf(mm, s_m[i]);
-            ww += s_w[i];
-        }
-        gref[0] = mm;
-        gref[1] = st->w_raw ? (float)((double)mm - log2(ww)) : mm;
-    }
-}
 
 // Per point: total over chunks (fixed order); (0, 1/total) and the natural-log
 // log-likelihood, or, if the total is below 2^-100, listed for the exact step.
@@ -1297,48 +1241,6 @@ __global__ void __launch_bounds__(COMBINE_THREADS) chunk_combine_kernel(const fl
             pref[i] = make_float2(0.f, 0.f);
             llpt[i] = 0.0;
             flags[atomicAdd(flag_count, 1)] = (int)i;
-        }
-    }
-}
-
-// One warp per listed point: exact maximum of the logits over all k components,
-// then (shift, 1/sum) relative to it (Eq. logestep's max-subtraction).
-__global__ void chunk_exact_kernel(const float4* __restrict__ pts8, const float* __restrict__ params, int k,
-                                   const float* __restrict__ gref, const int* __restrict__ flags,
-                                   const int* __restrict__ flag_count, float2* pref, double* llpt, DeviceState* st) {
-    const int count = *flag_count;
-    const float cmax = gref[0], ref0 = gref[1];
-    const int lane = threadIdx.x & 31;
-    const int wg = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
-    for (int f = wg; f < count; f += nw) {
-        const int64_t i = flags[f];
-        const float4 xy = pts8[2 * i], zz = pts8[2 * i + 1];
-        const float x0 = xy.x, x1 = xy.z, x2 = zz.x;
-        auto nlog = [&](int b) {   // q' = |P'(x - mu)|^2 + (cmax - c_b), as the E-step forms it
-            const float* p = chunk_slot(params, b);
-            const float d0 = x0 + p[2 * (SLOT_NMU + 0)], d1 = x1 + p[2 * (SLOT_NMU + 1)], d2 = x2 + p[2 * (SLOT_NMU + 2)];
-            const float y0 = p[2 * (SLOT_P + 0)] * d0;
-            const float y1 = fmaf(p[2 * (SLOT_P + 2)], d1, p[2 * (SLOT_P + 1)] * d0);
-            const float y2 = fmaf(p[2 * (SLOT_P + 5)], d2, fmaf(p[2 * (SLOT_P + 4)], d1, p[2 * (SLOT_P + 3)] * d0));
-            return fmaf(y2, y2, fmaf(y1, y1, fmaf(y0, y0, cmax - p[2 * SLOT_C])));
-        };
-        float mx = -INFINITY;
-        for (int b = lane; b < k; b += 32) mx = fmaxf(mx, -nlog(b));
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        float sum = 0.f;
-        if (mx > -INFINITY)
-            for (int b = lane; b < k; b += 32) sum += ex2_approx(-nlog(b) - mx);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-        if (lane == 0) {
-            if (!(mx > -INFINITY) || !(sum > 0.f)) {
-                set_error(st, GIRA_ERR_NUMERIC);
-                pref[i] = make_float2(0.f, 0.f);
-            } else {
-                pref[i] = make_float2(-mx, __frcp_rn(sum));
-                llpt[i] = (double)(lg2_approx(sum) + mx + ref0) * 0.693147180559945309417232121458;
-            }
         }
     }
 }
@@ -1990,31 +1892,15 @@ __global__ void __launch_bounds__(FIN_THREADS) reduce_finalize_kernel(const FinA
 
 // Every instance of a batch: block (instance i, index j) finalizes components
 // j * FIN_CPB .. of instance i from its own partials, into its own state.
-// shared: the entries are chunks of one fit (state, trace and log-likelihood
-// partials shared; the log-likelihood step runs in the block of (0, 0)).
 __global__ void __launch_bounds__(FIN_THREADS) reduce_finalize_batched_kernel(const FinArgs base,
                                                                               const BatchInst* __restrict__ insts,
                                                                               const int2* __restrict__ blocks,
-                                                                              DeviceState* states, int iters,
-                                                                              int shared) {
+                                                                              DeviceState* states, int iters) {
     const int2 bi = blocks[blockIdx.x];
     const BatchInst I = insts[bi.x];
     FinArgs f = base;
     f.partials = base.partials ? base.partials + I.part_off : nullptr;
     f.grid = I.ctas;
-    if (shared) {
-        f.stats64 = base.stats64 ? base.stats64 + (size_t)I.comp_off * NSTAT : nullptr;
-        f.shift4 = base.shift4 + I.comp_off;
-        f.k = I.k;
-        f.n = I.n;
-        f.model64 = base.model64 + (size_t)I.comp_off * MODEL;
-        f.params = base.params + I.par_off;
-        f.perm = base.perm ? base.perm + I.comp_off : nullptr;
-        f.st = states;
-        f.do_ll = (bi.x == 0);
-        reduce_finalize_body(f, bi.y);
-        return;
-    }
     f.llp = base.llp ? base.llp + I.ll_off : nullptr;
     f.perm = base.perm ? base.perm + I.comp_off : nullptr;
     if (base.masks) {   // point-stationary E-step: per-warp rows, live masks, one ll slot per CTA
@@ -2541,18 +2427,7 @@ cudaError_t launch_reduce_finalize_batched(const float* partials, const double* 
                                            const int* perm, const uint32_t* masks) {
     const FinArgs f{partials, 0, ll_partials, stats64, shift4, 0, 0, reg, tol, model64, params, trace, nullptr,
                     iter, em ? 1 : 0, 0, 1, perm, masks, 0};
-    reduce_finalize_batched_kernel<<<nblocks, FIN_THREADS, 0, s>>>(f, insts, blocks, states, std::max(iters, 1), 0);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_reduce_finalize_chunks(const float* partials, const double* ll_partials, int ll_count,
-                                          const double* stats64, float4* shift4, const BatchInst* insts,
-                                          const int2* blocks, int nblocks, int64_t n, double reg, double tol,
-                                          double* model64, float* params, double* trace, DeviceState* st, int iter,
-                                          bool em, cudaStream_t s, const int* perm) {
-    const FinArgs f{partials, 0, ll_partials, stats64, shift4, 0, n, reg, tol, model64, params, trace, nullptr,
-                    iter, em ? 1 : 0, ll_count, 1, perm};
-    reduce_finalize_batched_kernel<<<nblocks, FIN_THREADS, 0, s>>>(f, insts, blocks, st, 1, 1);
+    reduce_finalize_batched_kernel<<<nblocks, FIN_THREADS, 0, s>>>(f, insts, blocks, states, std::max(iters, 1));
     return cudaGetLastError();
 }
 
@@ -2685,22 +2560,11 @@ cudaError_t launch_grad_finalize_batched(const float* partials, const double* ll
 namespace gira {
 int chunk_combine_grid() { return COMBINE_BLOCKS; }
 
-cudaError_t launch_chunk_ref(const float* params, int k, const DeviceState* st, float* gref, cudaStream_t s) {
-    chunk_ref_kernel<<<1, 256, 0, s>>>(params, k, st, gref);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_chunk_combine(const float* psum, int chunks, int64_t n, const float* gref, float2* pref,
                                  double* llpt, int* flag_count, int* flags, DeviceState* st, cudaStream_t s) {
     (void)st;
     chunk_combine_kernel<<<COMBINE_BLOCKS, COMBINE_THREADS, 0, s>>>(psum, chunks, n, gref, pref, llpt, flag_count,
                                                                     flags);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_chunk_exact(const float4* pts8, const float* params, int k, const float* gref, const int* flags,
-                               const int* flag_count, float2* pref, double* llpt, DeviceState* st, cudaStream_t s) {
-    chunk_exact_kernel<<<152, 256, 0, s>>>(pts8, params, k, gref, flags, flag_count, pref, llpt, st);
     return cudaGetLastError();
 }
 

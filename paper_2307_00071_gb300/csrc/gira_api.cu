@@ -335,129 +335,65 @@ void build_tables(std::vector<BatchInst>& hi, std::vector<BatchClass>& cls, std:
 }  // namespace
 
 
-// ---------------------------------------------------------------- large K (chunked E-step)
+// ---------------------------------------------------------------- E-step over reach lists
 namespace {
 
-// The chunk table of one fit over n points with k components, and its unit list.
-struct ChunkPlan {
-    int chunks = 0;
-    int64_t ppc = 0;
-    std::vector<BatchInst> hi;
-    std::vector<BatchUnit> units;
-    std::vector<int2> blocks;
-    std::vector<int> comp_inst, npairs;
-    int64_t part_floats = 0;
+// Buffers of the E-step over reach lists (reach_kernels.cu) for n points and k
+// components; with stats, also those of its statistics.
+struct ReachBufs {
+    float4* ctr = nullptr;
+    float2 *aux = nullptr, *pref = nullptr;
+    float *gref = nullptr, *partials = nullptr;
+    uint32_t *masks = nullptr, *live2 = nullptr;
+    double* llp = nullptr;
+    int grid = 0, h = 0, words = 0, slices = 0;
+    int64_t rows = 0;
 };
 
-ChunkPlan plan_chunks(int64_t n, int k, int sms) {
-    ChunkPlan P;
-    const int KC = chunk_components();
-    P.chunks = (k + KC - 1) / KC;
-    const int Q = estep_batch_q();
-    const int occ = estep_occupancy(KC, true, 1024);
-    int64_t ppc = (n * P.chunks + 2LL * sms * occ - 1) / (2LL * sms * occ);
-    P.ppc = std::min<int64_t>(estep_ppc_max(), std::max<int64_t>(4 * Q, (ppc + Q - 1) / Q * Q));
-    const int ctas = (int)((n + P.ppc - 1) / P.ppc);
-    const int cpb = fin_components_per_block();
-    for (int c = 0; c < P.chunks; ++c) {
-        BatchInst I{};
-        I.pt_off = 0;
-        I.n = n;
-        I.ppc = P.ppc;
-        I.k = std::min(KC, k - c * KC);
-        I.comp_off = c * KC;
-        I.par_off = c * chunk_param_floats();
-        I.ctas = ctas;
-        I.part_off = P.part_floats;
-        I.ll_off = 0;
-        P.part_floats += (int64_t)ctas * I.k * NSTAT;
-        P.hi.push_back(I);
-        P.npairs.push_back((int)(chunk_param_floats() / PAIR_FLOATS));
-        for (int t = 0; t < ctas; ++t) P.units.push_back(BatchUnit{c, t});
-        for (int j = 0; j * cpb < I.k; ++j) P.blocks.push_back(make_int2(c, j));
-        for (int b = 0; b < I.k; ++b) P.comp_inst.push_back(c);
-    }
-    return P;
-}
-
-struct ChunkBufs {
-    float *params = nullptr, *partials = nullptr, *psum = nullptr, *gref = nullptr;
-    float2* pref = nullptr;
-    double *llpt = nullptr, *llp = nullptr;
-    int *flags = nullptr, *flag_count = nullptr, *comp_inst = nullptr, *npairs = nullptr;
-    BatchInst* insts = nullptr;
-    BatchUnit* units = nullptr;
-    int2* blocks = nullptr;
-};
-
-void carve_chunks(Carver& cv, const ChunkPlan& P, int64_t n, bool stats, ChunkBufs* b) {
-    b->params = cv.take<float>((size_t)P.chunks * chunk_param_floats());
-    b->partials = cv.take<float>(stats ? (size_t)P.part_floats : 0);
-    b->psum = cv.take<float>((size_t)P.chunks * n);
+void carve_reach(Carver& cv, int64_t n, int k, int nstat, bool stats, ReachBufs* b) {
+    int sl = 1;
+    b->grid = reach_grid(n);
+    b->h = reach_h(n);
+    b->words = reach_mask_words(k);
+    b->rows = reach_rows(n);
+    b->slices = reach_slices(n, &sl);
+    b->ctr = cv.take<float4>(k);
+    b->aux = cv.take<float2>(k);
     b->gref = cv.take<float>(2);
+    b->llp = cv.take<double>(b->grid);
+    if (!stats) return;
     b->pref = cv.take<float2>(n);
-    b->llpt = cv.take<double>(n);
-    b->llp = cv.take<double>(chunk_combine_grid());
-    b->flags = cv.take<int>(n);
-    b->flag_count = cv.take<int>(1);
-    b->comp_inst = cv.take<int>(P.comp_inst.size());
-    b->npairs = cv.take<int>(P.chunks);
-    b->insts = cv.take<BatchInst>(P.chunks);
-    b->units = cv.take<BatchUnit>(P.units.size());
-    b->blocks = cv.take<int2>(P.blocks.size());
+    b->masks = cv.take<uint32_t>((size_t)b->words * b->rows);
+    b->live2 = cv.take<uint32_t>((size_t)b->words * b->slices);
+    b->partials = cv.take<float>((size_t)b->slices * ((k + 1) / 2) * 2 * nstat);
 }
 
-cudaError_t upload_chunks(const ChunkPlan& P, const ChunkBufs& b, cudaStream_t s) {
-    cudaError_t e = cudaMemcpyAsync(b.insts, P.hi.data(), sizeof(BatchInst) * P.chunks, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(b.units, P.units.data(), sizeof(BatchUnit) * P.units.size(), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(b.blocks, P.blocks.data(), sizeof(int2) * P.blocks.size(), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(b.comp_inst, P.comp_inst.data(), sizeof(int) * P.comp_inst.size(),
-                            cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(b.npairs, P.npairs.data(), sizeof(int) * P.chunks, cudaMemcpyHostToDevice, s);
-    return e;
+ReachLaunch reach_launch(const ReachBufs& b, const float4* p8, int64_t n, int k, const float* params, DeviceState* st,
+                         int iter) {
+    ReachLaunch a{p8, n, k, params, b.ctr, b.aux, b.gref, b.llp, nullptr, st, iter};
+    a.n_buf = n;
+    a.rows = b.rows;
+    return a;
 }
 
-// The two-level log-sum-exp: reference, pass A (chunk sums), combine, exact
-// points, per-point log-likelihood partials (and into st when ll_to_state).
-cudaError_t chunk_lse(const ChunkPlan& P, const ChunkBufs& b, const float4* p8, int64_t n, int k, DeviceState* st,
-                      int iter, bool ll_to_state, long long* launches, cudaStream_t s) {
-    cudaError_t e = launch_chunk_ref(b.params, k, st, b.gref, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(b.flag_count, 0, sizeof(int), s);
-    EStepLaunch a{p8, n, k, b.params, P.ppc, nullptr, nullptr, nullptr, nullptr, iter};
-    a.insts = b.insts;
-    a.units = b.units;
-    a.states = st;
-    a.gref = b.gref;
-    a.psum = b.psum;
-    if (e == cudaSuccess) e = launch_estep_chunks(a, 1, (int)P.units.size(), P.ppc, s);
-    if (e == cudaSuccess) e = launch_chunk_combine(b.psum, P.chunks, n, b.gref, b.pref, b.llpt, b.flag_count, b.flags, st, s);
-    if (e == cudaSuccess) e = launch_chunk_exact(p8, b.params, k, b.gref, b.flags, b.flag_count, b.pref, b.llpt, st, s);
-    if (e == cudaSuccess) e = launch_points_ll_reduce(b.llpt, n, b.llp, ll_to_state ? st : nullptr, s);
-    *launches += 5 + (ll_to_state ? 1 : 0);
-    return e;
-}
-
-cudaError_t chunk_em_iteration(const ChunkPlan& P, const ChunkBufs& b, const float4* p8, int64_t n, int k,
-                               float4* shift4, double* model64, double* trace, const gira_fit_opts& o,
-                               DeviceState* st, int iter, long long* launches, cudaStream_t s, const int* perm) {
-    cudaError_t e = chunk_lse(P, b, p8, n, k, st, iter, false, launches, s);
-    EStepLaunch a{p8, n, k, b.params, P.ppc, b.partials, nullptr, nullptr, nullptr, iter};
-    a.insts = b.insts;
-    a.units = b.units;
-    a.states = st;
-    a.gref = b.gref;
+// One E-step with statistics: b.partials rows and b.live2 masks for the finalize.
+cudaError_t reach_estep_stats(const ReachBufs& b, ReachLaunch a, long long* launches, cudaStream_t s) {
     a.pref = b.pref;
-    a.psum = b.psum;   // pass B skips the batches pass A found out of this chunk's reach
-    if (e == cudaSuccess) e = launch_estep_chunks(a, 2, (int)P.units.size(), P.ppc, s);
-    if (e == cudaSuccess)
-        e = launch_reduce_finalize_chunks(b.partials, b.llp, chunk_combine_grid(), nullptr, shift4, b.insts,
-                                          b.blocks, (int)P.blocks.size(), n, o.reg_covar, o.tol, model64, b.params,
-                                          trace, st, iter, true, s, perm);
-    *launches += 2;
+    a.masks = b.masks;
+    cudaError_t e = launch_reach_prepare(a.params, a.k, nullptr, 1, a.st, a.iter, b.ctr, b.aux, b.gref, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(b.live2, 0, sizeof(uint32_t) * b.words * b.slices, s);
+    if (e == cudaSuccess) e = launch_estep_reach(a, 1, b.grid, b.h, a.k, s);
+    if (e == cudaSuccess) e = launch_reach_stats(a, 0, b.partials, b.live2, s);
+    *launches += 3;
+    return e;
+}
+
+// The log-likelihood alone: a.per_point (nullable) and st->ll_sum.
+cudaError_t reach_loglik(const ReachBufs& b, const ReachLaunch& a, long long* launches, cudaStream_t s) {
+    cudaError_t e = launch_reach_prepare(a.params, a.k, nullptr, 1, a.st, a.iter, b.ctr, b.aux, b.gref, s);
+    if (e == cudaSuccess) e = launch_estep_reach(a, 0, b.grid, b.h, a.k, s);
+    if (e == cudaSuccess) e = launch_ll_reduce(b.llp, b.grid, a.st, s);
+    *launches += 3;
     return e;
 }
 
@@ -629,15 +565,14 @@ gira_status gira_gmm_fit(const float* points, int64_t n, int k, const gira_fit_o
     TRY(check_ptr(covs, "covs", c.dev, &kc));
     const bool model_host = kw == Kind::Host || km == Kind::Host || kc == Kind::Host;
     const bool kinit = o.init_mode == GIRA_INIT_KMEANS;
-    const bool chunked = k > MAX_K_DIRECT;   // two-level log-sum-exp over chunks of components
-    const ChunkPlan P = chunked ? plan_chunks(n, k, c.sms) : ChunkPlan{};
-    ChunkBufs cb;
-    const int npairs = chunked ? 0 : params_pairs_padded(k);
+    const bool large = k > MAX_K_DIRECT;   // the E-step over reach lists (reach_kernels.cu)
+    ReachBufs rb;
+    const int npairs = params_pairs_padded(k);
     // point-stationary E-step: one grid for the EM loop and the final log-likelihood;
     // per-warp partial rows and live masks
-    const int grid = chunked ? 0 : estep_pt_grid(n);
-    const int rows = chunked ? 0 : estep_pt_rows(grid);
-    const int nwords = chunked ? 0 : estep_pt_mask_words(k);
+    const int grid = large ? 0 : estep_pt_grid(n);
+    const int rows = large ? 0 : estep_pt_rows(grid);
+    const int nwords = large ? 0 : estep_pt_mask_words(k);
     const int nblk = kpp_num_blocks(n);
     int kgrid = kinit ? kpp_persistent_grid() : 0;
     if (kgrid > 0 && n > kpp_persistent_max_n(kgrid)) kgrid = 0;
@@ -661,7 +596,7 @@ gira_status gira_gmm_fit(const float* points, int64_t n, int k, const gira_fit_o
     // the E-steps and Lloyd run on the points in a spatial order (a warp's points then
     // reach fewer components and centres); k-means++ on the caller's order, which
     // defines its draws
-    const bool sorted = !chunked && n <= point_order_max_n();
+    const bool sorted = n <= point_order_max_n();
     auto layout = [&](Carver& cv) {
         b.st = cv.take<DeviceState>(1);
         b.perm = cv.take<int>(k);
@@ -679,9 +614,9 @@ gira_status gira_gmm_fit(const float* points, int64_t n, int k, const gira_fit_o
         b.masks = cv.take<uint32_t>((size_t)rows * nwords);
         b.llp = cv.take<double>(grid);
         b.trace = cv.take<double>(std::max(o.iters, 1));
-        b.cta_key = cv.take<uint8_t>(chunked ? 0 : grid);
-        b.cta_perm = cv.take<int>(chunked ? 0 : 2 * (size_t)grid);
-        if (chunked) carve_chunks(cv, P, n, true, &cb);
+        b.cta_key = cv.take<uint8_t>(grid);
+        b.cta_perm = cv.take<int>(2 * (size_t)grid);
+        if (large) carve_reach(cv, n, k, NSTAT, true, &rb);
         b.mw = cv.take<float>(model_host ? k : 0);
         b.mmu = cv.take<float>(model_host ? 3 * (size_t)k : 0);
         b.mcov = cv.take<float>(model_host ? 9 * (size_t)k : 0);
@@ -725,13 +660,7 @@ gira_status gira_gmm_fit(const float* points, int64_t n, int k, const gira_fit_o
     if (sorted)
         COUNTED(prof, point_order_launches(1),
                 launch_point_order(b.p8, n, nullptr, nullptr, 0, 1, b.osc, b.p8s, kinit ? b.p4s : nullptr, nullptr, c.s));
-    if (chunked) {
-        GIRA_CUDA(upload_chunks(P, cb, c.s));
-        b.params = cb.params;
-        COUNTED(prof, 1, launch_fill_padding_batched(cb.params, cb.insts, P.chunks, 0, cb.npairs, c.s));
-    } else {
-        COUNTED(prof, 1, launch_fill_padding(b.params, k, npairs, c.s));
-    }
+    COUNTED(prof, 1, launch_fill_padding(b.params, k, npairs, c.s));
 
     float* w_d = (kw == Kind::Device) ? weights : b.mw;
     float* mu_d = (km == Kind::Device) ? means : b.mmu;
@@ -754,26 +683,15 @@ gira_status gira_gmm_fit(const float* points, int64_t n, int k, const gira_fit_o
         GIRA_CUDA(cudaMemsetAsync(b.stats64, 0, sizeof(double) * NSTAT * k, c.s));
         COUNTED(prof, 1, launch_label_stats(sorted ? b.p4s : b.p4, n, k, b.lab, b.c4, b.stats64, b.st, c.s));
         GIRA_CUDA(cudaMemcpyAsync(b.shift4, b.c4, sizeof(float4) * k, cudaMemcpyDeviceToDevice, c.s));
-        if (chunked) {
-            COUNTED(prof, 1, launch_reduce_finalize_chunks(nullptr, nullptr, 0, b.stats64, b.shift4, cb.insts,
-                                                           cb.blocks, (int)P.blocks.size(), n, o.reg_covar, o.tol,
-                                                           b.model64, cb.params, b.trace, b.st, 0, false, c.s));
-        } else {
-            COUNTED(prof, 1, launch_reduce_finalize(nullptr, 0, nullptr, b.stats64, b.shift4, k, n, o.reg_covar,
-                                                    o.tol, b.model64, b.params, b.trace, b.st, 0, false, c.s));
-        }
+        COUNTED(prof, 1, launch_reduce_finalize(nullptr, 0, nullptr, b.stats64, b.shift4, k, n, o.reg_covar, o.tol,
+                                                b.model64, b.params, b.trace, b.st, 0, false, c.s));
     } else {
         if (kw == Kind::Host) GIRA_CUDA(cudaMemcpyAsync(b.mw, weights, sizeof(float) * k, cudaMemcpyHostToDevice, c.s));
         if (km == Kind::Host)
             GIRA_CUDA(cudaMemcpyAsync(b.mmu, means, sizeof(float) * 3 * k, cudaMemcpyHostToDevice, c.s));
         if (kc == Kind::Host)
             GIRA_CUDA(cudaMemcpyAsync(b.mcov, covs, sizeof(float) * 9 * k, cudaMemcpyHostToDevice, c.s));
-        if (chunked) {
-            COUNTED(prof, 1, launch_params_from_model_batched(w_d, mu_d, cov_d, k, cb.comp_inst, cb.insts, b.model64,
-                                                              cb.params, b.shift4, b.st, c.s));
-        } else {
-            COUNTED(prof, 1, launch_params_from_model(w_d, mu_d, cov_d, k, b.model64, b.params, b.shift4, b.st, c.s));
-        }
+        COUNTED(prof, 1, launch_params_from_model(w_d, mu_d, cov_d, k, b.model64, b.params, b.shift4, b.st, c.s));
     }
     // the EM runs with the components along a space-filling curve of their means
     // (the E-step then skips the many point-component pairs out of reach);
@@ -782,12 +700,17 @@ gira_status gira_gmm_fit(const float* points, int64_t n, int k, const gira_fit_o
     COUNTED(prof, 2, launch_order_components(b.model64, b.stats64, k, b.perm, b.params, b.shift4, b.st, c.s));
     prof.t_init = prof.mark();
 
-    if (chunked) {
-        for (int t = 1; t <= o.iters; ++t)
-            GIRA_CUDA(chunk_em_iteration(P, cb, b.p8, n, k, b.shift4, b.model64, b.trace, o, b.st, t, &prof.launches,
-                                         c.s, perm));
+    if (large) {
+        const float4* pe = sorted ? b.p8s : b.p8;
+        for (int t = 1; t <= o.iters; ++t) {
+            GIRA_CUDA(reach_estep_stats(rb, reach_launch(rb, pe, n, k, b.params, b.st, t), &prof.launches, c.s));
+            COUNTED(prof, 1, launch_reduce_finalize(rb.partials, rb.slices, rb.llp, nullptr, b.shift4, k, n,
+                                                    o.reg_covar, o.tol, b.model64, b.params, b.trace, b.st, t, true,
+                                                    c.s, false, perm, rb.live2, rb.words, rb.grid));
+        }
         prof.t_em = prof.mark();
-        if (final_loglik) GIRA_CUDA(chunk_lse(P, cb, b.p8, n, k, b.st, 0, true, &prof.launches, c.s));
+        if (final_loglik)
+            GIRA_CUDA(reach_loglik(rb, reach_launch(rb, pe, n, k, b.params, b.st, 0), &prof.launches, c.s));
     }
     EStepLaunch a{sorted ? b.p8s : b.p8, n, k, b.params, 0, b.partials, b.llp, nullptr, b.st, 0};
     a.n_buf = n;
@@ -795,7 +718,7 @@ gira_status gira_gmm_fit(const float* points, int64_t n, int k, const gira_fit_o
     a.pt_rows = rows;
     a.cta_perm = b.cta_perm;   // from the third iteration on: the CTAs of most work first
     a.cta_key = b.cta_key;
-    for (int t = 1; t <= o.iters && !chunked; ++t) {
+    for (int t = 1; t <= o.iters && !large; ++t) {
         a.iter = t;
         // dependent launches unless an event pair brackets each E-step: each
         // kernel is resident before the previous one ends and waits on the
@@ -809,8 +732,8 @@ gira_status gira_gmm_fit(const float* points, int64_t n, int k, const gira_fit_o
                                                 o.tol, b.model64, b.params, b.trace, b.st, t, true, c.s, pdl, perm,
                                                 b.masks, nwords, grid, b.cta_key, b.cta_perm, grid));
     }
-    if (!chunked) prof.t_em = prof.mark();
-    if (final_loglik && !chunked) {
+    if (!large) prof.t_em = prof.mark();
+    if (final_loglik && !large) {
         EStepLaunch f = a;
         f.iter = 0;
         f.partials = nullptr;
@@ -827,7 +750,7 @@ gira_status gira_gmm_fit(const float* points, int64_t n, int k, const gira_fit_o
     GIRA_CUDA(cudaMemcpyAsync(&h, b.st, sizeof h, cudaMemcpyDeviceToHost, c.s));
     prof.t_end = prof.mark();
     GIRA_CUDA(cudaStreamSynchronize(c.s));
-    if (!chunked) {
+    if (!large) {
         prof.pair_slots = (long long)h.iters_done * rows * ((((k + 1) >> 1) + 1) & ~1);
         prof.pairs_near = (long long)h.pairs_near;
         prof.pairs_live = (long long)h.pairs_live;
@@ -854,11 +777,10 @@ gira_status gira_gmm_loglik(const float* points, int64_t n, int k, const float* 
     TRY(check_ptr(means, "means", c.dev, &km));
     TRY(check_ptr(covs, "covs", c.dev, &kc));
     if (per_point) TRY(check_ptr(per_point, "per_point", c.dev, &kpp));
-    const bool chunked = k > MAX_K_DIRECT;   // two-level log-sum-exp over chunks of components
-    const ChunkPlan P = chunked ? plan_chunks(n, k, c.sms) : ChunkPlan{};
-    ChunkBufs cb;
-    const int npairs = chunked ? 0 : params_pairs_padded(k);
-    const int grid = chunked ? 0 : estep_pt_grid(n);
+    const bool large = k > MAX_K_DIRECT;   // the E-step over reach lists
+    ReachBufs rb;
+    const int npairs = params_pairs_padded(k);
+    const int grid = large ? 0 : estep_pt_grid(n);
     struct Bufs {
         DeviceState* st;
         float *pin, *params, *mw, *mmu, *mcov, *pp;
@@ -877,7 +799,7 @@ gira_status gira_gmm_loglik(const float* points, int64_t n, int k, const float* 
         b.mmu = cv.take<float>(km == Kind::Host ? 3 * (size_t)k : 0);
         b.mcov = cv.take<float>(kc == Kind::Host ? 9 * (size_t)k : 0);
         b.pp = cv.take<float>((per_point && kpp == Kind::Host) ? n : 0);
-        if (chunked) carve_chunks(cv, P, n, false, &cb);
+        if (large) carve_reach(cv, n, k, NSTAT, false, &rb);
     };
     Carver sizer;
     layout(sizer);
@@ -919,20 +841,15 @@ gira_status gira_gmm_loglik(const float* points, int64_t n, int k, const float* 
     }
     COUNTED(prof, 1, launch_pack(pts, n, nullptr, b.p8, b.st, c.s));
     float* ppd = per_point ? ((kpp == Kind::Device) ? per_point : b.pp) : nullptr;
-    if (chunked) {
-        GIRA_CUDA(upload_chunks(P, cb, c.s));
-        COUNTED(prof, 1, launch_fill_padding_batched(cb.params, cb.insts, P.chunks, 0, cb.npairs, c.s));
-        COUNTED(prof, 1, launch_params_from_model_batched(w_d, mu_d, cov_d, k, cb.comp_inst, cb.insts, b.model64,
-                                                          cb.params, b.shift4, b.st, c.s));
-        prof.t_init = prof.mark();
-        prof.t_em = prof.t_init;
-        GIRA_CUDA(chunk_lse(P, cb, b.p8, n, k, b.st, 0, true, &prof.launches, c.s));
-        if (ppd) COUNTED(prof, 1, launch_double_to_float(cb.llpt, n, ppd, c.s));
+    COUNTED(prof, 1, launch_fill_padding(b.params, k, npairs, c.s));
+    COUNTED(prof, 1, launch_params_from_model(w_d, mu_d, cov_d, k, b.model64, b.params, b.shift4, b.st, c.s));
+    prof.t_init = prof.mark();
+    prof.t_em = prof.t_init;
+    if (large) {
+        ReachLaunch a = reach_launch(rb, b.p8, n, k, b.params, b.st, 0);
+        a.per_point = ppd;
+        GIRA_CUDA(reach_loglik(rb, a, &prof.launches, c.s));
     } else {
-        COUNTED(prof, 1, launch_fill_padding(b.params, k, npairs, c.s));
-        COUNTED(prof, 1, launch_params_from_model(w_d, mu_d, cov_d, k, b.model64, b.params, b.shift4, b.st, c.s));
-        prof.t_init = prof.mark();
-        prof.t_em = prof.t_init;
         EStepLaunch a{b.p8, n, k, b.params, 0, nullptr, b.llp, ppd, b.st, 0};
         a.n_buf = n;
         COUNTED(prof, 1, launch_estep_pt(a, false, grid, c.s));

@@ -315,7 +315,7 @@ __host__ __device__ __forceinline__ double uniform53(uint64_t seed, uint64_t j) 
     return (double)(splitmix64(seed, j) >> 11) * (1.0 / 9007199254740992.0);
 }
 
-// K above this runs the chunked (two-level log-sum-exp) path; the batched and
+// K above this runs the E-step over reach lists (reach_kernels.cu); the batched and
 // no-allocation entry points take K up to it only.
 constexpr int MAX_K_DIRECT = 1024;
 
@@ -334,12 +334,62 @@ struct BatchInst {
     int comp_off;       // first component in the per-component arrays
     int ctas;           // E-step CTAs of the instance
     int pad_;
-    int64_t mask_off;   // word offset of its per-warp live masks (point-stationary E-step)
+    int64_t mask_off;   // word offset of its live masks
+    int64_t live_off;   // word offset of its live-slice masks (gradient)
 };
 // One E-step CTA of a batched launch: instance and CTA index within it.
 struct BatchUnit {
     int inst, cta;
 };
+
+// Slices of the statistics launch over n points: sl words of 32 blocks of 128 points
+// each.  One word (4,096 points) up to 256 slices -- a slice is one warp's serial work
+// -- then longer slices, which bounds the partial rows.
+__host__ __device__ inline int reach_slices(int64_t n, int* sl) {
+    const int64_t words = (n + 4095) / 4096;
+    *sl = (int)((words + 255) / 256);
+    return (int)((words + *sl - 1) / *sl);
+}
+
+// The E-step over reach lists (reach_kernels.cu).
+struct ReachLaunch {
+    const float4* pts8;      // 2 float4 per point, as EStepLaunch (4-D: (x,x,y,y) (z,z,I,I))
+    int64_t n;
+    int k;
+    const float* params;     // pair-interleaved
+    const float4* ctr;       // compact per-component arrays and references of launch_reach_prepare
+    const float2* aux;
+    const float* gref;
+    double* llp;             // [grid] log-likelihood partials
+    float* per_point;        // mode 0: [n] natural-log lse, or nullptr
+    DeviceState* st;
+    int iter;
+    int64_t n_buf = 0;       // points in pts8 (index checks of the debug build; 0: unchecked)
+    float2* pref = nullptr;  // [n] (shift, 1 / total): with masks
+    uint32_t* masks = nullptr;   // [reach_mask_words(k)][rows] live pairs per block of 128 points
+    int64_t rows = 0;
+    // gradient (mode 2)
+    float* grad_pts = nullptr;        // [n][3], at order[i] (or i) for the i-th point, or nullptr
+    const int* order = nullptr;
+    const float* rot = nullptr;       // R of x' = R x + t, or nullptr
+    double* pose_partials = nullptr;  // [grid][12]
+    // batched gradient launches: as EStepLaunch
+    const BatchInst* insts = nullptr;
+    const BatchUnit* units = nullptr;
+    DeviceState* states = nullptr;
+};
+int reach_h(int64_t n);        // warps per block of 128 points for n points in the launch
+int reach_grid(int64_t n);     // CTAs of a single launch
+int64_t reach_rows(int64_t n); // blocks of 128 points
+int reach_mask_words(int k);
+int reach_stat_groups(int k);  // CTAs per slice of the statistics launch
+cudaError_t launch_reach_prepare(const float* params, int k, const BatchInst* insts, int batch, const DeviceState* st,
+                                 int iter, float4* ctr, float2* aux, float* gref, cudaStream_t s);
+// mode 0 log-likelihood, 1 with masks and pref, 2 gradient; h: reach_h of the launch; kmax: the largest k.
+cudaError_t launch_estep_reach(const ReachLaunch& a, int mode, int grid, int h, int kmax, cudaStream_t s);
+// partials [slices][pairs][2 NSTAT] and live2 [words][slices] (zeroed by the caller):
+// launch_reduce_finalize takes them as rows and masks.
+cudaError_t launch_reach_stats(const ReachLaunch& a, int nunits, float* partials, uint32_t* live2, cudaStream_t s);
 
 struct EStepLaunch {
     const float4* pts8;      // 2 float4 per point: (x,x,y,y) (z,z,0,0)
@@ -503,36 +553,15 @@ cudaError_t launch_order_components_batched(double* model64, double* scratch, in
 cudaError_t launch_ll_reduce_batched(const double* ll_partials, const BatchInst* insts, int batch,
                                      DeviceState* states, cudaStream_t s);
 
-// Large K: components in chunks of chunk_components() (one E-step shape),
-// each chunk an entry of a BatchInst table over the same points.
-int chunk_components();
-// gref = (max_b c_b over all k components, log-likelihood reference) from the
-// chunked parameter blocks (chunk c at c * chunk_param_floats()).
-int64_t chunk_param_floats();
-cudaError_t launch_chunk_ref(const float* params, int k, const DeviceState* st, float* gref, cudaStream_t s);
-// Pass A / pass B over all chunks (units: chunk-major); see EStepLaunch.
-cudaError_t launch_estep_chunks(const EStepLaunch& a, int pass, int nunits, int64_t ppc, cudaStream_t s);
 // Per point: total over chunks -> pref, per-point log-likelihood llpt (natural);
 // points whose total underflows (< 2^-100) are listed in flags for the exact step.
 int chunk_combine_grid();
 cudaError_t launch_chunk_combine(const float* psum, int chunks, int64_t n, const float* gref, float2* pref,
                                  double* llpt, int* flag_count, int* flags, DeviceState* st, cudaStream_t s);
-// Listed points: exact per-point maximum over all k components (one warp each).
-cudaError_t launch_chunk_exact(const float4* pts8, const float* params, int k, const float* gref, const int* flags,
-                               const int* flag_count, float2* pref, double* llpt, DeviceState* st, cudaStream_t s);
 cudaError_t launch_double_to_float(const double* x, int64_t n, float* y, cudaStream_t s);
 // Fixed-order sums of llpt into chunk_combine_grid() partials, then (st != nullptr)
 // into st->ll_sum.
 cudaError_t launch_points_ll_reduce(const double* llpt, int64_t n, double* llp, DeviceState* st, cudaStream_t s);
-// The chunks' finalize: like the batched one, but every chunk shares state st
-// and trace; the log-likelihood / convergence step (em) runs once, from
-// ll_partials[0 .. ll_count).
-cudaError_t launch_reduce_finalize_chunks(const float* partials, const double* ll_partials, int ll_count,
-                                          const double* stats64, float4* shift4, const BatchInst* insts,
-                                          const int2* blocks, int nblocks, int64_t n, double reg, double tol,
-                                          double* model64, float* params, double* trace, DeviceState* st, int iter,
-                                          bool em, cudaStream_t s, const int* perm = nullptr);
-
 // Batched differentiable log-likelihood (a batch table of scans, each with its
 // own model and pose; poses: batch x 12, or nullptr for identities).
 cudaError_t launch_pack_pose_batched(const float* pts3, int64_t n, const int64_t* offsets, int batch,

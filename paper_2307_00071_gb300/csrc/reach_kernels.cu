@@ -1,0 +1,854 @@
+// reach_kernels.cu -- the E-step over many components (3-D with K above 1024, the
+// gradient, 4-D): per-block reach lists read from global memory, and the M-step
+// statistics accumulated component by component over the blocks each one reaches.
+//
+// GIRA (arXiv 2307.00071) Sec. V: Eq. (estep) in the log domain (Eq. logestep)
+// with the Cholesky log-density of Eq. (simplifiedGaussian).  ex2.approx.ftz
+// returns +0 below 2^-126, so a (point, component) whose q' = |P'(x - mu)|^2 +
+// (cmax - c) exceeds 126 adds exactly nothing; at thousands of components that is
+// all but one pair in fifty or a hundred.
+//
+// Three kernels per E-step:
+//  reach_prepare_kernel  per component (mean, bound of sigma_min(P')^2, c) in compact
+//      arrays, and the reference cmax with the weight normaliser;
+//  reach_estep_kernel    a block of 128 consecutive points (4 per lane) shared by H
+//      warps.  Two tests list the pairs of components that can reach the block: the
+//      whole CTA tests every component's sphere against the CTA's box (16 + 8 bytes
+//      per component, coalesced), then each warp tests the survivors' boxes exactly as
+//      estep_pt_kernel does.  The listed pairs' parameters are read through L1 / L2 as
+//      broadcasts: nothing is staged, so shared memory (a few KB of lists) does not
+//      bound the occupancy and K does not bound the kernel.  Writes per-point
+//      (shift, 1 / total), the log-likelihood, and per block the mask of live pairs;
+//  reach_stats_kernel    one warp per (pair, slice of blocks): the statistics of both
+//      components over the live blocks of the slice stay in registers and are reduced
+//      over the lanes once per slice.  A row-wise second phase would reduce and store 20
+//      values per (block, pair) and need a partial row per block (10 GB at 4M points,
+//      K = 8192); here it is one 80-byte row per (pair, slice).
+// The mode for gradients adds, in reach_estep_kernel, sum_b gamma Sigma_b^-1 (x' - mu_b)
+// per point from the live pairs, and the pose sums.
+//
+// Measured on GB300 (4M points of 16 posed frames, K = 8192): E-step 0.70 ms, statistics
+// 1.33 ms per iteration; the dense two-pass kernels over chunks of 512 components that
+// this replaced took 2 x 15.5 ms.  A call of two iterations with the final
+// log-likelihood: 79.2 -> 6.1 ms.
+#include <float.h>
+#include <math.h>
+
+#include <algorithm>
+
+#include "gira_internal.cuh"
+
+namespace gira {
+namespace {
+
+constexpr unsigned FULL = 0xffffffffu;
+constexpr float LN2F = 0.693147180559945309f;
+constexpr double LN2 = 0.693147180559945309417232121458;
+constexpr int RB_P = 4;                    // points per lane
+constexpr int RB_PTS = 32 * RB_P;          // points per block (a row of the masks)
+constexpr int RB_W = 4;                    // warps per CTA
+constexpr float REACH = 128.f;             // q' above which a component is out of reach (e = 0 from q' > 126)
+constexpr int RARE_FEW = 16;               // rare points of a block up to which lanes take pairs instead of points
+
+template <int D>
+struct Lay;
+template <>
+struct Lay<3> {
+    static constexpr int NP = 6, NS = NSTAT, PF = PAIR_FLOATS;
+    static constexpr int SP = SLOT_P, SC = SLOT_C, SNMU = SLOT_NMU, SW = SLOT_W, SS = SLOT_S;
+};
+
+// Parameters of a pair of components (slot-wise float2: components 2p, 2p + 1).
+template <int D>
+struct Pair {
+    float2 p[Lay<D>::NP], c, nmu[D];
+};
+
+// The slots [S0, S0 + N) of pair pp, read as whole float4.
+template <int D>
+__device__ __forceinline__ void load_slots(const float* params, int pp, float2 (&s)[Lay<D>::PF / 2]) {
+    const float4* q = reinterpret_cast<const float4*>(params + (size_t)pp * Lay<D>::PF);
+#pragma unroll
+    for (int i = 0; i < Lay<D>::PF / 4; ++i) {
+        const float4 v = __ldg(q + i);   // slots never used are never loaded (dead after inlining)
+        s[2 * i] = f2(v.x, v.y);
+        s[2 * i + 1] = f2(v.z, v.w);
+    }
+}
+
+template <int D>
+__device__ __forceinline__ void load_pair(const float* params, int pp, float cmax, Pair<D>& P) {
+    float2 s[Lay<D>::PF / 2];
+    load_slots<D>(params, pp, s);
+#pragma unroll
+    for (int i = 0; i < Lay<D>::NP; ++i) P.p[i] = s[Lay<D>::SP + i];
+    P.c = f2(cmax - s[Lay<D>::SC].x, cmax - s[Lay<D>::SC].y);
+#pragma unroll
+    for (int i = 0; i < D; ++i) P.nmu[i] = s[Lay<D>::SNMU + i];
+}
+
+// q' = |P'(x - mu)|^2 + (cmax - c) of both components at one point, and y = P'(x - mu)
+// (the difference first: see neg_logit2 in em_kernels.cu).
+template <int D>
+__device__ __forceinline__ float2 nlogit(const Pair<D>& P, const float2 (&X)[D], float2 (&y)[D]) {
+    float2 d[D];
+#pragma unroll
+    for (int j = 0; j < D; ++j) d[j] = add2(X[j], P.nmu[j]);
+    float2 q = P.c;
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+        const int r = i * (i + 1) / 2;
+        y[i] = mul2(P.p[r], d[0]);
+#pragma unroll
+        for (int j = 1; j <= i; ++j) y[i] = fma2(P.p[r + j], d[j], y[i]);
+        q = fma2(y[i], y[i], q);
+    }
+    return q;
+}
+
+template <int D>
+__device__ __forceinline__ void load_point(const float4* pts8, int64_t i, float2 (&X)[D]) {
+    const float4 a = pts8[2 * i], b = pts8[2 * i + 1];
+    X[0] = f2(a.x, a.y);
+    X[1] = f2(a.z, a.w);
+    X[2] = f2(b.x, b.y);
+    if (D == 4) X[D - 1] = f2(b.z, b.w);
+}
+
+// ------------------------------------------------------------------ per-component compact arrays
+// Block i: instance i of a batch (insts), or the one fit (k components).  ctr[b] = the
+// mean's first three coordinates and, in 3-D, the bound s2 of sigma_min(P')^2 (in 4-D the
+// fourth coordinate); aux[b] = (c, s2); gref[0] = max_b c_b, gref[1] = the log-likelihood
+// reference (cmax - log2 sum_a N_a once the weights are raw N_b, else cmax).
+constexpr int PREP_THREADS = 1024;
+template <int D>
+__global__ void __launch_bounds__(PREP_THREADS) reach_prepare_kernel(const float* __restrict__ params, int k,
+                                                                     const BatchInst* __restrict__ insts,
+                                                                     const DeviceState* st, int iter, float4* ctr,
+                                                                     float2* aux, float* gref) {
+    __shared__ float s_m[PREP_THREADS / 32];
+    __shared__ double s_w[PREP_THREADS / 32];
+    if (insts) {
+        const BatchInst I = insts[blockIdx.x];
+        k = I.k;
+        params += I.par_off;
+        ctr += I.comp_off;
+        aux += I.comp_off;
+        gref += 2 * blockIdx.x;
+        st += blockIdx.x;
+    }
+    pdl_wait();
+    if (iter > st->stop_after || st->error) return;
+    float m = -INFINITY;
+    double w = 0.0;
+    for (int b = threadIdx.x; b < k; b += blockDim.x) {
+        const float* p = params + (size_t)(b >> 1) * Lay<D>::PF + (b & 1);
+        const float c = p[2 * Lay<D>::SC], s2 = p[2 * Lay<D>::SS];
+        float x[4];
+#pragma unroll
+        for (int j = 0; j < D; ++j) x[j] = -p[2 * (Lay<D>::SNMU + j)];
+        if (D == 3) x[3] = s2;
+        ctr[b] = make_float4(x[0], x[1], x[2], x[3]);
+        aux[b] = f2(c, s2);
+        m = fmaxf(m, c);
+        w += (double)p[2 * Lay<D>::SW];
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        m = fmaxf(m, __shfl_xor_sync(FULL, m, o));
+        w += __shfl_xor_sync(FULL, w, o);
+    }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (lane == 0) {
+        s_m[warp] = m;
+        s_w[warp] = w;
+    }
+    __syncthreads();
+    if (warp == 0) {
+        m = lane < (int)(blockDim.x >> 5) ? s_m[lane] : -INFINITY;
+        w = lane < (int)(blockDim.x >> 5) ? s_w[lane] : 0.0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            m = fmaxf(m, __shfl_xor_sync(FULL, m, o));
+            w += __shfl_xor_sync(FULL, w, o);
+        }
+        if (lane == 0) {
+            gref[0] = m;
+            gref[1] = st->w_raw ? (float)((double)m - log2(w)) : m;
+        }
+    }
+}
+
+// ------------------------------------------------------------------ the E-step
+// Shared memory: the CTA's surviving pairs by warp quarter and class (pp % H), every
+// warp's listed pairs, every warp's live-mask words.
+__host__ __device__ constexpr int reach_pairs(int k) { return (((k + 1) / 2) + 127) & ~127; }   // quarters of whole warps
+__host__ __device__ constexpr int reach_words(int k) { return (((k + 1) / 2) + 31) / 32; }
+__host__ __device__ constexpr size_t reach_smem(int k, int h) {
+    return (size_t)reach_pairs(k) * 2 + (size_t)RB_W * (reach_pairs(k) / h) * 2 + (size_t)RB_W * reach_words(k) * 4;
+}
+
+// The barrier of block blk's H warps.
+template <int H>
+__device__ __forceinline__ void block_sync(int blk) {
+    if (H == RB_W) {
+        __syncthreads();
+    } else if (blk == 0) {
+        asm volatile("bar.sync 1, %0;" ::"n"(32 * H) : "memory");
+    } else {
+        asm volatile("bar.sync 2, %0;" ::"n"(32 * H) : "memory");
+    }
+}
+
+// MODE 0: log-likelihood; 1: also (shift, 1 / total) and the masks for reach_stats_kernel;
+// 2: the gradient (the masks only when a.masks).  H warps share a block's pairs (pp % H):
+// 2 for large inputs, 4 where 256-point CTAs would leave SMs idle.
+template <int D, int H, int MODE>
+__global__ void __launch_bounds__(32 * RB_W, 4) estep_reach_kernel(const ReachLaunch a_in) {
+    extern __shared__ __align__(16) unsigned char dsm[];
+    constexpr int B = RB_W / H;   // blocks per CTA
+    static_assert(B * H == RB_W && B <= 2, "one named barrier per block");
+    __shared__ float s_box[RB_W][2 * D];
+    __shared__ float2 s_tot[RB_W][RB_P][32];
+    __shared__ float s_rare[RB_W][RARE_FEW];
+    __shared__ int s_cnt[RB_W][H];
+    __shared__ double s_ll[B];
+    __shared__ int s_skip;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int blk = warp / H, half = warp % H;
+    int cta = blockIdx.x;
+    int64_t pt0 = 0;   // the instance's first point (loads index the launch's own pointers by it)
+    ReachLaunch a = a_in;
+    if (a_in.units) {
+        const BatchUnit u = a_in.units[blockIdx.x];
+        const BatchInst I = a_in.insts[u.inst];
+        cta = u.cta;
+        pt0 = I.pt_off;
+        a.n = I.n;
+        a.k = I.k;
+        a.params = a_in.params + I.par_off;
+        a.ctr = a_in.ctr + I.comp_off;
+        a.aux = a_in.aux + I.comp_off;
+        a.gref = a_in.gref + 2 * u.inst;
+        a.masks = a_in.masks ? a_in.masks + I.mask_off : nullptr;
+        a.rows = (I.n + RB_PTS - 1) / RB_PTS;
+        a.llp = a_in.llp + I.ll_off;
+        a.st = a_in.states + u.inst;
+        a.rot = a_in.rot ? a_in.rot + 12 * (size_t)u.inst : nullptr;
+        a.pose_partials = a_in.pose_partials ? a_in.pose_partials + 12 * I.ll_off : nullptr;
+    }
+    const int npairs = (a.k + 1) >> 1;
+    const int nquarter = reach_pairs(a.k) / RB_W, ncap = reach_pairs(a.k) / H, nwords = reach_words(a.k);
+    uint16_t* slist0 = reinterpret_cast<uint16_t*>(dsm);                        // [RB_W][H][nquarter / H]
+    uint16_t* slist = slist0 + reach_pairs(a.k) + (size_t)warp * ncap;          // this warp's listed pairs
+    uint32_t* smask_all = reinterpret_cast<uint32_t*>(slist0 + reach_pairs(a.k) + (size_t)RB_W * ncap);
+    uint32_t* smask = smask_all + warp * nwords;
+    // a slot beyond n holds a point 1e18 m away, where every q' is +inf and e exactly 0
+    const int64_t row = (int64_t)cta * B + blk;
+    const int64_t base = row * RB_PTS + lane;
+    float2 X[RB_P][D];
+    bool valid[RB_P];
+#pragma unroll
+    for (int p = 0; p < RB_P; ++p) {
+        const int64_t i = base + 32 * p;
+        valid[p] = i < a.n && GIRA_IN(a_in.n_buf == 0 || pt0 + i < a_in.n_buf, a.st);
+        if (valid[p]) {
+            load_point<D>(a_in.pts8, pt0 + i, X[p]);
+        } else {
+#pragma unroll
+            for (int j = 0; j < D; ++j) X[p][j] = dup(1e18f);
+        }
+    }
+    float lo[D], hi[D];
+#pragma unroll
+    for (int j = 0; j < D; ++j) {
+        lo[j] = INFINITY;
+        hi[j] = -INFINITY;
+    }
+#pragma unroll
+    for (int p = 0; p < RB_P; ++p)
+        if (valid[p])
+#pragma unroll
+            for (int j = 0; j < D; ++j) {
+                lo[j] = fminf(lo[j], X[p][j].x);
+                hi[j] = fmaxf(hi[j], X[p][j].x);
+            }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int j = 0; j < D; ++j) {
+            lo[j] = fminf(lo[j], __shfl_xor_sync(FULL, lo[j], o));
+            hi[j] = fmaxf(hi[j], __shfl_xor_sync(FULL, hi[j], o));
+        }
+    if (lane == 0)
+#pragma unroll
+        for (int j = 0; j < D; ++j) {
+            s_box[warp][j] = lo[j];
+            s_box[warp][D + j] = hi[j];
+        }
+    pdl_wait();   // the parameters and the state written by the previous kernels
+    if (threadIdx.x == 0) s_skip = (a.iter > a.st->stop_after) || (a.st->error != 0);
+    __syncthreads();
+    if (s_skip) return;
+    pdl_allow_next();
+    const float cmax = a.gref[0], ref0 = a.gref[1];
+
+    // ---- the components whose sphere {x : sigma_min(P')^2 |x - mu|^2 <= room} meets the
+    // CTA's box: a superset of those the second test keeps (a larger box, more slack)
+    {
+        float blo[D], bhi[D];
+#pragma unroll
+        for (int j = 0; j < D; ++j) {
+            blo[j] = s_box[0][j];
+            bhi[j] = s_box[0][D + j];
+            if (B == 2) {
+                blo[j] = fminf(blo[j], s_box[H][j]);
+                bhi[j] = fmaxf(bhi[j], s_box[H][D + j]);
+            }
+        }
+        int cnt = 0;   // lanes of class c keep the count of their class: lane % H == pp % H
+        const uint32_t cls = H == 2 ? 0x55555555u << (lane & 1) : 0x11111111u << (lane & 3);
+        uint16_t* dst = slist0 + warp * nquarter + (lane % H) * (nquarter / H);
+        for (int j0 = 0; j0 < nquarter; j0 += 32) {
+            const int pp = warp * nquarter + j0 + lane;
+            bool live = false;
+#pragma unroll
+            for (int m = 0; m < 2; ++m) {
+                const int b = 2 * pp + m;
+                if (b < a.k) {
+                    const float4 ct = a.ctr[b];
+                    const float2 ax = a.aux[b];
+                    const float x[4] = {ct.x, ct.y, ct.z, ct.w};
+                    float d2 = 0.f;
+#pragma unroll
+                    for (int j = 0; j < D; ++j) {
+                        const float e = fmaxf(fmaxf(blo[j] - x[j], x[j] - bhi[j]), 0.f);
+                        d2 = fmaf(e, e, d2);
+                    }
+                    const float room = REACH - (cmax - ax.x);
+                    live = live || (room > 0.f && ax.y * d2 * (1.f - 1.f / 64.f) <= room);
+                }
+            }
+            const uint32_t m = __ballot_sync(FULL, live) & cls;
+            if (live) dst[cnt + __popc(m & ((1u << lane) - 1u))] = (uint16_t)pp;
+            cnt += __popc(m);
+        }
+        if (lane < H) s_cnt[warp][lane] = cnt;
+    }
+    for (int wd = lane; wd < nwords; wd += 32) smask[wd] = 0u;
+    __syncthreads();
+
+    // ---- of these, the pairs of this warp's class that can reach a point of its block
+    // (the two bounds of estep_pt_kernel's phase 0, over the block's box)
+    int nlive = 0;
+    if (lo[0] <= hi[0]) {
+        float ctr[D], h[D];
+#pragma unroll
+        for (int j = 0; j < D; ++j) {
+            ctr[j] = 0.5f * (lo[j] + hi[j]);
+            h[j] = fmaxf(hi[j] - ctr[j], ctr[j] - lo[j]);
+        }
+        for (int w = 0; w < RB_W; ++w) {
+            const uint16_t* src = slist0 + w * nquarter + half * (nquarter / H);
+            const int cnt = s_cnt[w][half];
+            for (int i0 = 0; i0 < cnt; i0 += 32) {
+                const int i = i0 + lane;
+                const int pp = i < cnt ? (int)src[i] : -1;
+                bool live = false;
+                if (pp >= 0 && GIRA_IN(pp < npairs, a.st)) {
+                    float2 s[Lay<D>::PF / 2];
+                    load_slots<D>(a.params, pp, s);
+#pragma unroll
+                    for (int m = 0; m < 2; ++m) {
+                        auto sl = [&](int q) { return m ? s[q].y : s[q].x; };
+                        const float room = REACH - (cmax - sl(Lay<D>::SC));   // q' budget left for |y|^2
+                        float d[D], yy = 0.f, r = 0.f, e2 = 0.f;
+#pragma unroll
+                        for (int j = 0; j < D; ++j) {
+                            d[j] = ctr[j] + sl(Lay<D>::SNMU + j);
+                            const float e = fmaxf(fabsf(d[j]) - h[j], 0.f);
+                            e2 = fmaf(e, e, e2);
+                            float col = 0.f;   // |column j of P'|^2
+#pragma unroll
+                            for (int i2 = j; i2 < D; ++i2) {
+                                const float v = sl(Lay<D>::SP + i2 * (i2 + 1) / 2 + j);
+                                col = fmaf(v, v, col);
+                            }
+                            r = fmaf(h[j], sqrtf(col), r);
+                        }
+#pragma unroll
+                        for (int i2 = 0; i2 < D; ++i2) {
+                            float y = 0.f;
+#pragma unroll
+                            for (int j = 0; j <= i2; ++j) y = fmaf(sl(Lay<D>::SP + i2 * (i2 + 1) / 2 + j), d[j], y);
+                            yy = fmaf(y, y, yy);
+                        }
+                        const float reach = (r + sqrtf(fmaxf(room, 0.f))) * (1.f + 1.f / 256.f);
+                        const float iso = sl(Lay<D>::SS) * e2 * (1.f - 1.f / 128.f);
+                        live = live || (room > 0.f && yy <= reach * reach && iso <= room);
+                    }
+                }
+                const uint32_t m = __ballot_sync(FULL, live);
+                const int at = nlive + __popc(m & ((1u << lane) - 1u));
+                if (live && GIRA_IN(at < ncap, a.st)) slist[at] = (uint16_t)pp;
+                nlive += __popc(m);
+            }
+        }
+    }
+    __syncwarp();
+
+    // ---- phase 1: the listed pairs at the lane's points; a pair with a nonzero e is live
+    float2 tot[RB_P];
+#pragma unroll
+    for (int p = 0; p < RB_P; ++p) tot[p] = f2(0.f, 0.f);
+    constexpr int U = D == 3 ? 2 : 1;   // pairs per step (4-D: one, for registers)
+    for (int i = 0; i < nlive; i += U) {
+        int pp[U];
+        Pair<D> P[U];
+        uint32_t nz[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            pp[u] = slist[min(i + u, nlive - 1)];
+            load_pair<D>(a.params, pp[u], cmax, P[u]);
+            if (i + u >= nlive) P[u].c = dup(INFINITY);   // no such pair: q' = inf, e = 0
+            nz[u] = 0u;
+        }
+#pragma unroll
+        for (int p = 0; p < RB_P; ++p) {
+            float2 y[D], s = f2(0.f, 0.f);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const float2 nq = nlogit<D>(P[u], X[p], y);
+                const float2 e = f2(ex2_approx(-nq.x), ex2_approx(-nq.y));
+                s = u == 0 ? e : add2(s, e);
+                if (MODE != 0) nz[u] |= __float_as_uint(e.x) | __float_as_uint(e.y);
+            }
+            tot[p] = add2(tot[p], s);
+        }
+        if (MODE != 0) {
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const bool v = __ballot_sync(FULL, nz[u] != 0u) != 0u;
+                if (v && lane == 0) smask[pp[u] >> 5] |= 1u << (pp[u] & 31);
+            }
+        }
+    }
+
+    // ---- totals: the block's warps add their sums in the same order
+#pragma unroll
+    for (int p = 0; p < RB_P; ++p) s_tot[warp][p][lane] = tot[p];
+    block_sync<H>(blk);
+    float t[RB_P], sh[RB_P];
+    uint32_t rare[RB_P];   // lanes whose point p has every component > 100 binades below cmax
+    int nrare = 0;
+#pragma unroll
+    for (int p = 0; p < RB_P; ++p) {
+        t[p] = 0.f;
+        sh[p] = 0.f;
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+            const float2 u = s_tot[blk * H + h][p][lane];
+            t[p] += u.x + u.y;
+        }
+        rare[p] = __ballot_sync(FULL, valid[p] && !(t[p] >= 0x1p-100f));
+        nrare += __popc(rare[p]);
+    }
+    // Rare points: the exact maximum over every pair (Eq. logestep's max-subtraction), then
+    // the sums relative to it; a pair with a nonzero term becomes live.  nrare is the same
+    // in the block's warps, which split the pairs as in phase 1.
+    if (nrare > 0 && nrare <= RARE_FEW) {   // few: lanes take pairs, one point at a time
+#pragma unroll 1
+        for (int pass = 0; pass < 2; ++pass) {
+            int f = 0;
+#pragma unroll
+            for (int p = 0; p < RB_P; ++p)
+                for (uint32_t m = rare[p]; m; m &= m - 1u, ++f) {
+                    const int src = __ffs(m) - 1;
+                    float2 Z[D], y[D];
+#pragma unroll
+                    for (int j = 0; j < D; ++j) Z[j] = dup(__shfl_sync(FULL, X[p][j].x, src));
+                    const float mx = pass ? __shfl_sync(FULL, -sh[p], src) : -INFINITY;
+                    float v = pass ? 0.f : -INFINITY;
+                    for (int pp = half + H * lane; pp < npairs; pp += 32 * H) {
+                        Pair<D> P;
+                        load_pair<D>(a.params, pp, cmax, P);
+                        const float2 nq = nlogit<D>(P, Z, y);
+                        if (pass == 0) {
+                            v = fmaxf(v, fmaxf(-nq.x, -nq.y));
+                        } else {
+                            const float e = ex2_approx(-nq.x - mx) + ex2_approx(-nq.y - mx);
+                            v += e;
+                            if (MODE != 0 && e != 0.f) atomicOr(&smask[pp >> 5], 1u << (pp & 31));
+                        }
+                    }
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) {
+                        const float w = __shfl_xor_sync(FULL, v, o);
+                        v = pass ? v + w : fmaxf(v, w);
+                    }
+                    if (lane == 0) s_rare[warp][f] = v;
+                }
+            block_sync<H>(blk);
+            f = 0;
+#pragma unroll
+            for (int p = 0; p < RB_P; ++p)
+                for (uint32_t m = rare[p]; m; m &= m - 1u, ++f) {
+                    float v = s_rare[blk * H][f];
+#pragma unroll
+                    for (int h = 1; h < H; ++h) v = pass ? v + s_rare[blk * H + h][f] : fmaxf(v, s_rare[blk * H + h][f]);
+                    if (lane == __ffs(m) - 1) {
+                        if (pass) t[p] = v;
+                        else sh[p] = v > -INFINITY ? -v : 0.f;
+                    }
+                }
+            block_sync<H>(blk);   // s_rare is free for the next pass
+        }
+    } else if (nrare > 0) {   // many: every lane its own points
+        float mx[RB_P];
+#pragma unroll
+        for (int p = 0; p < RB_P; ++p) mx[p] = -INFINITY;
+#pragma unroll 2
+        for (int pp = half; pp < npairs; pp += H) {
+            Pair<D> P;
+            load_pair<D>(a.params, pp, cmax, P);
+#pragma unroll
+            for (int p = 0; p < RB_P; ++p)
+                if (rare[p]) {
+                    float2 y[D];
+                    const float2 nq = nlogit<D>(P, X[p], y);
+                    mx[p] = fmaxf(mx[p], fmaxf(-nq.x, -nq.y));
+                }
+        }
+        block_sync<H>(blk);   // every warp has read the totals
+#pragma unroll
+        for (int p = 0; p < RB_P; ++p) s_tot[warp][p][lane] = dup(mx[p]);
+        block_sync<H>(blk);
+        bool mine[RB_P];
+#pragma unroll
+        for (int p = 0; p < RB_P; ++p) {
+            mine[p] = (rare[p] >> lane) & 1u;
+#pragma unroll
+            for (int h = 0; h < H; ++h) mx[p] = fmaxf(mx[p], s_tot[blk * H + h][p][lane].x);
+            if (mine[p]) sh[p] = mx[p] > -INFINITY ? -mx[p] : 0.f;
+            tot[p] = f2(0.f, 0.f);
+        }
+#pragma unroll 2
+        for (int pp = half; pp < npairs; pp += H) {
+            Pair<D> P;
+            load_pair<D>(a.params, pp, cmax, P);
+            uint32_t nz = 0u;
+#pragma unroll
+            for (int p = 0; p < RB_P; ++p)
+                if (rare[p]) {
+                    float2 y[D];
+                    const float2 nq = nlogit<D>(P, X[p], y);
+                    const float2 e = f2(ex2_approx(sh[p] - nq.x), ex2_approx(sh[p] - nq.y));
+                    tot[p] = add2(tot[p], e);
+                    if (mine[p]) nz |= __float_as_uint(e.x) | __float_as_uint(e.y);
+                }
+            if (MODE != 0) {
+                const bool v = __ballot_sync(FULL, nz != 0u) != 0u;
+                if (v && lane == 0) smask[pp >> 5] |= 1u << (pp & 31);
+            }
+        }
+        block_sync<H>(blk);
+#pragma unroll
+        for (int p = 0; p < RB_P; ++p) s_tot[warp][p][lane] = tot[p];
+        block_sync<H>(blk);
+#pragma unroll
+        for (int p = 0; p < RB_P; ++p)
+            if (mine[p]) {
+                t[p] = 0.f;
+#pragma unroll
+                for (int h = 0; h < H; ++h) {
+                    const float2 u = s_tot[blk * H + h][p][lane];
+                    t[p] += u.x + u.y;
+                }
+            }
+    }
+
+    // ---- (shift, 1 / total), log-likelihood
+    float2 pr[RB_P];
+    double ll = 0.0;
+#pragma unroll
+    for (int p = 0; p < RB_P; ++p) {
+        pr[p] = f2(0.f, 0.f);
+        if (valid[p]) {
+            if (t[p] > 0.f) {
+                pr[p] = f2(sh[p], __frcp_rn(t[p]));
+                const float lse2 = lg2_approx(t[p]) + ref0 - sh[p];   // log2 sum_b pi_b N(x|b)
+                if (half == 0) {
+                    ll += (double)lse2;
+                    if (MODE == 0 && a.per_point) a_in.per_point[pt0 + base + 32 * p] = lse2 * LN2F;
+                }
+            } else {
+                set_error(a.st, GIRA_ERR_NUMERIC);   // underflows under every component
+            }
+            if (MODE != 0 && half == 0 && a.masks) a_in.pref[pt0 + base + 32 * p] = pr[p];
+        }
+    }
+    if (half == 0) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) ll += __shfl_xor_sync(FULL, ll, o);
+        if (lane == 0) s_ll[blk] = ll;
+    }
+    if (MODE != 0) {
+        __syncwarp();
+        block_sync<H>(blk);   // the block's masks are final
+        if (a.masks && half == 0 && row < a.rows)
+            for (int wd = lane; wd < nwords; wd += 32) {
+                uint32_t m = 0u;
+#pragma unroll
+                for (int h = 0; h < H; ++h) m |= smask_all[(blk * H + h) * nwords + wd];
+                a.masks[wd * a.rows + row] = m;
+            }
+    }
+    if constexpr (MODE == 2) {
+        // ---- sum_b gamma P'^T P' (x' - mu) over this warp's live pairs (components packed)
+        float2 G[RB_P][D];
+#pragma unroll
+        for (int p = 0; p < RB_P; ++p)
+#pragma unroll
+            for (int j = 0; j < D; ++j) {
+                G[p][j] = f2(0.f, 0.f);
+                if (!valid[p]) X[p][j] = f2(0.f, 0.f);   // weight 0 at a finite place
+            }
+        for (int wd = 0; wd < nwords; ++wd)
+            for (uint32_t m = smask[wd]; m; m &= m - 1u) {
+                Pair<D> P;
+                load_pair<D>(a.params, wd * 32 + __ffs(m) - 1, cmax, P);
+#pragma unroll
+                for (int p = 0; p < RB_P; ++p) {
+                    float2 y[D];
+                    const float2 nq = nlogit<D>(P, X[p], y);
+                    const float2 e = f2(ex2_approx(pr[p].x - nq.x), ex2_approx(pr[p].x - nq.y));
+                    const float2 g = mul2(e, dup(pr[p].y));   // pr = 0 for invalid points: g = 0
+#pragma unroll
+                    for (int j = 0; j < D; ++j) {   // z_j = sum_i P'_ij y_i
+                        float2 z = mul2(P.p[j * (j + 1) / 2 + j], y[j]);
+#pragma unroll
+                        for (int i = j + 1; i < D; ++i) z = fma2(P.p[i * (i + 1) / 2 + j], y[i], z);
+                        G[p][j] = fma2(g, z, G[p][j]);
+                    }
+                }
+            }
+        // the block's warps in order; -(2 ln 2): P'^T P' = Sigma^{-1} log2(e) / 2
+        float g3[RB_P][D];
+#pragma unroll
+        for (int j = 0; j < D; ++j) {
+            block_sync<H>(blk);   // s_tot is free
+#pragma unroll
+            for (int p = 0; p < RB_P; ++p) s_tot[warp][p][lane] = G[p][j];
+            block_sync<H>(blk);
+#pragma unroll
+            for (int p = 0; p < RB_P; ++p) {
+                float v = 0.f;
+#pragma unroll
+                for (int h = 0; h < H; ++h) {
+                    const float2 u = s_tot[blk * H + h][p][lane];
+                    v += u.x + u.y;
+                }
+                g3[p][j] = -1.38629436111989061883f * v;
+            }
+        }
+        __shared__ double s_pose[B][12];
+        if (half == 0) {
+            float tw[12] = {};   // sum g x'^T (row-major), sum g
+#pragma unroll
+            for (int p = 0; p < RB_P; ++p) {
+                if (!valid[p]) continue;
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+#pragma unroll
+                    for (int j = 0; j < 3; ++j) tw[3 * i + j] = fmaf(g3[p][i], X[p][j].x, tw[3 * i + j]);
+                    tw[9 + i] += g3[p][i];
+                }
+                if (a.grad_pts) {
+                    const int64_t at = pt0 + base + 32 * p;
+                    float* gp = a_in.grad_pts + 3 * (a_in.order ? (int64_t)a_in.order[at] : at);
+                    if (a.rot) {
+                        const float* Rm = a.rot;
+                        gp[0] = fmaf(Rm[6], g3[p][2], fmaf(Rm[3], g3[p][1], Rm[0] * g3[p][0]));
+                        gp[1] = fmaf(Rm[7], g3[p][2], fmaf(Rm[4], g3[p][1], Rm[1] * g3[p][0]));
+                        gp[2] = fmaf(Rm[8], g3[p][2], fmaf(Rm[5], g3[p][1], Rm[2] * g3[p][0]));
+                    } else {
+                        gp[0] = g3[p][0];
+                        gp[1] = g3[p][1];
+                        gp[2] = g3[p][2];
+                    }
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < 12; ++i) {
+                double u = (double)tw[i];
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) u += __shfl_xor_sync(FULL, u, o);
+                if (lane == 0) s_pose[blk][i] = u;
+            }
+        }
+        __syncthreads();
+        if (threadIdx.x < 12) {
+            double u = s_pose[0][threadIdx.x];
+            if (B == 2) u += s_pose[B - 1][threadIdx.x];
+            a.pose_partials[(size_t)cta * 12 + threadIdx.x] = u;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double v = s_ll[0];
+        if (B == 2) v += s_ll[B - 1];
+        a.llp[cta] = v * LN2;
+    }
+}
+
+// ------------------------------------------------------------------ the statistics
+// One warp per (pair, slice of `sl` words of 32 blocks): S0 = sum r, S1 = sum r y, S2 =
+// sum r y y^T with y = P'(x - mu_old) of both components over the points of the live
+// blocks, e formed by the E-step's operations (the same bits).  Row (slice) of the
+// partials [slices][pairs][2 NS], written where it is not empty; live2 [words][slices]
+// (zeroed before the launch) gets the pair's bit there.  The 8 warps of a CTA take
+// neighbouring pairs (in Morton order), which reach much the same blocks: the points
+// come out of L1.
+constexpr int ST_W = 8;
+template <int D>
+__global__ void __launch_bounds__(32 * ST_W) reach_stats_kernel(const ReachLaunch a_in, int sl, float* partials,
+                                                                uint32_t* live2) {
+    constexpr int NS = Lay<D>::NS;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    ReachLaunch a = a_in;
+    int64_t pt0 = 0;
+    int slices = gridDim.y, pair0 = blockIdx.x * ST_W, slice = blockIdx.y;
+    if (a_in.units) {   // units: (instance, slice * pair groups + group)
+        const BatchUnit u = a_in.units[blockIdx.x];
+        const BatchInst I = a_in.insts[u.inst];
+        pt0 = I.pt_off;
+        a.n = I.n;
+        a.k = I.k;
+        a.params = a_in.params + I.par_off;
+        a.gref = a_in.gref + 2 * u.inst;
+        a.masks = a_in.masks + I.mask_off;
+        a.rows = (I.n + RB_PTS - 1) / RB_PTS;
+        a.st = a_in.states + u.inst;
+        const int groups = ((I.k + 1) / 2 + ST_W - 1) / ST_W;
+        slices = reach_slices(I.n, &sl);
+        slice = u.cta / groups;
+        pair0 = (u.cta % groups) * ST_W;
+        partials += I.part_off;
+        live2 += I.live_off;
+    }
+    pdl_wait();
+    if (a.iter > a.st->stop_after || a.st->error) return;
+    const int pp = pair0 + warp;
+    const int npairs = (a.k + 1) >> 1;
+    if (pp >= npairs) return;
+    const uint32_t* mw = a.masks + (size_t)(pp >> 5) * a.rows;
+    const int64_t r0 = (int64_t)slice * sl * 32;
+    const float cmax = a.gref[0];
+    Pair<D> P;
+    bool loaded = false;
+    float2 S[NS];
+#pragma unroll
+    for (int s = 0; s < NS; ++s) S[s] = f2(0.f, 0.f);
+    for (int w = 0; w < sl; ++w) {
+        const int64_t r = r0 + 32 * w + lane;
+        uint32_t m = __ballot_sync(FULL, r < a.rows && ((mw[r] >> (pp & 31)) & 1u));
+        if (m && !loaded) {
+            load_pair<D>(a.params, pp, cmax, P);
+            loaded = true;
+        }
+        for (; m; m &= m - 1u) {
+            const int64_t b0 = (r0 + 32 * w + __ffs(m) - 1) * RB_PTS + lane;
+#pragma unroll
+            for (int p = 0; p < RB_P; ++p) {
+                const int64_t i = b0 + 32 * p;
+                const bool ok = i < a.n;
+                const int64_t at = pt0 + (ok ? i : a.n - 1);   // an absent point: the last one with weight 0
+                float2 X[D], y[D];
+                load_point<D>(a_in.pts8, at, X);
+                const float2 pr = a_in.pref[at];
+                const float2 nq = nlogit<D>(P, X, y);
+                const float2 e = f2(ex2_approx(pr.x - nq.x), ex2_approx(pr.x - nq.y));
+                const float2 g = mul2(e, dup(ok ? pr.y : 0.f));
+                S[0] = add2(S[0], g);
+#pragma unroll
+                for (int i2 = 0, q = 1 + D; i2 < D; ++i2) {
+                    const float2 gy = mul2(g, y[i2]);
+                    S[1 + i2] = add2(S[1 + i2], gy);
+#pragma unroll
+                    for (int j = i2; j < D; ++j, ++q) S[q] = fma2(gy, y[j], S[q]);
+                }
+            }
+        }
+    }
+    if (!loaded) return;
+    // lanes 0-15 end with the first component's sums, 16-31 with the second's
+    float v[NS];
+    const bool hi16 = lane & 16;
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+        const float keep = hi16 ? S[s].y : S[s].x, send = hi16 ? S[s].x : S[s].y;
+        v[s] = keep + __shfl_xor_sync(FULL, send, 16);
+    }
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1)
+#pragma unroll
+        for (int s = 0; s < NS; ++s) v[s] += __shfl_xor_sync(FULL, v[s], o);
+    float mine = 0.f;
+#pragma unroll
+    for (int s = 0; s < NS; ++s)
+        if ((lane & 15) == s) mine = v[s];
+    if ((lane & 15) < NS) {
+        float* dst = partials + ((size_t)slice * npairs + pp) * (2 * NS);
+        dst[(hi16 ? NS : 0) + (lane & 15)] = mine;
+    }
+    if (lane == 0) atomicOr(live2 + (size_t)(pp >> 5) * slices + slice, 1u << (pp & 31));
+}
+
+template <int D>
+const void* reach_fn(int mode, int h) {
+    if (h == 2)
+        return mode == 0 ? (const void*)estep_reach_kernel<D, 2, 0>
+                         : mode == 1 ? (const void*)estep_reach_kernel<D, 2, 1> : (const void*)estep_reach_kernel<D, 2, 2>;
+    return mode == 0 ? (const void*)estep_reach_kernel<D, 4, 0>
+                     : mode == 1 ? (const void*)estep_reach_kernel<D, 4, 1> : (const void*)estep_reach_kernel<D, 4, 2>;
+}
+
+}  // namespace
+
+// Two warps per block of 128 points where that fills the chip's SMs with one CTA each
+// (152 x 256 points), else four: fewer points per CTA, a block's pairs in parallel.
+int reach_h(int64_t n) { return n > 152 * 2 * RB_PTS ? 2 : 4; }
+int reach_grid(int64_t n) {
+    const int64_t pts = (int64_t)(RB_W / reach_h(n)) * RB_PTS;
+    return (int)std::max<int64_t>(1, (n + pts - 1) / pts);
+}
+int64_t reach_rows(int64_t n) { return (n + RB_PTS - 1) / RB_PTS; }
+int reach_mask_words(int k) { return reach_words(k); }
+int reach_stat_groups(int k) { return ((k + 1) / 2 + ST_W - 1) / ST_W; }
+
+cudaError_t launch_reach_prepare(const float* params, int k, const BatchInst* insts, int batch, const DeviceState* st,
+                                 int iter, float4* ctr, float2* aux, float* gref, cudaStream_t s) {
+    const int threads = insts ? 256 : std::min(PREP_THREADS, (k + 31) / 32 * 32);
+    reach_prepare_kernel<3><<<insts ? batch : 1, threads, 0, s>>>(params, k, insts, st, iter, ctr, aux, gref);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_estep_reach(const ReachLaunch& a, int mode, int grid, int h, int kmax, cudaStream_t s) {
+    const void* fn = reach_fn<3>(mode, h);
+    note_estep_kernel(fn);
+    const size_t smem = reach_smem(kmax, h);
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    void* args[] = {(void*)&a};
+    return cudaLaunchKernel(fn, dim3(grid), dim3(32 * RB_W), args, smem, s);
+}
+
+cudaError_t launch_reach_stats(const ReachLaunch& a, int nunits, float* partials, uint32_t* live2, cudaStream_t s) {
+    int sl = 1;
+    const int slices = a.units ? 1 : reach_slices(a.n, &sl);
+    const dim3 grid = a.units ? dim3(nunits) : dim3(reach_stat_groups(a.k), slices);
+    reach_stats_kernel<3><<<grid, 32 * ST_W, 0, s>>>(a, sl, partials, live2);
+    return cudaGetLastError();
+}
+
+}  // namespace gira

@@ -1,0 +1,68 @@
+"""The E-step over reach lists (reach_kernels.cu) at the sizes where its tiling changes: blocks of
+128 points, two or four warps per block (38,912 points), slices of 4,096 points in the statistics,
+odd and padded component counts, and blocks holding a few (lanes take component pairs) or many
+(lanes take points) points whose every component lies more than 100 binades below the reference.
+
+Tolerances: per-point log-likelihoods within the derived bound of _parity.per_point_bound (which
+covers the summation order); one EM iteration within the fit's 1e-4 per component.  The points
+off the model there sit at q' of a few hundred, where the binary32 rounding of q' (a few 2^-24
+relative) moves a responsibility by less than 1e-4.
+"""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2307_00071_gb300 import synth
+from tests._parity import LL_ABS, assert_model_close, per_point_bound, to_np
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def gira():
+    from paper_2307_00071_gb300 import gira as g
+    return g
+
+
+@pytest.fixture(scope="module")
+def frame():
+    return synth.depth_frame(seed=4).points
+
+
+def ball_model(pts, k, rng, d=3, sigma=0.05):
+    """k isotropic components at scan points, with a jitter of their axes."""
+    means = pts[rng.choice(len(pts), k, replace=False)].astype(np.float64)
+    a = rng.normal(scale=0.2, size=(k, d, d))
+    covs = sigma ** 2 * (np.eye(d) + a @ np.transpose(a, (0, 2, 1)))
+    return rng.dirichlet(np.ones(k) * 5).astype(np.float32), means.astype(np.float32), covs.astype(np.float32)
+
+
+def off_model(pts, count, rng):
+    """count points of the cloud moved 0.8-1 m away, next to one another in the cloud's order."""
+    at = rng.integers(0, len(pts) - count) + np.arange(count)
+    out = pts.copy()
+    step = rng.normal(size=(count, 3))
+    out[at, :3] += (step / np.linalg.norm(step, axis=1)[:, None] * rng.uniform(0.8, 1.0, (count, 1))).astype(np.float32)
+    return out, at
+
+
+SIZES = [(1_100, 1_025, 0), (4_097, 1_500, 3), (38_912, 1_026, 16), (38_913, 1_999, 200), (12_289, 8_192, 700)]
+
+
+@pytest.mark.parametrize("n,k,off", SIZES)
+def test_large_k_reach(gira, frame, n, k, off):
+    rng = np.random.default_rng(n + k)
+    start = rng.integers(0, len(frame) - n)
+    pts, at = off_model(np.ascontiguousarray(frame[start:start + n]), off, rng)
+    w, m, c = ball_model(pts, k, rng)
+    mean, pp = gira.gira_gmm_loglik(pts, w, m, c, per_point=True)
+    pp = to_np(pp).astype(np.float64)
+    assert mean == pytest.approx(pp.mean(), rel=1e-6)
+    sample = np.unique(np.concatenate([at, [0, n - 1], rng.choice(n, 200, replace=False)]))
+    _, _, lse = oracle.estep(pts[sample], w, m, c, want_resp=False, want_lse=True)
+    err, bound = np.abs(pp[sample] - lse), per_point_bound(pts[sample], w, m, c)
+    assert np.all(err <= bound), np.max(err / bound)
+    r = gira.gira_gmm_fit(pts, k, iters=1, tol=0.0, init=(w, m, c))
+    ref = oracle.em_par(pts, w, m, c, iters=1, tol=0.0, reg=1e-6)
+    assert abs(r["trace"][0] - ref["trace"][0]) <= LL_ABS + 1e-7 * abs(ref["trace"][0])
+    assert_model_close((r["weights"], r["means"], r["covs"]), (ref["weights"], ref["means"], ref["covs"]))
