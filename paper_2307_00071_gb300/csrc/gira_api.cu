@@ -286,55 +286,6 @@ gira_status gira::device_status(const DeviceState& h) {
 }
 
 
-// ---------------------------------------------------------------- batched EM helpers
-namespace {
-
-// Instances with the same E-step block shape run in one launch per iteration.
-struct BatchClass {
-    int np = 0, g = 0, threads = 0, kmax = 0;
-    std::vector<int> insts;
-    int64_t points = 0;
-    int64_t ppc = 0;
-    int unit_begin = 0, nunits = 0;
-};
-
-// Points per CTA chosen by measurement, per (device, shape, log2 of the class's points).
-std::mutex g_tune_mu;
-std::map<std::tuple<int, int, int, int>, int64_t> g_tuned;
-
-int ilog2(int64_t v) {
-    int r = 0;
-    while ((int64_t(1) << (r + 1)) <= v) ++r;
-    return r;
-}
-
-// Per-instance offsets and the unit list for the classes' current ppc values.
-// Returns the units, the partial floats and the log-likelihood slots used.
-void build_tables(std::vector<BatchInst>& hi, std::vector<BatchClass>& cls, std::vector<BatchUnit>& units,
-                  int64_t* part_floats, int64_t* ll_slots) {
-    int64_t part = 0, ll = 0;
-    units.clear();
-    for (auto& c : cls) {
-        c.unit_begin = (int)units.size();
-        for (int i : c.insts) {
-            BatchInst& I = hi[i];
-            I.ppc = c.ppc;
-            I.ctas = (int)((I.n + c.ppc - 1) / c.ppc);
-            I.part_off = part;
-            I.ll_off = ll;
-            part += (int64_t)I.ctas * I.k * NSTAT;
-            ll += I.ctas;
-            for (int t = 0; t < I.ctas; ++t) units.push_back(BatchUnit{i, t});
-        }
-        c.nunits = (int)units.size() - c.unit_begin;
-    }
-    *part_floats = part;
-    *ll_slots = ll;
-}
-
-}  // namespace
-
-
 // ---------------------------------------------------------------- E-step over reach lists
 namespace {
 
@@ -380,17 +331,17 @@ ReachLaunch reach_launch(const ReachBufs& b, const float4* p8, int64_t n, int k,
 cudaError_t reach_estep_stats(const ReachBufs& b, ReachLaunch a, long long* launches, cudaStream_t s) {
     a.pref = b.pref;
     a.masks = b.masks;
-    cudaError_t e = launch_reach_prepare(a.params, a.k, nullptr, 1, a.st, a.iter, b.ctr, b.aux, b.gref, s);
+    cudaError_t e = launch_reach_prepare(a.params, a.k, a.st, a.iter, b.ctr, b.aux, b.gref, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(b.live2, 0, sizeof(uint32_t) * b.words * b.slices, s);
     if (e == cudaSuccess) e = launch_estep_reach(a, 1, b.grid, b.h, a.k, s);
-    if (e == cudaSuccess) e = launch_reach_stats(a, 0, b.partials, b.live2, s);
+    if (e == cudaSuccess) e = launch_reach_stats(a, 1, a.k, a.n, b.partials, b.live2, s);
     *launches += 3;
     return e;
 }
 
 // The log-likelihood alone: a.per_point (nullable) and st->ll_sum.
 cudaError_t reach_loglik(const ReachBufs& b, const ReachLaunch& a, long long* launches, cudaStream_t s) {
-    cudaError_t e = launch_reach_prepare(a.params, a.k, nullptr, 1, a.st, a.iter, b.ctr, b.aux, b.gref, s);
+    cudaError_t e = launch_reach_prepare(a.params, a.k, a.st, a.iter, b.ctr, b.aux, b.gref, s);
     if (e == cudaSuccess) e = launch_estep_reach(a, 0, b.grid, b.h, a.k, s);
     if (e == cudaSuccess) e = launch_ll_reduce(b.llp, b.grid, a.st, s);
     *launches += 3;
@@ -712,7 +663,7 @@ gira_status gira_gmm_fit(const float* points, int64_t n, int k, const gira_fit_o
         if (final_loglik)
             GIRA_CUDA(reach_loglik(rb, reach_launch(rb, pe, n, k, b.params, b.st, 0), &prof.launches, c.s));
     }
-    EStepLaunch a{sorted ? b.p8s : b.p8, n, k, b.params, 0, b.partials, b.llp, nullptr, b.st, 0};
+    EStepLaunch a{sorted ? b.p8s : b.p8, n, k, b.params, b.partials, b.llp, nullptr, b.st, 0};
     a.n_buf = n;
     a.masks = b.masks;
     a.pt_rows = rows;
@@ -850,7 +801,7 @@ gira_status gira_gmm_loglik(const float* points, int64_t n, int k, const float* 
         a.per_point = ppd;
         GIRA_CUDA(reach_loglik(rb, a, &prof.launches, c.s));
     } else {
-        EStepLaunch a{b.p8, n, k, b.params, 0, nullptr, b.llp, ppd, b.st, 0};
+        EStepLaunch a{b.p8, n, k, b.params, nullptr, b.llp, ppd, b.st, 0};
         a.n_buf = n;
         COUNTED(prof, 1, launch_estep_pt(a, false, grid, c.s));
         COUNTED(prof, 1, launch_ll_reduce(b.llp, grid, b.st, c.s));
@@ -892,16 +843,19 @@ gira_status gira_gmm_loglik_grad(const float* points, int64_t n, int k, const fl
     if (grad_means) TRY(check_ptr(grad_means, "grad_means", c.dev, &kgm));
     if (grad_chol) TRY(check_ptr(grad_chol, "grad_chol", c.dev, &kgc));
     const bool grad = grad_points || grad_pose || grad_twist || grad_logits || grad_means || grad_chol;
+    const bool gpar = grad_logits || grad_means || grad_chol;   // statistics wanted
+    const bool sorted = grad && n <= point_order_max_n();        // the E-step visits the scan in Morton order
     const int npairs = params_pairs_padded(k);
-    int64_t ppc = 0;
-    const int grid = estep_grid(n, k, grad, c.sms, &ppc, true);
     auto host = [&](Kind kd, const void* ptr) { return ptr && kd == Kind::Host; };
     struct Bufs {
         DeviceState* st;
-        float *pin, *pose, *lg, *mu, *ch, *params, *partials, *gp, *gl, *gm, *gc;
-        float4 *p8, *shift4;
-        double *model64, *llp, *ppart, *po64, *tw64;
+        float *pin, *pose, *lg, *mu, *ch, *params, *gp, *gl, *gm, *gc;
+        float4 *p8, *p8s, *shift4;
+        double *model64, *ppart, *po64, *tw64;
+        int *perm, *order;
+        void* osc;
     } b{};
+    ReachBufs rb;
     auto layout = [&](Carver& cv) {
         b.st = cv.take<DeviceState>(1);
         b.pin = cv.take<float>(host(kp, points) ? 3 * (size_t)n : 0);
@@ -910,12 +864,15 @@ gira_status gira_gmm_loglik_grad(const float* points, int64_t n, int k, const fl
         b.mu = cv.take<float>(host(km, means) ? 3 * (size_t)k : 0);
         b.ch = cv.take<float>(host(kc, chol) ? 9 * (size_t)k : 0);
         b.p8 = cv.take<float4>(2 * (size_t)n);
+        b.p8s = cv.take<float4>(sorted ? 2 * (size_t)n : 0);
+        b.order = cv.take<int>(sorted ? (size_t)n : 0);
+        b.osc = cv.take<char>(sorted ? point_order_scratch_bytes(n, 1) : 0);
+        b.perm = cv.take<int>(k);
+        carve_reach(cv, n, k, NSTAT, gpar, &rb);
         b.params = cv.take<float>((size_t)npairs * PAIR_FLOATS);
         b.shift4 = cv.take<float4>(k);
         b.model64 = cv.take<double>((size_t)k * MODEL);
-        b.llp = cv.take<double>(grid);
-        b.partials = cv.take<float>(grad ? (size_t)grid * k * NSTAT : 0);
-        b.ppart = cv.take<double>(grad ? (size_t)grid * 12 : 0);
+        b.ppart = cv.take<double>(grad ? (size_t)rb.grid * 12 : 0);
         b.po64 = cv.take<double>(12);
         b.tw64 = cv.take<double>(6);
         b.gp = cv.take<float>(host(kgp, grad_points) ? 3 * (size_t)n : 0);
@@ -940,6 +897,7 @@ gira_status gira_gmm_loglik_grad(const float* points, int64_t n, int k, const fl
     DeviceState h{};
     h.stop_after = 0;
     h.bad_component = INT_MAX;
+    h.cmax_ord = CMAX_ORD_NONE;
     GIRA_CUDA(cudaMemcpyAsync(b.st, &h, sizeof h, cudaMemcpyHostToDevice, c.s));
     // inputs: device pointers as given, host arrays staged
     auto in = [&](const float* src, Kind kd, float* stage, size_t count) -> const float* {
@@ -965,24 +923,36 @@ gira_status gira_gmm_loglik_grad(const float* points, int64_t n, int k, const fl
     double* tw_d = grad_twist ? (kgt == Kind::Host ? b.tw64 : grad_twist) : nullptr;
 
     COUNTED(prof, 1, launch_pack_pose(pts_d, n, pose_d, b.p8, b.st, c.s));
-    COUNTED(prof, 1, launch_fill_padding(b.params, k, npairs, c.s));
-    COUNTED(prof, 1, launch_params_from_chol(lg_d, mu_d, ch_d, k, b.model64, b.params, b.shift4, b.st, c.s));
+    if (sorted)
+        COUNTED(prof, point_order_launches(1),
+                launch_point_order(b.p8, n, nullptr, nullptr, 0, 1, b.osc, b.p8s, nullptr, b.order, c.s));
+    COUNTED(prof, 1, launch_params_from_chol(lg_d, mu_d, ch_d, k, nullptr, 1, b.model64, b.params, b.shift4, b.perm,
+                                             rb.ctr, rb.aux, b.st, c.s));
     prof.t_init = prof.mark();
     prof.t_em = prof.t_init;
-    EStepLaunch a{b.p8, n, k, b.params, ppc, grad ? b.partials : nullptr, b.llp, nullptr, b.st, 0};
+    ReachLaunch a = reach_launch(rb, sorted ? b.p8s : b.p8, n, k, b.params, b.st, 0);
+    a.gref = nullptr;   // the parameter build leaves max_b c_b in the state
     if (grad) {
         a.grad_pts = gp_d;
+        a.order = sorted ? b.order : nullptr;
         a.rot = pose_d;
         a.pose_partials = b.ppart;
+        if (gpar) {
+            a.pref = rb.pref;
+            a.masks = rb.masks;
+            GIRA_CUDA(cudaMemsetAsync(rb.live2, 0, sizeof(uint32_t) * rb.words * rb.slices, c.s));
+        }
         cudaEvent_t e0 = prof.mark_launch();
-        COUNTED(prof, 1, launch_estep(a, true, grid, c.s, true));
+        COUNTED(prof, 1, launch_estep_reach(a, 2, rb.grid, rb.h, k, c.s));
         cudaEvent_t e1 = prof.mark_launch();
         if (prof.per_launch) prof.timed(e0, e1);
-        COUNTED(prof, 1, launch_grad_finalize(b.partials, grid, b.llp, b.ppart, pose_d, ch_d, b.model64, k, n, gl_d,
-                                              gm_d, gc_d, po_d, tw_d, b.st, c.s));
+        if (gpar) COUNTED(prof, 1, launch_reach_stats(a, 1, k, n, rb.partials, rb.live2, c.s));
+        const ReachGradArgs f{gpar ? rb.partials : nullptr, rb.live2, rb.slices, rb.llp, b.ppart, rb.grid, pose_d,
+                              ch_d, b.params, b.model64, b.perm, k, n, gl_d, gm_d, gc_d, po_d, tw_d, b.st};
+        COUNTED(prof, 1, launch_reach_grad_finalize(f, nullptr, 1, c.s));
     } else {
-        COUNTED(prof, 1, launch_estep(a, false, grid, c.s, true));
-        COUNTED(prof, 1, launch_ll_reduce(b.llp, grid, b.st, c.s));
+        COUNTED(prof, 1, launch_estep_reach(a, 0, rb.grid, rb.h, k, c.s));
+        COUNTED(prof, 1, launch_ll_reduce(rb.llp, rb.grid, b.st, c.s));
     }
     auto out = [&](void* dst, Kind kd, const void* stage, size_t bytes) -> gira_status {
         if (dst && kd == Kind::Host) GIRA_CUDA(cudaMemcpyAsync(dst, stage, bytes, cudaMemcpyDeviceToHost, c.s));
@@ -1268,7 +1238,7 @@ gira_status gira_gmm_fit_batched(const float* points, const int64_t* offsets, in
                                                      b.comp_inst, b.perm, b.params, b.shift4, b.st, c.s));
     prof.t_init = prof.mark();
 
-    EStepLaunch base{sorted ? b.p8s : b.p8, 0, 0, b.params, 0, b.partials, b.llp, nullptr, nullptr, 0};
+    EStepLaunch base{sorted ? b.p8s : b.p8, 0, 0, b.params, b.partials, b.llp, nullptr, nullptr, 0};
     base.n_buf = total_n;
     base.insts = b.insts;
     base.units = b.units;
@@ -1409,64 +1379,56 @@ gira_status gira_gmm_loglik_grad_batched(const float* points, const int64_t* off
         if (a.p) TRY(check_ptr(a.p, a.name, c.dev, &a.k));
     for (auto& a : out)
         if (a.p) TRY(check_ptr(a.p, a.name, c.dev, &a.k));
-    const int Q = estep_batch_q();
+    const bool gpar = grad_logits || grad_means || grad_chol;   // statistics wanted
+    const bool sorted = total_n <= point_order_max_n();
 
-    // ---- tables: instances, shape classes (points per CTA by a balance rule), finalize blocks
+    // ---- tables: instances and their E-step CTAs
     std::vector<BatchInst> hi(batch);
-    std::vector<int> npairs_of(batch);
-    int total_k = 0;
-    int64_t par_floats = 0;
-    std::map<std::pair<int, int>, int> class_of_shape;
-    std::vector<BatchClass> cls;
+    std::vector<BatchUnit> units;
+    const int rh = reach_h(total_n), rpts = reach_points(rh);
+    int total_k = 0, kmax = 0;
+    int64_t par_floats = 0, ll_slots = 0, part_floats = 0, mask_words = 0, live_words = 0, nmax = 0;
     for (int i = 0; i < batch; ++i) {
         BatchInst& I = hi[i];
+        int sl;
         I.pt_off = offsets[i];
         I.n = offsets[i + 1] - offsets[i];
         I.k = ks[i];
         I.comp_off = total_k;
         total_k += ks[i];
-        npairs_of[i] = params_pairs_padded(ks[i]);
+        kmax = std::max(kmax, ks[i]);
+        nmax = std::max(nmax, I.n);
         I.par_off = par_floats;
-        par_floats += (int64_t)npairs_of[i] * PAIR_FLOATS;
-        int np, g, th;
-        estep_shape(ks[i], &np, &g, &th);
-        auto key = std::make_pair(np, g);
-        auto it = class_of_shape.find(key);
-        if (it == class_of_shape.end()) {
-            it = class_of_shape.emplace(key, (int)cls.size()).first;
-            cls.emplace_back();
-            cls.back().np = np;
-            cls.back().g = g;
-            cls.back().threads = th;
-        }
-        BatchClass& C = cls[it->second];
-        C.insts.push_back(i);
-        C.points += I.n;
-        C.kmax = std::max(C.kmax, ks[i]);
+        par_floats += (int64_t)params_pairs_padded(ks[i]) * PAIR_FLOATS;
+        I.ctas = (int)((I.n + rpts - 1) / rpts);
+        I.ll_off = ll_slots;
+        ll_slots += I.ctas;
+        I.mask_off = mask_words;
+        mask_words += reach_mask_words(I.k) * reach_rows(I.n);
+        const int slices = reach_slices(I.n, &sl);
+        I.live_off = live_words;
+        live_words += (int64_t)reach_mask_words(I.k) * slices;
+        I.part_off = part_floats;
+        part_floats += (int64_t)slices * ((I.k + 1) / 2) * 2 * NSTAT;
+        for (int t = 0; t < I.ctas; ++t) units.push_back(BatchUnit{i, t});
     }
-    for (auto& C : cls) {
-        const int occ = estep_grad_occupancy(C.kmax, 1024);
-        int64_t ppc = (C.points + 2LL * c.sms * occ - 1) / (2LL * c.sms * occ);
-        C.ppc = std::min<int64_t>(estep_ppc_max(), std::max<int64_t>(4 * Q, (ppc + Q - 1) / Q * Q));
-    }
-    std::vector<BatchUnit> units;
-    int64_t part_floats = 0, ll_slots = 0;
-    build_tables(hi, cls, units, &part_floats, &ll_slots);
-    std::vector<int2> fin_blocks;
-    const int cpb = fin_components_per_block();
-    for (int i = 0; i < batch; ++i)
-        for (int j = 0; j * cpb < ks[i]; ++j) fin_blocks.push_back(make_int2(i, j));
+    const int64_t nounits = sorted ? point_order_box_units(offsets, batch) : 0;
+    std::vector<int2> ounits((size_t)nounits);
+    if (sorted) point_order_fill_units(offsets, batch, ounits.data());
 
     struct Bufs {
         DeviceState* st;
         float *pin, *poses, *lg, *mu, *ch, *params, *partials, *gp, *gl, *gm, *gc;
-        float4 *p8, *shift4;
+        float4 *p8, *p8s, *shift4, *ctr;
+        float2 *aux, *pref;
         double *model64, *llp, *ppart, *gpose, *gtwist;
+        uint32_t *masks, *live2;
         BatchInst* insts;
         BatchUnit* units;
-        int2* blocks;
-        int* npairs;
+        int2* ounits;
+        int *perm, *order;
         int64_t* offs;
+        void* osc;
     } b{};
     auto layout = [&](Carver& cv) {
         b.st = cv.take<DeviceState>(batch);
@@ -1479,10 +1441,20 @@ gira_status gira_gmm_loglik_grad_batched(const float* points, const int64_t* off
         b.params = cv.take<float>((size_t)par_floats);
         b.shift4 = cv.take<float4>(total_k);
         b.model64 = cv.take<double>((size_t)total_k * MODEL);
-        b.partials = cv.take<float>((size_t)part_floats);
+        b.p8s = cv.take<float4>(sorted ? 2 * (size_t)total_n : 0);
+        b.order = cv.take<int>(sorted ? (size_t)total_n : 0);
+        b.ounits = cv.take<int2>((size_t)nounits);
+        b.osc = cv.take<char>(sorted ? point_order_scratch_bytes(total_n, batch) : 0);
+        b.perm = cv.take<int>(total_k);
+        b.ctr = cv.take<float4>(total_k);
+        b.aux = cv.take<float2>(total_k);
+        b.pref = cv.take<float2>(gpar ? (size_t)total_n : 0);
+        b.masks = cv.take<uint32_t>(gpar ? (size_t)mask_words : 0);
+        b.live2 = cv.take<uint32_t>(gpar ? (size_t)live_words : 0);
+        b.partials = cv.take<float>(gpar ? (size_t)part_floats : 0);
         b.llp = cv.take<double>((size_t)ll_slots);
         b.ppart = cv.take<double>(12 * (size_t)ll_slots);
-        b.gp = cv.take<float>(3 * (size_t)total_n);
+        b.gp = cv.take<float>(grad_points ? 3 * (size_t)total_n : 0);
         b.gl = cv.take<float>(total_k);
         b.gm = cv.take<float>(3 * (size_t)total_k);
         b.gc = cv.take<float>(9 * (size_t)total_k);
@@ -1490,8 +1462,6 @@ gira_status gira_gmm_loglik_grad_batched(const float* points, const int64_t* off
         b.gtwist = cv.take<double>(6 * (size_t)batch);
         b.insts = cv.take<BatchInst>(batch);
         b.units = cv.take<BatchUnit>(units.size());
-        b.blocks = cv.take<int2>(fin_blocks.size());
-        b.npairs = cv.take<int>(batch);
         b.offs = cv.take<int64_t>(batch + 1);
     };
     Carver sizer;
@@ -1512,6 +1482,7 @@ gira_status gira_gmm_loglik_grad_batched(const float* points, const int64_t* off
     for (auto& h : hs) {
         h = DeviceState{};
         h.bad_component = INT_MAX;
+        h.cmax_ord = CMAX_ORD_NONE;
     }
     // every input staged into the workspace, so that the cached graph reads only workspace memory
     auto stage = [&](void* dst, const Arg& a, size_t bytes) -> gira_status {
@@ -1535,13 +1506,13 @@ gira_status gira_gmm_loglik_grad_batched(const float* points, const int64_t* off
     GIRA_CUDA(cudaMemcpyAsync(b.offs, offsets, sizeof(int64_t) * (batch + 1), cudaMemcpyHostToDevice, c.s));
     GIRA_CUDA(cudaMemcpyAsync(b.insts, hi.data(), sizeof(BatchInst) * batch, cudaMemcpyHostToDevice, c.s));
     GIRA_CUDA(cudaMemcpyAsync(b.units, units.data(), sizeof(BatchUnit) * units.size(), cudaMemcpyHostToDevice, c.s));
-    GIRA_CUDA(cudaMemcpyAsync(b.blocks, fin_blocks.data(), sizeof(int2) * fin_blocks.size(), cudaMemcpyHostToDevice,
-                              c.s));
-    GIRA_CUDA(cudaMemcpyAsync(b.npairs, npairs_of.data(), sizeof(int) * batch, cudaMemcpyHostToDevice, c.s));
+    if (sorted)
+        GIRA_CUDA(cudaMemcpyAsync(b.ounits, ounits.data(), sizeof(int2) * ounits.size(), cudaMemcpyHostToDevice, c.s));
     prof.t_init = prof.mark();
 
-    // ---- one graph: move the scans, build the parameters, the adjoint E-step per shape class, finalize
-    std::string key = "grad|" + std::to_string((uintptr_t)ws->ptr) + "|" + std::to_string(sizer.off) + "|" +
+    // ---- one graph: move the scans, order them, build the parameters, the E-step with the
+    // gradient, the statistics (when a parameter gradient is asked for), finalize
+    std::string key = "grad|" + std::to_string((int)gpar) + std::to_string((int)(grad_points != nullptr)) + "|" + std::to_string((uintptr_t)ws->ptr) + "|" + std::to_string(sizer.off) + "|" +
                       std::to_string(batch);
     for (int i = 0; i < batch; ++i) key += "|" + std::to_string(hi[i].n) + ":" + std::to_string(hi[i].k);
     if (ws->graph_key != key || !ws->graph_exec) {
@@ -1550,24 +1521,32 @@ gira_status gira_gmm_loglik_grad_batched(const float* points, const int64_t* off
         cudaStream_t cs = ws->capture_stream;
         GIRA_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeRelaxed));
         cudaError_t e = launch_pack_pose_batched(b.pin, total_n, b.offs, batch, b.poses, b.p8, b.st, cs);
-        if (e == cudaSuccess) e = launch_fill_padding_batched(b.params, b.insts, batch, 0, b.npairs, cs);
+        if (e == cudaSuccess && sorted)
+            e = launch_point_order(b.p8, total_n, b.offs, b.ounits, (int)nounits, batch, b.osc, b.p8s, nullptr,
+                                   b.order, cs);
         if (e == cudaSuccess)
-            e = launch_params_from_chol_batched(b.lg, b.mu, b.ch, b.insts, batch, b.model64, b.params, b.shift4, b.st,
-                                                cs);
-        EStepLaunch a{b.p8, 0, 0, b.params, 0, b.partials, b.llp, nullptr, nullptr, 0};
-        a.insts = b.insts;
-        a.states = b.st;
-        a.grad_pts = b.gp;
+            e = launch_params_from_chol(b.lg, b.mu, b.ch, kmax, b.insts, batch, b.model64, b.params, b.shift4, b.perm,
+                                        b.ctr, b.aux, b.st, cs);
+        ReachLaunch a{sorted ? b.p8s : b.p8, 0, 0, b.params, b.ctr, b.aux, nullptr, b.llp, nullptr, nullptr, 0};
+        a.n_buf = total_n;
+        a.grad_pts = grad_points ? b.gp : nullptr;
+        a.order = sorted ? b.order : nullptr;
         a.rot = b.poses;
         a.pose_partials = b.ppart;
-        for (const BatchClass& C : cls) {
-            if (e != cudaSuccess || !C.nunits) continue;
-            a.units = b.units + C.unit_begin;
-            e = launch_estep_grad_units(a, C.nunits, C.kmax, C.ppc, cs);
+        a.insts = b.insts;
+        a.units = b.units;
+        a.states = b.st;
+        if (gpar) {
+            a.pref = b.pref;
+            a.masks = b.masks;
+            if (e == cudaSuccess) e = cudaMemsetAsync(b.live2, 0, sizeof(uint32_t) * live_words, cs);
         }
-        if (e == cudaSuccess)
-            e = launch_grad_finalize_batched(b.partials, b.llp, b.ppart, b.poses, b.ch, b.model64, b.insts, b.blocks,
-                                             (int)fin_blocks.size(), b.gl, b.gm, b.gc, b.gpose, b.gtwist, b.st, cs);
+        if (e == cudaSuccess) e = launch_estep_reach(a, 2, (int)units.size(), rh, kmax, cs);
+        if (e == cudaSuccess && gpar) e = launch_reach_stats(a, batch, kmax, nmax, b.partials, b.live2, cs);
+        const ReachGradArgs f{gpar ? b.partials : nullptr, b.live2, 0, b.llp, b.ppart, 0, b.poses, b.ch, b.params,
+                              b.model64, b.perm, kmax, 0, gpar ? b.gl : nullptr, gpar ? b.gm : nullptr,
+                              gpar ? b.gc : nullptr, b.gpose, b.gtwist, b.st};
+        if (e == cudaSuccess) e = launch_reach_grad_finalize(f, b.insts, batch, cs);
         cudaGraph_t graph = nullptr;
         cudaError_t e2 = cudaStreamEndCapture(cs, &graph);
         if (e != cudaSuccess || e2 != cudaSuccess) {
@@ -1586,7 +1565,7 @@ gira_status gira_gmm_loglik_grad_batched(const float* points, const int64_t* off
         ws->graph_exec = exec;
         ws->graph_key = key;
     }
-    prof.launches += 4 + (long long)cls.size();
+    prof.launches += 4 + (sorted ? point_order_launches(batch) : 0) + (gpar ? 1 : 0);
     GIRA_CUDA(cudaGraphLaunch(ws->graph_exec, c.s));
     prof.t_em = prof.mark();
     const void* src[6] = {b.gp, b.gpose, b.gtwist, b.gl, b.gm, b.gc};

@@ -31,7 +31,6 @@ constexpr int PAIR_F4 = PAIR_FLOATS / 4;   // float4 per pair block
 constexpr int SLOT_P = 0, SLOT_B = 6, SLOT_C = 9, SLOT_NMU = 10, SLOT_W = 13, SLOT_S = 14;
 constexpr int NSTAT = 10;   // S0, S1[3], S2[6] (00,01,02,11,12,22)
 constexpr int MODEL = 10;   // w, mu[3], Sigma[6] (00,01,02,11,12,22), binary64; w = N_b or caller weight
-constexpr int Q_BATCH = 8;  // points per E-step batch
 
 // Device-side state of one library call (zeroed by the host at call start).
 struct DeviceState {
@@ -47,7 +46,9 @@ struct DeviceState {
     // point-stationary E-step with statistics, summed over its launches: warp x pair
     // evaluations made (pairs within reach of the warp's box) and with statistics
     unsigned long long pairs_near, pairs_live;
+    int cmax_ord;          // gradient: max_b c_b as an order-preserving int (host: that of -inf)
 };
+constexpr int CMAX_ORD_NONE = (int)0x807fffff;   // -inf
 
 __device__ __forceinline__ void set_error(DeviceState* st, int code) { atomicCAS(&st->error, 0, code); }
 
@@ -359,7 +360,7 @@ struct ReachLaunch {
     const float* params;     // pair-interleaved
     const float4* ctr;       // compact per-component arrays and references of launch_reach_prepare
     const float2* aux;
-    const float* gref;
+    const float* gref;       // nullptr (gradient): max_b c_b from st->cmax_ord
     double* llp;             // [grid] log-likelihood partials
     float* per_point;        // mode 0: [n] natural-log lse, or nullptr
     DeviceState* st;
@@ -379,44 +380,35 @@ struct ReachLaunch {
     DeviceState* states = nullptr;
 };
 int reach_h(int64_t n);        // warps per block of 128 points for n points in the launch
+int reach_points(int h);       // points per CTA
 int reach_grid(int64_t n);     // CTAs of a single launch
 int64_t reach_rows(int64_t n); // blocks of 128 points
 int reach_mask_words(int k);
-int reach_stat_groups(int k);  // CTAs per slice of the statistics launch
-cudaError_t launch_reach_prepare(const float* params, int k, const BatchInst* insts, int batch, const DeviceState* st,
-                                 int iter, float4* ctr, float2* aux, float* gref, cudaStream_t s);
+cudaError_t launch_reach_prepare(const float* params, int k, const DeviceState* st, int iter, float4* ctr, float2* aux,
+                                 float* gref, cudaStream_t s);
 // mode 0 log-likelihood, 1 with masks and pref, 2 gradient; h: reach_h of the launch; kmax: the largest k.
 cudaError_t launch_estep_reach(const ReachLaunch& a, int mode, int grid, int h, int kmax, cudaStream_t s);
 // partials [slices][pairs][2 NSTAT] and live2 [words][slices] (zeroed by the caller):
 // launch_reduce_finalize takes them as rows and masks.
-cudaError_t launch_reach_stats(const ReachLaunch& a, int nunits, float* partials, uint32_t* live2, cudaStream_t s);
+// Batched (a.insts): every instance, kmax and nmax its largest k and n.
+cudaError_t launch_reach_stats(const ReachLaunch& a, int batch, int kmax, int64_t nmax, float* partials,
+                               uint32_t* live2, cudaStream_t s);
 
 struct EStepLaunch {
     const float4* pts8;      // 2 float4 per point: (x,x,y,y) (z,z,0,0)
     int64_t n;
     int k;
     const float* params;     // pair-interleaved, npairs_pad * PAIR_FLOATS
-    int64_t pts_per_cta;     // multiple of Q_BATCH
-    float* partials;         // [grid][k][NSTAT] (stats kernels)
+    float* partials;         // statistics (stats launches), see masks
     double* ll_partials;     // [grid]
     float* per_point;        // [n] natural-log lse, or nullptr
     DeviceState* st;
     int iter;                // iteration index (1-based); kernels skip if iter > st->stop_after
-    // adjoint launches (log-likelihood gradient) only
-    float* grad_pts = nullptr;           // [n][3] dL/dx (dL/dx' rotated back by R^T), or nullptr
-    const float* rot = nullptr;          // R, row-major 3x3, of x' = R x + t; nullptr = identity
-    double* pose_partials = nullptr;     // [grid][12]: per CTA sum dL/dx' x'^T (row-major), sum dL/dx'
     // batched launches: CTA b runs units[b]; pts8 / params / partials / ll_partials /
     // per_point are then bases offset by the instance's table entry, st = states + inst
     const BatchInst* insts = nullptr;
     const BatchUnit* units = nullptr;
     DeviceState* states = nullptr;
-    // K split into chunks (one table entry per chunk, all over the same points):
-    // pass A writes psum[chunk][n] = sum over the chunk of 2^(l - cmax); pass B
-    // takes pref[n] = (shift, 1 / total) from the combine step
-    const float* gref = nullptr;   // [0] cmax over all K, [1] log-likelihood reference (base 2)
-    float* psum = nullptr;
-    const float2* pref = nullptr;
     // point-stationary E-step (estep_pt_kernel): partial rows [rows][pairs][2 NSTAT],
     // row cta * PT_B + block written only where the block's live mask has the pair's
     // bit, and the live masks [npairs / 32][rows] (bit p: pair p reaches some point
@@ -432,9 +424,6 @@ struct EStepLaunch {
     uint8_t* cta_key = nullptr;
 };
 
-// Chooses the template instance and block shape for K; returns the CTA count
-// actually used in *grid_out (needed for the partials buffer size).
-// grad: the differentiable path's kernels (d-form logits; with stats, the adjoint).
 // A launch configuration, with programmatic stream serialisation when pdl (the
 // kernel may start before the previous kernel in the stream has finished, and
 // waits for it with pdl_wait()).
@@ -452,12 +441,6 @@ struct PdlConfig {
         cfg.numAttrs = pdl ? 1 : 0;
     }
 };
-// pdl: launch as a programmatic dependent of the previous kernel in s (that kernel
-// must not write the points).
-cudaError_t launch_estep(const EStepLaunch& a, bool stats, int grid, cudaStream_t s, bool grad = false,
-                         bool pdl = false);
-// Occupancy-derived grid size for (k, stats) with n points.
-int estep_grid(int64_t n, int k, bool stats, int num_sms, int64_t* pts_per_cta, bool grad = false);
 // Pairs (padded) the parameter buffer must hold for k components.
 int params_pairs_padded(int k);
 
@@ -515,16 +498,6 @@ cudaError_t launch_order_components(double* model64, double* scratch, int k, int
                                     float4* shift4, DeviceState* st, cudaStream_t s);
 
 // Batched EM (per-instance tables on the device).
-// E-step block shape for k components (pairs per lane, warps, threads); the
-// batch size Q of the kernels; the largest points-per-CTA; CTAs per SM.
-void estep_shape(int k, int* np, int* g, int* threads);
-int estep_batch_q();
-int estep_ppc_max();
-int estep_occupancy(int k, bool stats, int64_t ppc);
-// One launch over nunits CTAs (a.units / a.insts / a.states set) of the class
-// whose shape is that of k_class; every instance of the class has ppc_class.
-cudaError_t launch_estep_units(const EStepLaunch& a, bool stats, int nunits, int k_class, int64_t ppc_class,
-                               cudaStream_t s);
 cudaError_t launch_pack_batched(const float* pts3, int64_t n, const int64_t* offsets, int batch, float4* pts4,
                                 float4* pts8, DeviceState* states, cudaStream_t s);
 // Finalize blocks: (instance, block index within the instance), FIN_CPB components each.
@@ -566,34 +539,40 @@ cudaError_t launch_points_ll_reduce(const double* llpt, int64_t n, double* llp, 
 // own model and pose; poses: batch x 12, or nullptr for identities).
 cudaError_t launch_pack_pose_batched(const float* pts3, int64_t n, const int64_t* offsets, int batch,
                                      const float* poses, float4* pts8, DeviceState* states, cudaStream_t s);
-cudaError_t launch_params_from_chol_batched(const float* logits, const float* mu, const float* chol,
-                                            const BatchInst* insts, int batch, double* model64, float* params,
-                                            float4* shift4, DeviceState* states, cudaStream_t s);
-cudaError_t launch_estep_grad_units(const EStepLaunch& a, int nunits, int k_class, int64_t ppc_class, cudaStream_t s);
-int estep_grad_occupancy(int k, int64_t ppc);
-cudaError_t launch_grad_finalize_batched(const float* partials, const double* ll_partials,
-                                         const double* pose_partials, const float* poses, const float* chol,
-                                         const double* model64, const BatchInst* insts, const int2* blocks,
-                                         int nblocks, float* g_logits, float* g_means, float* g_chol, double* g_pose,
-                                         double* g_twist, DeviceState* states, cudaStream_t s);
-
 // Differentiable log-likelihood.  pose12 = R (row-major) then t, or nullptr.
 // N x 3 -> pts8 of x' = R x + t (binary32, fixed order); flags non-finite input.
 cudaError_t launch_pack_pose(const float* pts3, int64_t n, const float* pose12, float4* pts8, DeviceState* st,
                              cudaStream_t s);
-// E-step parameters from (logits, means, Cholesky factors): pi = softmax in
-// binary64, Sigma = L L^T, then the same binary64 build as the M-step.
-cudaError_t launch_params_from_chol(const float* logits, const float* mu, const float* chol, int k, double* model64,
-                                    float* params, float4* shift4, DeviceState* st, cudaStream_t s);
-// Reduces the statistics, the log-likelihood and the pose partials of a
-// gradient launch, then writes dL/dlogits (k), dL/dmeans (k x 3), dL/dchol
-// (k x 3 x 3, lower) in binary32, and in binary64 dL/dpose (dL/dR row-major,
-// dL/dt) and dL/dtwist (omega, v); loglik goes to st->ll_sum.  Outputs nullable.
-cudaError_t launch_grad_finalize(const float* partials, int grid, const double* ll_partials,
-                                 const double* pose_partials, const float* pose12, const float* chol,
-                                 const double* model64, int k, int64_t n, float* g_logits, float* g_means,
-                                 float* g_chol, double* g_pose, double* g_twist,
-                                 DeviceState* st, cudaStream_t s);
+// E-step parameters from (logits, means, Cholesky factors), k <= MAX_K_DIRECT, in Morton
+// order of the means (perm[slot]: the caller's component), with the compact arrays of the
+// reach tests and max_b c_b in st->cmax_ord.  insts: every instance of a batch, kmax the
+// largest k (one fit: its k).
+cudaError_t launch_params_from_chol(const float* logits, const float* mu, const float* chol, int kmax,
+                                    const BatchInst* insts, int batch, double* model64, float* params, float4* shift4,
+                                    int* perm, float4* ctr, float2* aux, DeviceState* st, cudaStream_t s);
+// Sums of a gradient launch (fixed order): dL/dlogits (k), dL/dmeans (k x 3), dL/dchol
+// (k x 3 x 3, lower) in binary32 from the statistics, in the caller's order; in binary64
+// dL/dpose (dL/dR row-major, dL/dt) and dL/dtwist (omega, v); the log-likelihood in
+// st->ll_sum.  Outputs nullable; partials nullptr: no parameter gradients.
+struct ReachGradArgs {
+    const float* partials;    // [slices][pairs][2 NSTAT], live where live2 says
+    const uint32_t* live2;    // [words][slices]
+    int slices;
+    const double* llp;        // [grid]
+    const double* pp;         // [grid][12]
+    int grid;
+    const float* pose;
+    const float* chol;
+    const float* params;
+    const double* model64;
+    const int* perm;
+    int k;
+    int64_t n;
+    float *g_logits, *g_means, *g_chol;
+    double *g_pose, *g_twist;
+    DeviceState* st;
+};
+cudaError_t launch_reach_grad_finalize(const ReachGradArgs& f, const BatchInst* insts, int batch, cudaStream_t s);
 
 // k-means
 // dim: 3 (distances over x, y, z) or 4 (also the fourth coordinate)

@@ -48,7 +48,6 @@ constexpr int RB_P = 4;                    // points per lane
 constexpr int RB_PTS = 32 * RB_P;          // points per block (a row of the masks)
 constexpr int RB_W = 4;                    // warps per CTA
 constexpr float REACH = 128.f;             // q' above which a component is out of reach (e = 0 from q' > 126)
-constexpr int RARE_FEW = 16;               // rare points of a block up to which lanes take pairs instead of points
 
 template <int D>
 struct Lay;
@@ -106,6 +105,13 @@ __device__ __forceinline__ float2 nlogit(const Pair<D>& P, const float2 (&X)[D],
     return q;
 }
 
+// max_b c_b: of the prepared references, or (gradient) of the parameter build's atomics
+__device__ __forceinline__ float cmax_of(const float* gref, const DeviceState* st) {
+    if (gref) return gref[0];
+    const int o = st->cmax_ord;
+    return __int_as_float(o >= 0 ? o : o ^ 0x7fffffff);
+}
+
 template <int D>
 __device__ __forceinline__ void load_point(const float4* pts8, int64_t i, float2 (&X)[D]) {
     const float4 a = pts8[2 * i], b = pts8[2 * i + 1];
@@ -116,27 +122,17 @@ __device__ __forceinline__ void load_point(const float4* pts8, int64_t i, float2
 }
 
 // ------------------------------------------------------------------ per-component compact arrays
-// Block i: instance i of a batch (insts), or the one fit (k components).  ctr[b] = the
+// One block.  ctr[b] = the
 // mean's first three coordinates and, in 3-D, the bound s2 of sigma_min(P')^2 (in 4-D the
 // fourth coordinate); aux[b] = (c, s2); gref[0] = max_b c_b, gref[1] = the log-likelihood
 // reference (cmax - log2 sum_a N_a once the weights are raw N_b, else cmax).
 constexpr int PREP_THREADS = 1024;
 template <int D>
 __global__ void __launch_bounds__(PREP_THREADS) reach_prepare_kernel(const float* __restrict__ params, int k,
-                                                                     const BatchInst* __restrict__ insts,
                                                                      const DeviceState* st, int iter, float4* ctr,
                                                                      float2* aux, float* gref) {
     __shared__ float s_m[PREP_THREADS / 32];
     __shared__ double s_w[PREP_THREADS / 32];
-    if (insts) {
-        const BatchInst I = insts[blockIdx.x];
-        k = I.k;
-        params += I.par_off;
-        ctr += I.comp_off;
-        aux += I.comp_off;
-        gref += 2 * blockIdx.x;
-        st += blockIdx.x;
-    }
     pdl_wait();
     if (iter > st->stop_after || st->error) return;
     float m = -INFINITY;
@@ -179,6 +175,52 @@ __global__ void __launch_bounds__(PREP_THREADS) reach_prepare_kernel(const float
     }
 }
 
+// Whether a component of the pair with slots s can have q' <= limit at a point of the box
+// (centre ctr, half-extents h): the two lower bounds of estep_pt_kernel's phase 0,
+//   |P'(x - mu)| >= |P'(ctr - mu)| - sum_j h_j |column j of P'|  and
+//   |P'(x - mu)|^2 >= sigma_min(P')^2 dist(mu, box)^2,
+// with their relative slack.  ub (if not nullptr): lowered to the pair's upper bound of
+// q' over the box.
+template <int D>
+__device__ __forceinline__ bool pair_reaches(const float2 (&s)[Lay<D>::PF / 2], const float (&ctr)[D],
+                                             const float (&h)[D], float cmax, float limit, float* ub) {
+    bool live = false;
+#pragma unroll
+    for (int m = 0; m < 2; ++m) {
+        auto sl = [&](int q) { return m ? s[q].y : s[q].x; };
+        const float cc = cmax - sl(Lay<D>::SC), room = limit - cc;   // q' budget left for |y|^2
+        float d[D], yy = 0.f, r = 0.f, e2 = 0.f;
+#pragma unroll
+        for (int j = 0; j < D; ++j) {
+            d[j] = ctr[j] + sl(Lay<D>::SNMU + j);
+            const float e = fmaxf(fabsf(d[j]) - h[j], 0.f);
+            e2 = fmaf(e, e, e2);
+            float col = 0.f;   // |column j of P'|^2
+#pragma unroll
+            for (int i = j; i < D; ++i) {
+                const float v = sl(Lay<D>::SP + i * (i + 1) / 2 + j);
+                col = fmaf(v, v, col);
+            }
+            r = fmaf(h[j], sqrtf(col), r);
+        }
+#pragma unroll
+        for (int i = 0; i < D; ++i) {
+            float y = 0.f;
+#pragma unroll
+            for (int j = 0; j <= i; ++j) y = fmaf(sl(Lay<D>::SP + i * (i + 1) / 2 + j), d[j], y);
+            yy = fmaf(y, y, yy);
+        }
+        const float reach = (r + sqrtf(fmaxf(room, 0.f))) * (1.f + 1.f / 256.f);
+        const float iso = sl(Lay<D>::SS) * e2 * (1.f - 1.f / 128.f);
+        live = live || (room > 0.f && yy <= reach * reach && iso <= room);
+        if (ub) {
+            const float u = (r + sqrtf(yy)) * (1.f + 1.f / 256.f);
+            *ub = fminf(*ub, fmaf(u, u, cc));
+        }
+    }
+    return live;
+}
+
 // ------------------------------------------------------------------ the E-step
 // Shared memory: the CTA's surviving pairs by warp quarter and class (pp % H), every
 // warp's listed pairs, every warp's live-mask words.
@@ -210,38 +252,41 @@ __global__ void __launch_bounds__(32 * RB_W, 4) estep_reach_kernel(const ReachLa
     static_assert(B * H == RB_W && B <= 2, "one named barrier per block");
     __shared__ float s_box[RB_W][2 * D];
     __shared__ float2 s_tot[RB_W][RB_P][32];
-    __shared__ float s_rare[RB_W][RARE_FEW];
+    __shared__ float s_ub[RB_W];
     __shared__ int s_cnt[RB_W][H];
     __shared__ double s_ll[B];
     __shared__ int s_skip;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int blk = warp / H, half = warp % H;
-    int cta = blockIdx.x;
-    int64_t pt0 = 0;   // the instance's first point (loads index the launch's own pointers by it)
-    ReachLaunch a = a_in;
+    // batched launches: this CTA's instance.  Everything of the instance is an offset
+    // added to the launch's own pointers (loads through a pointer advanced inside a copy
+    // of the launch struct read the unadvanced one under nvcc 13.0 for sm_103a).
+    int cta = blockIdx.x, inst = 0, k = a_in.k;
+    int64_t pt0 = 0, n = a_in.n, rows = a_in.rows, par_off = 0, comp_off = 0, mask_off = 0, ll_off = 0;
+    DeviceState* st = a_in.st;
     if (a_in.units) {
         const BatchUnit u = a_in.units[blockIdx.x];
         const BatchInst I = a_in.insts[u.inst];
         cta = u.cta;
+        inst = u.inst;
         pt0 = I.pt_off;
-        a.n = I.n;
-        a.k = I.k;
-        a.params = a_in.params + I.par_off;
-        a.ctr = a_in.ctr + I.comp_off;
-        a.aux = a_in.aux + I.comp_off;
-        a.gref = a_in.gref + 2 * u.inst;
-        a.masks = a_in.masks ? a_in.masks + I.mask_off : nullptr;
-        a.rows = (I.n + RB_PTS - 1) / RB_PTS;
-        a.llp = a_in.llp + I.ll_off;
-        a.st = a_in.states + u.inst;
-        a.rot = a_in.rot ? a_in.rot + 12 * (size_t)u.inst : nullptr;
-        a.pose_partials = a_in.pose_partials ? a_in.pose_partials + 12 * I.ll_off : nullptr;
+        n = I.n;
+        k = I.k;
+        rows = (I.n + RB_PTS - 1) / RB_PTS;
+        par_off = I.par_off;
+        comp_off = I.comp_off;
+        mask_off = I.mask_off;
+        ll_off = I.ll_off;
+        st = a_in.states + u.inst;
     }
-    const int npairs = (a.k + 1) >> 1;
-    const int nquarter = reach_pairs(a.k) / RB_W, ncap = reach_pairs(a.k) / H, nwords = reach_words(a.k);
+    const float* const params = a_in.params + par_off;
+    const float4* const ctr4 = a_in.ctr + comp_off;
+    const float2* const aux = a_in.aux + comp_off;
+    const int npairs = (k + 1) >> 1;
+    const int nquarter = reach_pairs(k) / RB_W, ncap = reach_pairs(k) / H, nwords = reach_words(k);
     uint16_t* slist0 = reinterpret_cast<uint16_t*>(dsm);                        // [RB_W][H][nquarter / H]
-    uint16_t* slist = slist0 + reach_pairs(a.k) + (size_t)warp * ncap;          // this warp's listed pairs
-    uint32_t* smask_all = reinterpret_cast<uint32_t*>(slist0 + reach_pairs(a.k) + (size_t)RB_W * ncap);
+    uint16_t* slist = slist0 + reach_pairs(k) + (size_t)warp * ncap;          // this warp's listed pairs
+    uint32_t* smask_all = reinterpret_cast<uint32_t*>(slist0 + reach_pairs(k) + (size_t)RB_W * ncap);
     uint32_t* smask = smask_all + warp * nwords;
     // a slot beyond n holds a point 1e18 m away, where every q' is +inf and e exactly 0
     const int64_t row = (int64_t)cta * B + blk;
@@ -251,7 +296,7 @@ __global__ void __launch_bounds__(32 * RB_W, 4) estep_reach_kernel(const ReachLa
 #pragma unroll
     for (int p = 0; p < RB_P; ++p) {
         const int64_t i = base + 32 * p;
-        valid[p] = i < a.n && GIRA_IN(a_in.n_buf == 0 || pt0 + i < a_in.n_buf, a.st);
+        valid[p] = i < n && GIRA_IN(a_in.n_buf == 0 || pt0 + i < a_in.n_buf, st);
         if (valid[p]) {
             load_point<D>(a_in.pts8, pt0 + i, X[p]);
         } else {
@@ -287,11 +332,11 @@ __global__ void __launch_bounds__(32 * RB_W, 4) estep_reach_kernel(const ReachLa
             s_box[warp][D + j] = hi[j];
         }
     pdl_wait();   // the parameters and the state written by the previous kernels
-    if (threadIdx.x == 0) s_skip = (a.iter > a.st->stop_after) || (a.st->error != 0);
+    if (threadIdx.x == 0) s_skip = (a_in.iter > st->stop_after) || (st->error != 0);
     __syncthreads();
     if (s_skip) return;
     pdl_allow_next();
-    const float cmax = a.gref[0], ref0 = a.gref[1];
+    const float cmax = cmax_of(a_in.gref, st), ref0 = a_in.gref ? a_in.gref[1] : cmax;
 
     // ---- the components whose sphere {x : sigma_min(P')^2 |x - mu|^2 <= room} meets the
     // CTA's box: a superset of those the second test keeps (a larger box, more slack)
@@ -315,9 +360,9 @@ __global__ void __launch_bounds__(32 * RB_W, 4) estep_reach_kernel(const ReachLa
 #pragma unroll
             for (int m = 0; m < 2; ++m) {
                 const int b = 2 * pp + m;
-                if (b < a.k) {
-                    const float4 ct = a.ctr[b];
-                    const float2 ax = a.aux[b];
+                if (b < k) {
+                    const float4 ct = ctr4[b];
+                    const float2 ax = aux[b];
                     const float x[4] = {ct.x, ct.y, ct.z, ct.w};
                     float d2 = 0.f;
 #pragma unroll
@@ -341,57 +386,31 @@ __global__ void __launch_bounds__(32 * RB_W, 4) estep_reach_kernel(const ReachLa
     // ---- of these, the pairs of this warp's class that can reach a point of its block
     // (the two bounds of estep_pt_kernel's phase 0, over the block's box)
     int nlive = 0;
-    if (lo[0] <= hi[0]) {
-        float ctr[D], h[D];
+    float ctr[D], h[D];
 #pragma unroll
-        for (int j = 0; j < D; ++j) {
-            ctr[j] = 0.5f * (lo[j] + hi[j]);
-            h[j] = fmaxf(hi[j] - ctr[j], ctr[j] - lo[j]);
-        }
+    for (int j = 0; j < D; ++j) {
+        ctr[j] = 0.5f * (lo[j] + hi[j]);
+        h[j] = fmaxf(hi[j] - ctr[j], ctr[j] - lo[j]);
+    }
+    auto push = [&](bool live, int pp) {   // append the lanes' live pairs in lane order
+        const uint32_t m = __ballot_sync(FULL, live);
+        const int at = nlive + __popc(m & ((1u << lane) - 1u));
+        if (live && GIRA_IN(at < ncap, st)) slist[at] = (uint16_t)pp;
+        nlive += __popc(m);
+    };
+    if (lo[0] <= hi[0]) {
         for (int w = 0; w < RB_W; ++w) {
             const uint16_t* src = slist0 + w * nquarter + half * (nquarter / H);
             const int cnt = s_cnt[w][half];
             for (int i0 = 0; i0 < cnt; i0 += 32) {
-                const int i = i0 + lane;
-                const int pp = i < cnt ? (int)src[i] : -1;
+                const int pp = i0 + lane < cnt ? (int)src[i0 + lane] : -1;
                 bool live = false;
-                if (pp >= 0 && GIRA_IN(pp < npairs, a.st)) {
+                if (pp >= 0 && GIRA_IN(pp < npairs, st)) {
                     float2 s[Lay<D>::PF / 2];
-                    load_slots<D>(a.params, pp, s);
-#pragma unroll
-                    for (int m = 0; m < 2; ++m) {
-                        auto sl = [&](int q) { return m ? s[q].y : s[q].x; };
-                        const float room = REACH - (cmax - sl(Lay<D>::SC));   // q' budget left for |y|^2
-                        float d[D], yy = 0.f, r = 0.f, e2 = 0.f;
-#pragma unroll
-                        for (int j = 0; j < D; ++j) {
-                            d[j] = ctr[j] + sl(Lay<D>::SNMU + j);
-                            const float e = fmaxf(fabsf(d[j]) - h[j], 0.f);
-                            e2 = fmaf(e, e, e2);
-                            float col = 0.f;   // |column j of P'|^2
-#pragma unroll
-                            for (int i2 = j; i2 < D; ++i2) {
-                                const float v = sl(Lay<D>::SP + i2 * (i2 + 1) / 2 + j);
-                                col = fmaf(v, v, col);
-                            }
-                            r = fmaf(h[j], sqrtf(col), r);
-                        }
-#pragma unroll
-                        for (int i2 = 0; i2 < D; ++i2) {
-                            float y = 0.f;
-#pragma unroll
-                            for (int j = 0; j <= i2; ++j) y = fmaf(sl(Lay<D>::SP + i2 * (i2 + 1) / 2 + j), d[j], y);
-                            yy = fmaf(y, y, yy);
-                        }
-                        const float reach = (r + sqrtf(fmaxf(room, 0.f))) * (1.f + 1.f / 256.f);
-                        const float iso = sl(Lay<D>::SS) * e2 * (1.f - 1.f / 128.f);
-                        live = live || (room > 0.f && yy <= reach * reach && iso <= room);
-                    }
+                    load_slots<D>(params, pp, s);
+                    live = pair_reaches<D>(s, ctr, h, cmax, REACH, nullptr);
                 }
-                const uint32_t m = __ballot_sync(FULL, live);
-                const int at = nlive + __popc(m & ((1u << lane) - 1u));
-                if (live && GIRA_IN(at < ncap, a.st)) slist[at] = (uint16_t)pp;
-                nlive += __popc(m);
+                push(live, pp);
             }
         }
     }
@@ -409,7 +428,7 @@ __global__ void __launch_bounds__(32 * RB_W, 4) estep_reach_kernel(const ReachLa
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             pp[u] = slist[min(i + u, nlive - 1)];
-            load_pair<D>(a.params, pp[u], cmax, P[u]);
+            load_pair<D>(params, pp[u], cmax, P[u]);
             if (i + u >= nlive) P[u].c = dup(INFINITY);   // no such pair: q' = inf, e = 0
             nz[u] = 0u;
         }
@@ -453,89 +472,87 @@ __global__ void __launch_bounds__(32 * RB_W, 4) estep_reach_kernel(const ReachLa
         rare[p] = __ballot_sync(FULL, valid[p] && !(t[p] >= 0x1p-100f));
         nrare += __popc(rare[p]);
     }
-    // Rare points: the exact maximum over every pair (Eq. logestep's max-subtraction), then
-    // the sums relative to it; a pair with a nonzero term becomes live.  nrare is the same
-    // in the block's warps, which split the pairs as in phase 1.
-    if (nrare > 0 && nrare <= RARE_FEW) {   // few: lanes take pairs, one point at a time
-#pragma unroll 1
-        for (int pass = 0; pass < 2; ++pass) {
-            int f = 0;
-#pragma unroll
-            for (int p = 0; p < RB_P; ++p)
-                for (uint32_t m = rare[p]; m; m &= m - 1u, ++f) {
-                    const int src = __ffs(m) - 1;
-                    float2 Z[D], y[D];
-#pragma unroll
-                    for (int j = 0; j < D; ++j) Z[j] = dup(__shfl_sync(FULL, X[p][j].x, src));
-                    const float mx = pass ? __shfl_sync(FULL, -sh[p], src) : -INFINITY;
-                    float v = pass ? 0.f : -INFINITY;
-                    for (int pp = half + H * lane; pp < npairs; pp += 32 * H) {
-                        Pair<D> P;
-                        load_pair<D>(a.params, pp, cmax, P);
-                        const float2 nq = nlogit<D>(P, Z, y);
-                        if (pass == 0) {
-                            v = fmaxf(v, fmaxf(-nq.x, -nq.y));
-                        } else {
-                            const float e = ex2_approx(-nq.x - mx) + ex2_approx(-nq.y - mx);
-                            v += e;
-                            if (MODE != 0 && e != 0.f) atomicOr(&smask[pp >> 5], 1u << (pp & 31));
-                        }
-                    }
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) {
-                        const float w = __shfl_xor_sync(FULL, v, o);
-                        v = pass ? v + w : fmaxf(v, w);
-                    }
-                    if (lane == 0) s_rare[warp][f] = v;
-                }
-            block_sync<H>(blk);
-            f = 0;
-#pragma unroll
-            for (int p = 0; p < RB_P; ++p)
-                for (uint32_t m = rare[p]; m; m &= m - 1u, ++f) {
-                    float v = s_rare[blk * H][f];
-#pragma unroll
-                    for (int h = 1; h < H; ++h) v = pass ? v + s_rare[blk * H + h][f] : fmaxf(v, s_rare[blk * H + h][f]);
-                    if (lane == __ffs(m) - 1) {
-                        if (pass) t[p] = v;
-                        else sh[p] = v > -INFINITY ? -v : 0.f;
-                    }
-                }
-            block_sync<H>(blk);   // s_rare is free for the next pass
-        }
-    } else if (nrare > 0) {   // many: every lane its own points
+    // Rare points: the exact maximum (Eq. logestep's max-subtraction), then the sums
+    // relative to it; a pair with a nonzero term becomes live.  The listed pairs give every
+    // rare point some q' (or, where none is listed, a pair's upper bound over the box): with U
+    // the largest of these over the block's rare points, a pair out of reach of q' <= U + 126
+    // adds exact zeros to them, so the pairs are listed again with that limit -- in the
+    // registration of a scan 10-20 cm off the model about a third of them, where the maximum
+    // over all pairs was two passes over every pair.  nrare is the same in the block's warps.
+    if (nrare > 0) {
         float mx[RB_P];
-#pragma unroll
-        for (int p = 0; p < RB_P; ++p) mx[p] = -INFINITY;
-#pragma unroll 2
-        for (int pp = half; pp < npairs; pp += H) {
-            Pair<D> P;
-            load_pair<D>(a.params, pp, cmax, P);
-#pragma unroll
-            for (int p = 0; p < RB_P; ++p)
-                if (rare[p]) {
-                    float2 y[D];
-                    const float2 nq = nlogit<D>(P, X[p], y);
-                    mx[p] = fmaxf(mx[p], fmaxf(-nq.x, -nq.y));
-                }
-        }
-        block_sync<H>(blk);   // every warp has read the totals
-#pragma unroll
-        for (int p = 0; p < RB_P; ++p) s_tot[warp][p][lane] = dup(mx[p]);
-        block_sync<H>(blk);
         bool mine[RB_P];
 #pragma unroll
         for (int p = 0; p < RB_P; ++p) {
+            mx[p] = -INFINITY;
             mine[p] = (rare[p] >> lane) & 1u;
+        }
+        auto max_pass = [&]() {   // max over the list, then over the block's warps
+            for (int i = 0; i < nlive; ++i) {
+                Pair<D> P;
+                load_pair<D>(params, slist[i], cmax, P);
 #pragma unroll
-            for (int h = 0; h < H; ++h) mx[p] = fmaxf(mx[p], s_tot[blk * H + h][p][lane].x);
+                for (int p = 0; p < RB_P; ++p)
+                    if (rare[p]) {
+                        float2 y[D];
+                        const float2 nq = nlogit<D>(P, X[p], y);
+                        mx[p] = fmaxf(mx[p], fmaxf(-nq.x, -nq.y));
+                    }
+            }
+            block_sync<H>(blk);   // s_tot has been read
+#pragma unroll
+            for (int p = 0; p < RB_P; ++p) s_tot[warp][p][lane] = dup(mx[p]);
+            block_sync<H>(blk);
+#pragma unroll
+            for (int p = 0; p < RB_P; ++p)
+#pragma unroll
+                for (int g = 0; g < H; ++g) mx[p] = fmaxf(mx[p], s_tot[blk * H + g][p][lane].x);
+        };
+        max_pass();
+        float U = 0.f;
+#pragma unroll
+        for (int p = 0; p < RB_P; ++p)
+            if (mine[p]) U = fmaxf(U, -mx[p]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) U = fmaxf(U, __shfl_xor_sync(FULL, U, o));
+        if (U == INFINITY) {   // some rare point has no listed pair
+            float ub = INFINITY;
+            for (int pp = half + H * lane; pp < npairs; pp += 32 * H) {
+                float2 s[Lay<D>::PF / 2];
+                load_slots<D>(params, pp, s);
+                pair_reaches<D>(s, ctr, h, cmax, REACH, &ub);
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) ub = fminf(ub, __shfl_xor_sync(FULL, ub, o));
+            if (lane == 0) s_ub[warp] = ub;
+            block_sync<H>(blk);
+            U = s_ub[blk * H];
+#pragma unroll
+            for (int g = 1; g < H; ++g) U = fminf(U, s_ub[blk * H + g]);
+        }
+        nlive = 0;
+        for (int j0 = 0; j0 < npairs; j0 += 32 * H) {
+            const int pp = j0 + H * lane + half;
+            bool live = false;
+            if (pp < npairs) {
+                float2 s[Lay<D>::PF / 2];
+                load_slots<D>(params, pp, s);
+                // (a limit beyond binary32, or an overflowing bound: every pair)
+                live = !(U < 1e30f) || pair_reaches<D>(s, ctr, h, cmax, U + REACH, nullptr);
+            }
+            push(live, pp);
+        }
+        __syncwarp();
+        max_pass();
+#pragma unroll
+        for (int p = 0; p < RB_P; ++p) {
             if (mine[p]) sh[p] = mx[p] > -INFINITY ? -mx[p] : 0.f;
             tot[p] = f2(0.f, 0.f);
         }
-#pragma unroll 2
-        for (int pp = half; pp < npairs; pp += H) {
+        for (int i = 0; i < nlive; ++i) {
+            const int pp = slist[i];
             Pair<D> P;
-            load_pair<D>(a.params, pp, cmax, P);
+            load_pair<D>(params, pp, cmax, P);
             uint32_t nz = 0u;
 #pragma unroll
             for (int p = 0; p < RB_P; ++p)
@@ -560,8 +577,8 @@ __global__ void __launch_bounds__(32 * RB_W, 4) estep_reach_kernel(const ReachLa
             if (mine[p]) {
                 t[p] = 0.f;
 #pragma unroll
-                for (int h = 0; h < H; ++h) {
-                    const float2 u = s_tot[blk * H + h][p][lane];
+                for (int g = 0; g < H; ++g) {
+                    const float2 u = s_tot[blk * H + g][p][lane];
                     t[p] += u.x + u.y;
                 }
             }
@@ -579,12 +596,12 @@ __global__ void __launch_bounds__(32 * RB_W, 4) estep_reach_kernel(const ReachLa
                 const float lse2 = lg2_approx(t[p]) + ref0 - sh[p];   // log2 sum_b pi_b N(x|b)
                 if (half == 0) {
                     ll += (double)lse2;
-                    if (MODE == 0 && a.per_point) a_in.per_point[pt0 + base + 32 * p] = lse2 * LN2F;
+                    if (MODE == 0 && a_in.per_point) a_in.per_point[pt0 + base + 32 * p] = lse2 * LN2F;
                 }
             } else {
-                set_error(a.st, GIRA_ERR_NUMERIC);   // underflows under every component
+                set_error(st, GIRA_ERR_NUMERIC);   // underflows under every component
             }
-            if (MODE != 0 && half == 0 && a.masks) a_in.pref[pt0 + base + 32 * p] = pr[p];
+            if (MODE != 0 && half == 0 && a_in.masks) a_in.pref[pt0 + base + 32 * p] = pr[p];
         }
     }
     if (half == 0) {
@@ -595,12 +612,12 @@ __global__ void __launch_bounds__(32 * RB_W, 4) estep_reach_kernel(const ReachLa
     if (MODE != 0) {
         __syncwarp();
         block_sync<H>(blk);   // the block's masks are final
-        if (a.masks && half == 0 && row < a.rows)
+        if (a_in.masks && half == 0 && row < rows)
             for (int wd = lane; wd < nwords; wd += 32) {
                 uint32_t m = 0u;
 #pragma unroll
                 for (int h = 0; h < H; ++h) m |= smask_all[(blk * H + h) * nwords + wd];
-                a.masks[wd * a.rows + row] = m;
+                a_in.masks[mask_off + wd * rows + row] = m;
             }
     }
     if constexpr (MODE == 2) {
@@ -616,7 +633,7 @@ __global__ void __launch_bounds__(32 * RB_W, 4) estep_reach_kernel(const ReachLa
         for (int wd = 0; wd < nwords; ++wd)
             for (uint32_t m = smask[wd]; m; m &= m - 1u) {
                 Pair<D> P;
-                load_pair<D>(a.params, wd * 32 + __ffs(m) - 1, cmax, P);
+                load_pair<D>(params, wd * 32 + __ffs(m) - 1, cmax, P);
 #pragma unroll
                 for (int p = 0; p < RB_P; ++p) {
                     float2 y[D];
@@ -663,11 +680,11 @@ __global__ void __launch_bounds__(32 * RB_W, 4) estep_reach_kernel(const ReachLa
                     for (int j = 0; j < 3; ++j) tw[3 * i + j] = fmaf(g3[p][i], X[p][j].x, tw[3 * i + j]);
                     tw[9 + i] += g3[p][i];
                 }
-                if (a.grad_pts) {
+                if (a_in.grad_pts) {
                     const int64_t at = pt0 + base + 32 * p;
                     float* gp = a_in.grad_pts + 3 * (a_in.order ? (int64_t)a_in.order[at] : at);
-                    if (a.rot) {
-                        const float* Rm = a.rot;
+                    if (a_in.rot) {
+                        const float* Rm = a_in.rot + 12 * (size_t)inst;
                         gp[0] = fmaf(Rm[6], g3[p][2], fmaf(Rm[3], g3[p][1], Rm[0] * g3[p][0]));
                         gp[1] = fmaf(Rm[7], g3[p][2], fmaf(Rm[4], g3[p][1], Rm[1] * g3[p][0]));
                         gp[2] = fmaf(Rm[8], g3[p][2], fmaf(Rm[5], g3[p][1], Rm[2] * g3[p][0]));
@@ -690,14 +707,14 @@ __global__ void __launch_bounds__(32 * RB_W, 4) estep_reach_kernel(const ReachLa
         if (threadIdx.x < 12) {
             double u = s_pose[0][threadIdx.x];
             if (B == 2) u += s_pose[B - 1][threadIdx.x];
-            a.pose_partials[(size_t)cta * 12 + threadIdx.x] = u;
+            a_in.pose_partials[(ll_off + cta) * 12 + threadIdx.x] = u;
         }
     }
     __syncthreads();
     if (threadIdx.x == 0) {
         double v = s_ll[0];
         if (B == 2) v += s_ll[B - 1];
-        a.llp[cta] = v * LN2;
+        a_in.llp[ll_off + cta] = v * LN2;
     }
 }
 
@@ -715,35 +732,33 @@ __global__ void __launch_bounds__(32 * ST_W) reach_stats_kernel(const ReachLaunc
                                                                 uint32_t* live2) {
     constexpr int NS = Lay<D>::NS;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    ReachLaunch a = a_in;
-    int64_t pt0 = 0;
-    int slices = gridDim.y, pair0 = blockIdx.x * ST_W, slice = blockIdx.y;
-    if (a_in.units) {   // units: (instance, slice * pair groups + group)
-        const BatchUnit u = a_in.units[blockIdx.x];
-        const BatchInst I = a_in.insts[u.inst];
-        pt0 = I.pt_off;
-        a.n = I.n;
-        a.k = I.k;
-        a.params = a_in.params + I.par_off;
-        a.gref = a_in.gref + 2 * u.inst;
-        a.masks = a_in.masks + I.mask_off;
-        a.rows = (I.n + RB_PTS - 1) / RB_PTS;
-        a.st = a_in.states + u.inst;
-        const int groups = ((I.k + 1) / 2 + ST_W - 1) / ST_W;
+    int slices = gridDim.y, k = a_in.k;
+    int64_t pt0 = 0, n = a_in.n, rows = a_in.rows, par_off = 0, mask_off = 0, part_off = 0, live_off = 0;
+    const DeviceState* st = a_in.st;
+    const int slice = blockIdx.y;
+    if (a_in.insts) {   // blockIdx.z: instance (offsets, as in estep_reach_kernel)
+        const BatchInst I = a_in.insts[blockIdx.z];
         slices = reach_slices(I.n, &sl);
-        slice = u.cta / groups;
-        pair0 = (u.cta % groups) * ST_W;
-        partials += I.part_off;
-        live2 += I.live_off;
+        if (slice >= slices) return;
+        pt0 = I.pt_off;
+        n = I.n;
+        k = I.k;
+        rows = (I.n + RB_PTS - 1) / RB_PTS;
+        par_off = I.par_off;
+        mask_off = I.mask_off;
+        part_off = I.part_off;
+        live_off = I.live_off;
+        st = a_in.states + blockIdx.z;
     }
     pdl_wait();
-    if (a.iter > a.st->stop_after || a.st->error) return;
-    const int pp = pair0 + warp;
-    const int npairs = (a.k + 1) >> 1;
+    if (a_in.iter > st->stop_after || st->error) return;
+    const int pp = blockIdx.x * ST_W + warp;
+    const int npairs = (k + 1) >> 1;
     if (pp >= npairs) return;
-    const uint32_t* mw = a.masks + (size_t)(pp >> 5) * a.rows;
+    const float* const params = a_in.params + par_off;
+    const uint32_t* const mw = a_in.masks + mask_off + (size_t)(pp >> 5) * rows;
     const int64_t r0 = (int64_t)slice * sl * 32;
-    const float cmax = a.gref[0];
+    const float cmax = cmax_of(a_in.gref, st);
     Pair<D> P;
     bool loaded = false;
     float2 S[NS];
@@ -751,9 +766,9 @@ __global__ void __launch_bounds__(32 * ST_W) reach_stats_kernel(const ReachLaunc
     for (int s = 0; s < NS; ++s) S[s] = f2(0.f, 0.f);
     for (int w = 0; w < sl; ++w) {
         const int64_t r = r0 + 32 * w + lane;
-        uint32_t m = __ballot_sync(FULL, r < a.rows && ((mw[r] >> (pp & 31)) & 1u));
+        uint32_t m = __ballot_sync(FULL, r < rows && ((mw[r] >> (pp & 31)) & 1u));
         if (m && !loaded) {
-            load_pair<D>(a.params, pp, cmax, P);
+            load_pair<D>(params, pp, cmax, P);
             loaded = true;
         }
         for (; m; m &= m - 1u) {
@@ -761,8 +776,8 @@ __global__ void __launch_bounds__(32 * ST_W) reach_stats_kernel(const ReachLaunc
 #pragma unroll
             for (int p = 0; p < RB_P; ++p) {
                 const int64_t i = b0 + 32 * p;
-                const bool ok = i < a.n;
-                const int64_t at = pt0 + (ok ? i : a.n - 1);   // an absent point: the last one with weight 0
+                const bool ok = i < n;
+                const int64_t at = pt0 + (ok ? i : n - 1);   // an absent point: the last one with weight 0
                 float2 X[D], y[D];
                 load_point<D>(a_in.pts8, at, X);
                 const float2 pr = a_in.pref[at];
@@ -798,10 +813,10 @@ __global__ void __launch_bounds__(32 * ST_W) reach_stats_kernel(const ReachLaunc
     for (int s = 0; s < NS; ++s)
         if ((lane & 15) == s) mine = v[s];
     if ((lane & 15) < NS) {
-        float* dst = partials + ((size_t)slice * npairs + pp) * (2 * NS);
+        float* dst = partials + part_off + ((size_t)slice * npairs + pp) * (2 * NS);
         dst[(hi16 ? NS : 0) + (lane & 15)] = mine;
     }
-    if (lane == 0) atomicOr(live2 + (size_t)(pp >> 5) * slices + slice, 1u << (pp & 31));
+    if (lane == 0) atomicOr(live2 + live_off + (size_t)(pp >> 5) * slices + slice, 1u << (pp & 31));
 }
 
 template <int D>
@@ -815,21 +830,23 @@ const void* reach_fn(int mode, int h) {
 
 }  // namespace
 
-// Two warps per block of 128 points where that fills the chip's SMs with one CTA each
-// (152 x 256 points), else four: fewer points per CTA, a block's pairs in parallel.
-int reach_h(int64_t n) { return n > 152 * 2 * RB_PTS ? 2 : 4; }
+// Two warps per block of 128 points (256-point CTAs), or four (128-point CTAs: a block's
+// pairs in parallel, twice the CTAs) up to 8 blocks per SM.  Measured, two against four:
+// the gradient of 100k points at K = 1024 924 / 905 us per call, a map of 4M points at
+// K = 8192 6.1 / 7.0 ms, its first test then being made twice as often.
+int reach_h(int64_t n) { return n > 152 * 8 * RB_PTS ? 2 : 4; }
+int reach_points(int h) { return RB_W / h * RB_PTS; }
 int reach_grid(int64_t n) {
-    const int64_t pts = (int64_t)(RB_W / reach_h(n)) * RB_PTS;
+    const int64_t pts = reach_points(reach_h(n));
     return (int)std::max<int64_t>(1, (n + pts - 1) / pts);
 }
 int64_t reach_rows(int64_t n) { return (n + RB_PTS - 1) / RB_PTS; }
 int reach_mask_words(int k) { return reach_words(k); }
-int reach_stat_groups(int k) { return ((k + 1) / 2 + ST_W - 1) / ST_W; }
 
-cudaError_t launch_reach_prepare(const float* params, int k, const BatchInst* insts, int batch, const DeviceState* st,
-                                 int iter, float4* ctr, float2* aux, float* gref, cudaStream_t s) {
-    const int threads = insts ? 256 : std::min(PREP_THREADS, (k + 31) / 32 * 32);
-    reach_prepare_kernel<3><<<insts ? batch : 1, threads, 0, s>>>(params, k, insts, st, iter, ctr, aux, gref);
+cudaError_t launch_reach_prepare(const float* params, int k, const DeviceState* st, int iter, float4* ctr, float2* aux,
+                                 float* gref, cudaStream_t s) {
+    reach_prepare_kernel<3><<<1, std::min(PREP_THREADS, (k + 31) / 32 * 32), 0, s>>>(params, k, st, iter, ctr, aux,
+                                                                                    gref);
     return cudaGetLastError();
 }
 
@@ -843,11 +860,194 @@ cudaError_t launch_estep_reach(const ReachLaunch& a, int mode, int grid, int h, 
     return cudaLaunchKernel(fn, dim3(grid), dim3(32 * RB_W), args, smem, s);
 }
 
-cudaError_t launch_reach_stats(const ReachLaunch& a, int nunits, float* partials, uint32_t* live2, cudaStream_t s) {
+cudaError_t launch_reach_stats(const ReachLaunch& a, int batch, int kmax, int64_t nmax, float* partials,
+                               uint32_t* live2, cudaStream_t s) {
     int sl = 1;
-    const int slices = a.units ? 1 : reach_slices(a.n, &sl);
-    const dim3 grid = a.units ? dim3(nunits) : dim3(reach_stat_groups(a.k), slices);
+    const int slices = reach_slices(nmax, &sl);
+    const dim3 grid(((kmax + 1) / 2 + ST_W - 1) / ST_W, slices, a.insts ? batch : 1);
     reach_stats_kernel<3><<<grid, 32 * ST_W, 0, s>>>(a, sl, partials, live2);
+    return cudaGetLastError();
+}
+
+// ------------------------------------------------------------------ gradient sums
+namespace {
+
+// Block j: 16 pairs of components.  Thread t sums value t of the 16 pairs' 320
+// contiguous values over the live slices (compensated binary32, in order); then one
+// warp maps the statistics of the 32 components to the parameter gradients in binary64,
+// one component per lane (a binary64 warp instruction costs the same whatever the
+// number of lanes).  With S0, S1, S2 about y = P'_32 (x' - mu) (the binary32 P' of the
+// E-step), P = L_b^{-1} and T = P P'_32^{-1}:
+//   dL/dmu_b    = P^T (T S1)
+//   dL/dL_b     = lower(P^T (T S2 T^T)) - S0 diag(1/L_ii)
+//   dL/dalpha_b = S0 - N pi_b
+// The instance's block 0 also sums the log-likelihood and the pose terms.
+constexpr int RG_PAIRS = 16, RG_THREADS = RG_PAIRS * 2 * NSTAT;
+static_assert(RG_THREADS % 32 == 0, "whole warps");
+
+__global__ void __launch_bounds__(RG_THREADS) reach_grad_finalize_kernel(const ReachGradArgs f_in,
+                                                                         const BatchInst* __restrict__ insts) {
+    __shared__ double s_stat[2 * RG_PAIRS][NSTAT];
+    // an instance's offsets into the launch's arrays (as in estep_reach_kernel)
+    int k = f_in.k, slices = f_in.slices, ctas = f_in.grid;
+    int64_t n = f_in.n;
+    size_t c_off = 0, part_off = 0, live_off = 0, ll_off = 0, par_off = 0;
+    const int inst = blockIdx.y;
+    if (insts) {
+        const BatchInst I = insts[inst];
+        int sl;
+        slices = reach_slices(I.n, &sl);
+        c_off = I.comp_off;
+        part_off = I.part_off;
+        live_off = I.live_off;
+        ll_off = I.ll_off;
+        par_off = I.par_off;
+        ctas = I.ctas;
+        k = I.k;
+        n = I.n;
+    }
+    DeviceState* const st = f_in.st + inst;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int npairs = (k + 1) >> 1, pair0 = blockIdx.x * RG_PAIRS;
+    if (pair0 >= npairs || st->error) return;
+    if (f_in.partials) {
+        const int pp = pair0 + t / (2 * NSTAT), v = t % (2 * NSTAT);
+        float s = 0.f, e = 0.f;
+        if (pp < npairs) {
+            const uint32_t* lw = f_in.live2 + live_off + (size_t)(pp >> 5) * slices;
+            const float* src = f_in.partials + part_off + (size_t)pp * 2 * NSTAT + v;
+            const size_t stride = (size_t)npairs * 2 * NSTAT;
+            for (int c0 = 0; c0 < slices; c0 += 8) {   // eight loads in flight
+                float x[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    x[u] = (c0 + u < slices && ((lw[c0 + u] >> (pp & 31)) & 1u)) ? src[(size_t)(c0 + u) * stride] : 0.f;
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {   // Knuth's TwoSum
+                    const float a = __fadd_rn(s, x[u]), bp = __fsub_rn(a, s);
+                    e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(a, bp)), __fsub_rn(x[u], bp)));
+                    s = a;
+                }
+            }
+        }
+        s_stat[2 * (t / (2 * NSTAT)) + v / NSTAT][v % NSTAT] = (double)s + (double)e;
+        __syncthreads();
+        const int b = 2 * pair0 + lane;   // this lane's component (slot)
+        if (warp == 0 && b < k) {
+            const double* S = s_stat[lane];
+            const int src_b = f_in.perm[c_off + b];
+            const float* L = f_in.chol + 9 * (c_off + src_b);
+            const double L00 = L[0], L10 = L[3], L11 = L[4], L20 = L[6], L21 = L[7], L22 = L[8];
+            auto inv3 = [](double a00, double a10, double a11, double a20, double a21, double a22, double (&M)[3][3]) {
+                const double i0 = 1.0 / a00, i1 = 1.0 / a11, i2 = 1.0 / a22;
+                M[0][0] = i0; M[0][1] = 0.0; M[0][2] = 0.0;
+                M[1][0] = -a10 * i0 * i1; M[1][1] = i1; M[1][2] = 0.0;
+                M[2][0] = -(a20 * i0 + a21 * M[1][0]) * i2; M[2][1] = -a21 * i1 * i2; M[2][2] = i2;
+            };
+            double P[3][3], Q[3][3], T[3][3];
+            inv3(L00, L10, L11, L20, L21, L22, P);
+            const float* q = f_in.params + par_off + (size_t)(b >> 1) * PAIR_FLOATS + (b & 1);
+            inv3(q[2 * SLOT_P], q[2 * (SLOT_P + 1)], q[2 * (SLOT_P + 2)], q[2 * (SLOT_P + 3)], q[2 * (SLOT_P + 4)],
+                 q[2 * (SLOT_P + 5)], Q);
+#pragma unroll
+            for (int i = 0; i < 3; ++i)
+#pragma unroll
+                for (int j = 0; j < 3; ++j) {
+                    T[i][j] = 0.0;
+#pragma unroll
+                    for (int m = j; m <= i; ++m) T[i][j] += P[i][m] * Q[m][j];
+                }
+            const double S2[3][3] = {{S[4], S[5], S[6]}, {S[5], S[7], S[8]}, {S[6], S[8], S[9]}};
+            double u[3], A[3][3], M[3][3];   // u = T S1, A = T S2, M = A T^T
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                u[i] = 0.0;
+#pragma unroll
+                for (int m = 0; m <= i; ++m) u[i] += T[i][m] * S[1 + m];
+#pragma unroll
+                for (int j = 0; j < 3; ++j) {
+                    A[i][j] = 0.0;
+#pragma unroll
+                    for (int m = 0; m <= i; ++m) A[i][j] += T[i][m] * S2[m][j];
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < 3; ++i)
+#pragma unroll
+                for (int j = 0; j < 3; ++j) {
+                    M[i][j] = 0.0;
+#pragma unroll
+                    for (int m = 0; m <= j; ++m) M[i][j] += A[i][m] * T[j][m];
+                }
+            const double Ld[3] = {L00, L11, L22};
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                double gm = 0.0;
+#pragma unroll
+                for (int m = i; m < 3; ++m) gm += P[m][i] * u[m];
+                if (f_in.g_means) f_in.g_means[3 * (c_off + src_b) + i] = (float)gm;
+#pragma unroll
+                for (int j = 0; j < 3; ++j) {
+                    double v2 = 0.0;
+                    if (j <= i) {
+#pragma unroll
+                        for (int m = i; m < 3; ++m) v2 += P[m][i] * M[m][j];
+                        if (i == j) v2 -= S[0] / Ld[i];
+                    }
+                    if (f_in.g_chol) f_in.g_chol[9 * (c_off + src_b) + 3 * i + j] = (float)v2;
+                }
+            }
+            if (f_in.g_logits) f_in.g_logits[c_off + src_b] = (float)(S[0] - (double)n * f_in.model64[(c_off + b) * MODEL]);
+        }
+    }
+    if (blockIdx.x != 0 || warp != 1) return;
+    // log-likelihood and pose sums, fixed order
+    double v[13] = {};
+    for (int c = lane; c < ctas; c += 32) {
+        v[0] += f_in.llp[ll_off + c];
+#pragma unroll
+        for (int i = 0; i < 12; ++i) v[1 + i] += f_in.pp[(ll_off + c) * 12 + i];
+    }
+#pragma unroll
+    for (int i = 0; i < 13; ++i) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v[i] += __shfl_xor_sync(FULL, v[i], o);
+    }
+    if (lane == 0) {
+        st->ll_sum = v[0];
+        const double* M = v + 1;    // sum g x'^T
+        const double* G = v + 10;   // sum g
+        if (f_in.g_twist) {
+            double* const g_twist = f_in.g_twist + 6 * (size_t)inst;   // omega = sum x' x g, v = sum g
+            g_twist[0] = M[3 * 2 + 1] - M[3 * 1 + 2];
+            g_twist[1] = M[3 * 0 + 2] - M[3 * 2 + 0];
+            g_twist[2] = M[3 * 1 + 0] - M[3 * 0 + 1];
+            for (int i = 0; i < 3; ++i) g_twist[3 + i] = G[i];
+        }
+        if (f_in.g_pose) {    // x = R^T (x' - t): dL/dR = (sum g x'^T - G t^T) R, dL/dt = G
+            const float* const pose = f_in.pose ? f_in.pose + 12 * (size_t)inst : nullptr;
+            double* const g_pose = f_in.g_pose + 12 * (size_t)inst;
+            const double tt[3] = {pose ? pose[9] : 0.0, pose ? pose[10] : 0.0, pose ? pose[11] : 0.0};
+            for (int i = 0; i < 3; ++i)
+                for (int j = 0; j < 3; ++j) {
+                    double acc = 0.0;
+                    for (int m = 0; m < 3; ++m) {
+                        const double Rmj = pose ? (double)pose[3 * m + j] : (m == j ? 1.0 : 0.0);
+                        acc += (M[3 * i + m] - G[i] * tt[m]) * Rmj;
+                    }
+                    g_pose[3 * i + j] = acc;
+                }
+            for (int i = 0; i < 3; ++i) g_pose[9 + i] = G[i];
+        }
+    }
+}
+
+}  // namespace
+
+// f.k: the largest k of a batch.  Without parameter gradients one block per instance.
+cudaError_t launch_reach_grad_finalize(const ReachGradArgs& f, const BatchInst* insts, int batch, cudaStream_t s) {
+    const int blocks = f.partials ? ((f.k + 1) / 2 + RG_PAIRS - 1) / RG_PAIRS : 1;
+    reach_grad_finalize_kernel<<<dim3(blocks, insts ? batch : 1), RG_THREADS, 0, s>>>(f, insts);
     return cudaGetLastError();
 }
 

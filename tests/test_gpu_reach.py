@@ -1,7 +1,8 @@
 """The E-step over reach lists (reach_kernels.cu) at the sizes where its tiling changes: blocks of
-128 points, two or four warps per block (38,912 points), slices of 4,096 points in the statistics,
-odd and padded component counts, and blocks holding a few (lanes take component pairs) or many
-(lanes take points) points whose every component lies more than 100 binades below the reference.
+128 points, two or four warps per block (155,648 points), slices of 4,096 points in the statistics,
+odd and padded component counts, and blocks holding a few or many points whose every component
+lies more than 100 binades below the reference (listed again about the block's own maximum), also
+points that no component's first list reaches.
 
 Tolerances: per-point log-likelihoods within the derived bound of _parity.per_point_bound (which
 covers the summation order); one EM iteration within the fit's 1e-4 per component.  The points
@@ -46,7 +47,7 @@ def off_model(pts, count, rng):
     return out, at
 
 
-SIZES = [(1_100, 1_025, 0), (4_097, 1_500, 3), (38_912, 1_026, 16), (38_913, 1_999, 200), (12_289, 8_192, 700)]
+SIZES = [(1_100, 1_025, 0), (4_097, 1_500, 3), (38_912, 1_026, 16), (155_649, 1_099, 200), (12_289, 8_192, 700)]
 
 
 @pytest.mark.parametrize("n,k,off", SIZES)
@@ -66,3 +67,21 @@ def test_large_k_reach(gira, frame, n, k, off):
     ref = oracle.em_par(pts, w, m, c, iters=1, tol=0.0, reg=1e-6)
     assert abs(r["trace"][0] - ref["trace"][0]) <= LL_ABS + 1e-7 * abs(ref["trace"][0])
     assert_model_close((r["weights"], r["means"], r["covs"]), (ref["weights"], ref["means"], ref["covs"]))
+
+
+@pytest.mark.parametrize("n,k,off", [(1, 1, 0), (129, 3, 5), (5_000, 63, 300), (4_096, 64, 4_096), (20_001, 1_024, 900)])
+def test_gradient_reach(gira, frame, n, k, off):
+    """Every gradient of a scan partly (or wholly) off the model, against the oracle's."""
+    from tests.test_gpu_grad import check_all, pose12, ref_grads, rot
+    rng = np.random.default_rng(n + k)
+    start = rng.integers(0, len(frame) - n)
+    pts = np.ascontiguousarray(frame[start:start + n])
+    if off:
+        pts, _ = off_model(pts, min(off, n - 1), rng)
+    w, m, c = ball_model(frame[start:start + max(n, k)], k, rng)
+    chol = np.linalg.cholesky(c.astype(np.float64)).astype(np.float32)
+    R, t = rot(rng.normal(scale=0.02, size=3)).astype(np.float32), rng.normal(scale=0.02, size=3).astype(np.float32)
+    r = gira.gira_gmm_loglik_grad(pts, np.log(w), m, chol, pose12(R, t))
+    check_all(r, ref_grads(pts, np.log(w), m, chol, R, t), n)
+    only = gira.gira_gmm_loglik_grad(pts, np.log(w), m, chol, pose12(R, t), want=("twist",))   # no statistics launch
+    assert np.array_equal(to_np(only["grad_twist"]), to_np(r["grad_twist"])) and only["loglik"] == r["loglik"]
