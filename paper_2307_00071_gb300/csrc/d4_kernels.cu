@@ -9,13 +9,9 @@
 // given positions (conditional mean and variance) and points resampled from
 // the joint distribution.
 //
-// The E-step here is the component-stationary design of the 3D kernel with one
-// component per lane (scalar FP32): G = ceil(K / 32) warps hold all K <= 1024
-// components, a CTA's points arrive by one TMA bulk copy (one float4 each),
-// per batch of 8 points the sums over components are reduced across lanes
-// (transpose-reduce) and warps (shared memory, one barrier), and pass 2
-// accumulates S0, S1 (4), S2 (10) about mu_b.  Logits use d = x - mu_b
-// (P'd, not P'x + b': intensity and metres-scale coordinates share a point).
+// The E-step and its statistics are reach_kernels.cu with D = 4 (logits from d = x - mu_b:
+// intensity and metre-scale coordinates share a point); here are the M-step, KInit's
+// Lloyd iterations and one-hot statistics, the regression and the sampling.
 #include <float.h>
 #include <math.h>
 
@@ -28,12 +24,6 @@ namespace gira {
 namespace {
 
 constexpr unsigned FULL = 0xffffffffu;
-constexpr int Q4 = 8;
-constexpr int PPC4_MAX = 2048;                          // points staged per CTA (64 KB)
-constexpr long long MBAR_LIMIT4 = 2000000000ll;         // bound on the TMA wait: 2 s of wall time
-constexpr float LN2F4 = 0.693147180559945309f;
-constexpr double LN2_4 = 0.693147180559945309417232121458;
-
 // lower-triangular index of (i, j), j <= i: 00,10,11,20,21,22,30,31,32,33
 __host__ __device__ constexpr int tri4(int i, int j) { return i * (i + 1) / 2 + j; }
 
@@ -42,229 +32,19 @@ __host__ __device__ __forceinline__ size_t slot4(int b, int s) {
     return (size_t)(b >> 1) * PAIR4_FLOATS + 2 * s + (b & 1);
 }
 
-// CH = 0: the whole E-step of one CTA (every component); CH = 1: pass A of a
-// chunk (per-point sums only); CH = 2: pass B of a chunk (statistics from pref).
-template <bool STATS, int CH = 0>
-__global__ void __launch_bounds__(512, 1) estep4_kernel(const EStep4Launch a) {
-    extern __shared__ __align__(128) unsigned char dsm4[];
-    __shared__ __align__(8) uint64_t bar_tma;
-    __shared__ float red_sum[2][16][Q4];
-    __shared__ float red_aux[2][16][Q4];
-    __shared__ float s_cmax[16], s_wsum[16];
-    __shared__ int s_skip, s_norm, s_dead;
-    constexpr int LPQ = 32 / Q4;
-    const int G = blockDim.x >> 5;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int chunk = (CH != 0) ? (int)blockIdx.y : 0;
-    const int pr = threadIdx.x;   // this lane's component pair: components 2 pr, 2 pr + 1 of the chunk
-    const int k_here = (CH != 0) ? min(CHUNK4, a.k - chunk * CHUNK4) : a.k;
-    const float* params = a.params + (size_t)chunk * (CHUNK4 / 2) * PAIR4_FLOATS;
-    const int64_t begin = (int64_t)blockIdx.x * a.pts_per_cta;
-    const int64_t end = min(a.n, begin + a.pts_per_cta);
-    const int npts = (int)(end - begin);
-    const int nb = (npts + Q4 - 1) / Q4;
-    const float4* spts = reinterpret_cast<const float4*>(dsm4);   // (x,x,y,y)(z,z,w,w) per point
-    if (threadIdx.x == 0) {
-        // the points are never written by the kernel this one may overlap
-        // (dependent launch), so their copy starts before the wait below
-        mbar_init(&bar_tma, 1);
-        mbar_fence_init();
-        mbar_expect_tx(&bar_tma, (uint32_t)npts * 32u);
-        tma_load_1d(reinterpret_cast<void*>(dsm4), a.pts8 + 2 * begin, (uint32_t)npts * 32u, &bar_tma);
-    }
-    pdl_wait();   // the parameters and the state written by the previous kernel
-    if (threadIdx.x == 0) {
-        s_skip = (a.iter > a.st->stop_after) || (a.st->error != 0);
-        s_norm = a.st->w_raw;
-        s_dead = 0;
-    }
-    __syncthreads();
-    if (s_skip) {   // let the copy land before leaving
-        if (threadIdx.x == 0) mbar_wait_bounded(&bar_tma, 0u, MBAR_LIMIT4);
-        return;
-    }
-    pdl_allow_next();
-    // ---- this lane's pair -> registers (padding components: c = -inf, never contribute)
-    float2 P[10], nmu[4], c, w;
-    {
-        const float4* src = reinterpret_cast<const float4*>(params + (size_t)pr * PAIR4_FLOATS);
-        float4 v[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) v[i] = src[i];
-        const float2* f = reinterpret_cast<const float2*>(v);
-#pragma unroll
-        for (int i = 0; i < 10; ++i) P[i] = f[SLOT4_P + i];
-        c = f[SLOT4_C];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) nmu[i] = f[SLOT4_NMU + i];
-        w = f[SLOT4_W];
-    }
-    float cm = fmaxf(c.x, c.y), ws = w.x + w.y;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        cm = fmaxf(cm, __shfl_xor_sync(FULL, cm, o));
-        ws += __shfl_xor_sync(FULL, ws, o);
-    }
-    if (lane == 0) {
-        s_cmax[warp] = cm;
-        s_wsum[warp] = ws;
-    }
-    if (!mbar_wait_bounded(&bar_tma, 0u, MBAR_LIMIT4)) s_dead = 1;
-    __syncthreads();
-    if (s_dead) {
-        if (threadIdx.x == 0) {
-            set_error(a.st, GIRA_ERR_TIMEOUT);
-            mbar_wait_bounded(&bar_tma, 0u, MBAR_LIMIT4);
-        }
-        return;
-    }
-    float cmax = s_cmax[0], wsum = s_wsum[0];
-    for (int i = 1; i < G; ++i) {
-        cmax = fmaxf(cmax, s_cmax[i]);
-        wsum += s_wsum[i];
-    }
-    if (CH != 0) cmax = a.gref[0];   // chunks: one reference for all K components
-    const float2 cc = f2(cmax - c.x, cmax - c.y);   // >= 0; +inf for padding
-    const float ref0 = s_norm ? cmax - __log2f(wsum) : cmax;
-    float2 S[NSTAT4];   // statistics of the lane's two components, packed
-    if (STATS)
-#pragma unroll
-        for (int i = 0; i < NSTAT4; ++i) S[i] = f2(0.f, 0.f);
-    double ll_acc = 0.0;
-    const int myq = q_of_lane<Q4>(lane);
-    const bool owner = (warp == 0) && ((lane & (LPQ - 1)) == 0);
+constexpr double ALPHA4 = 0.84932180028801904272;     // sqrt(log2(e) / 2)
+constexpr double LOG2_2PI4 = 2.6514961294723187980;   // log2(2 pi)
 
-    // q' = |P'(x - mu)|^2 + (cmax - c) for both components: minus the base-2
-    // logit relative to cmax (packed: one FFMA2 / FADD2 / FMUL2 per pair)
-    auto qform = [&](int li) {
-        const float4 xy = spts[2 * li], zw = spts[2 * li + 1];
-        const float2 d0 = add2(f2(xy.x, xy.y), nmu[0]), d1 = add2(f2(xy.z, xy.w), nmu[1]);
-        const float2 d2 = add2(f2(zw.x, zw.y), nmu[2]), d3 = add2(f2(zw.z, zw.w), nmu[3]);
-        const float2 y0 = mul2(P[0], d0);
-        const float2 y1 = fma2(P[2], d1, mul2(P[1], d0));
-        const float2 y2 = fma2(P[5], d2, fma2(P[4], d1, mul2(P[3], d0)));
-        const float2 y3 = fma2(P[9], d3, fma2(P[8], d2, fma2(P[7], d1, mul2(P[6], d0))));
-        return fma2(y3, y3, fma2(y2, y2, fma2(y1, y1, fma2(y0, y0, cc))));
-    };
-    // pass 2: S0 = sum g, S1 = sum g d, S2 = sum g d d^T about mu_b for both
-    // components at once (packed); g = e * R with R the owner lane's 1 / total
-    // (r != nullptr) or already folded into e (pass B)
-    auto accumulate = [&](int lb, int nvalid, const float2 (&Eq)[Q4], const float* r) {
-#pragma unroll
-        for (int q = 0; q < Q4; ++q) {
-            const int li = (q < nvalid) ? lb + q : lb;
-            const float4 xy = spts[2 * li], zw = spts[2 * li + 1];
-            const float2 g = r ? mul2(Eq[q], dup(__shfl_sync(FULL, *r, q * LPQ))) : Eq[q];
-            const float2 d[4] = {add2(f2(xy.x, xy.y), nmu[0]), add2(f2(xy.z, xy.w), nmu[1]),
-                                 add2(f2(zw.x, zw.y), nmu[2]), add2(f2(zw.z, zw.w), nmu[3])};
-            float2 gd[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) gd[i] = mul2(g, d[i]);
-            S[0] = add2(S[0], g);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) S[1 + i] = add2(S[1 + i], gd[i]);
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = i; j < 4; ++j) S[5 + sym4(i, j)] = fma2(gd[i], d[j], S[5 + sym4(i, j)]);
-        }
-    };
-    float2 E[Q4];
-    for (int t = 0; t < nb; ++t) {
-        const int lb = t * Q4, nvalid = min(Q4, npts - lb);
-        if (CH == 2) {
-            // pass B: e relative to the point's reference, times 1 / total, into the statistics
-#pragma unroll
-            for (int q = 0; q < Q4; ++q) {
-                const float2 prq = (q < nvalid) ? a.pref[begin + lb + q] : f2(0.f, 0.f);
-                const float2 nq = qform((q < nvalid) ? lb + q : lb);
-                E[q] = f2(ex2_approx(prq.x - nq.x) * prq.y, ex2_approx(prq.x - nq.y) * prq.y);
-            }
-            if (STATS) accumulate(lb, nvalid, E, nullptr);
-            continue;
-        }
-        // pass 1: e for (point, own components), per-point sums over the CTA
-        float part[Q4];
-#pragma unroll
-        for (int q = 0; q < Q4; ++q) {
-            const float2 nq = qform((q < nvalid) ? lb + q : lb);
-            E[q] = f2(ex2_approx(-nq.x), ex2_approx(-nq.y));
-            part[q] = E[q].x + E[q].y;
-        }
-        const float wt = warp_transpose_reduce<Q4>(part, lane, AddOp());
-        if ((lane & (LPQ - 1)) == 0) red_sum[t & 1][warp][myq] = wt;
-        __syncthreads();
-        float tot = red_sum[t & 1][0][myq];
-        for (int i = 1; i < G; ++i) tot += red_sum[t & 1][i][myq];
-        const bool myvalid = myq < nvalid;
-        if (CH == 1) {   // pass A: the chunk's sum for each point
-            if (owner && myvalid) a.psum[(size_t)chunk * a.n + begin + lb + myq] = tot;
-            continue;
-        }
-        float ref = ref0;
-        if (__any_sync(FULL, myvalid && !(tot >= 0x1p-100f))) {
-            // rare: a point > 100 binades below cmax everywhere; exact per-point maximum
-            float m[Q4];
-#pragma unroll
-            for (int q = 0; q < Q4; ++q) {
-                const float2 nq = qform((q < nvalid) ? lb + q : lb);
-                E[q] = f2(-nq.x, -nq.y);
-                m[q] = fmaxf(E[q].x, E[q].y);
-            }
-            float mt = warp_transpose_reduce<Q4>(m, lane, MaxOp());
-            if ((lane & (LPQ - 1)) == 0) red_aux[0][warp][myq] = mt;
-            __syncthreads();
-            mt = red_aux[0][0][myq];
-            for (int i = 1; i < G; ++i) mt = fmaxf(mt, red_aux[0][i][myq]);
-            float p2[Q4];
-#pragma unroll
-            for (int q = 0; q < Q4; ++q) {
-                float mq = __shfl_sync(FULL, mt, q * LPQ);
-                mq = (mq > -INFINITY) ? mq : 0.f;
-                E[q] = f2(ex2_approx(E[q].x - mq), ex2_approx(E[q].y - mq));
-                p2[q] = E[q].x + E[q].y;
-            }
-            const float w2 = warp_transpose_reduce<Q4>(p2, lane, AddOp());
-            if ((lane & (LPQ - 1)) == 0) red_aux[1][warp][myq] = w2;
-            __syncthreads();
-            tot = red_aux[1][0][myq];
-            for (int i = 1; i < G; ++i) tot += red_aux[1][i][myq];
-            if (myvalid && !(mt > -INFINITY)) set_error(a.st, GIRA_ERR_NUMERIC);
-            ref = ref0 + ((mt > -INFINITY) ? mt : 0.f);
-        }
-        const bool ok = myvalid && tot > 0.f;
-        const float lse2 = lg2_approx(tot) + ref;
-        if (owner && ok) {
-            ll_acc += (double)lse2;
-            if (!STATS && a.per_point) a.per_point[begin + lb + myq] = lse2 * LN2F4;
-        }
-        const float r = ok ? __frcp_rn(tot) : 0.f;
-        if (STATS) accumulate(lb, nvalid, E, &r);
-    }
-    if (STATS) {
-        const int kc = (CH != 0) ? CHUNK4 : a.k;   // components per partial block
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int b = 2 * pr + h;
-            if (b < k_here) {
-                float* dst = a.partials + (((size_t)chunk * gridDim.x + blockIdx.x) * kc + b) * NSTAT4;
-#pragma unroll
-                for (int i = 0; i < NSTAT4; ++i) dst[i] = h ? S[i].y : S[i].x;
-            }
-        }
-    }
-    if (CH != 0) return;
-    if (warp == 0) {
-        double v = ll_acc;
-#pragma unroll
-        for (int o = LPQ; o < 32; o <<= 1) v += __shfl_xor_sync(FULL, v, o);
-        if (lane == 0) a.ll_partials[blockIdx.x] = v * LN2_4;
-    }
+// A lower bound of sigma_min(P')^2 = alpha^2 / lambda_max(Sigma) from the sum of Sigma's
+// squared entries: lambda_max <= ||Sigma||_F (and >= half of it).
+__device__ __forceinline__ float sigma_min_sq_bound4(double fro2) {
+    return (float)(ALPHA4 * ALPHA4) / (sqrtf((float)fro2) * (1.f + 1e-4f)) * (1.f - 1e-4f);
 }
 
 // From (w, mu, Sigma) in binary64: Cholesky, P = L^{-1}, the base-2 constants.
+// report: the caller's index of the component (slot b may hold another one).
 __device__ bool build_component4(int b, double w, const double mu[4], const double S[16], float* params,
-                                 double* model64, DeviceState* st) {
+                                 double* model64, DeviceState* st, int report) {
     double L[16] = {0};
     bool pd = true;
     for (int j = 0; j < 4 && pd; ++j) {
@@ -279,7 +59,7 @@ __device__ bool build_component4(int b, double w, const double mu[4], const doub
         }
     }
     if (!pd) {
-        atomicMin(&st->bad_component, b);
+        atomicMin(&st->bad_component, report);
         set_error(st, GIRA_ERR_NOT_PD);
         return false;
     }
@@ -290,12 +70,13 @@ __device__ bool build_component4(int b, double w, const double mu[4], const doub
             for (int k = cidx; k < i; ++k) t -= L[4 * i + k] * P[4 * k + cidx];
             P[4 * i + cidx] = t / L[4 * i + i];
         }
-    const double alpha = 0.84932180028801904272;   // sqrt(log2(e) / 2)
-    const double LOG2_2PI = 2.6514961294723187980;  // log2(2 pi)
+    double fro2 = 0.0;
+    for (int i = 0; i < 16; ++i) fro2 += S[i] * S[i];
+    params[slot4(b, SLOT4_S)] = sigma_min_sq_bound4(fro2);
     for (int i = 0; i < 4; ++i)
-        for (int j = 0; j <= i; ++j) params[slot4(b, SLOT4_P + tri4(i, j))] = (float)(alpha * P[4 * i + j]);
+        for (int j = 0; j <= i; ++j) params[slot4(b, SLOT4_P + tri4(i, j))] = (float)(ALPHA4 * P[4 * i + j]);
     // log2 w + sum_j log2 P_jj - (4/2) log2(2 pi)
-    params[slot4(b, SLOT4_C)] = (float)(log2(w * (P[0] * P[5] * P[10] * P[15])) - 2.0 * LOG2_2PI);
+    params[slot4(b, SLOT4_C)] = (float)(log2(w * (P[0] * P[5] * P[10] * P[15])) - 2.0 * LOG2_2PI4);
     for (int i = 0; i < 4; ++i) params[slot4(b, SLOT4_NMU + i)] = -(float)mu[i];
     params[slot4(b, SLOT4_W)] = (float)w;
     double* m = model64 + (size_t)b * MODEL4;
@@ -306,85 +87,220 @@ __device__ bool build_component4(int b, double w, const double mu[4], const doub
     return true;
 }
 
-// One block per component: fixed-order binary64 sum of its per-CTA partials
-// (32 slices, binary32 groups of 8 inside a slice), then the M-step and build.
-// The E-step kept mu_b (as binary32) as the shift, so the statistics are about
-// the previous mean, and the update un-shifts them exactly in binary64.
-__global__ void __launch_bounds__(NSTAT4 * 32) reduce_finalize4_kernel(
-    const float* __restrict__ partials, int grid, int kc, const double* __restrict__ llp, int ll_count,
-    const double* __restrict__ stats64, const float4* __restrict__ shift4, int k, int64_t n, double reg, double tol,
-    double* model64, float* params, double* trace, DeviceState* st, int iter, int em) {
-    __shared__ double part[32][NSTAT4];
-    __shared__ double Sb[NSTAT4];
-    __shared__ int s_skip;
+// The M-step of one pair of components per block.  Sums: warp w adds, value by lane, the
+// pair's live rows among the w-th quarter of the slices (compensated binary32, Knuth's
+// TwoSum), warp 0 joins the quarters in order.  Update: warp 0, lanes 16 h + 4 i + j for
+// entry (i, j) of component h's 4 x 4 matrices, every stage in parallel lanes through
+// shared memory: GB300 issues one binary64 warp instruction per 64 cycles per warp whatever
+// the number of active lanes, so a stage costs what one entry costs (~170 instructions in
+// all; one thread per component, one block each, ran ~500 in a row: 58 us per launch at
+// K = 512, 9 us now).  The statistics are about y = P'(x - s) with the binary32 P' of
+// the E-step (a component thin in one direction keeps that direction's digits): with M =
+// P'^{-1}, mu = (S0 / N_b) s + M ybar, Sigma = M (S2 / N_b - ybar ybar^T) M^T + reg I; one-hot
+// statistics are about shift4 with M = I.
+struct Fin4Args {
+    const float* partials;
+    const uint32_t* live2;
+    int slices;
+    const double* llp;
+    int ll_count;
+    const double* stats64;
+    const float4* shift4;
+    int k;
+    int64_t n;
+    double reg, tol;
+    double* model64;
+    float* params;
+    double* trace;
+    const int* perm;
+    DeviceState* st;
+    int iter, em;
+};
+constexpr int FIN4_WARPS = 4;
+__global__ void __launch_bounds__(32 * FIN4_WARPS) reduce_finalize4_kernel(const Fin4Args f) {
+    __shared__ float s_hi[FIN4_WARPS][2][32];
+    __shared__ double s_stat[2][NSTAT4], s_P[2][10], s_r[2][5], s_M[2][16], s_C[2][16], s_A[2][16], s_mu[2][4];
+    __shared__ double s_ll[FIN4_WARPS];
+    DeviceState* const st = f.st;
     pdl_wait();         // the E-step's partials (dependent launch)
-    pdl_allow_next();   // the next E-step may stage its points meanwhile
-    if (threadIdx.x == 0) s_skip = (em && iter > st->stop_after) || st->error != 0;
-    __syncthreads();
-    if (s_skip) return;
-    const int b = blockIdx.x, t = threadIdx.x;
-    if (partials) {
-        const int o = t % NSTAT4, q = t / NSTAT4;
-        const int c0 = q * grid / 32, c1 = (q + 1) * grid / 32;
-        const float* src = partials + ((size_t)(b / kc) * grid * kc + b % kc) * NSTAT4 + o;
-        double acc = 0.0;
-        for (int cta = c0; cta < c1; cta += 8) {
-            float f = 0.f;
+    pdl_allow_next();
+    if ((f.em && f.iter > st->stop_after) || st->error) return;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int pp = blockIdx.x;
+    const bool white = f.partials != nullptr;
+    if (white) {
+        const int npairs = (f.k + 1) >> 1;
+        const uint32_t* lw = f.live2 + (size_t)(pp >> 5) * f.slices;
+        const float* src = f.partials + (size_t)pp * 2 * NSTAT4 + lane;
+        const size_t stride = (size_t)npairs * 2 * NSTAT4;
+        const int c0 = warp * f.slices / FIN4_WARPS, c1 = (warp + 1) * f.slices / FIN4_WARPS;
+        float s = 0.f, e = 0.f;
+        auto add = [&](float x) {
+            const float a = __fadd_rn(s, x), bp = __fsub_rn(a, s);
+            e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(a, bp)), __fsub_rn(x, bp)));
+            s = a;
+        };
+        for (int c = c0; c < c1; c += 8) {   // eight loads in flight
+            float x[8];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) f += (cta + u < c1) ? __ldcg(src + (size_t)(cta + u) * kc * NSTAT4) : 0.f;
-            acc += (double)f;
+            for (int u = 0; u < 8; ++u)
+                x[u] = (c + u < c1 && lane < 2 * NSTAT4 && ((lw[c + u] >> (pp & 31)) & 1u)) ? src[(size_t)(c + u) * stride]
+                                                                                           : 0.f;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) add(x[u]);
         }
-        part[q][o] = acc;
+        s_hi[warp][0][lane] = s;
+        s_hi[warp][1][lane] = e;
         __syncthreads();
-        if (t < NSTAT4) {
-            double v = 0.0;
-            for (int q2 = 0; q2 < 32; ++q2) v += part[q2][t];
-            Sb[t] = v;
-        }
-    } else if (t < NSTAT4) {
-        Sb[t] = stats64[(size_t)b * NSTAT4 + t];
-    }
-    __syncthreads();
-    if (t == 0) {
-        double s[4];
-        if (shift4) {
-            const float4 v = shift4[b];
-            s[0] = v.x; s[1] = v.y; s[2] = v.z; s[3] = v.w;
-        } else {
-            for (int i = 0; i < 4; ++i) s[i] = -(double)params[slot4(b, SLOT4_NMU + i)];
-        }
-        const double s0 = Sb[0];
-        const double nbw = s0 + 10.0 * DBL_EPSILON;
-        const double inv = 1.0 / nbw;
-        double mu[4], dl[4];
-        for (int i = 0; i < 4; ++i) {
-            mu[i] = (s0 * s[i] + Sb[1 + i]) * inv;
-            dl[i] = mu[i] - s[i];
-        }
-        double S[16];
-        for (int i = 0; i < 4; ++i)
-            for (int j = i; j < 4; ++j) {
-                const double v = Sb[5 + sym4(i, j)] - dl[i] * Sb[1 + j] - Sb[1 + i] * dl[j] + s0 * dl[i] * dl[j];
-                S[4 * i + j] = S[4 * j + i] = v * inv + ((i == j) ? reg : 0.0);
-            }
-        build_component4(b, nbw, mu, S, params, model64, st);
-        if (b == 0) st->w_raw = 1;
-    }
-    if (em && b == 0 && t >= 32 && t < 64) {   // warp 1: log-likelihood, trace, convergence
-        const int lane = t - 32;
-        double v = 0.0;
-        for (int cta = lane; cta < ll_count; cta += 32) v += llp[cta];
+        if (warp == 0) {
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
-        if (lane == 0) {
-            st->ll_sum = v;
-            const double ll = v / (double)n;
-            trace[iter - 1] = ll;
-            if (iter > 1 && fabs(ll - st->prev_ll) < tol) st->stop_after = iter;
-            st->prev_ll = ll;
-            st->iters_done = iter;
+            for (int w = 1; w < FIN4_WARPS; ++w) {
+                e = __fadd_rn(e, s_hi[w][1][lane]);
+                add(s_hi[w][0][lane]);
+            }
+            if (lane < 2 * NSTAT4) s_stat[lane / NSTAT4][lane % NSTAT4] = (double)s + (double)e;
         }
+    } else if (warp == 0 && lane < 2 * NSTAT4 && 2 * pp + lane / NSTAT4 < f.k) {
+        s_stat[lane / NSTAT4][lane % NSTAT4] = f.stats64[(size_t)2 * pp * NSTAT4 + lane];
     }
+    if (warp == 0) {
+        const int h = lane >> 4, l = lane & 15, i = l >> 2, j = l & 3;
+        const int b = 2 * pp + h;
+        const bool on = b < f.k;
+        double* P = s_P[h];
+        double* r = s_r[h];
+        double* M = s_M[h];
+        double* C = s_C[h];
+        double* A = s_A[h];
+        double* mu = s_mu[h];
+        const double* S = s_stat[h];
+        if (on && l < 10) P[l] = white ? (double)f.params[slot4(b, SLOT4_P + l)] : 0.0;
+        __syncwarp();
+        const double nbw = on ? S[0] + 10.0 * DBL_EPSILON : 1.0;
+        if (on && l < 5) r[l] = __drcp_rn(l == 4 ? nbw : white ? P[tri4(l, l)] : 1.0);
+        __syncwarp();
+        const double inv = on ? r[4] : 0.0;
+        // M = P'^{-1}, row by row (columns in parallel)
+        if (on) M[l] = i == j ? r[i] : 0.0;
+        __syncwarp();
+        if (white)
+            for (int row = 1; row < 4; ++row) {
+                if (on && i == row && j < row) {
+                    double v = 0.0;
+                    for (int m = j; m < row; ++m) v = __fma_rn(P[tri4(row, m)], M[4 * m + j], v);
+                    M[l] = -v * r[row];
+                }
+                __syncwarp();
+            }
+        // C = S2 / N_b - ybar ybar^T
+        if (on) C[l] = __fma_rn(-(S[1 + i] * inv), S[1 + j] * inv, S[5 + sym4(min(i, j), max(i, j))] * inv);
+        __syncwarp();
+        // mu = (S0 / N_b) s + M ybar (lanes 0 .. 3), A = M C
+        if (on && l < 4) {
+            double s;
+            if (white) s = -(double)f.params[slot4(b, SLOT4_NMU + l)];
+            else s = l == 0 ? f.shift4[b].x : l == 1 ? f.shift4[b].y : l == 2 ? f.shift4[b].z : f.shift4[b].w;
+            s *= S[0] * inv;   // sum_n r x / N_b: 0 for a component without support
+            for (int m = 0; m <= l; ++m) s = __fma_rn(M[4 * l + m], S[1 + m] * inv, s);
+            mu[l] = s;
+        }
+        double v = 0.0;
+        if (on)
+#pragma unroll
+            for (int m = 0; m < 4; ++m) v = __fma_rn(M[4 * i + m], C[4 * m + j], v);
+        if (on) A[l] = v;
+        __syncwarp();
+        // Sigma = A M^T + reg I (symmetric: entry (i, j) computed as (max, min))
+        if (on) {
+            const int hi = max(i, j), lo = min(i, j);
+            v = i == j ? f.reg : 0.0;
+#pragma unroll
+            for (int m = 0; m < 4; ++m) v = __fma_rn(A[4 * hi + m], M[4 * lo + m], v);
+            C[l] = v;
+        }
+        __syncwarp();
+        const double sig = on ? C[l] : 0.0;
+        double fro2 = sig * sig;
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) fro2 += __shfl_xor_sync(FULL, fro2, o);
+        // Cholesky by Schur complements, r = the pivots' reciprocal square roots; A = L
+        bool pd = true;
+        double prod = 1.0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const double piv = on ? C[5 * q] : 1.0;
+            pd = pd && piv > 0.0;
+            const double u = rsqrt(piv);
+            prod *= u;
+            if (on && l == 0) r[q] = u;
+            if (on && j == q && i >= q) A[l] = C[l] * u;
+            __syncwarp();
+            if (on && i > q && j > q) C[l] = __fma_rn(-A[4 * i + q], A[4 * j + q], C[l]);
+            __syncwarp();
+        }
+        if (on && !pd && l == 0) {
+            atomicMin(&st->bad_component, f.perm ? f.perm[b] : b);
+            set_error(st, GIRA_ERR_NOT_PD);
+        }
+        const bool ok = on && pd;
+        // P = L^{-1}
+        if (ok) M[l] = i == j ? r[i] : 0.0;
+        __syncwarp();
+        for (int row = 1; row < 4; ++row) {
+            if (ok && i == row && j < row) {
+                v = 0.0;
+                for (int m = j; m < row; ++m) v = __fma_rn(A[4 * row + m], M[4 * m + j], v);
+                M[l] = -v * r[row];
+            }
+            __syncwarp();
+        }
+        const float c32 = (float)(log2(nbw * prod) - 2.0 * LOG2_2PI4);
+        if (ok) {
+            if (j <= i) f.params[slot4(b, SLOT4_P + tri4(i, j))] = (float)(ALPHA4 * M[l]);
+            if (l < 4) f.params[slot4(b, SLOT4_NMU + l)] = -(float)mu[l];
+            if (l == 4) f.params[slot4(b, SLOT4_C)] = c32;
+            if (l == 5) f.params[slot4(b, SLOT4_W)] = (float)nbw;
+            if (l == 6) f.params[slot4(b, SLOT4_S)] = sigma_min_sq_bound4(fro2);
+            double* m = f.model64 + (size_t)b * MODEL4;
+            if (l == 7) m[0] = nbw;
+            if (l < 4) m[1 + l] = mu[l];
+            if (i <= j) m[5 + sym4(i, j)] = sig;
+        }
+        if (t == 0 && pp == 0) st->w_raw = 1;
+    }
+    if (!f.em || pp != 0) return;
+    // log-likelihood, trace, convergence (fixed order)
+    double v = 0.0;
+    if (warp > 0)
+        for (int c = t - 32; c < f.ll_count; c += 32 * (FIN4_WARPS - 1)) v += f.llp[c];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
+    if (lane == 0) s_ll[warp] = v;
+    __syncthreads();
+    if (t == 32) {
+        v = 0.0;
+        for (int w = 1; w < FIN4_WARPS; ++w) v += s_ll[w];
+        st->ll_sum = v;
+        const double ll = v / (double)f.n;
+        f.trace[f.iter - 1] = ll;
+        if (f.iter > 1 && fabs(ll - st->prev_ll) < f.tol) st->stop_after = f.iter;
+        st->prev_ll = ll;
+        st->iters_done = f.iter;
+    }
+}
+
+// Slot s takes component perm[s]: its row of `old` rebuilt into slot s.
+__global__ void rebuild_components4_kernel(const double* __restrict__ old, const int* __restrict__ perm, int k,
+                                           double* model64, float* params, DeviceState* st) {
+    const int slot = blockIdx.x * blockDim.x + threadIdx.x;
+    if (slot >= k) return;
+    const int b = perm[slot];
+    if (!GIRA_IN(b >= 0 && b < k, st)) return;
+    const double* r = old + (size_t)b * MODEL4;
+    double S[16];
+    for (int i = 0; i < 4; ++i)
+        for (int j = 0; j < 4; ++j) S[4 * i + j] = r[5 + sym4(min(i, j), max(i, j))];
+    build_component4(slot, r[0], r + 1, S, params, model64, st, b);
 }
 
 __global__ void params_from_model4_kernel(const float* __restrict__ w, const float* __restrict__ mu,
@@ -408,12 +324,12 @@ __global__ void params_from_model4_kernel(const float* __restrict__ w, const flo
         }
     if (!fin) { set_error(st, GIRA_ERR_NONFINITE_INPUT); return; }
     if (!(pi > 0.0)) { set_error(st, GIRA_ERR_INVALID_ARG); return; }
-    build_component4(b, pi, m, S, params, model64, st);
+    build_component4(b, pi, m, S, params, model64, st, b);
 }
 
 __global__ void model_out4_kernel(const double* __restrict__ model64, int k, float* w, float* mu, float* cov,
-                                  const DeviceState* st) {
-    __shared__ double s_part[2];
+                                  const int* __restrict__ perm, const DeviceState* st) {
+    __shared__ double s_part[2];   // (the same sum in every block)
     double part = 0.0;
     for (int a2 = threadIdx.x; a2 < k; a2 += blockDim.x) part += model64[(size_t)a2 * MODEL4];
 #pragma unroll
@@ -421,8 +337,10 @@ __global__ void model_out4_kernel(const double* __restrict__ model64, int k, flo
     if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = part;
     __syncthreads();
     const double nsum = s_part[0] + s_part[1];
-    for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < k; b += gridDim.x * blockDim.x) {
-        const double* m = model64 + (size_t)b * MODEL4;
+    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < k; s += gridDim.x * blockDim.x) {
+        const int b = perm ? perm[s] : s;   // slot s holds the caller's component b
+        if (!GIRA_IN(b >= 0 && b < k, const_cast<DeviceState*>(st))) continue;
+        const double* m = model64 + (size_t)s * MODEL4;
         w[b] = (float)(st->w_raw ? m[0] / nsum : m[0]);
         for (int i = 0; i < 4; ++i) mu[4 * (size_t)b + i] = (float)m[1 + i];
         for (int i = 0; i < 4; ++i)
@@ -664,86 +582,6 @@ __global__ void sample_kernel(int64_t m, int k, int d, const float* __restrict__
     if (comp) comp[i] = b;
 }
 
-// ------------------------------------------------------------------ chunks (K above MAX_K4_DIRECT)
-// gref[0] = max_b c_b over all k components; gref[1] = the log-likelihood
-// reference (gref[0] - log2 sum_a w_a once the weights are raw N_b).
-__global__ void chunk_ref4_kernel(const float* __restrict__ params, int k, const DeviceState* st, float* gref) {
-    __shared__ float s_m[8];
-    __shared__ double s_w[8];
-    float m = -INFINITY;
-    double w = 0.0;
-    for (int b = threadIdx.x; b < k; b += blockDim.x) {
-        m = fmaxf(m, params[slot4(b, SLOT4_C)]);
-        w += (double)params[slot4(b, SLOT4_W)];
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        m = fmaxf(m, __shfl_xor_sync(FULL, m, o));
-        w += __shfl_xor_sync(FULL, w, o);
-    }
-    if ((threadIdx.x & 31) == 0) {
-        s_m[threadIdx.x >> 5] = m;
-        s_w[threadIdx.x >> 5] = w;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float mm = s_m[0];
-        double ww = s_w[0];
-        for (int i = 1; i < (int)(blockDim.x >> 5); ++i) {
-            mm = fmaxf(mm, s_m[i]);
-            ww += s_w[i];
-        }
-        gref[0] = mm;
-        gref[1] = st->w_raw ? (float)((double)mm - log2(ww)) : mm;
-    }
-}
-
-// One warp per listed point (total over the chunks below 2^-100): the exact
-// maximum of the logits over all k components, then (shift, 1 / sum) relative
-// to it, with the E-step's arithmetic.
-__global__ void chunk_exact4_kernel(const float4* __restrict__ pts8, const float* __restrict__ params, int k,
-                                    const float* __restrict__ gref, const int* __restrict__ flags,
-                                    const int* __restrict__ flag_count, float2* pref, double* llpt, DeviceState* st) {
-    const int count = *flag_count;
-    const float cmax = gref[0], ref0 = gref[1];
-    const int lane = threadIdx.x & 31;
-    const int wg = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
-    for (int f = wg; f < count; f += nw) {
-        const int64_t i = flags[f];
-        const float4 xy = pts8[2 * i], zw = pts8[2 * i + 1];
-        const float x[4] = {xy.x, xy.z, zw.x, zw.z};
-        auto nlog = [&](int b) {   // q' = |P'(x - mu)|^2 + (cmax - c_b)
-            float P[10], d[4];
-            for (int j = 0; j < 10; ++j) P[j] = params[slot4(b, SLOT4_P + j)];
-            for (int j = 0; j < 4; ++j) d[j] = x[j] + params[slot4(b, SLOT4_NMU + j)];
-            const float y0 = P[0] * d[0];
-            const float y1 = fmaf(P[2], d[1], P[1] * d[0]);
-            const float y2 = fmaf(P[5], d[2], fmaf(P[4], d[1], P[3] * d[0]));
-            const float y3 = fmaf(P[9], d[3], fmaf(P[8], d[2], fmaf(P[7], d[1], P[6] * d[0])));
-            const float cc = cmax - params[slot4(b, SLOT4_C)];
-            return fmaf(y3, y3, fmaf(y2, y2, fmaf(y1, y1, fmaf(y0, y0, cc))));
-        };
-        float mx = -INFINITY;
-        for (int b = lane; b < k; b += 32) mx = fmaxf(mx, -nlog(b));
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(FULL, mx, o));
-        float sum = 0.f;
-        if (mx > -INFINITY)
-            for (int b = lane; b < k; b += 32) sum += ex2_approx(-nlog(b) - mx);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(FULL, sum, o);
-        if (lane == 0) {
-            if (!(mx > -INFINITY) || !(sum > 0.f)) {
-                set_error(st, GIRA_ERR_NUMERIC);
-                pref[i] = make_float2(0.f, 0.f);
-            } else {
-                pref[i] = make_float2(-mx, __frcp_rn(sum));
-                llpt[i] = (double)(lg2_approx(sum) + mx + ref0) * LN2_4;
-            }
-        }
-    }
-}
-
 // ------------------------------------------------------------------ k-means in four dimensions
 // labels = argmin_b ||x - c_b||^2 (binary32 in the order of dist2_f32_4, ties to
 // the lowest b); binary64 sums of the coordinates and counts per label;
@@ -887,74 +725,22 @@ cudaError_t launch_label_stats4(const float4* pts4, int64_t n, int k, const int3
     return cudaGetLastError();
 }
 
-int estep4_threads(int k) { return 32 * ((k + 63) / 64); }
-
-// CTAs per SM of the statistics kernel for k components and ppc staged points.
-static int estep4_occupancy(int k, int64_t ppc) {
-    int occ = 0;
-    const int smem = (int)(ppc * 32);
-    cudaFuncSetAttribute(estep4_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, PPC4_MAX * 32);
-    cudaFuncSetAttribute(estep4_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, PPC4_MAX * 32);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, estep4_kernel<true>, estep4_threads(k), smem) !=
-            cudaSuccess ||
-        occ < 1) {
-        cudaGetLastError();
-        occ = 1;
-    }
-    return occ;
-}
-
-// One wave of CTAs (SMs x resident CTAs) over the points, at most PPC4_MAX
-// points each (more waves beyond that).
-int estep4_grid(int64_t n, int k, int num_sms, int64_t* ppc) {
-    auto plan = [&](int occ) {
-        const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((n + Q4 - 1) / Q4, (int64_t)num_sms * occ));
-        return std::min<int64_t>(((n + grid - 1) / grid + Q4 - 1) / Q4 * Q4, PPC4_MAX);
-    };
-    int64_t p = plan(estep4_occupancy(k, 1024));
-    if (p > 1024) p = plan(estep4_occupancy(k, p));
-    *ppc = p;
-    return (int)((n + p - 1) / p);
-}
-
-cudaError_t launch_estep4(const EStep4Launch& a, bool stats, int grid, cudaStream_t s, bool pdl) {
-    const size_t smem = (size_t)a.pts_per_cta * 32;
-    const void* fn = stats ? (const void*)estep4_kernel<true> : (const void*)estep4_kernel<false>;
-    note_estep_kernel(fn);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    void* args[] = {(void*)&a};
-    PdlConfig c(dim3(grid), dim3(estep4_threads(a.k)), smem, s, pdl);
-    return cudaLaunchKernelExC(&c.cfg, fn, args);
-}
-
-cudaError_t launch_reduce_finalize4(const float* partials, int grid, int kc, const double* ll_partials,
+cudaError_t launch_reduce_finalize4(const float* partials, const uint32_t* live2, int slices, const double* llp,
                                     int ll_count, const double* stats64, const float4* shift4, int k, int64_t n,
                                     double reg, double tol, double* model64, float* params, double* trace,
-                                    DeviceState* st, int iter, bool em, cudaStream_t s, bool pdl) {
-    PdlConfig c(dim3(k), dim3(NSTAT4 * 32), 0, s, pdl);
-    return cudaLaunchKernelEx(&c.cfg, reduce_finalize4_kernel, partials, grid, kc, ll_partials, ll_count, stats64,
-                              shift4, k, n, reg, tol, model64, params, trace, st, iter, em ? 1 : 0);
-}
-
-cudaError_t launch_chunk_ref4(const float* params, int k, const DeviceState* st, float* gref, cudaStream_t s) {
-    chunk_ref4_kernel<<<1, 256, 0, s>>>(params, k, st, gref);
+                                    const int* perm, DeviceState* st, int iter, bool em, cudaStream_t s) {
+    const Fin4Args f{partials, live2, slices, llp, ll_count, stats64, shift4, k, n, reg, tol, model64, params, trace,
+                     perm, st, iter, em ? 1 : 0};
+    reduce_finalize4_kernel<<<(k + 1) / 2, 32 * FIN4_WARPS, 0, s>>>(f);
     return cudaGetLastError();
 }
 
-cudaError_t launch_estep4_chunks(const EStep4Launch& a, int pass, int grid, cudaStream_t s) {
-    const size_t smem = (size_t)a.pts_per_cta * 32;
-    const void* fn = (pass == 1) ? (const void*)estep4_kernel<false, 1> : (const void*)estep4_kernel<true, 2>;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+cudaError_t launch_order_components4(double* model64, double* scratch, int k, int* perm, float* params,
+                                     DeviceState* st, cudaStream_t s) {
+    cudaError_t e = cudaMemcpyAsync(scratch, model64, sizeof(double) * (size_t)k * MODEL4, cudaMemcpyDeviceToDevice, s);
+    if (e == cudaSuccess) e = launch_order_means(scratch, MODEL4, k, perm, s);
     if (e != cudaSuccess) return e;
-    const int chunks = (a.k + CHUNK4 - 1) / CHUNK4;
-    void* args[] = {(void*)&a};
-    return cudaLaunchKernel(fn, dim3(grid, chunks), dim3(CHUNK4 / 2), args, smem, s);
-}
-
-cudaError_t launch_chunk_exact4(const float4* pts8, const float* params, int k, const float* gref, const int* flags,
-                                const int* flag_count, float2* pref, double* llpt, DeviceState* st, cudaStream_t s) {
-    chunk_exact4_kernel<<<152, 256, 0, s>>>(pts8, params, k, gref, flags, flag_count, pref, llpt, st);
+    rebuild_components4_kernel<<<(k + 63) / 64, 64, 0, s>>>(scratch, perm, k, model64, params, st);
     return cudaGetLastError();
 }
 
@@ -964,15 +750,13 @@ cudaError_t launch_params_from_model4(const float* w, const float* mu, const flo
     return cudaGetLastError();
 }
 
-cudaError_t launch_model_out4(const double* model64, int k, float* w, float* mu, float* cov, const DeviceState* st,
-                              cudaStream_t s) {
-    model_out4_kernel<<<1, 64, 0, s>>>(model64, k, w, mu, cov, st);
+cudaError_t launch_model_out4(const double* model64, int k, float* w, float* mu, float* cov, const int* perm,
+                              const DeviceState* st, cudaStream_t s) {
+    model_out4_kernel<<<(k + 63) / 64, 64, 0, s>>>(model64, k, w, mu, cov, perm, st);
     return cudaGetLastError();
 }
 
-int params4_pairs(int k) {
-    return k > MAX_K4_DIRECT ? ((k + CHUNK4 - 1) / CHUNK4) * (CHUNK4 / 2) : estep4_threads(k);
-}
+int params4_pairs(int k) { return (k + 1) / 2; }
 
 cudaError_t launch_fill_padding4(float* params, int k, cudaStream_t s) {
     const int kpad = 2 * params4_pairs(k);

@@ -538,10 +538,8 @@ void note_estep_kernel(const void* fn) {
     char* dem = abi::__cxa_demangle(raw, nullptr, nullptr, &ok);
     std::string name = (ok == 0 && dem) ? dem : raw;
     std::free(dem);
-    size_t at = name.find("estep_kernel<");
-    if (at == std::string::npos) at = name.find("estep_pt_kernel<");
+    size_t at = name.find("estep_pt_kernel<");
     if (at == std::string::npos) at = name.find("estep_reach_kernel<");
-    if (at == std::string::npos) at = name.find("estep4_kernel<");
     if (at != std::string::npos) name = name.substr(at);
     const size_t par = name.rfind(">(");
     if (par != std::string::npos) name = name.substr(0, par + 1);
@@ -657,49 +655,6 @@ cudaError_t launch_fill_padding(float* params, int k, int npairs_pad, cudaStream
 
 // ------------------------------------------------------------------ log-likelihood reduce
 namespace {
-// ------------------------------------------------------------------ two-level log-sum-exp (4-D chunks)
-constexpr int COMBINE_BLOCKS = 608;
-constexpr int COMBINE_THREADS = 256;
-
-// Per point: total over chunks (fixed order); (0, 1/total) and the natural-log
-// log-likelihood, or, if the total is below 2^-100, listed for the exact step.
-__global__ void __launch_bounds__(COMBINE_THREADS) chunk_combine_kernel(const float* __restrict__ psum, int chunks,
-                                                                        int64_t n, const float* __restrict__ gref,
-                                                                        float2* pref, double* llpt, int* flag_count,
-                                                                        int* flags) {
-    const float ref0 = gref[1];
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        float tot = 0.f;
-        for (int c = 0; c < chunks; ++c) tot += psum[(size_t)c * n + i];
-        if (tot >= 0x1p-100f) {
-            pref[i] = make_float2(0.f, __frcp_rn(tot));
-            llpt[i] = (double)(lg2_approx(tot) + ref0) * 0.693147180559945309417232121458;
-        } else {
-            pref[i] = make_float2(0.f, 0.f);
-            llpt[i] = 0.0;
-            flags[atomicAdd(flag_count, 1)] = (int)i;
-        }
-    }
-}
-
-// Fixed-order per-block sums of the per-point log-likelihoods.
-__global__ void __launch_bounds__(COMBINE_THREADS) points_ll_reduce_kernel(const double* __restrict__ llpt, int64_t n,
-                                                                           double* llp) {
-    __shared__ double s_w[COMBINE_THREADS / 32];
-    double v = 0.0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        v += llpt[i];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0) s_w[threadIdx.x >> 5] = v;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int w = 0; w < COMBINE_THREADS / 32; ++w) t += s_w[w];
-        llp[blockIdx.x] = t;
-    }
-}
-
 __global__ void ll_reduce_batched_kernel(const double* __restrict__ llp, const BatchInst* __restrict__ insts,
                                          DeviceState* states) {
     const BatchInst I = insts[blockIdx.x];
@@ -1421,22 +1376,16 @@ __device__ __forceinline__ unsigned spread10(unsigned v) {   // bit i -> bit 3 i
 }
 
 // insts (batched fits): block i orders instance i (its own k, offsets and state).
-__global__ void __launch_bounds__(ORDER_THREADS) order_components_kernel(const double* __restrict__ old, int k,
-                                                                        int kp2, int* perm, double* model64,
-                                                                        float* params, float4* shift4,
-                                                                        DeviceState* st,
+__global__ void __launch_bounds__(ORDER_THREADS) order_components_kernel(const double* __restrict__ old,
+                                                                        int stride, int k, int kp2, int* perm,
                                                                         const BatchInst* __restrict__ insts) {
     extern __shared__ unsigned long long keys[];   // kp2 = power of two >= k
     __shared__ float s_lo[3][32], s_hi[3][32];
     if (insts) {
         const BatchInst I = insts[blockIdx.x];
         k = I.k;
-        old += (size_t)I.comp_off * MODEL;
-        model64 += (size_t)I.comp_off * MODEL;
+        old += (size_t)I.comp_off * stride;
         perm += I.comp_off;
-        params += I.par_off;
-        shift4 += I.comp_off;
-        st += blockIdx.x;
         kp2 = 1;
         while (kp2 < k) kp2 <<= 1;
     }
@@ -1445,7 +1394,7 @@ __global__ void __launch_bounds__(ORDER_THREADS) order_components_kernel(const d
     float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
     for (int b = t; b < k; b += blockDim.x)
         for (int i = 0; i < 3; ++i) {
-            const float v = (float)old[(size_t)b * MODEL + 1 + i];
+            const float v = (float)old[(size_t)b * stride + 1 + i];
             lo[i] = fminf(lo[i], v);
             hi[i] = fmaxf(hi[i], v);
         }
@@ -1477,7 +1426,7 @@ __global__ void __launch_bounds__(ORDER_THREADS) order_components_kernel(const d
         if (b < k) {
             unsigned code = 0;
             for (int i = 0; i < 3; ++i) {
-                const float u = ((float)old[(size_t)b * MODEL + 1 + i] - lo[i]) * scale[i];
+                const float u = ((float)old[(size_t)b * stride + 1 + i] - lo[i]) * scale[i];
                 const unsigned q = (unsigned)fminf(1023.f, fmaxf(0.f, floorf(u)));
                 code |= spread10(q) << i;
             }
@@ -1487,9 +1436,9 @@ __global__ void __launch_bounds__(ORDER_THREADS) order_components_kernel(const d
     }
     __syncthreads();
     for (int size = 2; size <= kp2; size <<= 1)
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
+        for (int hop = size >> 1; hop > 0; hop >>= 1) {
             for (int i = t; i < kp2; i += blockDim.x) {
-                const int j = i ^ stride;
+                const int j = i ^ hop;
                 if (j > i) {
                     const unsigned long long a = keys[i], c = keys[j];
                     const bool up = (i & size) == 0;
@@ -1796,18 +1745,25 @@ cudaError_t launch_model_out(const double* model64, int k, float* w, float* mu, 
     return cudaGetLastError();
 }
 
+cudaError_t launch_order_means(const double* old, int stride, int k, int* perm, cudaStream_t s) {
+    if (k > ORDER_MAX_K) return cudaErrorInvalidValue;
+    int kp2 = 1;
+    while (kp2 < k) kp2 <<= 1;
+    const size_t smem = sizeof(unsigned long long) * (size_t)kp2;
+    const cudaError_t e =
+        cudaFuncSetAttribute(order_components_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    order_components_kernel<<<1, ORDER_THREADS, smem, s>>>(old, stride, k, kp2, perm, nullptr);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_order_components(double* model64, double* scratch, int k, int* perm, float* params,
                                     float4* shift4, DeviceState* st, cudaStream_t s) {
     if (k > ORDER_MAX_K) return cudaErrorInvalidValue;
     cudaError_t e = cudaMemcpyAsync(scratch, model64, sizeof(double) * (size_t)k * MODEL, cudaMemcpyDeviceToDevice, s);
     if (e != cudaSuccess) return e;
-    int kp2 = 1;
-    while (kp2 < k) kp2 <<= 1;
-    const size_t smem = sizeof(unsigned long long) * (size_t)kp2;
-    e = cudaFuncSetAttribute(order_components_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = launch_order_means(scratch, MODEL, k, perm, s);
     if (e != cudaSuccess) return e;
-    order_components_kernel<<<1, ORDER_THREADS, smem, s>>>(scratch, k, kp2, perm, model64, params, shift4, st,
-                                                           nullptr);
     rebuild_components_kernel<<<(k + 63) / 64, 64, 0, s>>>(scratch, perm, k, model64, params, shift4, st, nullptr,
                                                            nullptr);
     return cudaGetLastError();
@@ -1825,8 +1781,7 @@ cudaError_t launch_order_components_batched(double* model64, double* scratch, in
     const size_t smem = sizeof(unsigned long long) * (size_t)kp2;
     e = cudaFuncSetAttribute(order_components_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    order_components_kernel<<<batch, ORDER_THREADS, smem, s>>>(scratch, 0, 0, perm, model64, params, shift4, states,
-                                                               insts);
+    order_components_kernel<<<batch, ORDER_THREADS, smem, s>>>(scratch, MODEL, 0, 0, perm, insts);
     rebuild_components_kernel<<<(total_k + 63) / 64, 64, 0, s>>>(scratch, perm, total_k, model64, params, shift4,
                                                                  states, insts, comp_inst);
     return cudaGetLastError();
@@ -1857,36 +1812,4 @@ cudaError_t launch_pack_pose_batched(const float* pts3, int64_t n, const int64_t
     return cudaGetLastError();
 }
 
-}  // namespace gira
-
-namespace gira {
-int chunk_combine_grid() { return COMBINE_BLOCKS; }
-
-cudaError_t launch_chunk_combine(const float* psum, int chunks, int64_t n, const float* gref, float2* pref,
-                                 double* llpt, int* flag_count, int* flags, DeviceState* st, cudaStream_t s) {
-    (void)st;
-    chunk_combine_kernel<<<COMBINE_BLOCKS, COMBINE_THREADS, 0, s>>>(psum, chunks, n, gref, pref, llpt, flag_count,
-                                                                    flags);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_points_ll_reduce(const double* llpt, int64_t n, double* llp, DeviceState* st, cudaStream_t s) {
-    points_ll_reduce_kernel<<<COMBINE_BLOCKS, COMBINE_THREADS, 0, s>>>(llpt, n, llp);
-    if (!st) return cudaGetLastError();
-    return launch_ll_reduce(llp, COMBINE_BLOCKS, st, s);
-}
-}  // namespace gira
-
-namespace gira {
-namespace {
-__global__ void double_to_float_kernel(const double* __restrict__ x, int64_t n, float* y) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) y[i] = (float)x[i];
-}
-}  // namespace
-
-cudaError_t launch_double_to_float(const double* x, int64_t n, float* y, cudaStream_t s) {
-    double_to_float_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(x, n, y);
-    return cudaGetLastError();
-}
 }  // namespace gira

@@ -328,21 +328,21 @@ ReachLaunch reach_launch(const ReachBufs& b, const float4* p8, int64_t n, int k,
 }
 
 // One E-step with statistics: b.partials rows and b.live2 masks for the finalize.
-cudaError_t reach_estep_stats(const ReachBufs& b, ReachLaunch a, long long* launches, cudaStream_t s) {
+cudaError_t reach_estep_stats(int d, const ReachBufs& b, ReachLaunch a, long long* launches, cudaStream_t s) {
     a.pref = b.pref;
     a.masks = b.masks;
-    cudaError_t e = launch_reach_prepare(a.params, a.k, a.st, a.iter, b.ctr, b.aux, b.gref, s);
+    cudaError_t e = launch_reach_prepare(d, a.params, a.k, a.st, a.iter, b.ctr, b.aux, b.gref, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(b.live2, 0, sizeof(uint32_t) * b.words * b.slices, s);
-    if (e == cudaSuccess) e = launch_estep_reach(a, 1, b.grid, b.h, a.k, s);
-    if (e == cudaSuccess) e = launch_reach_stats(a, 1, a.k, a.n, b.partials, b.live2, s);
+    if (e == cudaSuccess) e = launch_estep_reach(d, a, 1, b.grid, b.h, a.k, s);
+    if (e == cudaSuccess) e = launch_reach_stats(d, a, 1, a.k, a.n, b.partials, b.live2, s);
     *launches += 3;
     return e;
 }
 
 // The log-likelihood alone: a.per_point (nullable) and st->ll_sum.
-cudaError_t reach_loglik(const ReachBufs& b, const ReachLaunch& a, long long* launches, cudaStream_t s) {
-    cudaError_t e = launch_reach_prepare(a.params, a.k, a.st, a.iter, b.ctr, b.aux, b.gref, s);
-    if (e == cudaSuccess) e = launch_estep_reach(a, 0, b.grid, b.h, a.k, s);
+cudaError_t reach_loglik(int d, const ReachBufs& b, const ReachLaunch& a, long long* launches, cudaStream_t s) {
+    cudaError_t e = launch_reach_prepare(d, a.params, a.k, a.st, a.iter, b.ctr, b.aux, b.gref, s);
+    if (e == cudaSuccess) e = launch_estep_reach(d, a, 0, b.grid, b.h, a.k, s);
     if (e == cudaSuccess) e = launch_ll_reduce(b.llp, b.grid, a.st, s);
     *launches += 3;
     return e;
@@ -654,14 +654,14 @@ gira_status gira_gmm_fit(const float* points, int64_t n, int k, const gira_fit_o
     if (large) {
         const float4* pe = sorted ? b.p8s : b.p8;
         for (int t = 1; t <= o.iters; ++t) {
-            GIRA_CUDA(reach_estep_stats(rb, reach_launch(rb, pe, n, k, b.params, b.st, t), &prof.launches, c.s));
+            GIRA_CUDA(reach_estep_stats(3, rb, reach_launch(rb, pe, n, k, b.params, b.st, t), &prof.launches, c.s));
             COUNTED(prof, 1, launch_reduce_finalize(rb.partials, rb.slices, rb.llp, nullptr, b.shift4, k, n,
                                                     o.reg_covar, o.tol, b.model64, b.params, b.trace, b.st, t, true,
                                                     c.s, false, perm, rb.live2, rb.words, rb.grid));
         }
         prof.t_em = prof.mark();
         if (final_loglik)
-            GIRA_CUDA(reach_loglik(rb, reach_launch(rb, pe, n, k, b.params, b.st, 0), &prof.launches, c.s));
+            GIRA_CUDA(reach_loglik(3, rb, reach_launch(rb, pe, n, k, b.params, b.st, 0), &prof.launches, c.s));
     }
     EStepLaunch a{sorted ? b.p8s : b.p8, n, k, b.params, b.partials, b.llp, nullptr, b.st, 0};
     a.n_buf = n;
@@ -799,7 +799,7 @@ gira_status gira_gmm_loglik(const float* points, int64_t n, int k, const float* 
     if (large) {
         ReachLaunch a = reach_launch(rb, b.p8, n, k, b.params, b.st, 0);
         a.per_point = ppd;
-        GIRA_CUDA(reach_loglik(rb, a, &prof.launches, c.s));
+        GIRA_CUDA(reach_loglik(3, rb, a, &prof.launches, c.s));
     } else {
         EStepLaunch a{b.p8, n, k, b.params, nullptr, b.llp, ppd, b.st, 0};
         a.n_buf = n;
@@ -943,15 +943,15 @@ gira_status gira_gmm_loglik_grad(const float* points, int64_t n, int k, const fl
             GIRA_CUDA(cudaMemsetAsync(rb.live2, 0, sizeof(uint32_t) * rb.words * rb.slices, c.s));
         }
         cudaEvent_t e0 = prof.mark_launch();
-        COUNTED(prof, 1, launch_estep_reach(a, 2, rb.grid, rb.h, k, c.s));
+        COUNTED(prof, 1, launch_estep_reach(3, a, 2, rb.grid, rb.h, k, c.s));
         cudaEvent_t e1 = prof.mark_launch();
         if (prof.per_launch) prof.timed(e0, e1);
-        if (gpar) COUNTED(prof, 1, launch_reach_stats(a, 1, k, n, rb.partials, rb.live2, c.s));
+        if (gpar) COUNTED(prof, 1, launch_reach_stats(3, a, 1, k, n, rb.partials, rb.live2, c.s));
         const ReachGradArgs f{gpar ? rb.partials : nullptr, rb.live2, rb.slices, rb.llp, b.ppart, rb.grid, pose_d,
                               ch_d, b.params, b.model64, b.perm, k, n, gl_d, gm_d, gc_d, po_d, tw_d, b.st};
         COUNTED(prof, 1, launch_reach_grad_finalize(f, nullptr, 1, c.s));
     } else {
-        COUNTED(prof, 1, launch_estep_reach(a, 0, rb.grid, rb.h, k, c.s));
+        COUNTED(prof, 1, launch_estep_reach(3, a, 0, rb.grid, rb.h, k, c.s));
         COUNTED(prof, 1, launch_ll_reduce(rb.llp, rb.grid, b.st, c.s));
     }
     auto out = [&](void* dst, Kind kd, const void* stage, size_t bytes) -> gira_status {
@@ -1541,8 +1541,8 @@ gira_status gira_gmm_loglik_grad_batched(const float* points, const int64_t* off
             a.masks = b.masks;
             if (e == cudaSuccess) e = cudaMemsetAsync(b.live2, 0, sizeof(uint32_t) * live_words, cs);
         }
-        if (e == cudaSuccess) e = launch_estep_reach(a, 2, (int)units.size(), rh, kmax, cs);
-        if (e == cudaSuccess && gpar) e = launch_reach_stats(a, batch, kmax, nmax, b.partials, b.live2, cs);
+        if (e == cudaSuccess) e = launch_estep_reach(3, a, 2, (int)units.size(), rh, kmax, cs);
+        if (e == cudaSuccess && gpar) e = launch_reach_stats(3, a, batch, kmax, nmax, b.partials, b.live2, cs);
         const ReachGradArgs f{gpar ? b.partials : nullptr, b.live2, 0, b.llp, b.ppart, 0, b.poses, b.ch, b.params,
                               b.model64, b.perm, kmax, 0, gpar ? b.gl : nullptr, gpar ? b.gm : nullptr,
                               gpar ? b.gc : nullptr, b.gpose, b.gtwist, b.st};
@@ -1610,45 +1610,6 @@ gira_status check_nk4(int64_t n, int k) {
     if (k > n) return fail(GIRA_ERR_INVALID_ARG, "k = %d > n = %lld", k, (long long)n);
     return GIRA_OK;
 }
-
-// K above MAX_K4_DIRECT: per-point state of the two-level log-sum-exp.
-struct Chunk4Bufs {
-    float* gref = nullptr;     // [2]: max_b c_b, log-likelihood reference
-    float* psum = nullptr;     // [chunks][n]
-    float2* pref = nullptr;    // [n] (shift, 1 / total)
-    double* llpt = nullptr;    // [n] natural-log per-point log-likelihood
-    int* flags = nullptr;      // [n] points for the exact step
-    int* flag_count = nullptr;
-};
-
-void carve_chunk4(Carver& cv, int64_t n, int chunks, Chunk4Bufs* b) {
-    b->gref = cv.take<float>(2);
-    b->psum = cv.take<float>((size_t)chunks * n);
-    b->pref = cv.take<float2>(n);
-    b->llpt = cv.take<double>(n);
-    b->flags = cv.take<int>(n);
-    b->flag_count = cv.take<int>(1);
-}
-
-// Reference, pass A, per-point totals, exact step for underflowing points, and
-// the fixed-order log-likelihood partials (into st->ll_sum when ll_to_state).
-cudaError_t chunk4_lse(const Chunk4Bufs& b, EStep4Launch a, int grid, double* llp, bool ll_to_state,
-                       long long* launches, cudaStream_t s) {
-    const int chunks = (a.k + CHUNK4 - 1) / CHUNK4;
-    a.partials = nullptr;
-    a.gref = b.gref;
-    a.psum = b.psum;
-    cudaError_t e = launch_chunk_ref4(a.params, a.k, a.st, b.gref, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(b.flag_count, 0, sizeof(int), s);
-    if (e == cudaSuccess) e = launch_estep4_chunks(a, 1, grid, s);
-    if (e == cudaSuccess)
-        e = launch_chunk_combine(b.psum, chunks, a.n, b.gref, b.pref, b.llpt, b.flag_count, b.flags, a.st, s);
-    if (e == cudaSuccess)
-        e = launch_chunk_exact4(a.pts8, a.params, a.k, b.gref, b.flags, b.flag_count, b.pref, b.llpt, a.st, s);
-    if (e == cudaSuccess) e = launch_points_ll_reduce(b.llpt, a.n, llp, ll_to_state ? a.st : nullptr, s);
-    *launches += 5 + (ll_to_state ? 1 : 0);
-    return e;
-}
 }  // namespace
 
 gira_status gira_gmm_fit4(const float* points, int64_t n, int k, const gira_fit_opts* opts, float* weights,
@@ -1669,39 +1630,37 @@ gira_status gira_gmm_fit4(const float* points, int64_t n, int k, const gira_fit_
     TRY(check_ptr(means, "means", c.dev, &km));
     TRY(check_ptr(covs, "covs", c.dev, &kc));
     const bool kinit = o.init_mode == GIRA_INIT_KMEANS;
-    const bool chunked = k > MAX_K4_DIRECT;   // two-level log-sum-exp over chunks of CHUNK4 components
-    const int chunks = chunked ? (k + CHUNK4 - 1) / CHUNK4 : 1;
     const int kpad = params4_pairs(k);
-    int64_t ppc = 0;
-    const int grid = estep4_grid(n, chunked ? CHUNK4 : k, c.sms, &ppc);   // CTAs per chunk when chunked
-    const int kblk = chunked ? CHUNK4 : k;                                 // components per partial block
+    const bool sorted = n <= point_order_max_n();   // the E-steps visit the points in Morton order of (x, y, z)
     const int nblk = kpp_num_blocks(n);
     int kgrid = kinit ? kpp_persistent_grid() : 0;
     if (kgrid > 0 && n > kpp_persistent_max_n(kgrid)) kgrid = 0;
-    Chunk4Bufs cb;
+    ReachBufs rb;
     struct Bufs {
         DeviceState* st;
-        float *pin, *params, *partials, *d2, *mw, *mmu, *mcov;
-        float4 *p4, *p8, *c4;
-        double *model64, *stats64, *llp, *trace, *sums;
+        float *pin, *params, *d2, *mw, *mmu, *mcov;
+        float4 *p4, *p8, *p8s, *p4s, *c4;
+        double *model64, *stats64, *trace, *sums;
         u128 *bs, *ksums;
         int64_t* ch;
         int32_t* lab;
         int *ksync, *perm;
         unsigned long long* chg;
+        void* osc;
     } b{};
     auto layout = [&](Carver& cv) {
         b.st = cv.take<DeviceState>(1);
         b.perm = cv.take<int>(k);
         b.pin = cv.take<float>(kp == Kind::Host ? 4 * n : 0);
-        b.p4 = cv.take<float4>(n);
+        b.p4 = cv.take<float4>(kinit ? n : 0);
+        b.p8s = cv.take<float4>(sorted ? 2 * (size_t)n : 0);
+        b.p4s = cv.take<float4>(sorted && kinit ? (size_t)n : 0);
+        b.osc = cv.take<char>(sorted ? point_order_scratch_bytes(n, 1) : 0);
         b.p8 = cv.take<float4>(2 * (size_t)n);
         b.params = cv.take<float>((size_t)kpad * PAIR4_FLOATS);
         b.model64 = cv.take<double>((size_t)k * MODEL4);
         b.stats64 = cv.take<double>((size_t)k * NSTAT4);
-        b.partials = cv.take<float>((size_t)chunks * grid * kblk * NSTAT4);
-        b.llp = cv.take<double>(std::max(grid, chunk_combine_grid()));
-        if (chunked) carve_chunk4(cv, n, chunks, &cb);
+        carve_reach(cv, n, k, NSTAT4, true, &rb);
         b.trace = cv.take<double>(std::max(o.iters, 1));
         b.mw = cv.take<float>(kw == Kind::Host ? k : 0);
         b.mmu = cv.take<float>(km == Kind::Host ? 4 * (size_t)k : 0);
@@ -1742,7 +1701,10 @@ gira_status gira_gmm_fit4(const float* points, int64_t n, int k, const gira_fit_
         GIRA_CUDA(cudaMemcpyAsync(b.pin, points, sizeof(float) * 4 * n, cudaMemcpyHostToDevice, c.s));
         pts = b.pin;
     }
-    COUNTED(prof, 1, launch_pack4(pts, n, b.p4, b.p8, b.st, c.s));
+    COUNTED(prof, 1, launch_pack4(pts, n, kinit ? b.p4 : nullptr, b.p8, b.st, c.s));
+    if (sorted)
+        COUNTED(prof, point_order_launches(1),
+                launch_point_order(b.p8, n, nullptr, nullptr, 0, 1, b.osc, b.p8s, kinit ? b.p4s : nullptr, nullptr, c.s));
     COUNTED(prof, 1, launch_fill_padding4(b.params, k, c.s));
     float* w_d = (kw == Kind::Device) ? weights : b.mw;
     float* mu_d = (km == Kind::Device) ? means : b.mmu;
@@ -1761,8 +1723,8 @@ gira_status gira_gmm_fit4(const float* points, int64_t n, int k, const gira_fit_
                                                           b.st, c.s));
         GIRA_CUDA(cudaMemsetAsync(b.stats64, 0, sizeof(double) * NSTAT4 * k, c.s));
         COUNTED(prof, 1, launch_label_stats4(b.p4, n, k, b.lab, b.c4, b.stats64, b.st, c.s));
-        COUNTED(prof, 1, launch_reduce_finalize4(nullptr, 0, k, nullptr, 0, b.stats64, b.c4, k, n, o.reg_covar,
-                                                 o.tol, b.model64, b.params, b.trace, b.st, 0, false, c.s));
+        COUNTED(prof, 1, launch_reduce_finalize4(nullptr, nullptr, 0, nullptr, 0, b.stats64, b.c4, k, n, o.reg_covar,
+                                                 o.tol, b.model64, b.params, b.trace, nullptr, b.st, 0, false, c.s));
     } else {
         if (kw == Kind::Host) GIRA_CUDA(cudaMemcpyAsync(b.mw, weights, sizeof(float) * k, cudaMemcpyHostToDevice, c.s));
         if (km == Kind::Host)
@@ -1771,43 +1733,24 @@ gira_status gira_gmm_fit4(const float* points, int64_t n, int k, const gira_fit_
             GIRA_CUDA(cudaMemcpyAsync(b.mcov, covs, sizeof(float) * 16 * k, cudaMemcpyHostToDevice, c.s));
         COUNTED(prof, 1, launch_params_from_model4(w_d, mu_d, cov_d, k, b.model64, b.params, b.st, c.s));
     }
+    // components in Morton order of their means, as in the 3-D fit
+    COUNTED(prof, 2, launch_order_components4(b.model64, b.stats64, k, b.perm, b.params, b.st, c.s));
     prof.t_init = prof.mark();
-    EStep4Launch a{b.p8, n, k, b.params, ppc, b.partials, b.llp, nullptr, b.st, 0};
+    const float4* pe = sorted ? b.p8s : b.p8;
     for (int t = 1; t <= o.iters; ++t) {
-        a.iter = t;
-        if (chunked) {
-            GIRA_CUDA(chunk4_lse(cb, a, grid, b.llp, false, &prof.launches, c.s));
-            EStep4Launch pb = a;
-            pb.gref = cb.gref;
-            pb.pref = cb.pref;
-            COUNTED(prof, 1, launch_estep4_chunks(pb, 2, grid, c.s));
-            COUNTED(prof, 1, launch_reduce_finalize4(b.partials, grid, kblk, b.llp, chunk_combine_grid(), nullptr,
-                                                     nullptr, k, n, o.reg_covar, o.tol, b.model64, b.params, b.trace,
-                                                     b.st, t, true, c.s));
-            continue;
-        }
-        const bool pdl = !prof.per_launch;   // dependent launches, as in the 3-D loop
+        const ReachLaunch a = reach_launch(rb, pe, n, k, b.params, b.st, t);
         cudaEvent_t e0 = prof.mark_launch();
-        COUNTED(prof, 1, launch_estep4(a, true, grid, c.s, pdl));
+        GIRA_CUDA(reach_estep_stats(4, rb, a, &prof.launches, c.s));
         cudaEvent_t e1 = prof.mark_launch();
         if (prof.per_launch) prof.timed(e0, e1);
-        COUNTED(prof, 1, launch_reduce_finalize4(b.partials, grid, kblk, b.llp, grid, nullptr, nullptr, k, n,
-                                                 o.reg_covar, o.tol, b.model64, b.params, b.trace, b.st, t, true,
-                                                 c.s, pdl));
+        COUNTED(prof, 1, launch_reduce_finalize4(rb.partials, rb.live2, rb.slices, rb.llp, rb.grid, nullptr, nullptr, k,
+                                                 n, o.reg_covar, o.tol, b.model64, b.params, b.trace, b.perm, b.st, t,
+                                                 true, c.s));
     }
     prof.t_em = prof.mark();
-    if (final_loglik) {
-        EStep4Launch f = a;
-        f.iter = 0;
-        f.partials = nullptr;
-        if (chunked) {
-            GIRA_CUDA(chunk4_lse(cb, f, grid, b.llp, true, &prof.launches, c.s));
-        } else {
-            COUNTED(prof, 1, launch_estep4(f, false, grid, c.s));
-            COUNTED(prof, 1, launch_ll_reduce(b.llp, grid, b.st, c.s));
-        }
-    }
-    COUNTED(prof, 1, launch_model_out4(b.model64, k, w_d, mu_d, cov_d, b.st, c.s));
+    if (final_loglik)
+        GIRA_CUDA(reach_loglik(4, rb, reach_launch(rb, pe, n, k, b.params, b.st, 0), &prof.launches, c.s));
+    COUNTED(prof, 1, launch_model_out4(b.model64, k, w_d, mu_d, cov_d, b.perm, b.st, c.s));
     if (kw == Kind::Host) GIRA_CUDA(cudaMemcpyAsync(weights, b.mw, sizeof(float) * k, cudaMemcpyDeviceToHost, c.s));
     if (km == Kind::Host) GIRA_CUDA(cudaMemcpyAsync(means, b.mmu, sizeof(float) * 4 * k, cudaMemcpyDeviceToHost, c.s));
     if (kc == Kind::Host) GIRA_CUDA(cudaMemcpyAsync(covs, b.mcov, sizeof(float) * 16 * k, cudaMemcpyDeviceToHost, c.s));
@@ -1837,17 +1780,13 @@ gira_status gira_gmm_loglik4(const float* points, int64_t n, int k, const float*
     TRY(check_ptr(means, "means", c.dev, &km));
     TRY(check_ptr(covs, "covs", c.dev, &kc));
     if (per_point) TRY(check_ptr(per_point, "per_point", c.dev, &kpp));
-    const bool chunked = k > MAX_K4_DIRECT;
-    const int chunks = chunked ? (k + CHUNK4 - 1) / CHUNK4 : 1;
     const int kpad = params4_pairs(k);
-    int64_t ppc = 0;
-    const int grid = estep4_grid(n, chunked ? CHUNK4 : k, c.sms, &ppc);
-    Chunk4Bufs cb;
+    ReachBufs rb;
     struct Bufs {
         DeviceState* st;
         float *pin, *params, *mw, *mmu, *mcov, *pp;
         float4* p8;
-        double *model64, *llp;
+        double* model64;
     } b{};
     auto layout = [&](Carver& cv) {
         b.st = cv.take<DeviceState>(1);
@@ -1855,8 +1794,7 @@ gira_status gira_gmm_loglik4(const float* points, int64_t n, int k, const float*
         b.p8 = cv.take<float4>(2 * (size_t)n);
         b.params = cv.take<float>((size_t)kpad * PAIR4_FLOATS);
         b.model64 = cv.take<double>((size_t)k * MODEL4);
-        b.llp = cv.take<double>(std::max(grid, chunk_combine_grid()));
-        if (chunked) carve_chunk4(cv, n, chunks, &cb);
+        carve_reach(cv, n, k, NSTAT4, false, &rb);
         b.mw = cv.take<float>(kw == Kind::Host ? k : 0);
         b.mmu = cv.take<float>(km == Kind::Host ? 4 * (size_t)k : 0);
         b.mcov = cv.take<float>(kc == Kind::Host ? 16 * (size_t)k : 0);
@@ -1906,14 +1844,9 @@ gira_status gira_gmm_loglik4(const float* points, int64_t n, int k, const float*
     prof.t_init = prof.mark();
     prof.t_em = prof.t_init;
     float* ppd = per_point ? ((kpp == Kind::Device) ? per_point : b.pp) : nullptr;
-    EStep4Launch a{b.p8, n, k, b.params, ppc, nullptr, b.llp, ppd, b.st, 0};
-    if (chunked) {
-        GIRA_CUDA(chunk4_lse(cb, a, grid, b.llp, true, &prof.launches, c.s));
-        if (ppd) COUNTED(prof, 1, launch_double_to_float(cb.llpt, n, ppd, c.s));
-    } else {
-        COUNTED(prof, 1, launch_estep4(a, false, grid, c.s));
-        COUNTED(prof, 1, launch_ll_reduce(b.llp, grid, b.st, c.s));
-    }
+    ReachLaunch a = reach_launch(rb, b.p8, n, k, b.params, b.st, 0);
+    a.per_point = ppd;
+    GIRA_CUDA(reach_loglik(4, rb, a, &prof.launches, c.s));
     if (per_point && kpp == Kind::Host)
         GIRA_CUDA(cudaMemcpyAsync(per_point, b.pp, sizeof(float) * n, cudaMemcpyDeviceToHost, c.s));
     GIRA_CUDA(cudaMemcpyAsync(&h, b.st, sizeof h, cudaMemcpyDeviceToHost, c.s));

@@ -384,14 +384,14 @@ int reach_points(int h);       // points per CTA
 int reach_grid(int64_t n);     // CTAs of a single launch
 int64_t reach_rows(int64_t n); // blocks of 128 points
 int reach_mask_words(int k);
-cudaError_t launch_reach_prepare(const float* params, int k, const DeviceState* st, int iter, float4* ctr, float2* aux,
+cudaError_t launch_reach_prepare(int d, const float* params, int k, const DeviceState* st, int iter, float4* ctr, float2* aux,
                                  float* gref, cudaStream_t s);
-// mode 0 log-likelihood, 1 with masks and pref, 2 gradient; h: reach_h of the launch; kmax: the largest k.
-cudaError_t launch_estep_reach(const ReachLaunch& a, int mode, int grid, int h, int kmax, cudaStream_t s);
-// partials [slices][pairs][2 NSTAT] and live2 [words][slices] (zeroed by the caller):
+// d: 3 or 4 dimensions.  mode 0 log-likelihood, 1 with masks and pref, 2 gradient (3-D); h: reach_h of the launch; kmax: the largest k.
+cudaError_t launch_estep_reach(int d, const ReachLaunch& a, int mode, int grid, int h, int kmax, cudaStream_t s);
+// partials [slices][pairs][2 NSTAT (4-D: NSTAT4)] and live2 [words][slices] (zeroed by the caller):
 // launch_reduce_finalize takes them as rows and masks.
 // Batched (a.insts): every instance, kmax and nmax its largest k and n.
-cudaError_t launch_reach_stats(const ReachLaunch& a, int batch, int kmax, int64_t nmax, float* partials,
+cudaError_t launch_reach_stats(int d, const ReachLaunch& a, int batch, int kmax, int64_t nmax, float* partials,
                                uint32_t* live2, cudaStream_t s);
 
 struct EStepLaunch {
@@ -491,6 +491,8 @@ cudaError_t launch_params_from_model(const float* w, const float* mu, const floa
 // perm (nullable): slot s of model64 is the caller's component perm[s].
 cudaError_t launch_model_out(const double* model64, int k, float* w, float* mu, float* cov, const DeviceState* st,
                              cudaStream_t s, const int* perm = nullptr);
+// Morton order of the k <= 8192 means at old[b * stride + 1 ..] (rows of a binary64 model): perm.
+cudaError_t launch_order_means(const double* old, int stride, int k, int* perm, cudaStream_t s);
 // Reorder the k <= 8192 components of model64 along a space-filling curve of
 // their means (Morton order) and rebuild params / shift4 / model64 in that order:
 // slot s holds the caller's component perm[s].  scratch: k * MODEL doubles.
@@ -526,15 +528,6 @@ cudaError_t launch_order_components_batched(double* model64, double* scratch, in
 cudaError_t launch_ll_reduce_batched(const double* ll_partials, const BatchInst* insts, int batch,
                                      DeviceState* states, cudaStream_t s);
 
-// Per point: total over chunks -> pref, per-point log-likelihood llpt (natural);
-// points whose total underflows (< 2^-100) are listed in flags for the exact step.
-int chunk_combine_grid();
-cudaError_t launch_chunk_combine(const float* psum, int chunks, int64_t n, const float* gref, float2* pref,
-                                 double* llpt, int* flag_count, int* flags, DeviceState* st, cudaStream_t s);
-cudaError_t launch_double_to_float(const double* x, int64_t n, float* y, cudaStream_t s);
-// Fixed-order sums of llpt into chunk_combine_grid() partials, then (st != nullptr)
-// into st->ll_sum.
-cudaError_t launch_points_ll_reduce(const double* llpt, int64_t n, double* llp, DeviceState* st, cudaStream_t s);
 // Batched differentiable log-likelihood (a batch table of scans, each with its
 // own model and pose; poses: batch x 12, or nullptr for identities).
 cudaError_t launch_pack_pose_batched(const float* pts3, int64_t n, const int64_t* offsets, int batch,
@@ -630,69 +623,37 @@ cudaError_t launch_centers_out(const float4* centers4, int k, float* centers3, c
 //   slot 10     c = log2 w + sum_j log2 (L^{-1})_jj - (4/2) log2(2 pi)
 //   slot 11..14 -mu (binary32; also the shift of the M-step statistics)
 //   slot 15     w (N_b after an M-step, or the caller's weight)
-// Statistics (NSTAT4): S0, S1[4], S2[10] in the order 00,01,02,03,11,12,13,22,23,33;
+//   slot 16     a lower bound of sigma_min(P')^2, as slot 14 in 3-D; slot 17 padding
+// Statistics (NSTAT4, about y = P'(x - mu)): S0, S1[4], S2[10] in the order 00,01,02,03,11,12,13,22,23,33;
 // binary64 model (MODEL4): w, mu[4], Sigma[10] in the same order.
-constexpr int PAIR4_FLOATS = 32;
-constexpr int SLOT4_P = 0, SLOT4_C = 10, SLOT4_NMU = 11, SLOT4_W = 15;
+constexpr int PAIR4_FLOATS = 36;
+constexpr int SLOT4_P = 0, SLOT4_C = 10, SLOT4_NMU = 11, SLOT4_W = 15, SLOT4_S = 16;
 constexpr int NSTAT4 = 15;
 constexpr int MODEL4 = 15;
 // index of (i, j), i <= j, in the upper-triangle order 00,01,02,03,11,12,13,22,23,33
 __host__ __device__ constexpr int sym4(int i, int j) { return i * (7 - i) / 2 + j; }
 
-struct EStep4Launch {
-    const float4* pts8;    // 2 float4 per point: (x,x,y,y) (z,z,I,I)
-    int64_t n;
-    int k;
-    const float* params;   // estep4_threads(k) pairs * PAIR4_FLOATS (padding components: c = -inf)
-    int64_t pts_per_cta;   // multiple of 8
-    float* partials;       // [grid][k][NSTAT4] (stats launches)
-    double* ll_partials;   // [grid]
-    float* per_point;      // [n] natural-log lse, or nullptr
-    DeviceState* st;
-    int iter;              // 1-based EM iteration; skipped when iter > st->stop_after
-    // K above MAX_K4_DIRECT: chunks of CHUNK4 components (blockIdx.y = chunk, all over
-    // the same points, logits relative to gref[0] = max_b c_b).  Pass A writes
-    // psum[chunk][n] = sum over the chunk of 2^(l - cmax); pass B takes
-    // pref[n] = (shift, 1 / total) and writes the statistics, partials laid out
-    // [chunk][grid][CHUNK4][NSTAT4].
-    const float* gref = nullptr;
-    float* psum = nullptr;
-    const float2* pref = nullptr;
-};
-
-constexpr int MAX_K4_DIRECT = 1024;   // one CTA holds every component up to here
-constexpr int CHUNK4 = 512;           // components per chunk above it
-
-// Threads of the E-step block for k components (one pair per lane).
-int estep4_threads(int k);
-// Component pairs the parameter buffer holds for k (chunks padded to CHUNK4).
+// Component pairs the parameter buffer holds for k.
 int params4_pairs(int k);
-int estep4_grid(int64_t n, int k, int num_sms, int64_t* pts_per_cta);
-// pdl: as for launch_estep.
-cudaError_t launch_estep4(const EStep4Launch& a, bool stats, int grid, cudaStream_t s, bool pdl = false);
 // N x 4 -> pts4 (x,y,z,I) (nullable) and pts8 (x,x,y,y)(z,z,I,I); flags non-finite input.
 cudaError_t launch_pack4(const float* pts4in, int64_t n, float4* pts4, float4* pts8, DeviceState* st,
                          cudaStream_t s);
 cudaError_t launch_fill_padding4(float* params, int k, cudaStream_t s);
-// M-step from the per-CTA partials (or binary64 stats64 when partials is nullptr),
-// about the shift shift4 (nullptr: the means held in params); em as in launch_reduce_finalize.
-// kc: components per partial block (k for the direct E-step, CHUNK4 for chunks:
-// component b's partials at ((b / kc) * grid + cta) * kc + b % kc); the
-// log-likelihood is the sum of ll_partials[0 .. ll_count).
-cudaError_t launch_reduce_finalize4(const float* partials, int grid, int kc, const double* ll_partials,
+// M-step from the slices' partials of launch_reach_stats ([slices][pairs][2 NSTAT4], live
+// where live2 says) or, when partials is nullptr, from binary64 one-hot statistics stats64
+// about shift4; em as in launch_reduce_finalize, the log-likelihood being the sum of
+// llp[0 .. ll_count).  Slot b holds the caller's component perm[b] (nullptr: b).
+cudaError_t launch_reduce_finalize4(const float* partials, const uint32_t* live2, int slices, const double* llp,
                                     int ll_count, const double* stats64, const float4* shift4, int k, int64_t n,
                                     double reg, double tol, double* model64, float* params, double* trace,
-                                    DeviceState* st, int iter, bool em, cudaStream_t s, bool pdl = false);
-// Chunked E-step (K > MAX_K4_DIRECT): gref from all k components; pass A / B over
-// chunks x grid CTAs (pass 1 or 2); exact maximum for the points combine listed.
-cudaError_t launch_chunk_ref4(const float* params, int k, const DeviceState* st, float* gref, cudaStream_t s);
-cudaError_t launch_estep4_chunks(const EStep4Launch& a, int pass, int grid, cudaStream_t s);
-cudaError_t launch_chunk_exact4(const float4* pts8, const float* params, int k, const float* gref, const int* flags,
-                                const int* flag_count, float2* pref, double* llpt, DeviceState* st, cudaStream_t s);
+                                    const int* perm, DeviceState* st, int iter, bool em, cudaStream_t s);
+// Components in Morton order of their means, as launch_order_components (scratch: k * MODEL4 doubles).
+cudaError_t launch_order_components4(double* model64, double* scratch, int k, int* perm, float* params,
+                                     DeviceState* st, cudaStream_t s);
 cudaError_t launch_params_from_model4(const float* w, const float* mu, const float* cov, int k, double* model64,
                                       float* params, DeviceState* st, cudaStream_t s);
-cudaError_t launch_model_out4(const double* model64, int k, float* w, float* mu, float* cov, const DeviceState* st,
-                              cudaStream_t s);
+cudaError_t launch_model_out4(const double* model64, int k, float* w, float* mu, float* cov, const int* perm,
+                              const DeviceState* st, cudaStream_t s);
 // Lloyd in four dimensions and the one-hot statistics about the final centres.
 cudaError_t launch_lloyd4(const float4* pts4, int64_t n, int k, int lloyd_iters, float4* centers, int32_t* labels,
                           double* sums, unsigned long long* changed, DeviceState* st, cudaStream_t s);

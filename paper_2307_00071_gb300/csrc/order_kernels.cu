@@ -285,7 +285,8 @@ __global__ void __launch_bounds__(256) radix_scatter_kernel(const uint32_t* __re
     }
 }
 
-// The points in the sorted order: p8_out[j] = p8[order[j]] (and p4_out: (x, y, z, 0)).
+// The points in the sorted order: p8_out[j] = p8[order[j]] (and p4_out: (x, y, z, 0 or the
+// fourth coordinate)).
 __global__ void __launch_bounds__(256) gather_kernel(const int* __restrict__ order, int64_t n,
                                                      const float4* __restrict__ p8, float4* p8_out, float4* p4_out) {
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -295,7 +296,7 @@ __global__ void __launch_bounds__(256) gather_kernel(const int* __restrict__ ord
     const float4 a = p8[2 * s], b = p8[2 * s + 1];
     p8_out[2 * j] = a;
     p8_out[2 * j + 1] = b;
-    if (p4_out) p4_out[j] = make_float4(a.x, a.z, b.x, 0.f);
+    if (p4_out) p4_out[j] = make_float4(a.x, a.z, b.x, b.z);   // b.z: the fourth coordinate (0 in 3-D)
 }
 
 int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }

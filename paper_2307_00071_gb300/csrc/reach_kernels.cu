@@ -57,6 +57,12 @@ struct Lay<3> {
     static constexpr int SP = SLOT_P, SC = SLOT_C, SNMU = SLOT_NMU, SW = SLOT_W, SS = SLOT_S;
 };
 
+template <>
+struct Lay<4> {
+    static constexpr int NP = 10, NS = NSTAT4, PF = PAIR4_FLOATS;
+    static constexpr int SP = SLOT4_P, SC = SLOT4_C, SNMU = SLOT4_NMU, SW = SLOT4_W, SS = SLOT4_S;
+};
+
 // Parameters of a pair of components (slot-wise float2: components 2p, 2p + 1).
 template <int D>
 struct Pair {
@@ -819,13 +825,12 @@ __global__ void __launch_bounds__(32 * ST_W) reach_stats_kernel(const ReachLaunc
     if (lane == 0) atomicOr(live2 + live_off + (size_t)(pp >> 5) * slices + slice, 1u << (pp & 31));
 }
 
-template <int D>
-const void* reach_fn(int mode, int h) {
-    if (h == 2)
-        return mode == 0 ? (const void*)estep_reach_kernel<D, 2, 0>
-                         : mode == 1 ? (const void*)estep_reach_kernel<D, 2, 1> : (const void*)estep_reach_kernel<D, 2, 2>;
-    return mode == 0 ? (const void*)estep_reach_kernel<D, 4, 0>
-                     : mode == 1 ? (const void*)estep_reach_kernel<D, 4, 1> : (const void*)estep_reach_kernel<D, 4, 2>;
+template <int D, int H>
+const void* reach_fn(int mode) {
+    if (mode == 0) return (const void*)estep_reach_kernel<D, H, 0>;
+    if constexpr (D == 3)   // the gradient is 3-D
+        if (mode == 2) return (const void*)estep_reach_kernel<D, H, 2>;
+    return (const void*)estep_reach_kernel<D, H, 1>;
 }
 
 }  // namespace
@@ -843,15 +848,17 @@ int reach_grid(int64_t n) {
 int64_t reach_rows(int64_t n) { return (n + RB_PTS - 1) / RB_PTS; }
 int reach_mask_words(int k) { return reach_words(k); }
 
-cudaError_t launch_reach_prepare(const float* params, int k, const DeviceState* st, int iter, float4* ctr, float2* aux,
-                                 float* gref, cudaStream_t s) {
-    reach_prepare_kernel<3><<<1, std::min(PREP_THREADS, (k + 31) / 32 * 32), 0, s>>>(params, k, st, iter, ctr, aux,
-                                                                                    gref);
+cudaError_t launch_reach_prepare(int d, const float* params, int k, const DeviceState* st, int iter, float4* ctr,
+                                 float2* aux, float* gref, cudaStream_t s) {
+    const int threads = std::min(PREP_THREADS, (k + 31) / 32 * 32);
+    if (d == 3) reach_prepare_kernel<3><<<1, threads, 0, s>>>(params, k, st, iter, ctr, aux, gref);
+    else reach_prepare_kernel<4><<<1, threads, 0, s>>>(params, k, st, iter, ctr, aux, gref);
     return cudaGetLastError();
 }
 
-cudaError_t launch_estep_reach(const ReachLaunch& a, int mode, int grid, int h, int kmax, cudaStream_t s) {
-    const void* fn = reach_fn<3>(mode, h);
+cudaError_t launch_estep_reach(int d, const ReachLaunch& a, int mode, int grid, int h, int kmax, cudaStream_t s) {
+    const void* fn = d == 3 ? (h == 2 ? reach_fn<3, 2>(mode) : reach_fn<3, 4>(mode))
+                            : (h == 2 ? reach_fn<4, 2>(mode) : reach_fn<4, 4>(mode));
     note_estep_kernel(fn);
     const size_t smem = reach_smem(kmax, h);
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -860,12 +867,13 @@ cudaError_t launch_estep_reach(const ReachLaunch& a, int mode, int grid, int h, 
     return cudaLaunchKernel(fn, dim3(grid), dim3(32 * RB_W), args, smem, s);
 }
 
-cudaError_t launch_reach_stats(const ReachLaunch& a, int batch, int kmax, int64_t nmax, float* partials,
+cudaError_t launch_reach_stats(int d, const ReachLaunch& a, int batch, int kmax, int64_t nmax, float* partials,
                                uint32_t* live2, cudaStream_t s) {
     int sl = 1;
     const int slices = reach_slices(nmax, &sl);
     const dim3 grid(((kmax + 1) / 2 + ST_W - 1) / ST_W, slices, a.insts ? batch : 1);
-    reach_stats_kernel<3><<<grid, 32 * ST_W, 0, s>>>(a, sl, partials, live2);
+    if (d == 3) reach_stats_kernel<3><<<grid, 32 * ST_W, 0, s>>>(a, sl, partials, live2);
+    else reach_stats_kernel<4><<<grid, 32 * ST_W, 0, s>>>(a, sl, partials, live2);
     return cudaGetLastError();
 }
 

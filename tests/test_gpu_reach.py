@@ -85,3 +85,26 @@ def test_gradient_reach(gira, frame, n, k, off):
     check_all(r, ref_grads(pts, np.log(w), m, chol, R, t), n)
     only = gira.gira_gmm_loglik_grad(pts, np.log(w), m, chol, pose12(R, t), want=("twist",))   # no statistics launch
     assert np.array_equal(to_np(only["grad_twist"]), to_np(r["grad_twist"])) and only["loglik"] == r["loglik"]
+
+
+@pytest.mark.parametrize("n,k,off", [(1, 1, 0), (127, 2, 0), (4_097, 33, 5), (30_001, 1_023, 128), (8_193, 1_025, 600)])
+def test_4d_reach(gira, frame, n, k, off):
+    """Per-point log-likelihoods and one EM iteration in four dimensions."""
+    rng = np.random.default_rng(n + k)
+    start = rng.integers(0, len(frame) - n)
+    full = np.concatenate([frame, synth.frame_intensity(frame)[:, None]], axis=1)
+    pts = np.ascontiguousarray(full[start:start + n])
+    at = np.zeros(0, np.int64)
+    if off:
+        pts, at = off_model(pts, off, rng)
+    w, m, c = ball_model(full[start:start + max(n, k)], k, rng, d=4)
+    mean, pp = gira.gira_gmm_loglik4(pts, w, m, c, per_point=True)
+    pp = to_np(pp).astype(np.float64)
+    sample = np.unique(np.concatenate([at, [0, n - 1], rng.integers(0, n, 200)]))
+    _, _, lse = oracle.estep(pts[sample], w, m, c, want_resp=False, want_lse=True)
+    err, bound = np.abs(pp[sample] - lse), per_point_bound(pts[sample], w, m, c, form="d")
+    assert np.all(err <= bound), np.max(err / bound)
+    r = gira.gira_gmm_fit4(pts, k, iters=1, tol=0.0, init=(w, m, c))
+    ref = oracle.em(pts, w, m, c, iters=1, tol=0.0, reg=1e-6)
+    assert abs(r["trace"][0] - ref["trace"][0]) <= LL_ABS + 1e-7 * abs(ref["trace"][0])
+    assert_model_close((r["weights"], r["means"], r["covs"]), (ref["weights"], ref["means"], ref["covs"]))
