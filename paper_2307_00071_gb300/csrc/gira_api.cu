@@ -262,6 +262,45 @@ struct CallProfile {
     }
 };
 
+// k-means++ of one cloud (pts4 in the caller's order, which defines the draws), by the
+// first form that applies; every form draws the same points.
+//  - 3-D up to 294,912 points: one cluster with the points in shared memory;
+//  - 4-D, or more points: one cluster with the points in L2, when each of its warps has at
+//    most 8 sub-blocks of 32 points or the points' order is coherent (one kernel and one
+//    host round trip decide: 20 us against the milliseconds of a seeding).  A shuffled cloud
+//    of 1M points would touch all of a warp's 123 sub-blocks at every centre, several times
+//    the 12.4 us of the two launches; the figures are at kpp_blocks_kernel;
+//  - the persistent cooperative kernel (grid > 0), else two launches per centre.
+gira_status seed_centres(CallProfile& prof, Ctx& c, const float4* p4, int64_t n, int dim, int k, uint64_t seed,
+                         float4* c4, int64_t* ch, float* d2, u128* bs, int* ksync, u128* ksums, int kgrid,
+                         DeviceState* st) {
+    const int kcs = dim == 3 ? kpp_cluster_size(n) : 0;
+    if (kcs > 0) {
+        COUNTED(prof, 1, launch_kpp_cluster(p4, n, k, seed, c4, ch, kcs, st, c.s));
+        return GIRA_OK;
+    }
+    const int nsb = kpp_blocks_per_warp(n, dim);
+    if (nsb > 0) {
+        int coherent = 1;
+        if (nsb > 8) {
+            COUNTED(prof, 1, launch_kpp_coherence(p4, n, dim, st, c.s));
+            GIRA_CUDA(cudaMemcpyAsync(&coherent, &st->coherent, sizeof(int), cudaMemcpyDeviceToHost, c.s));
+            GIRA_CUDA(cudaStreamSynchronize(c.s));
+        }
+        if (coherent) {
+            COUNTED(prof, 1, launch_kpp_blocks(p4, n, k, seed, c4, ch, d2, nsb, st, c.s, dim));
+            return GIRA_OK;
+        }
+    }
+    if (kgrid > 0) {
+        GIRA_CUDA(cudaMemsetAsync(ksync, 0, sizeof(int) * (k + 1), c.s));
+        COUNTED(prof, 1, launch_kpp_persistent(p4, n, k, seed, c4, d2, ch, ksync, ksums, kgrid, st, c.s, dim));
+    } else {
+        COUNTED(prof, 2 * k - 1, launch_kpp(p4, n, k, seed, c4, d2, bs, ch, st, c.s, dim));
+    }
+    return GIRA_OK;
+}
+
 }  // namespace
 
 void gira::record_error(const char* msg, int component) {
@@ -467,15 +506,7 @@ gira_status gira_kmeans_init(const float* points, int64_t n, int k, uint64_t see
         pts = pin;
     }
     COUNTED(prof, 1, launch_pack(pts, n, p4, nullptr, st, c.s));
-    const int kcs = kpp_cluster_size(n);
-    if (kcs > 0) {
-        COUNTED(prof, 1, launch_kpp_cluster(p4, n, k, seed, c4, ch, kcs, st, c.s));
-    } else if (kgrid > 0) {
-        GIRA_CUDA(cudaMemsetAsync(ksync, 0, sizeof(int) * (k + 1), c.s));
-        COUNTED(prof, 1, launch_kpp_persistent(p4, n, k, seed, c4, d2, ch, ksync, ksums, kgrid, st, c.s));
-    } else {
-        COUNTED(prof, 2 * k - 1, launch_kpp(p4, n, k, seed, c4, d2, bs, ch, st, c.s));
-    }
+    TRY(seed_centres(prof, c, p4, n, 3, k, seed, c4, ch, d2, bs, ksync, ksums, kgrid, st));
     GIRA_CUDA(cudaMemsetAsync(sums, 0, sizeof(double) * 4 * k, c.s));
     GIRA_CUDA(cudaMemsetAsync(chg, 0, sizeof(unsigned long long) * (lloyd_iters + 1), c.s));
     COUNTED(prof, 1 + 2 * lloyd_iters, launch_lloyd(p4, n, k, lloyd_iters, c4, lab, sums, chg, st, c.s));
@@ -617,16 +648,7 @@ gira_status gira_gmm_fit(const float* points, int64_t n, int k, const gira_fit_o
     float* mu_d = (km == Kind::Device) ? means : b.mmu;
     float* cov_d = (kc == Kind::Device) ? covs : b.mcov;
     if (kinit) {
-        const int kcs = kpp_cluster_size(n);
-        if (kcs > 0) {
-            COUNTED(prof, 1, launch_kpp_cluster(b.p4, n, k, o.seed, b.c4, b.ch, kcs, b.st, c.s));
-        } else if (kgrid > 0) {
-            GIRA_CUDA(cudaMemsetAsync(b.ksync, 0, sizeof(int) * (k + 1), c.s));
-            COUNTED(prof, 1, launch_kpp_persistent(b.p4, n, k, o.seed, b.c4, b.d2, b.ch, b.ksync, b.ksums, kgrid, b.st,
-                                                   c.s));
-        } else {
-            COUNTED(prof, 2 * k - 1, launch_kpp(b.p4, n, k, o.seed, b.c4, b.d2, b.bs, b.ch, b.st, c.s));
-        }
+        TRY(seed_centres(prof, c, b.p4, n, 3, k, o.seed, b.c4, b.ch, b.d2, b.bs, b.ksync, b.ksums, kgrid, b.st));
         GIRA_CUDA(cudaMemsetAsync(b.sums, 0, sizeof(double) * 4 * k, c.s));
         GIRA_CUDA(cudaMemsetAsync(b.chg, 0, sizeof(unsigned long long) * (o.lloyd_iters + 1), c.s));
         COUNTED(prof, 1 + 2 * o.lloyd_iters,
@@ -1207,11 +1229,10 @@ gira_status gira_gmm_fit_batched(const float* points, const int64_t* offsets, in
                                                         sc.first, b.st, c.s));
             seed_off += sc.second;
         }
-        for (int i : seed_alone) {   // beyond one 16-CTA cluster: two launches per centre
+        for (int i : seed_alone) {   // beyond one 16-CTA cluster
             const BatchInst& I = hi[i];
-            COUNTED(prof, 2 * I.k - 1, launch_kpp(b.p4 + I.pt_off, I.n, I.k, o.seed, b.c4 + I.comp_off,
-                                                  b.d2 + I.pt_off, b.bs + nblk_off[i], b.ch + I.comp_off, b.st + i,
-                                                  c.s));
+            TRY(seed_centres(prof, c, b.p4 + I.pt_off, I.n, 3, I.k, o.seed, b.c4 + I.comp_off, b.ch + I.comp_off,
+                             b.d2 + I.pt_off, b.bs + nblk_off[i], nullptr, nullptr, 0, b.st + i));
         }
         const float4* p4l = sorted ? b.p4s : b.p4;   // Lloyd and the one-hot statistics: sorted points
         COUNTED(prof, 1 + 2 * o.lloyd_iters,
@@ -1710,13 +1731,7 @@ gira_status gira_gmm_fit4(const float* points, int64_t n, int k, const gira_fit_
     float* mu_d = (km == Kind::Device) ? means : b.mmu;
     float* cov_d = (kc == Kind::Device) ? covs : b.mcov;
     if (kinit) {
-        if (kgrid > 0) {
-            GIRA_CUDA(cudaMemsetAsync(b.ksync, 0, sizeof(int) * (k + 1), c.s));
-            COUNTED(prof, 1, launch_kpp_persistent(b.p4, n, k, o.seed, b.c4, b.d2, b.ch, b.ksync, b.ksums, kgrid, b.st,
-                                                   c.s, 4));
-        } else {
-            COUNTED(prof, 2 * k - 1, launch_kpp(b.p4, n, k, o.seed, b.c4, b.d2, b.bs, b.ch, b.st, c.s, 4));
-        }
+        TRY(seed_centres(prof, c, b.p4, n, 4, k, o.seed, b.c4, b.ch, b.d2, b.bs, b.ksync, b.ksums, kgrid, b.st));
         GIRA_CUDA(cudaMemsetAsync(b.sums, 0, sizeof(double) * 5 * k, c.s));
         GIRA_CUDA(cudaMemsetAsync(b.chg, 0, sizeof(unsigned long long) * (o.lloyd_iters + 1), c.s));
         COUNTED(prof, 1 + 2 * o.lloyd_iters, launch_lloyd4(b.p4, n, k, o.lloyd_iters, b.c4, b.lab, b.sums, b.chg,

@@ -46,6 +46,7 @@ struct DeviceState {
     // point-stationary E-step with statistics, summed over its launches: warp x pair
     // evaluations made (pairs within reach of the warp's box) and with statistics
     unsigned long long pairs_near, pairs_live;
+    int coherent;          // k-means++: the points' order keeps neighbours together (launch_kpp_coherence)
     int cmax_ord;          // gradient: max_b c_b as an order-preserving int (host: that of -inf)
 };
 constexpr int CMAX_ORD_NONE = (int)0x807fffff;   // -inf
@@ -583,6 +584,13 @@ int64_t kpp_persistent_max_n(int grid);
 cudaError_t launch_kpp_persistent(const float4* pts4, int64_t n, int k, uint64_t seed, float4* centers, float* d2,
                                   int64_t* chosen, int* sync_ints, u128* sums, int grid, DeviceState* st,
                                   cudaStream_t s, int dim = 3);
+// k-means++ by one cluster over sub-blocks of 32 points kept in L2 (any dim): sub-blocks per
+// warp for n points (0: not applicable); worth it when the points' order is coherent
+// (launch_kpp_coherence sets st->coherent) or each warp has few.  d2: n floats.
+int kpp_blocks_per_warp(int64_t n, int dim);
+cudaError_t launch_kpp_coherence(const float4* pts4, int64_t n, int dim, DeviceState* st, cudaStream_t s);
+cudaError_t launch_kpp_blocks(const float4* pts4, int64_t n, int k, uint64_t seed, float4* centers, int64_t* chosen,
+                              float* d2, int nsb, DeviceState* st, cudaStream_t s, int dim);
 // Batched KInit: one entry per instance.
 struct KppInst {
     int64_t pt_off, n;

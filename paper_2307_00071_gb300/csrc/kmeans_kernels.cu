@@ -509,6 +509,92 @@ __device__ __forceinline__ unsigned long long fx48_join(unsigned ah, unsigned am
            (unsigned long long)(al - bias);
 }
 
+// One warp, every block's total present: the block (CTA, warp) holding the threshold and
+// the threshold within it.  Returns whether every weight is zero.
+__device__ __forceinline__ bool kc_select(KcShared& sh, int b, int nblk, int cs, bool m64, unsigned long long k53,
+                                          int lane) {
+    constexpr int PER = KC_PER;   // blocks per lane, in order
+    bool tz;
+    if (m64) {
+        // 64-bit totals: lane l's blocks in registers, their sum, the warp's prefix
+        const unsigned long long* c64 = reinterpret_cast<const unsigned long long*>(sh.csum[b]);
+        unsigned long long run = 0ull;
+#pragma unroll
+        for (int q = 0; q < PER; ++q) run += lane * PER + q < nblk ? c64[q * 32 + lane] : 0ull;
+        const unsigned long long lincl = u64_warp_incl_scan(run, lane);
+        const unsigned long long T = __shfl_sync(FULL, lincl, 31);
+        tz = T == 0ull;
+        if (!tz) {
+            const unsigned long long t = fx_threshold(k53, u128{T, 0ull}).lo;   // t < T
+            const unsigned hits = __ballot_sync(FULL, lincl > t);
+            const int hl = hits ? __ffs(hits) - 1 : 0;
+            if (lane == hl) {   // the first of this lane's blocks whose running sum exceeds r
+                const unsigned long long r = t - (lincl - run);
+                unsigned long long pre = 0ull, prev = 0ull;   // pre: the running sum through block u
+                int q = -1;
+                unsigned long long v[PER];   // the lane's blocks again (independent loads)
+#pragma unroll
+                for (int u = 0; u < PER; ++u) v[u] = lane * PER + u < nblk ? c64[u * 32 + lane] : 0ull;
+#pragma unroll
+                for (int u = 0; u < PER; ++u) {
+                    const unsigned long long nx = pre + v[u];
+                    if (q < 0 && nx > r) {
+                        q = u;
+                        prev = pre;
+                    }
+                    pre = nx;
+                }
+                if (q < 0) {   // never: r is below the lane's sum
+                    q = PER - 1;
+                    prev = pre - v[PER - 1];
+                }
+                const int gw = lane * PER + q;
+                sh.win = gw % cs;
+                sh.wwin = gw / cs;
+                sh.rel = u128{r - prev, 0ull};
+                sh.mode = 0;
+            }
+        }
+    } else {
+        u128 run{0ull, 0ull};
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            const int gq = lane * PER + q;
+            run = u128_add(run, gq < nblk ? sh.csum[b][q * 32 + lane] : u128{0ull, 0ull});
+        }
+        const u128 lincl = u128_warp_incl_scan(run, lane);
+        const u128 before = u128_sub(lincl, run);   // the blocks of lower lanes
+        const u128 T = u128_shfl(lincl, 31);
+        tz = u128_zero(T);
+        if (lane == 0 && T.hi == 0ull) sh.m64 = 1;   // from the next centre on: 64-bit totals
+        if (!tz) {
+            const u128 t = fx_threshold(k53, T);
+            const unsigned hits = __ballot_sync(FULL, u128_gt(lincl, t));   // t < T: not empty
+            const int hl = hits ? __ffs(hits) - 1 : 0;
+            if (lane == hl) {   // the first of this lane's blocks whose running sum exceeds r
+                const u128 r = u128_sub(t, before);
+                u128 acc{0ull, 0ull}, prev{0ull, 0ull};
+                int q = PER - 1;
+                for (int u = 0; u < PER; ++u) {
+                    const int gq = lane * PER + u;
+                    acc = u128_add(acc, gq < nblk ? sh.csum[b][u * 32 + lane] : u128{0ull, 0ull});
+                    if (u128_gt(acc, r)) {
+                        q = u;
+                        break;
+                    }
+                    prev = acc;
+                }
+                const int gw = lane * PER + q;
+                sh.win = gw % cs;
+                sh.wwin = gw / cs;
+                sh.rel = u128_sub(r, prev);
+                sh.mode = 0;
+            }
+        }
+    }
+    return tz;
+}
+
 // table (batched seeding): cluster c of the launch seeds instance table[c]; the
 // pointers are then bases offset by its entry.
 __global__ void __launch_bounds__(KC_THREADS, 1) kpp_cluster_kernel(const float4* __restrict__ pts0, int64_t n0,
@@ -670,85 +756,7 @@ __global__ void __launch_bounds__(KC_THREADS, 1) kpp_cluster_kernel(const float4
                 dead = true;
                 set_error(st, GIRA_ERR_TIMEOUT);
             }
-            constexpr int PER = KC_PER;   // blocks per lane, in order
-            bool tz;   // every weight is zero
-            if (m64) {
-                // 64-bit totals: lane l's blocks in registers, their sum, the warp's prefix
-                const unsigned long long* c64 = reinterpret_cast<const unsigned long long*>(sh.csum[b]);
-                unsigned long long run = 0ull;
-#pragma unroll
-                for (int q = 0; q < PER; ++q) run += lane * PER + q < nblk ? c64[q * 32 + lane] : 0ull;
-                const unsigned long long lincl = u64_warp_incl_scan(run, lane);
-                const unsigned long long T = __shfl_sync(FULL, lincl, 31);
-                tz = T == 0ull;
-                if (!tz) {
-                    const unsigned long long t = fx_threshold(k53, u128{T, 0ull}).lo;   // t < T
-                    const unsigned hits = __ballot_sync(FULL, lincl > t);
-                    const int hl = hits ? __ffs(hits) - 1 : 0;
-                    if (lane == hl) {   // the first of this lane's blocks whose running sum exceeds r
-                        const unsigned long long r = t - (lincl - run);
-                        unsigned long long pre = 0ull, prev = 0ull;   // pre: the running sum through block u
-                        int q = -1;
-                        unsigned long long v[PER];   // the lane's blocks again (independent loads)
-#pragma unroll
-                        for (int u = 0; u < PER; ++u) v[u] = lane * PER + u < nblk ? c64[u * 32 + lane] : 0ull;
-#pragma unroll
-                        for (int u = 0; u < PER; ++u) {
-                            const unsigned long long nx = pre + v[u];
-                            if (q < 0 && nx > r) {
-                                q = u;
-                                prev = pre;
-                            }
-                            pre = nx;
-                        }
-                        if (q < 0) {   // never: r is below the lane's sum
-                            q = PER - 1;
-                            prev = pre - v[PER - 1];
-                        }
-                        const int gw = lane * PER + q;
-                        sh.win = gw % cs;
-                        sh.wwin = gw / cs;
-                        sh.rel = u128{r - prev, 0ull};
-                        sh.mode = 0;
-                    }
-                }
-            } else {
-                u128 run{0ull, 0ull};
-#pragma unroll
-                for (int q = 0; q < PER; ++q) {
-                    const int gq = lane * PER + q;
-                    run = u128_add(run, gq < nblk ? sh.csum[b][q * 32 + lane] : u128{0ull, 0ull});
-                }
-                const u128 lincl = u128_warp_incl_scan(run, lane);
-                const u128 before = u128_sub(lincl, run);   // the blocks of lower lanes
-                const u128 T = u128_shfl(lincl, 31);
-                tz = u128_zero(T);
-                if (lane == 0 && T.hi == 0ull) sh.m64 = 1;   // from the next centre on: 64-bit totals
-                if (!tz) {
-                    const u128 t = fx_threshold(k53, T);
-                    const unsigned hits = __ballot_sync(FULL, u128_gt(lincl, t));   // t < T: not empty
-                    const int hl = hits ? __ffs(hits) - 1 : 0;
-                    if (lane == hl) {   // the first of this lane's blocks whose running sum exceeds r
-                        const u128 r = u128_sub(t, before);
-                        u128 acc{0ull, 0ull}, prev{0ull, 0ull};
-                        int q = PER - 1;
-                        for (int u = 0; u < PER; ++u) {
-                            const int gq = lane * PER + u;
-                            acc = u128_add(acc, gq < nblk ? sh.csum[b][u * 32 + lane] : u128{0ull, 0ull});
-                            if (u128_gt(acc, r)) {
-                                q = u;
-                                break;
-                            }
-                            prev = acc;
-                        }
-                        const int gw = lane * PER + q;
-                        sh.win = gw % cs;
-                        sh.wwin = gw / cs;
-                        sh.rel = u128_sub(r, prev);
-                        sh.mode = 0;
-                    }
-                }
-            }
+            const bool tz = kc_select(sh, b, nblk, cs, m64, k53, lane);
             if (!tz) {
                 // this phase of bar_cen[b] expects the chosen point and its index
                 if (lane == 0 && !dead) mbar_expect_tx(&sh.bar_cen[b], (uint32_t)(sizeof(float4) + sizeof(long long)));
@@ -834,6 +842,335 @@ __global__ void __launch_bounds__(KC_THREADS, 1) kpp_cluster_kernel(const float4
         idx = sh.idx[b];
     }
     cluster.sync();   // no CTA leaves while a peer may still address its shared memory
+}
+
+// ---------------------------------------------------------------- k-means++ in one cluster, points in L2
+// For 4-D points and for more 3-D points than kpp_cluster_kernel's shared memory holds,
+// when the points come in an order that keeps neighbours together (a sensor's): the same
+// protocol, but the points and their D^2 stay in global memory (L2) and a warp keeps, per
+// sub-block of 32 consecutive points, the box, the largest D^2 and the exact total in
+// shared memory.  A new centre reaches the few sub-blocks whose box is nearer than their
+// largest D^2: the lanes test the boxes of their warp's sub-blocks into a list of the CTA,
+// and the CTA's warps share the listed ones (a patch of rows lies in one or two warps'
+// blocks of each CTA: taken by their owners alone, a warp had 20 of them in turn at 1M
+// points, 13.3 us per centre), one point per lane, up to four sub-blocks' loads in flight,
+// the exact total by three integer reductions of the fixed-point pieces.  The warp that
+// holds the threshold scans its sub-block totals, then one sub-block's 32 weights.
+// What bounds it: the chain of one centre (an L2 round trip to update, the totals to every
+// CTA, the search, another round trip, the point to every CTA), not the points.  Measured
+// (GB300): 1M points of 4 frames, K = 768, 5.9 us per centre (two launches per centre:
+// 12.4); the 276,348-point frame with intensity, K = 512, 3.9 us (the persistent kernel: 8.3).
+template <int DIM>
+__device__ __forceinline__ float dist2_dim(float4 x, float4 c) {
+    return DIM == 4 ? dist2_f32_4(x, c) : dist2_f32(x, c);
+}
+__device__ __forceinline__ int ord_f(float f) {   // order-preserving int, its own inverse
+    const int i = __float_as_int(f);
+    return i >= 0 ? i : i ^ 0x7fffffff;
+}
+__device__ __forceinline__ float f_ord(int i) { return __int_as_float(i >= 0 ? i : i ^ 0x7fffffff); }
+// fx48 of a weight below 2^10 as its three pieces (fx48_parts without the biases)
+__device__ __forceinline__ void fx48_pieces(float d, unsigned& h, unsigned& m, unsigned& l) {
+    h = m = l = 0u;
+    fx48_parts(d, h, m, l);
+    h -= 0x4B000000u;
+    m -= 0x4B000000u;
+    l -= 0x4B000000u;
+}
+// shared memory per sub-block: box, total, largest D^2, list entry
+constexpr size_t kb_sub_bytes(int dim) { return (size_t)dim * 8 + sizeof(u128) + 4 + 2; }
+constexpr int KB_FLIGHT = 4;   // reached sub-blocks loaded at once
+
+template <int DIM>
+__global__ void __launch_bounds__(KC_THREADS, 1) kpp_blocks_kernel(const float4* __restrict__ pts, int64_t n, int k,
+                                                                   uint64_t seed, float4* centers, int64_t* chosen,
+                                                                   float* __restrict__ d2, int nsb, DeviceState* st) {
+    extern __shared__ __align__(16) unsigned char kb_dsm[];
+    KcShared& sh = *reinterpret_cast<KcShared*>(kb_dsm);
+    const int ns = KC_WARPS * nsb;   // sub-blocks of the CTA (nsb per warp)
+    u128* tot = reinterpret_cast<u128*>(kb_dsm + ((sizeof(KcShared) + 15) & ~size_t(15)));
+    float* box = reinterpret_cast<float*>(tot + ns);   // [2 DIM][ns]: lows, then highs
+    float* dmax = box + 2 * DIM * ns;
+    uint16_t* list = reinterpret_cast<uint16_t*>(dmax + ns);   // the reached sub-blocks of this centre
+    __shared__ unsigned long long s_wtot[KC_WARPS][2];         // every block's total (lo, hi)
+    __shared__ int s_cnt[2];                                   // list length, by parity of j
+    cg::cluster_group cluster = cg::this_cluster();
+    const int cs = (int)cluster.num_blocks(), me = (int)cluster.block_rank();
+    if (st->error) return;   // set before the launch: every CTA of the cluster leaves
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // block g of 32 nsb consecutive points belongs to warp g / cs of CTA g % cs
+    const int g = warp * cs + me;
+    const int64_t p0 = (int64_t)g * nsb * 32;
+    const int nsub = (int)max((int64_t)0, min((int64_t)nsb, (n - p0 + 31) / 32));
+    const int w0 = warp * nsb;   // the warp's first sub-block in the CTA's arrays
+    for (int q = 0; q < nsub; ++q) {
+        const int64_t i = p0 + 32 * q + lane;
+        const bool ok = i < n;
+        const float4 x = __ldg(pts + (ok ? i : n - 1));   // an absent point: the last one, inside the box
+        const float v[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+        for (int c = 0; c < DIM; ++c) {
+            const int lo = __reduce_min_sync(FULL, ord_f(v[c])), hi = __reduce_max_sync(FULL, ord_f(v[c]));
+            if (lane == 0) {
+                box[c * ns + w0 + q] = f_ord(lo);
+                box[(DIM + c) * ns + w0 + q] = f_ord(hi);
+            }
+        }
+        if (lane == 0) {
+            tot[w0 + q] = u128{0ull, 0ull};
+            dmax[w0 + q] = INFINITY;   // the first centre reaches every sub-block
+        }
+    }
+    if (tid < 2) s_cnt[tid] = 0;
+    if (lane < 2) s_wtot[warp][lane] = 0ull;
+    int64_t idx = (int64_t)floor(uniform53(seed, 0) * (double)n);
+    if (idx > n - 1) idx = n - 1;
+    float4 cen = __ldg(pts + idx);
+    if (me == 0 && tid == 0) {
+        centers[0] = cen;
+        chosen[0] = idx;
+    }
+    if (tid == 0) {
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&sh.bar_sum[b], 1);
+            mbar_init(&sh.bar_cen[b], 1);
+        }
+        sh.m64 = 0;
+        mbar_fence_init();
+    }
+    cluster.sync();   // every CTA has started and initialised its mbarriers before any DSMEM access
+    unsigned ph_sum = 0u, ph_cen = 0u;   // per parity b: the parity of the phase to wait for next
+    bool dead = false;                    // this thread gave up a wait: stop waiting, run to the end
+    const int nblk = cs * KC_WARPS;
+    for (int j = 1; j < k; ++j) {
+        const int b = j & 1;
+        const bool m64 = sh.m64 != 0;   // as in kpp_cluster_kernel
+        // ---- 1. the sub-blocks within reach of the centre
+        const float cv[4] = {cen.x, cen.y, cen.z, cen.w};
+        for (int r0 = 0; r0 < nsub; r0 += 32) {
+            const int q = r0 + lane;
+            bool in = false;
+            if (q < nsub) {
+                float e2 = 0.f;
+#pragma unroll
+                for (int c = 0; c < DIM; ++c) {
+                    const float e = fmaxf(fmaxf(box[c * ns + w0 + q] - cv[c], cv[c] - box[(DIM + c) * ns + w0 + q]), 0.f);
+                    e2 = fmaf(e, e, e2);
+                }
+                // (the slack covers the rounding of the box distance and of every D^2)
+                in = e2 * (1.f - 1e-5f) <= dmax[w0 + q];
+            }
+            const unsigned m = __ballot_sync(FULL, in);
+            int base = 0;
+            if (lane == 0 && m) base = atomicAdd(&s_cnt[b], __popc(m));
+            base = __shfl_sync(FULL, base, 0);
+            if (in) list[base + __popc(m & ((1u << lane) - 1u))] = (uint16_t)(w0 + q);
+        }
+        __syncthreads();
+        const int cnt = s_cnt[b];
+        if (tid == 0) s_cnt[b ^ 1] = 0;   // free since the barrier: read before the previous centre's end
+        if (cnt > 0) {
+            for (int e0 = warp; e0 < cnt; e0 += KC_WARPS * KB_FLIGHT) {
+                int at[KB_FLIGHT];
+                float4 x[KB_FLIGHT];
+                float dn[KB_FLIGHT], dold[KB_FLIGHT];
+                int64_t i[KB_FLIGHT];
+                bool ok[KB_FLIGHT];
+#pragma unroll
+                for (int u = 0; u < KB_FLIGHT; ++u) {
+                    const int e = e0 + u * KC_WARPS;
+                    at[u] = e < cnt ? (int)list[e] : -1;
+                    // sub-block at[u] % nsb of warp at[u] / nsb
+                    const int w = max(at[u], 0) / nsb;
+                    i[u] = ((int64_t)(w * cs + me) * nsb + (max(at[u], 0) - w * nsb)) * 32 + lane;
+                    ok[u] = at[u] >= 0 && i[u] < n;
+                    x[u] = ok[u] ? __ldg(pts + i[u]) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    dold[u] = (ok[u] && j > 1) ? d2[i[u]] : INFINITY;
+                }
+#pragma unroll
+                for (int u = 0; u < KB_FLIGHT; ++u) {
+                    if (at[u] < 0) continue;
+                    dn[u] = ok[u] ? fminf(dold[u], dist2_dim<DIM>(x[u], cen)) : 0.f;
+                    const bool low = ok[u] && dn[u] < dold[u];
+                    if (low) d2[i[u]] = dn[u];
+                    if (!__any_sync(FULL, low) && j > 1) continue;   // no D^2 dropped
+                    u128 t{0ull, 0ull};
+                    if (__any_sync(FULL, !(dn[u] < 1024.f))) {   // a weight >= 2^10: sum in 128 bits
+                        t = u128_shfl(u128_warp_incl_scan(fx48(dn[u]), lane), 31);
+                    } else {
+                        unsigned ph, pm, pl;
+                        fx48_pieces(dn[u], ph, pm, pl);
+                        ph = __reduce_add_sync(FULL, ph);
+                        pm = __reduce_add_sync(FULL, pm);
+                        pl = __reduce_add_sync(FULL, pl);
+                        t.lo = ((unsigned long long)ph << 35) + ((unsigned long long)pm << 12) + pl;   // < 2^63
+                    }
+                    const unsigned mx = __reduce_max_sync(FULL, __float_as_uint(dn[u]));   // D^2 >= 0
+                    if (lane == 0) {   // the block's total by the difference (mod 2^128: any order)
+                        const u128 dt = u128_sub(t, tot[at[u]]);
+                        unsigned long long* wt = s_wtot[at[u] / nsb];
+                        const unsigned long long was = atomicAdd(&wt[0], dt.lo);
+                        const unsigned long long up = dt.hi + (was + dt.lo < was ? 1ull : 0ull);
+                        if (up) atomicAdd(&wt[1], up);
+                        tot[at[u]] = t;
+                        dmax[at[u]] = __uint_as_float(mx);
+                    }
+                }
+            }
+            __syncthreads();   // totals, D^2 and boxes' maxima of the CTA
+        }
+        const u128 wtot{s_wtot[warp][0], s_wtot[warp][1]};
+        if (tid == 0 && !dead) mbar_expect_tx(&sh.bar_sum[b], (uint32_t)nblk * (m64 ? 8u : 16u));
+        const unsigned long long k53 = splitmix64(seed, (uint64_t)j) >> 11;
+        {   // this warp's block total, to every CTA's slot of block g
+            const int slot = (g % KC_PER) * 32 + g / KC_PER;
+            if (lane < cs && !dead) {
+                const uint32_t bar = kc_peer(&sh.bar_sum[b], lane);
+                if (m64) kc_send_s64(kc_peer(reinterpret_cast<unsigned long long*>(sh.csum[b]) + slot, lane),
+                                     (long long)wtot.lo, bar);
+                else kc_send_u128(kc_peer(&sh.csum[b][slot], lane), wtot, bar);
+            }
+        }
+        if (warp == 0) {
+            // ---- 2. every block's total has arrived: the block holding the threshold
+            if (!dead && !kc_wait(&sh.bar_sum[b], (ph_sum >> b) & 1u)) {
+                dead = true;
+                set_error(st, GIRA_ERR_TIMEOUT);
+            }
+            const bool tz = kc_select(sh, b, nblk, cs, m64, k53, lane);
+            if (!tz) {
+                if (lane == 0 && !dead) mbar_expect_tx(&sh.bar_cen[b], (uint32_t)(sizeof(float4) + sizeof(long long)));
+            } else if (lane == 0) {   // every weight is zero: uniform index, the same in every CTA
+                long long id2 = (long long)floor(uniform53(seed, (uint64_t)j) * (double)n);
+                if (id2 > n - 1) id2 = n - 1;
+                sh.idx[b] = id2;
+                sh.cen[b] = __ldg(pts + id2);
+                sh.mode = 2;
+                if (me == 0) {
+                    centers[j] = sh.cen[b];
+                    chosen[j] = id2;
+                }
+            }
+        }
+        ph_sum ^= 1u << b;
+        __syncthreads();
+        const int mode = sh.mode;
+        if (mode == 0 && sh.win == me && warp == sh.wwin) {
+            // ---- 3. this warp holds the point: the sub-block, then its points
+            const u128 rel = sh.rel;
+            const int per = (nsub + 31) / 32, a0 = min(nsub, lane * per), a1 = min(nsub, a0 + per);
+            u128 loc{0ull, 0ull}, inc;
+            if (m64) {   // every total is below 2^64
+                for (int q = a0; q < a1; ++q) loc.lo += tot[w0 + q].lo;
+                inc = u128{u64_warp_incl_scan(loc.lo, lane), 0ull};
+            } else {
+                for (int q = a0; q < a1; ++q) loc = u128_add(loc, tot[w0 + q]);
+                inc = u128_warp_incl_scan(loc, lane);
+            }
+            const unsigned lh = __ballot_sync(FULL, u128_gt(inc, rel));   // rel < the block's total: not empty
+            const int src = lh ? __ffs(lh) - 1 : 0;
+            int sub = 0;
+            u128 rem{0ull, 0ull};
+            if (lane == src) {
+                u128 run = u128_sub(inc, loc);
+                sub = max(a1 - 1, 0);
+                for (int q = a0; q < a1; ++q) {
+                    const u128 nx = u128_add(run, tot[w0 + q]);
+                    if (u128_gt(nx, rel)) {
+                        sub = q;
+                        break;
+                    }
+                    run = nx;
+                }
+                rem = u128_sub(rel, run);
+            }
+            sub = __shfl_sync(FULL, sub, src);
+            rem = u128_shfl(rem, src);
+            const int64_t i = p0 + 32 * (int64_t)sub + lane;
+            const bool ok = sub < nsub && i < n;
+            const float4 x = __ldg(pts + (ok ? i : n - 1));
+            const float d = ok ? d2[i] : 0.f;
+            unsigned hh;
+            if (m64) {   // the sub-block's total is below 2^64
+                hh = __ballot_sync(FULL, u64_warp_incl_scan(fx48(d).lo, lane) > rem.lo);
+            } else {
+                hh = __ballot_sync(FULL, u128_gt(u128_warp_incl_scan(fx48(d), lane), rem));
+            }
+            const int hl = hh ? __ffs(hh) - 1 : 0;
+            const float4 pf = make_float4(__shfl_sync(FULL, x.x, hl), __shfl_sync(FULL, x.y, hl),
+                                          __shfl_sync(FULL, x.z, hl), __shfl_sync(FULL, x.w, hl));
+            const long long found = min((long long)n - 1, (long long)(p0 + 32 * (int64_t)sub + hl));   // clamp never taken
+            if (lane < cs && !dead) {
+                const uint32_t bar = kc_peer(&sh.bar_cen[b], lane);
+                kc_send_f4(kc_peer(&sh.cen[b], lane), pf, bar);
+                kc_send_s64(kc_peer(&sh.idx[b], lane), found, bar);
+            }
+            if (lane == 0) {
+                centers[j] = pf;
+                chosen[j] = found;
+            }
+        }
+        if (mode == 0) {   // uniform over the cluster: the same totals give the same mode
+            if (!dead && !kc_wait(&sh.bar_cen[b], (ph_cen >> b) & 1u)) {
+                dead = true;
+                set_error(st, GIRA_ERR_TIMEOUT);
+            }
+            ph_cen ^= 1u << b;
+        }
+        cen = sh.cen[b];
+    }
+    cluster.sync();   // no CTA leaves while a peer may still address its shared memory
+}
+
+// Whether the points come in an order that keeps neighbours together: over up to 1,024
+// sub-blocks of 32 consecutive points, spread evenly, the mean of the largest box extent
+// against the extent of all of them (st->coherent = 1 when below a quarter; a shuffled
+// cloud has about 0.9, a depth image's rows 0.02 .. 0.1).
+__global__ void __launch_bounds__(1024) kpp_coherence_kernel(const float4* __restrict__ pts, int64_t n, int dim,
+                                                             DeviceState* st) {
+    __shared__ float s_sum[32], s_lo[32][4], s_hi[32][4];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t subs = (n + 31) / 32;
+    const int take = (int)min(subs, (int64_t)1024);
+    float sum = 0.f, LO[4], HI[4];
+    for (int c = 0; c < 4; ++c) {
+        LO[c] = INFINITY;
+        HI[c] = -INFINITY;
+    }
+    for (int t = warp; t < take; t += 32) {
+        const int64_t i = min(n - 1, (int64_t)t * subs / take * 32 + lane);
+        const float4 x = __ldg(pts + i);
+        const float v[4] = {x.x, x.y, x.z, x.w};
+        float ext = 0.f;
+        for (int c = 0; c < dim; ++c) {
+            const float lo = f_ord(__reduce_min_sync(FULL, ord_f(v[c]))), hi = f_ord(__reduce_max_sync(FULL, ord_f(v[c])));
+            ext = fmaxf(ext, hi - lo);
+            LO[c] = fminf(LO[c], lo);
+            HI[c] = fmaxf(HI[c], hi);
+        }
+        sum += ext;
+    }
+    if (lane == 0) {
+        s_sum[warp] = sum;
+        for (int c = 0; c < 4; ++c) {
+            s_lo[warp][c] = LO[c];
+            s_hi[warp][c] = HI[c];
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        float ext = 0.f, tot = 0.f;
+        for (int c = 0; c < dim; ++c) {
+            float lo = INFINITY, hi = -INFINITY;
+            for (int w = 0; w < 32; ++w) {
+                lo = fminf(lo, s_lo[w][c]);
+                hi = fmaxf(hi, s_hi[w][c]);
+            }
+            ext = fmaxf(ext, hi - lo);
+        }
+        for (int w = 0; w < 32; ++w) tot += s_sum[w];
+        st->coherent = tot <= 0.25f * ext * (float)take ? 1 : 0;
+    }
 }
 
 // ---------------------------------------------------------------- Lloyd
@@ -1263,6 +1600,65 @@ cudaError_t launch_kpp_cluster(const float4* pts4, int64_t n, int k, uint64_t se
     cfg.attrs = at;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kpp_cluster_kernel, pts4, n, k, seed, centers, chosen, st, (const KppInst*)nullptr);
+}
+
+namespace {
+// Shared memory of the seeding over sub-blocks: nsb sub-blocks per warp.
+size_t kb_smem_bytes(int dim, int nsb) {
+    return ((sizeof(KcShared) + 15) & ~size_t(15)) + (size_t)KC_WARPS * nsb * kb_sub_bytes(dim);
+}
+cudaLaunchConfig_t kb_config(int cs, size_t smem, cudaLaunchAttribute* at, cudaStream_t s) {
+    cudaLaunchConfig_t cfg{};
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = cs;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(cs);
+    cfg.blockDim = dim3(KC_THREADS);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+constexpr size_t KB_SMEM_MAX = 224 * 1024;
+}  // namespace
+
+// Sub-blocks per warp for the one-cluster seeding of n points in L2, or 0 when it does not
+// apply (too many points, or a cluster of 16 does not fit on this GPU).
+int kpp_blocks_per_warp(int64_t n, int dim) {
+    static std::atomic<int> usable{-1};
+    int ok = usable.load();
+    if (ok < 0) {
+        ok = 1;
+        for (int d = 3; d <= 4 && ok; ++d) {
+            const void* fn = d == 3 ? (const void*)kpp_blocks_kernel<3> : (const void*)kpp_blocks_kernel<4>;
+            cudaLaunchAttribute at[1];
+            const cudaLaunchConfig_t cfg = kb_config(KC_MAX_CS, KB_SMEM_MAX, at, nullptr);
+            int nclusters = 0;
+            ok = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)KB_SMEM_MAX) == cudaSuccess &&
+                 cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+                 cudaOccupancyMaxActiveClusters(&nclusters, fn, &cfg) == cudaSuccess && nclusters >= 1;
+        }
+        cudaGetLastError();
+        usable.store(ok);   // racing first calls compute the same value
+    }
+    const int64_t nsb = ((n + 31) / 32 + KC_MAX_CS * KC_WARPS - 1) / (KC_MAX_CS * KC_WARPS);
+    if (!ok || nsb > INT_MAX / 64 || kb_smem_bytes(dim, (int)nsb) > KB_SMEM_MAX) return 0;
+    return (int)nsb;
+}
+
+cudaError_t launch_kpp_coherence(const float4* pts4, int64_t n, int dim, DeviceState* st, cudaStream_t s) {
+    kpp_coherence_kernel<<<1, 1024, 0, s>>>(pts4, n, dim, st);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_kpp_blocks(const float4* pts4, int64_t n, int k, uint64_t seed, float4* centers, int64_t* chosen,
+                              float* d2, int nsb, DeviceState* st, cudaStream_t s, int dim) {
+    cudaLaunchAttribute at[1];
+    const cudaLaunchConfig_t cfg = kb_config(KC_MAX_CS, kb_smem_bytes(dim, nsb), at, s);
+    return dim == 4 ? cudaLaunchKernelEx(&cfg, kpp_blocks_kernel<4>, pts4, n, k, seed, centers, chosen, d2, nsb, st)
+                    : cudaLaunchKernelEx(&cfg, kpp_blocks_kernel<3>, pts4, n, k, seed, centers, chosen, d2, nsb, st);
 }
 
 cudaError_t launch_kpp(const float4* pts4, int64_t n, int k, uint64_t seed, float4* centers, float* d2,

@@ -1,0 +1,50 @@
+"""k-means++ over sub-blocks in L2 (kpp_blocks_kernel): the drawn centres are the oracle's bit for
+bit, at one point per warp and less, ragged last sub-blocks, several sub-blocks per warp and per
+lane of the search, weights above 2^10 (128-bit totals), all-zero weights, and a shuffled cloud of
+the same size, which takes another kernel."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2307_00071_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def gira():
+    from paper_2307_00071_gb300 import gira as g
+    return g
+
+
+@pytest.fixture(scope="module")
+def frames():
+    return np.concatenate([synth.depth_frame(seed=s).points for s in (5, 6)])
+
+
+def seeds(gira, pts, k, seed):
+    """The seeding alone (no Lloyd update): 3-D centres, or a 4-D fit's one-hot means of it."""
+    return np.asarray(gira.gira_kmeans_init(pts, k, seed=seed, lloyd_iters=0, want_labels=False)[0])
+
+
+@pytest.mark.parametrize("n,k,scale,order", [(294_913, 40, 1.0, "sensor"), (500_001, 24, 1.0, "sensor"),
+                                             (540_000, 12, 60.0, "sensor"), (300_000, 12, 1.0, "shuffled"),
+                                             (300_001, 6, 0.0, "sensor")])
+def test_large_3d(gira, frames, n, k, scale, order):
+    pts = np.ascontiguousarray(frames[:n] * np.float32(scale))
+    if order == "shuffled":
+        pts = pts[np.random.default_rng(n).permutation(n)]
+    assert np.array_equal(seeds(gira, pts, k, 3), oracle.kmeanspp(pts, k, 3)[0].astype(np.float32))
+
+
+@pytest.mark.parametrize("n,k,scale", [(5, 5, 1.0), (33, 7, 1.0), (8_191, 30, 1.0), (70_001, 16, 1.0), (276_000, 16, 60.0),
+                                       (9_000, 4, 0.0)])
+def test_4d(gira, frames, n, k, scale):
+    """KInit with Lloyd in four dimensions, no EM iteration: the one-hot model of the oracle's labels."""
+    full = np.concatenate([frames[:n], synth.frame_intensity(frames[:n])[:, None]], axis=1) * np.float32(scale)
+    full = np.ascontiguousarray(full.astype(np.float32))
+    r = gira.gira_gmm_fit4(full, k, iters=0, seed=2, lloyd_iters=1, reg_covar=1e-3, final_loglik=False)
+    ref = oracle.kinit(full, k, 2, 1, 1e-3)
+    for key in ("weights", "means", "covs"):
+        got, want = np.asarray(r[key], np.float64), np.asarray(ref[key], np.float64)
+        assert np.all(np.abs(got - want) <= 2e-7 * np.abs(want).max() + 1e-12), key   # binary32 outputs
