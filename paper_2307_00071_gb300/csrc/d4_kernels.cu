@@ -583,45 +583,190 @@ __global__ void sample_kernel(int64_t m, int k, int d, const float* __restrict__
 }
 
 // ------------------------------------------------------------------ k-means in four dimensions
-// labels = argmin_b ||x - c_b||^2 (binary32 in the order of dist2_f32_4, ties to
-// the lowest b); binary64 sums of the coordinates and counts per label;
+// labels = argmin_b ||x - c_b||^2 (binary32 in the order of dist2_f32_4, every operation
+// rounded, ties to the lowest b); binary64 sums of the coordinates and counts per label;
 // changed[it] counts labels that moved (all of them for it == 0).
-constexpr int LL4_THREADS = 256;
+// A warp takes 128 consecutive points (Morton order in a fit), four per lane, two centres
+// per packed operation.  It scans only the centre pairs that can hold a nearest centre:
+// with U an upper bound of every point's nearest distance -- the largest distance to the
+// previous centres, or in the first assignment the smallest over the centres of the largest
+// distance to the box of the points -- a centre farther than U from the box (with slack for
+// the binary32 rounding of both) is farther than that from every point.  The pairs are
+// scanned in increasing order, so the argmin and its ties are those of the full scan.  Runs
+// of equal labels over the lanes are summed before the atomics, as in 3-D.
+// Bound by the scan's packed arithmetic and the binary64 scan of the sums; one point per
+// thread over every centre with five binary64 atomics per point took 104 us per launch on
+// the 276,348-point frame, K = 512.
+constexpr int LL4_THREADS = 256, LL4_PPT = 4;
+constexpr int LL4_LIST_MAX = 1024;   // centre pairs up to which the warps keep lists
+
+struct CPair4 {
+    float2 c[4];   // negated coordinates of centres 2p and 2p + 1
+};
+
+__host__ __device__ constexpr size_t lloyd4_smem(int npair) {
+    return sizeof(CPair4) * (size_t)npair + (npair <= LL4_LIST_MAX ? (LL4_THREADS / 32) * (size_t)npair * 2 : 0);
+}
 
 __global__ void __launch_bounds__(LL4_THREADS) lloyd4_assign_kernel(const float4* __restrict__ pts, int64_t n, int k,
                                                                     const float4* __restrict__ centers,
                                                                     int32_t* labels, double* sums,
-                                                                    unsigned long long* changed, int it,
+                                                                    unsigned long long* changed, int it, float2 nz,
                                                                     DeviceState* st) {
-    extern __shared__ float4 sc4[];
+    extern __shared__ CPair4 sc4[];
     if (st->error) return;
     if (it > 0 && changed[it - 1] == 0) return;
-    for (int b = threadIdx.x; b < k; b += blockDim.x) sc4[b] = centers[b];
+    const int npair = (k + 1) / 2;
+    for (int p = threadIdx.x; p < npair; p += blockDim.x) {
+        const float4 a = centers[2 * p];
+        const float4 b = (2 * p + 1 < k) ? centers[2 * p + 1] : make_float4(INFINITY, INFINITY, INFINITY, INFINITY);
+        sc4[p].c[0] = f2(-a.x, -b.x);
+        sc4[p].c[1] = f2(-a.y, -b.y);
+        sc4[p].c[2] = f2(-a.z, -b.z);
+        sc4[p].c[3] = f2(-a.w, -b.w);
+    }
     __syncthreads();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint16_t* slist = npair <= LL4_LIST_MAX ? reinterpret_cast<uint16_t*>(sc4 + npair) + warp * npair : nullptr;
     unsigned long long cnt = 0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const float4 x = pts[i];
-        int best = 0;
-        float bd = dist2_f32_4(x, sc4[0]);
-        for (int b = 1; b < k; ++b) {
-            const float d = dist2_f32_4(x, sc4[b]);
-            if (d < bd) {
-                bd = d;
-                best = b;
+    constexpr int64_t group = (int64_t)LL4_THREADS * LL4_PPT;
+    for (int64_t g0 = (int64_t)blockIdx.x * group; g0 < n; g0 += (int64_t)gridDim.x * group) {
+        const int64_t wb = g0 + (int64_t)warp * 32 * LL4_PPT;   // point r of this lane: wb + 32 r + lane
+        float2 X[LL4_PPT][4];
+        float bd[LL4_PPT];
+        int best[LL4_PPT];
+#pragma unroll
+        for (int r = 0; r < LL4_PPT; ++r) {
+            const float4 x = pts[min(wb + r * 32 + lane, n - 1)];
+            X[r][0] = dup(x.x);
+            X[r][1] = dup(x.y);
+            X[r][2] = dup(x.z);
+            X[r][3] = dup(x.w);
+            bd[r] = INFINITY;
+            best[r] = 0;
+        }
+        int nl = npair;
+        if (slist && wb < n) {
+            float lo[4], hi[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                lo[j] = fminf(fminf(X[0][j].x, X[1][j].x), fminf(X[2][j].x, X[3][j].x));
+                hi[j] = fmaxf(fmaxf(X[0][j].x, X[1][j].x), fmaxf(X[2][j].x, X[3][j].x));
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) {
+                    lo[j] = fminf(lo[j], __shfl_xor_sync(FULL, lo[j], o));
+                    hi[j] = fmaxf(hi[j], __shfl_xor_sync(FULL, hi[j], o));
+                }
+            }
+            float U;
+            if (it > 0) {
+                U = 0.f;
+#pragma unroll
+                for (int r = 0; r < LL4_PPT; ++r) {
+                    const int lp = labels[min(wb + r * 32 + lane, n - 1)];
+                    const CPair4 c = sc4[lp >> 1];
+                    float s = 0.f;
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float d = __fadd_rn(X[r][j].x, (lp & 1) ? c.c[j].y : c.c[j].x);
+                        s = __fadd_rn(s, __fmul_rn(d, d));
+                    }
+                    U = fmaxf(U, s);
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) U = fmaxf(U, __shfl_xor_sync(FULL, U, o));
+            } else {
+                U = INFINITY;
+                for (int b = lane; b < k; b += 32) {
+                    const CPair4 c = sc4[b >> 1];
+                    float s = 0.f;
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float nc = (b & 1) ? c.c[j].y : c.c[j].x;
+                        const float e = fmaxf(fabsf(lo[j] + nc), fabsf(hi[j] + nc));
+                        s = fmaf(e, e, s);
+                    }
+                    U = fminf(U, s);
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) U = fminf(U, __shfl_xor_sync(FULL, U, o));
+            }
+            nl = 0;
+            for (int j0 = 0; j0 < npair; j0 += 32) {
+                const int p = j0 + lane;
+                bool live = false;
+                if (p < npair) {
+                    const CPair4 c = sc4[p];
+#pragma unroll
+                    for (int m = 0; m < 2; ++m) {   // the centre is -nc
+                        float s = 0.f;
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            const float nc = m ? c.c[j].y : c.c[j].x;
+                            const float e = fmaxf(fmaxf(lo[j] + nc, -nc - hi[j]), 0.f);
+                            s = fmaf(e, e, s);
+                        }
+                        live = live || !(s * (1.f - 1e-5f) > U);
+                    }
+                }
+                const uint32_t mk = __ballot_sync(FULL, live);
+                if (live) slist[nl + __popc(mk & ((1u << lane) - 1u))] = (uint16_t)p;
+                nl += __popc(mk);
+            }
+            __syncwarp();
+        }
+        for (int q = 0; q < nl; ++q) {
+            const int p = nl == npair ? q : slist[q];
+            const CPair4 c = sc4[p];
+#pragma unroll
+            for (int r = 0; r < LL4_PPT; ++r) {
+                float2 s = f2(0.f, 0.f);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float2 d = add2(X[r][j], c.c[j]);
+                    const float2 dd = mul2_alone(d, d, nz);
+                    s = j == 0 ? dd : add2(s, dd);
+                }
+                if (s.x < bd[r]) { bd[r] = s.x; best[r] = 2 * p; }
+                if (s.y < bd[r]) { bd[r] = s.y; best[r] = 2 * p + 1; }
             }
         }
-        if (it == 0 || labels[i] != best) ++cnt;
-        labels[i] = best;
-        double* S = sums + 5 * (size_t)best;
-        atomicAdd(&S[0], (double)x.x);
-        atomicAdd(&S[1], (double)x.y);
-        atomicAdd(&S[2], (double)x.z);
-        atomicAdd(&S[3], (double)x.w);
-        atomicAdd(&S[4], 1.0);
+#pragma unroll
+        for (int r = 0; r < LL4_PPT; ++r) {
+            const int64_t i = wb + r * 32 + lane;
+            int key = -1;
+            double v[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+            if (i < n) {
+                if (it == 0 || labels[i] != best[r]) ++cnt;
+                labels[i] = best[r];
+                key = best[r];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) v[j] = (double)X[r][j].x;
+                v[4] = 1.0;
+            }
+            // segmented inclusive scan over runs of equal keys (fixed order)
+            const int prev = __shfl_up_sync(FULL, key, 1);
+            const bool head = (lane == 0) || (prev != key);
+            const unsigned heads = __ballot_sync(FULL, head);
+            const int start = 31 - __clz(heads & (0xffffffffu >> (31 - lane)));
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                if (__all_sync(FULL, lane - o < start)) break;   // no run is longer
+#pragma unroll
+                for (int q = 0; q < 5; ++q) {
+                    const double u = __shfl_up_sync(FULL, v[q], o);
+                    if (lane - o >= start) v[q] += u;
+                }
+            }
+            const bool tail = (lane == 31) || ((heads >> (lane + 1)) & 1u);
+            if (tail && key >= 0)
+#pragma unroll
+                for (int q = 0; q < 5; ++q) atomicAdd(&sums[5 * (size_t)key + q], v[q]);
+        }
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(FULL, cnt, o);
-    if ((threadIdx.x & 31) == 0 && cnt) atomicAdd(&changed[it], cnt);
+    if (lane == 0 && cnt) atomicAdd(&changed[it], cnt);
 }
 
 __global__ void lloyd4_update_kernel(int k, double* sums, float4* centers, const unsigned long long* changed, int it,
@@ -700,18 +845,19 @@ static int num_sms_now() {
 
 cudaError_t launch_lloyd4(const float4* pts4, int64_t n, int k, int lloyd_iters, float4* centers, int32_t* labels,
                           double* sums, unsigned long long* changed, DeviceState* st, cudaStream_t s) {
-    const size_t smem = sizeof(float4) * (size_t)k;
-    const int64_t want = (n + LL4_THREADS - 1) / LL4_THREADS;
+    const float2 nz = make_float2(-0.f, -0.f);
+    const size_t smem = lloyd4_smem((k + 1) / 2);
+    const int64_t want = (n + (int64_t)LL4_THREADS * LL4_PPT - 1) / ((int64_t)LL4_THREADS * LL4_PPT);
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)num_sms_now() * 8));
     if (smem > 48 * 1024) {
         const cudaError_t e =
             cudaFuncSetAttribute(lloyd4_assign_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    lloyd4_assign_kernel<<<grid, LL4_THREADS, smem, s>>>(pts4, n, k, centers, labels, sums, changed, 0, st);
+    lloyd4_assign_kernel<<<grid, LL4_THREADS, smem, s>>>(pts4, n, k, centers, labels, sums, changed, 0, nz, st);
     for (int it = 1; it <= lloyd_iters; ++it) {
         lloyd4_update_kernel<<<(k + 127) / 128, 128, 0, s>>>(k, sums, centers, changed, it, st);
-        lloyd4_assign_kernel<<<grid, LL4_THREADS, smem, s>>>(pts4, n, k, centers, labels, sums, changed, it, st);
+        lloyd4_assign_kernel<<<grid, LL4_THREADS, smem, s>>>(pts4, n, k, centers, labels, sums, changed, it, nz, st);
     }
     return cudaGetLastError();
 }

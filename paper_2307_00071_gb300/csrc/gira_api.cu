@@ -1734,10 +1734,10 @@ gira_status gira_gmm_fit4(const float* points, int64_t n, int k, const gira_fit_
         TRY(seed_centres(prof, c, b.p4, n, 4, k, o.seed, b.c4, b.ch, b.d2, b.bs, b.ksync, b.ksums, kgrid, b.st));
         GIRA_CUDA(cudaMemsetAsync(b.sums, 0, sizeof(double) * 5 * k, c.s));
         GIRA_CUDA(cudaMemsetAsync(b.chg, 0, sizeof(unsigned long long) * (o.lloyd_iters + 1), c.s));
-        COUNTED(prof, 1 + 2 * o.lloyd_iters, launch_lloyd4(b.p4, n, k, o.lloyd_iters, b.c4, b.lab, b.sums, b.chg,
+        COUNTED(prof, 1 + 2 * o.lloyd_iters, launch_lloyd4(sorted ? b.p4s : b.p4, n, k, o.lloyd_iters, b.c4, b.lab, b.sums, b.chg,
                                                           b.st, c.s));
         GIRA_CUDA(cudaMemsetAsync(b.stats64, 0, sizeof(double) * NSTAT4 * k, c.s));
-        COUNTED(prof, 1, launch_label_stats4(b.p4, n, k, b.lab, b.c4, b.stats64, b.st, c.s));
+        COUNTED(prof, 1, launch_label_stats4(sorted ? b.p4s : b.p4, n, k, b.lab, b.c4, b.stats64, b.st, c.s));
         COUNTED(prof, 1, launch_reduce_finalize4(nullptr, nullptr, 0, nullptr, 0, b.stats64, b.c4, k, n, o.reg_covar,
                                                  o.tol, b.model64, b.params, b.trace, nullptr, b.st, 0, false, c.s));
     } else {

@@ -74,6 +74,12 @@ __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
 
+// a * b rounded on its own: ptxas contracts a packed multiplication whose result is added
+// (__fmul2_rn, and mul.rn.f32x2 too: a probe against the scalar _rn form differed in 21 % of
+// random squared distances) and folds an fma with a literal -0; with a -0 it cannot see
+// (nz = (-0, -0), a kernel argument) the product stays one rounded operation.
+__device__ __forceinline__ float2 mul2_alone(float2 a, float2 b, float2 nz) { return fma2(a, b, nz); }
+
 __device__ __forceinline__ float ex2_approx(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));

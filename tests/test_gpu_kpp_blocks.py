@@ -48,3 +48,17 @@ def test_4d(gira, frames, n, k, scale):
     for key in ("weights", "means", "covs"):
         got, want = np.asarray(r[key], np.float64), np.asarray(ref[key], np.float64)
         assert np.all(np.abs(got - want) <= 2e-7 * np.abs(want).max() + 1e-12), key   # binary32 outputs
+
+
+@pytest.mark.parametrize("n,k,lloyd", [(1, 1, 2), (130, 100, 3), (60_000, 700, 4), (20_000, 2_049, 2)])
+def test_lloyd_4d(gira, frames, n, k, lloyd):
+    """Pruned and full (above 2,048 centres) assignments: every label as the oracle's, so the one-hot weights
+    (counts / n, exact to binary32) agree, and the model with them."""
+    full = np.concatenate([frames[:n], synth.frame_intensity(frames[:n])[:, None]], axis=1).astype(np.float32)
+    full = np.ascontiguousarray(full)
+    r = gira.gira_gmm_fit4(full, k, iters=0, seed=4, lloyd_iters=lloyd, reg_covar=1e-3, final_loglik=False)
+    ref = oracle.kinit(full, k, 4, lloyd, 1e-3)
+    assert np.array_equal(np.rint(np.asarray(r["weights"], np.float64) * n), np.bincount(ref["labels"], minlength=k))
+    for key in ("means", "covs"):
+        got, want = np.asarray(r[key], np.float64), np.asarray(ref[key], np.float64)
+        assert np.all(np.abs(got - want) <= 2e-7 * np.abs(want).max() + 1e-12), key
