@@ -88,8 +88,8 @@ __device__ bool build_component4(int b, double w, const double mu[4], const doub
 }
 
 // The M-step of one pair of components per block.  Sums: warp w adds, value by lane, the
-// pair's live rows among the w-th quarter of the slices (compensated binary32, Knuth's
-// TwoSum), warp 0 joins the quarters in order.  Update: warp 0, lanes 16 h + 4 i + j for
+// pair's live rows among the w-th eighth of the slices (compensated binary32, Knuth's
+// TwoSum), warp 0 joins them in order.  Update: warp 0, lanes 16 h + 4 i + j for
 // entry (i, j) of component h's 4 x 4 matrices, every stage in parallel lanes through
 // shared memory: GB300 issues one binary64 warp instruction per 64 cycles per warp whatever
 // the number of active lanes, so a stage costs what one entry costs (~170 instructions in
@@ -116,7 +116,7 @@ struct Fin4Args {
     DeviceState* st;
     int iter, em;
 };
-constexpr int FIN4_WARPS = 4;
+constexpr int FIN4_WARPS = 8;
 __global__ void __launch_bounds__(32 * FIN4_WARPS) reduce_finalize4_kernel(const Fin4Args f) {
     __shared__ float s_hi[FIN4_WARPS][2][32];
     __shared__ double s_stat[2][NSTAT4], s_P[2][10], s_r[2][5], s_M[2][16], s_C[2][16], s_A[2][16], s_mu[2][4];

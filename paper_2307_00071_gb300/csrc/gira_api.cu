@@ -334,7 +334,8 @@ struct ReachBufs {
     float4* ctr = nullptr;
     float2 *aux = nullptr, *pref = nullptr;
     float *gref = nullptr, *partials = nullptr;
-    uint32_t *masks = nullptr, *live2 = nullptr;
+    uint32_t *masks = nullptr, *live2 = nullptr;   // live2: words * slices, then the two unit counters
+    uint2* units = nullptr;
     double* llp = nullptr;
     int grid = 0, h = 0, words = 0, slices = 0;
     int64_t rows = 0;
@@ -354,7 +355,8 @@ void carve_reach(Carver& cv, int64_t n, int k, int nstat, bool stats, ReachBufs*
     if (!stats) return;
     b->pref = cv.take<float2>(n);
     b->masks = cv.take<uint32_t>((size_t)b->words * b->rows);
-    b->live2 = cv.take<uint32_t>((size_t)b->words * b->slices);
+    b->live2 = cv.take<uint32_t>((size_t)b->words * b->slices + 2);
+    b->units = cv.take<uint2>((size_t)b->slices * ((k + 1) / 2));
     b->partials = cv.take<float>((size_t)b->slices * ((k + 1) / 2) * 2 * nstat);
 }
 
@@ -366,14 +368,24 @@ ReachLaunch reach_launch(const ReachBufs& b, const float4* p8, int64_t n, int k,
     return a;
 }
 
+void reach_with_stats(const ReachBufs& b, ReachLaunch* a) {
+    a->pref = b.pref;
+    a->masks = b.masks;
+    a->live2 = b.live2;
+    a->stat_units = b.units;
+    a->unit_count = reinterpret_cast<int*>(b.live2 + (size_t)b.words * b.slices);
+}
+cudaError_t reach_zero_live(const ReachBufs& b, cudaStream_t s) {
+    return cudaMemsetAsync(b.live2, 0, sizeof(uint32_t) * ((size_t)b.words * b.slices + 2), s);
+}
+
 // One E-step with statistics: b.partials rows and b.live2 masks for the finalize.
 cudaError_t reach_estep_stats(int d, const ReachBufs& b, ReachLaunch a, long long* launches, cudaStream_t s) {
-    a.pref = b.pref;
-    a.masks = b.masks;
+    reach_with_stats(b, &a);
     cudaError_t e = launch_reach_prepare(d, a.params, a.k, a.st, a.iter, b.ctr, b.aux, b.gref, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(b.live2, 0, sizeof(uint32_t) * b.words * b.slices, s);
+    if (e == cudaSuccess) e = reach_zero_live(b, s);
     if (e == cudaSuccess) e = launch_estep_reach(d, a, 1, b.grid, b.h, a.k, s);
-    if (e == cudaSuccess) e = launch_reach_stats(d, a, 1, a.k, a.n, b.partials, b.live2, s);
+    if (e == cudaSuccess) e = launch_reach_stats(d, a, b.partials, s);
     *launches += 3;
     return e;
 }
@@ -960,15 +972,14 @@ gira_status gira_gmm_loglik_grad(const float* points, int64_t n, int k, const fl
         a.rot = pose_d;
         a.pose_partials = b.ppart;
         if (gpar) {
-            a.pref = rb.pref;
-            a.masks = rb.masks;
-            GIRA_CUDA(cudaMemsetAsync(rb.live2, 0, sizeof(uint32_t) * rb.words * rb.slices, c.s));
+            reach_with_stats(rb, &a);
+            GIRA_CUDA(reach_zero_live(rb, c.s));
         }
         cudaEvent_t e0 = prof.mark_launch();
         COUNTED(prof, 1, launch_estep_reach(3, a, 2, rb.grid, rb.h, k, c.s));
         cudaEvent_t e1 = prof.mark_launch();
         if (prof.per_launch) prof.timed(e0, e1);
-        if (gpar) COUNTED(prof, 1, launch_reach_stats(3, a, 1, k, n, rb.partials, rb.live2, c.s));
+        if (gpar) COUNTED(prof, 1, launch_reach_stats(3, a, rb.partials, c.s));
         const ReachGradArgs f{gpar ? rb.partials : nullptr, rb.live2, rb.slices, rb.llp, b.ppart, rb.grid, pose_d,
                               ch_d, b.params, b.model64, b.perm, k, n, gl_d, gm_d, gc_d, po_d, tw_d, b.st};
         COUNTED(prof, 1, launch_reach_grad_finalize(f, nullptr, 1, c.s));
@@ -1408,7 +1419,7 @@ gira_status gira_gmm_loglik_grad_batched(const float* points, const int64_t* off
     std::vector<BatchUnit> units;
     const int rh = reach_h(total_n), rpts = reach_points(rh);
     int total_k = 0, kmax = 0;
-    int64_t par_floats = 0, ll_slots = 0, part_floats = 0, mask_words = 0, live_words = 0, nmax = 0;
+    int64_t par_floats = 0, ll_slots = 0, part_floats = 0, mask_words = 0, live_words = 0;
     for (int i = 0; i < batch; ++i) {
         BatchInst& I = hi[i];
         int sl;
@@ -1418,7 +1429,6 @@ gira_status gira_gmm_loglik_grad_batched(const float* points, const int64_t* off
         I.comp_off = total_k;
         total_k += ks[i];
         kmax = std::max(kmax, ks[i]);
-        nmax = std::max(nmax, I.n);
         I.par_off = par_floats;
         par_floats += (int64_t)params_pairs_padded(ks[i]) * PAIR_FLOATS;
         I.ctas = (int)((I.n + rpts - 1) / rpts);
@@ -1447,6 +1457,7 @@ gira_status gira_gmm_loglik_grad_batched(const float* points, const int64_t* off
         BatchInst* insts;
         BatchUnit* units;
         int2* ounits;
+        uint2* sunits;
         int *perm, *order;
         int64_t* offs;
         void* osc;
@@ -1471,7 +1482,8 @@ gira_status gira_gmm_loglik_grad_batched(const float* points, const int64_t* off
         b.aux = cv.take<float2>(total_k);
         b.pref = cv.take<float2>(gpar ? (size_t)total_n : 0);
         b.masks = cv.take<uint32_t>(gpar ? (size_t)mask_words : 0);
-        b.live2 = cv.take<uint32_t>(gpar ? (size_t)live_words : 0);
+        b.live2 = cv.take<uint32_t>(gpar ? (size_t)live_words + 2 : 0);   // then the two unit counters
+        b.sunits = cv.take<uint2>(gpar ? (size_t)part_floats / (2 * NSTAT) : 0);
         b.partials = cv.take<float>(gpar ? (size_t)part_floats : 0);
         b.llp = cv.take<double>((size_t)ll_slots);
         b.ppart = cv.take<double>(12 * (size_t)ll_slots);
@@ -1560,10 +1572,13 @@ gira_status gira_gmm_loglik_grad_batched(const float* points, const int64_t* off
         if (gpar) {
             a.pref = b.pref;
             a.masks = b.masks;
-            if (e == cudaSuccess) e = cudaMemsetAsync(b.live2, 0, sizeof(uint32_t) * live_words, cs);
+            a.live2 = b.live2;
+            a.stat_units = b.sunits;
+            a.unit_count = reinterpret_cast<int*>(b.live2 + live_words);
+            if (e == cudaSuccess) e = cudaMemsetAsync(b.live2, 0, sizeof(uint32_t) * (live_words + 2), cs);
         }
         if (e == cudaSuccess) e = launch_estep_reach(3, a, 2, (int)units.size(), rh, kmax, cs);
-        if (e == cudaSuccess && gpar) e = launch_reach_stats(3, a, batch, kmax, nmax, b.partials, b.live2, cs);
+        if (e == cudaSuccess && gpar) e = launch_reach_stats(3, a, b.partials, cs);
         const ReachGradArgs f{gpar ? b.partials : nullptr, b.live2, 0, b.llp, b.ppart, 0, b.poses, b.ch, b.params,
                               b.model64, b.perm, kmax, 0, gpar ? b.gl : nullptr, gpar ? b.gm : nullptr,
                               gpar ? b.gc : nullptr, b.gpose, b.gtwist, b.st};

@@ -350,13 +350,16 @@ struct BatchUnit {
     int inst, cta;
 };
 
-// Slices of the statistics launch over n points: sl words of 32 blocks of 128 points
-// each.  One word (4,096 points) up to 256 slices -- a slice is one warp's serial work
-// -- then longer slices, which bounds the partial rows.
-__host__ __device__ inline int reach_slices(int64_t n, int* sl) {
-    const int64_t words = (n + 4095) / 4096;
-    *sl = (int)((words + 255) / 256);
-    return (int)((words + *sl - 1) / *sl);
+// Slices of the statistics over n points, of *sr blocks of 128 points each: the unit of
+// work is one (slice, pair).  8 blocks (in Morton order a pair's live blocks lie in a few
+// slices, and longer ones leave few, long units), more above 512 slices, which bounds the
+// partial rows.
+__host__ __device__ inline int reach_slices(int64_t n, int* sr) {
+    const int64_t rows = (n + 127) / 128;
+    int r = 8;
+    while (rows > 512 * (int64_t)r) r *= 2;
+    *sr = r;
+    return (int)((rows + r - 1) / r);
 }
 
 // The E-step over reach lists (reach_kernels.cu).
@@ -376,6 +379,12 @@ struct ReachLaunch {
     float2* pref = nullptr;  // [n] (shift, 1 / total): with masks
     uint32_t* masks = nullptr;   // [reach_mask_words(k)][rows] live pairs per block of 128 points
     int64_t rows = 0;
+    // with masks: the same per slice, [reach_mask_words(k)][slices], and the (slice, pair)s
+    // with work: units[0 .. count), count in unit_count[0] ([1]: the statistics' cursor);
+    // live2 and unit_count are zeroed before the launch
+    uint32_t* live2 = nullptr;
+    uint2* stat_units = nullptr;   // (instance, slice << 16 | pair)
+    int* unit_count = nullptr;
     // gradient (mode 2)
     float* grad_pts = nullptr;        // [n][3], at order[i] (or i) for the i-th point, or nullptr
     const int* order = nullptr;
@@ -395,11 +404,9 @@ cudaError_t launch_reach_prepare(int d, const float* params, int k, const Device
                                  float* gref, cudaStream_t s);
 // d: 3 or 4 dimensions.  mode 0 log-likelihood, 1 with masks and pref, 2 gradient (3-D); h: reach_h of the launch; kmax: the largest k.
 cudaError_t launch_estep_reach(int d, const ReachLaunch& a, int mode, int grid, int h, int kmax, cudaStream_t s);
-// partials [slices][pairs][2 NSTAT (4-D: NSTAT4)] and live2 [words][slices] (zeroed by the caller):
-// launch_reduce_finalize takes them as rows and masks.
-// Batched (a.insts): every instance, kmax and nmax its largest k and n.
-cudaError_t launch_reach_stats(int d, const ReachLaunch& a, int batch, int kmax, int64_t nmax, float* partials,
-                               uint32_t* live2, cudaStream_t s);
+// partials [slices][pairs][2 NSTAT (4-D: NSTAT4)], written where a.live2 has the bit:
+// launch_reduce_finalize takes the two as rows and masks.
+cudaError_t launch_reach_stats(int d, const ReachLaunch& a, float* partials, cudaStream_t s);
 
 struct EStepLaunch {
     const float4* pts8;      // 2 float4 per point: (x,x,y,y) (z,z,0,0)

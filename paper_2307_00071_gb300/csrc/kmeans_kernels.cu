@@ -1122,7 +1122,7 @@ __global__ void __launch_bounds__(KC_THREADS, 1) kpp_blocks_kernel(const float4*
     cluster.sync();   // no CTA leaves while a peer may still address its shared memory
 }
 
-// Whether the points come in an order that keeps neighbours together: over up to 1,024
+// Whether the points come in an order that keeps neighbours together: over up to 256
 // sub-blocks of 32 consecutive points, spread evenly, the mean of the largest box extent
 // against the extent of all of them (st->coherent = 1 when below a quarter; a shuffled
 // cloud has about 0.9, a depth image's rows 0.02 .. 0.1).
@@ -1131,7 +1131,7 @@ __global__ void __launch_bounds__(1024) kpp_coherence_kernel(const float4* __res
     __shared__ float s_sum[32], s_lo[32][4], s_hi[32][4];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t subs = (n + 31) / 32;
-    const int take = (int)min(subs, (int64_t)1024);
+    const int take = (int)min(subs, (int64_t)256);
     float sum = 0.f, LO[4], HI[4];
     for (int c = 0; c < 4; ++c) {
         LO[c] = INFINITY;

@@ -19,7 +19,7 @@
 //      broadcasts: nothing is staged, so shared memory (a few KB of lists) does not
 //      bound the occupancy and K does not bound the kernel.  Writes per-point
 //      (shift, 1 / total), the log-likelihood, and per block the mask of live pairs;
-//  reach_stats_kernel    one warp per (pair, slice of blocks): the statistics of both
+//  reach_stats_kernel    one warp at a time per (pair, slice of blocks): the statistics of both
 //      components over the live blocks of the slice stay in registers and are reduced
 //      over the lanes once per slice.  A row-wise second phase would reduce and store 20
 //      values per (block, pair) and need a partial row per block (10 GB at 4M points,
@@ -28,9 +28,9 @@
 // per point from the live pairs, and the pose sums.
 //
 // Measured on GB300 (4M points of 16 posed frames, K = 8192): E-step 0.70 ms, statistics
-// 1.33 ms per iteration; the dense two-pass kernels over chunks of 512 components that
+// 0.50 ms per iteration; the dense two-pass kernels over chunks of 512 components that
 // this replaced took 2 x 15.5 ms.  A call of two iterations with the final
-// log-likelihood: 79.2 -> 6.1 ms.
+// log-likelihood: 79.2 -> 3.9 ms.
 #include <float.h>
 #include <math.h>
 
@@ -248,11 +248,14 @@ __device__ __forceinline__ void block_sync(int blk) {
     }
 }
 
+// Registers: 3-D without the gradient fits 96 a thread (5 CTAs per SM: the 4M-point map's
+// call 3.90 ms, 4.04 with 4); the others would spill (4-D 5.04 against 4.95 ms per frame fit,
+// 16 registrations 763 against 698 us).
 // MODE 0: log-likelihood; 1: also (shift, 1 / total) and the masks for reach_stats_kernel;
 // 2: the gradient (the masks only when a.masks).  H warps share a block's pairs (pp % H):
 // 2 for large inputs, 4 where 256-point CTAs would leave SMs idle.
 template <int D, int H, int MODE>
-__global__ void __launch_bounds__(32 * RB_W, 4) estep_reach_kernel(const ReachLaunch a_in) {
+__global__ void __launch_bounds__(32 * RB_W, D == 3 && MODE != 2 ? 5 : 4) estep_reach_kernel(const ReachLaunch a_in) {
     extern __shared__ __align__(16) unsigned char dsm[];
     constexpr int B = RB_W / H;   // blocks per CTA
     static_assert(B * H == RB_W && B <= 2, "one named barrier per block");
@@ -268,7 +271,7 @@ __global__ void __launch_bounds__(32 * RB_W, 4) estep_reach_kernel(const ReachLa
     // added to the launch's own pointers (loads through a pointer advanced inside a copy
     // of the launch struct read the unadvanced one under nvcc 13.0 for sm_103a).
     int cta = blockIdx.x, inst = 0, k = a_in.k;
-    int64_t pt0 = 0, n = a_in.n, rows = a_in.rows, par_off = 0, comp_off = 0, mask_off = 0, ll_off = 0;
+    int64_t pt0 = 0, n = a_in.n, rows = a_in.rows, par_off = 0, comp_off = 0, mask_off = 0, ll_off = 0, live_off = 0;
     DeviceState* st = a_in.st;
     if (a_in.units) {
         const BatchUnit u = a_in.units[blockIdx.x];
@@ -283,6 +286,7 @@ __global__ void __launch_bounds__(32 * RB_W, 4) estep_reach_kernel(const ReachLa
         comp_off = I.comp_off;
         mask_off = I.mask_off;
         ll_off = I.ll_off;
+        live_off = I.live_off;
         st = a_in.states + u.inst;
     }
     const float* const params = a_in.params + par_off;
@@ -618,13 +622,32 @@ __global__ void __launch_bounds__(32 * RB_W, 4) estep_reach_kernel(const ReachLa
     if (MODE != 0) {
         __syncwarp();
         block_sync<H>(blk);   // the block's masks are final
-        if (a_in.masks && half == 0 && row < rows)
-            for (int wd = lane; wd < nwords; wd += 32) {
+        if (a_in.masks && half == 0 && row < rows) {
+            // the block's mask; the slice's, whose bits first set here become units of work
+            int sr;
+            const int slices = reach_slices(n, &sr), slice = (int)(row / sr);
+            for (int w0 = 0; w0 < nwords; w0 += 32) {
+                const int wd = w0 + lane;
                 uint32_t m = 0u;
+                if (wd < nwords) {
 #pragma unroll
-                for (int h = 0; h < H; ++h) m |= smask_all[(blk * H + h) * nwords + wd];
-                a_in.masks[mask_off + wd * rows + row] = m;
+                    for (int h2 = 0; h2 < H; ++h2) m |= smask_all[(blk * H + h2) * nwords + wd];
+                    a_in.masks[mask_off + wd * rows + row] = m;
+                }
+                uint32_t fresh = m ? m & ~atomicOr(a_in.live2 + live_off + (int64_t)wd * slices + slice, m) : 0u;
+                int incl = __popc(fresh);
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int v = __shfl_up_sync(FULL, incl, o);
+                    if (lane >= o) incl += v;
+                }
+                int at = 0;
+                if (lane == 31 && incl) at = atomicAdd(a_in.unit_count, incl);
+                at = __shfl_sync(FULL, at, 31) + incl - __popc(fresh);
+                for (; fresh; fresh &= fresh - 1u, ++at)
+                    a_in.stat_units[at] = make_uint2((unsigned)inst, ((unsigned)slice << 16) | (unsigned)(wd * 32 + __ffs(fresh) - 1));
             }
+        }
     }
     if constexpr (MODE == 2) {
         // ---- sum_b gamma P'^T P' (x' - mu) over this warp's live pairs (components packed)
@@ -725,104 +748,102 @@ __global__ void __launch_bounds__(32 * RB_W, 4) estep_reach_kernel(const ReachLa
 }
 
 // ------------------------------------------------------------------ the statistics
-// One warp per (pair, slice of `sl` words of 32 blocks): S0 = sum r, S1 = sum r y, S2 =
-// sum r y y^T with y = P'(x - mu_old) of both components over the points of the live
-// blocks, e formed by the E-step's operations (the same bits).  Row (slice) of the
-// partials [slices][pairs][2 NS], written where it is not empty; live2 [words][slices]
-// (zeroed before the launch) gets the pair's bit there.  The 8 warps of a CTA take
-// neighbouring pairs (in Morton order), which reach much the same blocks: the points
-// come out of L1.
-constexpr int ST_W = 8;
+// The E-step listed the (slice, pair)s with work; each warp takes the next one (the order in
+// which they were listed and taken decides nothing but who does them): S0 = sum r, S1 = sum
+// r y, S2 = sum r y y^T with y = P'(x - mu_old) of both components over the points of the
+// slice's live blocks, e formed by the E-step's operations (the same bits), reduced over the
+// lanes once and written to row `slice` of the partials [slices][pairs][2 NS].
+// Bound by the latency of a block's loads and the length of a warp's chain of blocks.
+// Measured: one warp per (pair, slice of 32 or 128 blocks), empty ones among them, 51 us per
+// launch on the 276,348-point frame in 4-D at K = 512 and 1.33 ms on the 4M-point map at
+// K = 8192, with 9 of 16 resident warps active (CTAs of 8 such warps); 38 us and 0.50 ms now.
+// Copying a unit's next block to shared memory meanwhile (cp.async) changed nothing.
+constexpr int ST_W = 4;   // warps per CTA
 template <int D>
-__global__ void __launch_bounds__(32 * ST_W) reach_stats_kernel(const ReachLaunch a_in, int sl, float* partials,
-                                                                uint32_t* live2) {
+__global__ void __launch_bounds__(32 * ST_W) reach_stats_kernel(const ReachLaunch a_in, float* partials) {
     constexpr int NS = Lay<D>::NS;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    int slices = gridDim.y, k = a_in.k;
-    int64_t pt0 = 0, n = a_in.n, rows = a_in.rows, par_off = 0, mask_off = 0, part_off = 0, live_off = 0;
-    const DeviceState* st = a_in.st;
-    const int slice = blockIdx.y;
-    if (a_in.insts) {   // blockIdx.z: instance (offsets, as in estep_reach_kernel)
-        const BatchInst I = a_in.insts[blockIdx.z];
-        slices = reach_slices(I.n, &sl);
-        if (slice >= slices) return;
-        pt0 = I.pt_off;
-        n = I.n;
-        k = I.k;
-        rows = (I.n + RB_PTS - 1) / RB_PTS;
-        par_off = I.par_off;
-        mask_off = I.mask_off;
-        part_off = I.part_off;
-        live_off = I.live_off;
-        st = a_in.states + blockIdx.z;
-    }
+    const int lane = threadIdx.x & 31;
     pdl_wait();
-    if (a_in.iter > st->stop_after || st->error) return;
-    const int pp = blockIdx.x * ST_W + warp;
-    const int npairs = (k + 1) >> 1;
-    if (pp >= npairs) return;
-    const float* const params = a_in.params + par_off;
-    const uint32_t* const mw = a_in.masks + mask_off + (size_t)(pp >> 5) * rows;
-    const int64_t r0 = (int64_t)slice * sl * 32;
-    const float cmax = cmax_of(a_in.gref, st);
-    Pair<D> P;
-    bool loaded = false;
-    float2 S[NS];
-#pragma unroll
-    for (int s = 0; s < NS; ++s) S[s] = f2(0.f, 0.f);
-    for (int w = 0; w < sl; ++w) {
-        const int64_t r = r0 + 32 * w + lane;
-        uint32_t m = __ballot_sync(FULL, r < rows && ((mw[r] >> (pp & 31)) & 1u));
-        if (m && !loaded) {
-            load_pair<D>(params, pp, cmax, P);
-            loaded = true;
+    const int count = a_in.unit_count[0];
+    auto take = [&]() {
+        int u = 0;
+        if (lane == 0) u = atomicAdd(a_in.unit_count + 1, 1);
+        return __shfl_sync(FULL, u, 0);
+    };
+    for (int u = take(); u < count; u = take()) {
+        const uint2 unit = a_in.stat_units[u];
+        const int inst = (int)unit.x, slice = (int)(unit.y >> 16), pp = (int)(unit.y & 0xffffu);
+        int k = a_in.k;
+        int64_t pt0 = 0, n = a_in.n, rows = a_in.rows, par_off = 0, mask_off = 0, part_off = 0;
+        const DeviceState* st = a_in.st;
+        if (a_in.insts) {   // offsets into the launch's arrays, as in estep_reach_kernel
+            const BatchInst I = a_in.insts[inst];
+            pt0 = I.pt_off;
+            n = I.n;
+            k = I.k;
+            rows = (I.n + RB_PTS - 1) / RB_PTS;
+            par_off = I.par_off;
+            mask_off = I.mask_off;
+            part_off = I.part_off;
+            st = a_in.states + inst;
         }
-        for (; m; m &= m - 1u) {
-            const int64_t b0 = (r0 + 32 * w + __ffs(m) - 1) * RB_PTS + lane;
+        const int npairs = (k + 1) >> 1;
+        int sr;
+        reach_slices(n, &sr);
+        const int64_t r0 = (int64_t)slice * sr, r1 = min(rows, r0 + sr);
+        const uint32_t* const mw = a_in.masks + mask_off + (int64_t)(pp >> 5) * rows;
+        Pair<D> P;
+        load_pair<D>(a_in.params + par_off, pp, cmax_of(a_in.gref, st), P);
+        float2 S[NS];
 #pragma unroll
-            for (int p = 0; p < RB_P; ++p) {
-                const int64_t i = b0 + 32 * p;
-                const bool ok = i < n;
-                const int64_t at = pt0 + (ok ? i : n - 1);   // an absent point: the last one with weight 0
-                float2 X[D], y[D];
-                load_point<D>(a_in.pts8, at, X);
-                const float2 pr = a_in.pref[at];
-                const float2 nq = nlogit<D>(P, X, y);
-                const float2 e = f2(ex2_approx(pr.x - nq.x), ex2_approx(pr.x - nq.y));
-                const float2 g = mul2(e, dup(ok ? pr.y : 0.f));
-                S[0] = add2(S[0], g);
+        for (int s = 0; s < NS; ++s) S[s] = f2(0.f, 0.f);
+        for (int64_t rb = r0; rb < r1; rb += 32) {
+            uint32_t m = __ballot_sync(FULL, rb + lane < r1 && ((mw[rb + lane] >> (pp & 31)) & 1u));
+            for (; m; m &= m - 1u) {
+                const int64_t b0 = (rb + __ffs(m) - 1) * RB_PTS + lane;
 #pragma unroll
-                for (int i2 = 0, q = 1 + D; i2 < D; ++i2) {
-                    const float2 gy = mul2(g, y[i2]);
-                    S[1 + i2] = add2(S[1 + i2], gy);
+                for (int p = 0; p < RB_P; ++p) {
+                    const int64_t i = b0 + 32 * p;
+                    const bool ok = i < n;
+                    const int64_t at = pt0 + (ok ? i : n - 1);   // an absent point: the last one with weight 0
+                    float2 X[D], y[D];
+                    load_point<D>(a_in.pts8, at, X);
+                    const float2 pr = a_in.pref[at];
+                    const float2 nq = nlogit<D>(P, X, y);
+                    const float2 e = f2(ex2_approx(pr.x - nq.x), ex2_approx(pr.x - nq.y));
+                    const float2 g = mul2(e, dup(ok ? pr.y : 0.f));
+                    S[0] = add2(S[0], g);
 #pragma unroll
-                    for (int j = i2; j < D; ++j, ++q) S[q] = fma2(gy, y[j], S[q]);
+                    for (int i2 = 0, q = 1 + D; i2 < D; ++i2) {
+                        const float2 gy = mul2(g, y[i2]);
+                        S[1 + i2] = add2(S[1 + i2], gy);
+#pragma unroll
+                        for (int j = i2; j < D; ++j, ++q) S[q] = fma2(gy, y[j], S[q]);
+                    }
                 }
             }
         }
+        // lanes 0-15 end with the first component's sums, 16-31 with the second's
+        float v[NS];
+        const bool hi16 = lane & 16;
+#pragma unroll
+        for (int s = 0; s < NS; ++s) {
+            const float keep = hi16 ? S[s].y : S[s].x, send = hi16 ? S[s].x : S[s].y;
+            v[s] = keep + __shfl_xor_sync(FULL, send, 16);
+        }
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1)
+#pragma unroll
+            for (int s = 0; s < NS; ++s) v[s] += __shfl_xor_sync(FULL, v[s], o);
+        float mine = 0.f;
+#pragma unroll
+        for (int s = 0; s < NS; ++s)
+            if ((lane & 15) == s) mine = v[s];
+        if ((lane & 15) < NS && GIRA_IN(pp < npairs, const_cast<DeviceState*>(st))) {
+            float* dst = partials + part_off + ((int64_t)slice * npairs + pp) * (2 * NS);
+            dst[(hi16 ? NS : 0) + (lane & 15)] = mine;
+        }
     }
-    if (!loaded) return;
-    // lanes 0-15 end with the first component's sums, 16-31 with the second's
-    float v[NS];
-    const bool hi16 = lane & 16;
-#pragma unroll
-    for (int s = 0; s < NS; ++s) {
-        const float keep = hi16 ? S[s].y : S[s].x, send = hi16 ? S[s].x : S[s].y;
-        v[s] = keep + __shfl_xor_sync(FULL, send, 16);
-    }
-#pragma unroll
-    for (int o = 8; o > 0; o >>= 1)
-#pragma unroll
-        for (int s = 0; s < NS; ++s) v[s] += __shfl_xor_sync(FULL, v[s], o);
-    float mine = 0.f;
-#pragma unroll
-    for (int s = 0; s < NS; ++s)
-        if ((lane & 15) == s) mine = v[s];
-    if ((lane & 15) < NS) {
-        float* dst = partials + part_off + ((size_t)slice * npairs + pp) * (2 * NS);
-        dst[(hi16 ? NS : 0) + (lane & 15)] = mine;
-    }
-    if (lane == 0) atomicOr(live2 + live_off + (size_t)(pp >> 5) * slices + slice, 1u << (pp & 31));
 }
 
 template <int D, int H>
@@ -867,13 +888,13 @@ cudaError_t launch_estep_reach(int d, const ReachLaunch& a, int mode, int grid, 
     return cudaLaunchKernel(fn, dim3(grid), dim3(32 * RB_W), args, smem, s);
 }
 
-cudaError_t launch_reach_stats(int d, const ReachLaunch& a, int batch, int kmax, int64_t nmax, float* partials,
-                               uint32_t* live2, cudaStream_t s) {
-    int sl = 1;
-    const int slices = reach_slices(nmax, &sl);
-    const dim3 grid(((kmax + 1) / 2 + ST_W - 1) / ST_W, slices, a.insts ? batch : 1);
-    if (d == 3) reach_stats_kernel<3><<<grid, 32 * ST_W, 0, s>>>(a, sl, partials, live2);
-    else reach_stats_kernel<4><<<grid, 32 * ST_W, 0, s>>>(a, sl, partials, live2);
+cudaError_t launch_reach_stats(int d, const ReachLaunch& a, float* partials, cudaStream_t s) {
+    int dev = 0, sms = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int grid = sms * (d == 3 ? 7 : 5);   // as many warps as fit (72 and 96 registers a thread)
+    if (d == 3) reach_stats_kernel<3><<<grid, 32 * ST_W, 0, s>>>(a, partials);
+    else reach_stats_kernel<4><<<grid, 32 * ST_W, 0, s>>>(a, partials);
     return cudaGetLastError();
 }
 
