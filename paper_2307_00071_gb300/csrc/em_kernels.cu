@@ -539,6 +539,7 @@ void note_estep_kernel(const void* fn) {
     std::string name = (ok == 0 && dem) ? dem : raw;
     std::free(dem);
     size_t at = name.find("estep_pt_kernel<");
+    if (at == std::string::npos) at = name.find("estep_adjoint_kernel<");
     if (at == std::string::npos) at = name.find("estep_reach_kernel<");
     if (at != std::string::npos) name = name.substr(at);
     const size_t par = name.rfind(">(");
@@ -1553,9 +1554,11 @@ __global__ void __launch_bounds__(PFC_THREADS) params_from_chol_kernel(
         model64 += c * MODEL;
         params += I.par_off;
         shift4 += c;
-        perm += c;
-        ctr += c;
-        aux += c;
+        if (perm) {
+            perm += c;
+            ctr += c;
+            aux += c;
+        }
         st += blockIdx.y;
     }
     const int c0 = blockIdx.x * PFC_COMPS;
@@ -1642,8 +1645,8 @@ __global__ void __launch_bounds__(PFC_THREADS) params_from_chol_kernel(
     const int b = c0 + lane;
     float cc = -INFINITY;
     if (b < k) {
-        const int slot = s_slot[lane];
-        perm[slot] = b;
+        const int slot = perm ? s_slot[lane] : b;
+        if (perm) perm[slot] = b;
         const float* L = chol + 9 * (size_t)b;
         const double m3[3] = {mu[3 * b], mu[3 * b + 1], mu[3 * b + 2]};
         bool ok = isfinite(m3[0]) && isfinite(m3[1]) && isfinite(m3[2]);
@@ -1661,8 +1664,10 @@ __global__ void __launch_bounds__(PFC_THREADS) params_from_chol_kernel(
                 const float* base = params + (size_t)(slot >> 1) * PAIR_FLOATS + (slot & 1);
                 cc = base[2 * SLOT_C];
                 const float s2 = base[2 * SLOT_S];
-                ctr[slot] = make_float4((float)m3[0], (float)m3[1], (float)m3[2], s2);
-                aux[slot] = f2(cc, s2);
+                if (perm) {
+                    ctr[slot] = make_float4((float)m3[0], (float)m3[1], (float)m3[2], s2);
+                    aux[slot] = f2(cc, s2);
+                }
             }
         }
     }

@@ -877,19 +877,16 @@ gira_status gira_gmm_loglik_grad(const float* points, int64_t n, int k, const fl
     if (grad_means) TRY(check_ptr(grad_means, "grad_means", c.dev, &kgm));
     if (grad_chol) TRY(check_ptr(grad_chol, "grad_chol", c.dev, &kgc));
     const bool grad = grad_points || grad_pose || grad_twist || grad_logits || grad_means || grad_chol;
-    const bool gpar = grad_logits || grad_means || grad_chol;   // statistics wanted
-    const bool sorted = grad && n <= point_order_max_n();        // the E-step visits the scan in Morton order
     const int npairs = params_pairs_padded(k);
+    int64_t ppc = 0;
+    const int grid = adjoint_grid(n, k, grad, c.sms, &ppc);
     auto host = [&](Kind kd, const void* ptr) { return ptr && kd == Kind::Host; };
     struct Bufs {
         DeviceState* st;
-        float *pin, *pose, *lg, *mu, *ch, *params, *gp, *gl, *gm, *gc;
-        float4 *p8, *p8s, *shift4;
-        double *model64, *ppart, *po64, *tw64;
-        int *perm, *order;
-        void* osc;
+        float *pin, *pose, *lg, *mu, *ch, *params, *partials, *gp, *gl, *gm, *gc;
+        float4 *p8, *shift4;
+        double *model64, *llp, *ppart, *po64, *tw64;
     } b{};
-    ReachBufs rb;
     auto layout = [&](Carver& cv) {
         b.st = cv.take<DeviceState>(1);
         b.pin = cv.take<float>(host(kp, points) ? 3 * (size_t)n : 0);
@@ -898,15 +895,12 @@ gira_status gira_gmm_loglik_grad(const float* points, int64_t n, int k, const fl
         b.mu = cv.take<float>(host(km, means) ? 3 * (size_t)k : 0);
         b.ch = cv.take<float>(host(kc, chol) ? 9 * (size_t)k : 0);
         b.p8 = cv.take<float4>(2 * (size_t)n);
-        b.p8s = cv.take<float4>(sorted ? 2 * (size_t)n : 0);
-        b.order = cv.take<int>(sorted ? (size_t)n : 0);
-        b.osc = cv.take<char>(sorted ? point_order_scratch_bytes(n, 1) : 0);
-        b.perm = cv.take<int>(k);
-        carve_reach(cv, n, k, NSTAT, gpar, &rb);
         b.params = cv.take<float>((size_t)npairs * PAIR_FLOATS);
         b.shift4 = cv.take<float4>(k);
         b.model64 = cv.take<double>((size_t)k * MODEL);
-        b.ppart = cv.take<double>(grad ? (size_t)rb.grid * 12 : 0);
+        b.llp = cv.take<double>(grid);
+        b.partials = cv.take<float>(grad ? (size_t)grid * k * NSTAT : 0);
+        b.ppart = cv.take<double>(grad ? (size_t)grid * 12 : 0);
         b.po64 = cv.take<double>(12);
         b.tw64 = cv.take<double>(6);
         b.gp = cv.take<float>(host(kgp, grad_points) ? 3 * (size_t)n : 0);
@@ -957,35 +951,23 @@ gira_status gira_gmm_loglik_grad(const float* points, int64_t n, int k, const fl
     double* tw_d = grad_twist ? (kgt == Kind::Host ? b.tw64 : grad_twist) : nullptr;
 
     COUNTED(prof, 1, launch_pack_pose(pts_d, n, pose_d, b.p8, b.st, c.s));
-    if (sorted)
-        COUNTED(prof, point_order_launches(1),
-                launch_point_order(b.p8, n, nullptr, nullptr, 0, 1, b.osc, b.p8s, nullptr, b.order, c.s));
-    COUNTED(prof, 1, launch_params_from_chol(lg_d, mu_d, ch_d, k, nullptr, 1, b.model64, b.params, b.shift4, b.perm,
-                                             rb.ctr, rb.aux, b.st, c.s));
+    COUNTED(prof, 1, launch_fill_padding(b.params, k, npairs, c.s));
+    COUNTED(prof, 1, launch_params_from_chol(lg_d, mu_d, ch_d, k, nullptr, 1, b.model64, b.params, b.shift4, nullptr,
+                                             nullptr, nullptr, b.st, c.s));
     prof.t_init = prof.mark();
     prof.t_em = prof.t_init;
-    ReachLaunch a = reach_launch(rb, sorted ? b.p8s : b.p8, n, k, b.params, b.st, 0);
-    a.gref = nullptr;   // the parameter build leaves max_b c_b in the state
+    const AdjointLaunch a{b.p8, n, k, b.params, ppc, grad ? b.partials : nullptr, b.llp, b.st, 0, gp_d, pose_d, b.ppart};
     if (grad) {
-        a.grad_pts = gp_d;
-        a.order = sorted ? b.order : nullptr;
-        a.rot = pose_d;
-        a.pose_partials = b.ppart;
-        if (gpar) {
-            reach_with_stats(rb, &a);
-            GIRA_CUDA(reach_zero_live(rb, c.s));
-        }
         cudaEvent_t e0 = prof.mark_launch();
-        COUNTED(prof, 1, launch_estep_reach(3, a, 2, rb.grid, rb.h, k, c.s));
+        COUNTED(prof, 1, launch_estep_adjoint(a, true, grid, k, c.s));
         cudaEvent_t e1 = prof.mark_launch();
         if (prof.per_launch) prof.timed(e0, e1);
-        if (gpar) COUNTED(prof, 1, launch_reach_stats(3, a, rb.partials, c.s));
-        const ReachGradArgs f{gpar ? rb.partials : nullptr, rb.live2, rb.slices, rb.llp, b.ppart, rb.grid, pose_d,
-                              ch_d, b.params, b.model64, b.perm, k, n, gl_d, gm_d, gc_d, po_d, tw_d, b.st};
-        COUNTED(prof, 1, launch_reach_grad_finalize(f, nullptr, 1, c.s));
+        const AdjointFinArgs f{b.partials, grid, b.llp, b.ppart, pose_d, ch_d, b.model64, k, n,
+                               gl_d, gm_d, gc_d, po_d, tw_d, b.st};
+        COUNTED(prof, 1, launch_adjoint_finalize(f, nullptr, nullptr, 0, b.st, c.s));
     } else {
-        COUNTED(prof, 1, launch_estep_reach(3, a, 0, rb.grid, rb.h, k, c.s));
-        COUNTED(prof, 1, launch_ll_reduce(rb.llp, rb.grid, b.st, c.s));
+        COUNTED(prof, 1, launch_estep_adjoint(a, false, grid, k, c.s));
+        COUNTED(prof, 1, launch_ll_reduce(b.llp, grid, b.st, c.s));
     }
     auto out = [&](void* dst, Kind kd, const void* stage, size_t bytes) -> gira_status {
         if (dst && kd == Kind::Host) GIRA_CUDA(cudaMemcpyAsync(dst, stage, bytes, cudaMemcpyDeviceToHost, c.s));
@@ -1411,8 +1393,9 @@ gira_status gira_gmm_loglik_grad_batched(const float* points, const int64_t* off
         if (a.p) TRY(check_ptr(a.p, a.name, c.dev, &a.k));
     for (auto& a : out)
         if (a.p) TRY(check_ptr(a.p, a.name, c.dev, &a.k));
-    const bool gpar = grad_logits || grad_means || grad_chol;   // statistics wanted
-    const bool sorted = total_n <= point_order_max_n();
+    const bool dense = grad_chol != nullptr;   // every component (adjoint_kernels.cu says why); else reach lists
+    const bool gpar = !dense && (grad_logits || grad_means);
+    const bool sorted = !dense && total_n <= point_order_max_n();
 
     // ---- tables: instances and their E-step CTAs
     std::vector<BatchInst> hi(batch);
@@ -1441,7 +1424,44 @@ gira_status gira_gmm_loglik_grad_batched(const float* points, const int64_t* off
         live_words += (int64_t)reach_mask_words(I.k) * slices;
         I.part_off = part_floats;
         part_floats += (int64_t)slices * ((I.k + 1) / 2) * 2 * NSTAT;
-        for (int t = 0; t < I.ctas; ++t) units.push_back(BatchUnit{i, t});
+        if (!dense)
+            for (int t = 0; t < I.ctas; ++t) units.push_back(BatchUnit{i, t});
+    }
+    // dense: one launch per block shape; points per CTA from the class's points
+    struct Class {
+        int kmax = 0, unit_begin = 0, nunits = 0;
+        int64_t points = 0, ppc = 0;
+        std::vector<int> insts;
+    };
+    std::map<int, Class> classes;
+    std::vector<int2> fin_blocks;
+    if (dense) {
+        for (int i = 0; i < batch; ++i) {
+            Class& C = classes[adjoint_class(ks[i])];
+            C.insts.push_back(i);
+            C.points += hi[i].n;
+            C.kmax = std::max(C.kmax, ks[i]);
+        }
+        part_floats = ll_slots = 0;
+        for (auto& kv : classes) {
+            Class& C = kv.second;
+            C.ppc = adjoint_class_points(C.kmax, C.points, c.sms);
+            C.unit_begin = (int)units.size();
+            for (int i : C.insts) {
+                BatchInst& I = hi[i];
+                I.ppc = C.ppc;
+                I.ctas = (int)((I.n + C.ppc - 1) / C.ppc);
+                I.part_off = part_floats;
+                I.ll_off = ll_slots;
+                part_floats += (int64_t)I.ctas * I.k * NSTAT;
+                ll_slots += I.ctas;
+                for (int t = 0; t < I.ctas; ++t) units.push_back(BatchUnit{i, t});
+            }
+            C.nunits = (int)units.size() - C.unit_begin;
+        }
+        const int cpb = adjoint_components_per_block();
+        for (int i = 0; i < batch; ++i)
+            for (int j = 0; j * cpb < ks[i]; ++j) fin_blocks.push_back(make_int2(i, j));
     }
     const int64_t nounits = sorted ? point_order_box_units(offsets, batch) : 0;
     std::vector<int2> ounits((size_t)nounits);
@@ -1456,12 +1476,14 @@ gira_status gira_gmm_loglik_grad_batched(const float* points, const int64_t* off
         uint32_t *masks, *live2;
         BatchInst* insts;
         BatchUnit* units;
-        int2* ounits;
+        int2 *ounits, *blocks;
         uint2* sunits;
-        int *perm, *order;
+        int *perm, *order, *npairs;
         int64_t* offs;
         void* osc;
     } b{};
+    std::vector<int> npairs_of(batch);
+    for (int i = 0; i < batch; ++i) npairs_of[i] = params_pairs_padded(ks[i]);
     auto layout = [&](Carver& cv) {
         b.st = cv.take<DeviceState>(batch);
         b.pin = cv.take<float>(3 * (size_t)total_n);
@@ -1484,7 +1506,9 @@ gira_status gira_gmm_loglik_grad_batched(const float* points, const int64_t* off
         b.masks = cv.take<uint32_t>(gpar ? (size_t)mask_words : 0);
         b.live2 = cv.take<uint32_t>(gpar ? (size_t)live_words + 2 : 0);   // then the two unit counters
         b.sunits = cv.take<uint2>(gpar ? (size_t)part_floats / (2 * NSTAT) : 0);
-        b.partials = cv.take<float>(gpar ? (size_t)part_floats : 0);
+        b.partials = cv.take<float>(gpar || dense ? (size_t)part_floats : 0);
+        b.blocks = cv.take<int2>(fin_blocks.size());
+        b.npairs = cv.take<int>(dense ? batch : 0);
         b.llp = cv.take<double>((size_t)ll_slots);
         b.ppart = cv.take<double>(12 * (size_t)ll_slots);
         b.gp = cv.take<float>(grad_points ? 3 * (size_t)total_n : 0);
@@ -1539,13 +1563,19 @@ gira_status gira_gmm_loglik_grad_batched(const float* points, const int64_t* off
     GIRA_CUDA(cudaMemcpyAsync(b.offs, offsets, sizeof(int64_t) * (batch + 1), cudaMemcpyHostToDevice, c.s));
     GIRA_CUDA(cudaMemcpyAsync(b.insts, hi.data(), sizeof(BatchInst) * batch, cudaMemcpyHostToDevice, c.s));
     GIRA_CUDA(cudaMemcpyAsync(b.units, units.data(), sizeof(BatchUnit) * units.size(), cudaMemcpyHostToDevice, c.s));
+    if (dense) {
+        GIRA_CUDA(cudaMemcpyAsync(b.blocks, fin_blocks.data(), sizeof(int2) * fin_blocks.size(),
+                                  cudaMemcpyHostToDevice, c.s));
+        GIRA_CUDA(cudaMemcpyAsync(b.npairs, npairs_of.data(), sizeof(int) * batch, cudaMemcpyHostToDevice, c.s));
+    }
     if (sorted)
         GIRA_CUDA(cudaMemcpyAsync(b.ounits, ounits.data(), sizeof(int2) * ounits.size(), cudaMemcpyHostToDevice, c.s));
     prof.t_init = prof.mark();
 
     // ---- one graph: move the scans, order them, build the parameters, the E-step with the
     // gradient, the statistics (when a parameter gradient is asked for), finalize
-    std::string key = "grad|" + std::to_string((int)gpar) + std::to_string((int)(grad_points != nullptr)) + "|" + std::to_string((uintptr_t)ws->ptr) + "|" + std::to_string(sizer.off) + "|" +
+    std::string key = "grad|" + std::to_string((int)gpar) + std::to_string((int)dense) +
+                      std::to_string((int)(grad_points != nullptr)) + "|" + std::to_string((uintptr_t)ws->ptr) + "|" + std::to_string(sizer.off) + "|" +
                       std::to_string(batch);
     for (int i = 0; i < batch; ++i) key += "|" + std::to_string(hi[i].n) + ":" + std::to_string(hi[i].k);
     if (ws->graph_key != key || !ws->graph_exec) {
@@ -1557,32 +1587,45 @@ gira_status gira_gmm_loglik_grad_batched(const float* points, const int64_t* off
         if (e == cudaSuccess && sorted)
             e = launch_point_order(b.p8, total_n, b.offs, b.ounits, (int)nounits, batch, b.osc, b.p8s, nullptr,
                                    b.order, cs);
+        if (e == cudaSuccess && dense) e = launch_fill_padding_batched(b.params, b.insts, batch, 0, b.npairs, cs);
         if (e == cudaSuccess)
-            e = launch_params_from_chol(b.lg, b.mu, b.ch, kmax, b.insts, batch, b.model64, b.params, b.shift4, b.perm,
-                                        b.ctr, b.aux, b.st, cs);
-        ReachLaunch a{sorted ? b.p8s : b.p8, 0, 0, b.params, b.ctr, b.aux, nullptr, b.llp, nullptr, nullptr, 0};
-        a.n_buf = total_n;
-        a.grad_pts = grad_points ? b.gp : nullptr;
-        a.order = sorted ? b.order : nullptr;
-        a.rot = b.poses;
-        a.pose_partials = b.ppart;
-        a.insts = b.insts;
-        a.units = b.units;
-        a.states = b.st;
-        if (gpar) {
-            a.pref = b.pref;
-            a.masks = b.masks;
-            a.live2 = b.live2;
-            a.stat_units = b.sunits;
-            a.unit_count = reinterpret_cast<int*>(b.live2 + live_words);
-            if (e == cudaSuccess) e = cudaMemsetAsync(b.live2, 0, sizeof(uint32_t) * (live_words + 2), cs);
+            e = launch_params_from_chol(b.lg, b.mu, b.ch, kmax, b.insts, batch, b.model64, b.params, b.shift4,
+                                        dense ? nullptr : b.perm, b.ctr, b.aux, b.st, cs);
+        if (dense) {
+            for (auto& kv : classes) {
+                const Class& C = kv.second;
+                AdjointLaunch d{b.p8, 0, 0, b.params, C.ppc, b.partials, b.llp, nullptr, 0,
+                                grad_points ? b.gp : nullptr, b.poses, b.ppart, b.insts, b.units + C.unit_begin, b.st};
+                if (e == cudaSuccess) e = launch_estep_adjoint(d, true, C.nunits, C.kmax, cs);
+            }
+            const AdjointFinArgs f{b.partials, 0, b.llp, b.ppart, b.poses, b.ch, b.model64, 0, 0,
+                                   b.gl, b.gm, b.gc, b.gpose, b.gtwist, nullptr};
+            if (e == cudaSuccess)
+                e = launch_adjoint_finalize(f, b.insts, b.blocks, (int)fin_blocks.size(), b.st, cs);
+        } else {
+            ReachLaunch a{sorted ? b.p8s : b.p8, 0, 0, b.params, b.ctr, b.aux, nullptr, b.llp, nullptr, nullptr, 0};
+            a.n_buf = total_n;
+            a.grad_pts = grad_points ? b.gp : nullptr;
+            a.order = sorted ? b.order : nullptr;
+            a.rot = b.poses;
+            a.pose_partials = b.ppart;
+            a.insts = b.insts;
+            a.units = b.units;
+            a.states = b.st;
+            if (gpar) {
+                a.pref = b.pref;
+                a.masks = b.masks;
+                a.live2 = b.live2;
+                a.stat_units = b.sunits;
+                a.unit_count = reinterpret_cast<int*>(b.live2 + live_words);
+                if (e == cudaSuccess) e = cudaMemsetAsync(b.live2, 0, sizeof(uint32_t) * (live_words + 2), cs);
+            }
+            if (e == cudaSuccess) e = launch_estep_reach(3, a, 2, (int)units.size(), rh, kmax, cs);
+            if (e == cudaSuccess && gpar) e = launch_reach_stats(3, a, b.partials, cs);
+            const ReachGradArgs f{gpar ? b.partials : nullptr, b.live2, 0, b.llp, b.ppart, 0, b.poses, b.params, b.model64,
+                                  b.perm, kmax, 0, gpar ? b.gl : nullptr, gpar ? b.gm : nullptr, b.gpose, b.gtwist, b.st};
+            if (e == cudaSuccess) e = launch_reach_grad_finalize(f, b.insts, batch, cs);
         }
-        if (e == cudaSuccess) e = launch_estep_reach(3, a, 2, (int)units.size(), rh, kmax, cs);
-        if (e == cudaSuccess && gpar) e = launch_reach_stats(3, a, b.partials, cs);
-        const ReachGradArgs f{gpar ? b.partials : nullptr, b.live2, 0, b.llp, b.ppart, 0, b.poses, b.ch, b.params,
-                              b.model64, b.perm, kmax, 0, gpar ? b.gl : nullptr, gpar ? b.gm : nullptr,
-                              gpar ? b.gc : nullptr, b.gpose, b.gtwist, b.st};
-        if (e == cudaSuccess) e = launch_reach_grad_finalize(f, b.insts, batch, cs);
         cudaGraph_t graph = nullptr;
         cudaError_t e2 = cudaStreamEndCapture(cs, &graph);
         if (e != cudaSuccess || e2 != cudaSuccess) {
@@ -1601,7 +1644,7 @@ gira_status gira_gmm_loglik_grad_batched(const float* points, const int64_t* off
         ws->graph_exec = exec;
         ws->graph_key = key;
     }
-    prof.launches += 4 + (sorted ? point_order_launches(batch) : 0) + (gpar ? 1 : 0);
+    prof.launches += 4 + (sorted ? point_order_launches(batch) : 0) + (gpar ? 1 : 0) + (long long)classes.size();
     GIRA_CUDA(cudaGraphLaunch(ws->graph_exec, c.s));
     prof.t_em = prof.mark();
     const void* src[6] = {b.gp, b.gpose, b.gtwist, b.gl, b.gm, b.gc};

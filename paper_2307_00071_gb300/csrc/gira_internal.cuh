@@ -546,6 +546,48 @@ cudaError_t launch_ll_reduce_batched(const double* ll_partials, const BatchInst*
 // own model and pose; poses: batch x 12, or nullptr for identities).
 cudaError_t launch_pack_pose_batched(const float* pts3, int64_t n, const int64_t* offsets, int batch,
                                      const float* poses, float4* pts8, DeviceState* states, cudaStream_t s);
+// The gradient with every component, statistics in world axes (adjoint_kernels.cu).
+struct AdjointLaunch {
+    const float4* pts8;      // as EStepLaunch, in the caller's order
+    int64_t n;
+    int k;
+    const float* params;     // in the caller's order, padded to params_pairs_padded(k)
+    int64_t pts_per_cta;     // batched: the largest of the launch (its instances' ppc)
+    float* partials;         // [grid][k][NSTAT]
+    double* ll_partials;     // [grid]
+    DeviceState* st;
+    int iter;
+    float* grad_pts;         // [n][3] dL/dx, or nullptr
+    const float* rot;        // R, row-major 3x3, of x' = R x + t; nullptr = identity
+    double* pose_partials;   // [grid][12]: per CTA sum dL/dx' x'^T (row-major), sum dL/dx'
+    // batched: CTA b runs units[b]; the pointers are bases offset by the instance's entry
+    const BatchInst* insts = nullptr;
+    const BatchUnit* units = nullptr;
+    DeviceState* states = nullptr;
+};
+struct AdjointFinArgs {
+    const float* partials;
+    int grid;
+    const double* llp;
+    const double* pp;
+    const float* pose;
+    const float* chol;
+    const double* model64;
+    int k;
+    int64_t n;
+    float *g_logits, *g_means, *g_chol;
+    double *g_pose, *g_twist;
+    DeviceState* st;
+};
+int adjoint_grid(int64_t n, int k, bool grad, int num_sms, int64_t* pts_per_cta);
+int adjoint_class(int k);   // instances of equal class run in one launch
+int64_t adjoint_class_points(int k, int64_t points, int num_sms);   // points per CTA of a class
+// grad = false: the log-likelihood alone.
+cudaError_t launch_estep_adjoint(const AdjointLaunch& a, bool grad, int grid, int k_class, cudaStream_t s);
+int adjoint_components_per_block();
+cudaError_t launch_adjoint_finalize(const AdjointFinArgs& f, const BatchInst* insts, const int2* blocks, int nblocks,
+                                    DeviceState* states, cudaStream_t s);
+
 // Differentiable log-likelihood.  pose12 = R (row-major) then t, or nullptr.
 // N x 3 -> pts8 of x' = R x + t (binary32, fixed order); flags non-finite input.
 cudaError_t launch_pack_pose(const float* pts3, int64_t n, const float* pose12, float4* pts8, DeviceState* st,
@@ -553,13 +595,12 @@ cudaError_t launch_pack_pose(const float* pts3, int64_t n, const float* pose12, 
 // E-step parameters from (logits, means, Cholesky factors), k <= MAX_K_DIRECT, in Morton
 // order of the means (perm[slot]: the caller's component), with the compact arrays of the
 // reach tests and max_b c_b in st->cmax_ord.  insts: every instance of a batch, kmax the
-// largest k (one fit: its k).
+// largest k (one fit: its k).  perm nullptr: the caller's order (ctr and aux are not written).
 cudaError_t launch_params_from_chol(const float* logits, const float* mu, const float* chol, int kmax,
                                     const BatchInst* insts, int batch, double* model64, float* params, float4* shift4,
                                     int* perm, float4* ctr, float2* aux, DeviceState* st, cudaStream_t s);
-// Sums of a gradient launch (fixed order): dL/dlogits (k), dL/dmeans (k x 3), dL/dchol
-// (k x 3 x 3, lower) in binary32 from the statistics, in the caller's order; in binary64
-// dL/dpose (dL/dR row-major, dL/dt) and dL/dtwist (omega, v); the log-likelihood in
+// Sums of a gradient launch (fixed order): dL/dlogits (k), dL/dmeans (k x 3) in binary32
+// from the statistics, in the caller's order; in binary64 dL/dpose (dL/dR row-major, dL/dt) and dL/dtwist (omega, v); the log-likelihood in
 // st->ll_sum.  Outputs nullable; partials nullptr: no parameter gradients.
 struct ReachGradArgs {
     const float* partials;    // [slices][pairs][2 NSTAT], live where live2 says
@@ -569,13 +610,12 @@ struct ReachGradArgs {
     const double* pp;         // [grid][12]
     int grid;
     const float* pose;
-    const float* chol;
     const float* params;
     const double* model64;
     const int* perm;
     int k;
     int64_t n;
-    float *g_logits, *g_means, *g_chol;
+    float *g_logits, *g_means;
     double *g_pose, *g_twist;
     DeviceState* st;
 };

@@ -905,12 +905,12 @@ namespace {
 // contiguous values over the live slices (compensated binary32, in order); then one
 // warp maps the statistics of the 32 components to the parameter gradients in binary64,
 // one component per lane (a binary64 warp instruction costs the same whatever the
-// number of lanes).  With S0, S1, S2 about y = P'_32 (x' - mu) (the binary32 P' of the
-// E-step), P = L_b^{-1} and T = P P'_32^{-1}:
-//   dL/dmu_b    = P^T (T S1)
-//   dL/dL_b     = lower(P^T (T S2 T^T)) - S0 diag(1/L_ii)
+// number of lanes).  With S0, S1 about y = P'_32 (x' - mu) (the binary32 P' of the E-step;
+// P'^T P' = Sigma^{-1} log2(e) / 2):
+//   dL/dmu_b    = 2 ln 2 P'^T S1
 //   dL/dalpha_b = S0 - N pi_b
-// The instance's block 0 also sums the log-likelihood and the pose terms.
+// (dL/dL_b: adjoint_kernels.cu).  The instance's block 0 also sums the log-likelihood and
+// the pose terms.
 constexpr int RG_PAIRS = 16, RG_THREADS = RG_PAIRS * 2 * NSTAT;
 static_assert(RG_THREADS % 32 == 0, "whole warps");
 
@@ -965,67 +965,15 @@ __global__ void __launch_bounds__(RG_THREADS) reach_grad_finalize_kernel(const R
         if (warp == 0 && b < k) {
             const double* S = s_stat[lane];
             const int src_b = f_in.perm[c_off + b];
-            const float* L = f_in.chol + 9 * (c_off + src_b);
-            const double L00 = L[0], L10 = L[3], L11 = L[4], L20 = L[6], L21 = L[7], L22 = L[8];
-            auto inv3 = [](double a00, double a10, double a11, double a20, double a21, double a22, double (&M)[3][3]) {
-                const double i0 = 1.0 / a00, i1 = 1.0 / a11, i2 = 1.0 / a22;
-                M[0][0] = i0; M[0][1] = 0.0; M[0][2] = 0.0;
-                M[1][0] = -a10 * i0 * i1; M[1][1] = i1; M[1][2] = 0.0;
-                M[2][0] = -(a20 * i0 + a21 * M[1][0]) * i2; M[2][1] = -a21 * i1 * i2; M[2][2] = i2;
-            };
-            double P[3][3], Q[3][3], T[3][3];
-            inv3(L00, L10, L11, L20, L21, L22, P);
             const float* q = f_in.params + par_off + (size_t)(b >> 1) * PAIR_FLOATS + (b & 1);
-            inv3(q[2 * SLOT_P], q[2 * (SLOT_P + 1)], q[2 * (SLOT_P + 2)], q[2 * (SLOT_P + 3)], q[2 * (SLOT_P + 4)],
-                 q[2 * (SLOT_P + 5)], Q);
+            if (f_in.g_means)
 #pragma unroll
-            for (int i = 0; i < 3; ++i)
+                for (int i = 0; i < 3; ++i) {
+                    double gm = 0.0;
 #pragma unroll
-                for (int j = 0; j < 3; ++j) {
-                    T[i][j] = 0.0;
-#pragma unroll
-                    for (int m = j; m <= i; ++m) T[i][j] += P[i][m] * Q[m][j];
+                    for (int m = i; m < 3; ++m) gm += (double)q[2 * (SLOT_P + m * (m + 1) / 2 + i)] * S[1 + m];
+                    f_in.g_means[3 * (c_off + src_b) + i] = (float)(1.3862943611198906 * gm);
                 }
-            const double S2[3][3] = {{S[4], S[5], S[6]}, {S[5], S[7], S[8]}, {S[6], S[8], S[9]}};
-            double u[3], A[3][3], M[3][3];   // u = T S1, A = T S2, M = A T^T
-#pragma unroll
-            for (int i = 0; i < 3; ++i) {
-                u[i] = 0.0;
-#pragma unroll
-                for (int m = 0; m <= i; ++m) u[i] += T[i][m] * S[1 + m];
-#pragma unroll
-                for (int j = 0; j < 3; ++j) {
-                    A[i][j] = 0.0;
-#pragma unroll
-                    for (int m = 0; m <= i; ++m) A[i][j] += T[i][m] * S2[m][j];
-                }
-            }
-#pragma unroll
-            for (int i = 0; i < 3; ++i)
-#pragma unroll
-                for (int j = 0; j < 3; ++j) {
-                    M[i][j] = 0.0;
-#pragma unroll
-                    for (int m = 0; m <= j; ++m) M[i][j] += A[i][m] * T[j][m];
-                }
-            const double Ld[3] = {L00, L11, L22};
-#pragma unroll
-            for (int i = 0; i < 3; ++i) {
-                double gm = 0.0;
-#pragma unroll
-                for (int m = i; m < 3; ++m) gm += P[m][i] * u[m];
-                if (f_in.g_means) f_in.g_means[3 * (c_off + src_b) + i] = (float)gm;
-#pragma unroll
-                for (int j = 0; j < 3; ++j) {
-                    double v2 = 0.0;
-                    if (j <= i) {
-#pragma unroll
-                        for (int m = i; m < 3; ++m) v2 += P[m][i] * M[m][j];
-                        if (i == j) v2 -= S[0] / Ld[i];
-                    }
-                    if (f_in.g_chol) f_in.g_chol[9 * (c_off + src_b) + 3 * i + j] = (float)v2;
-                }
-            }
             if (f_in.g_logits) f_in.g_logits[c_off + src_b] = (float)(S[0] - (double)n * f_in.model64[(c_off + b) * MODEL]);
         }
     }

@@ -71,8 +71,9 @@ def test_large_k_reach(gira, frame, n, k, off):
 
 @pytest.mark.parametrize("n,k,off", [(1, 1, 0), (129, 3, 5), (5_000, 63, 300), (4_096, 64, 4_096), (20_001, 1_024, 900)])
 def test_gradient_reach(gira, frame, n, k, off):
-    """Every gradient of a scan partly (or wholly) off the model, against the oracle's."""
-    from tests.test_gpu_grad import check_all, pose12, ref_grads, rot
+    """The gradients of a scan partly (or wholly) off the model against the oracle's: on one scan, and in a
+    batch over reach lists (with and without the statistics launch)."""
+    from tests.test_gpu_grad import assert_group, assert_points, check_all, ll_tol, pose12, ref_grads, rot
     rng = np.random.default_rng(n + k)
     start = rng.integers(0, len(frame) - n)
     pts = np.ascontiguousarray(frame[start:start + n])
@@ -81,10 +82,19 @@ def test_gradient_reach(gira, frame, n, k, off):
     w, m, c = ball_model(frame[start:start + max(n, k)], k, rng)
     chol = np.linalg.cholesky(c.astype(np.float64)).astype(np.float32)
     R, t = rot(rng.normal(scale=0.02, size=3)).astype(np.float32), rng.normal(scale=0.02, size=3).astype(np.float32)
-    r = gira.gira_gmm_loglik_grad(pts, np.log(w), m, chol, pose12(R, t))
-    check_all(r, ref_grads(pts, np.log(w), m, chol, R, t), n)
-    only = gira.gira_gmm_loglik_grad(pts, np.log(w), m, chol, pose12(R, t), want=("twist",))   # no statistics launch
-    assert np.array_equal(to_np(only["grad_twist"]), to_np(r["grad_twist"])) and only["loglik"] == r["loglik"]
+    args, ref = (pts, np.log(w), m, chol, pose12(R, t)), ref_grads(pts, np.log(w), m, chol, R, t)
+    check_all(gira.gira_gmm_loglik_grad(*args), ref, n)
+    twice = [np.concatenate([pts, pts]), [0, n, 2 * n], [k, k], *(np.concatenate([a, a]) for a in args[1:4]),
+             np.stack([args[4], args[4]])]
+    r = gira.gira_gmm_loglik_grad_batched(*twice, want=("points", "pose", "twist", "logits", "means"))
+    only = gira.gira_gmm_loglik_grad_batched(*twice, want=("twist",))   # no statistics launch
+    assert np.array_equal(to_np(only["grad_twist"]), to_np(r["grad_twist"])) and np.array_equal(only["loglik"], r["loglik"])
+    for i in range(2):
+        assert abs(r["loglik"][i] - ref["loglik"]) <= ll_tol(ref["loglik"], n)
+        for g, per in (("logits", k), ("means", k), ("twist", 0), ("pose", 0)):
+            got = to_np(r["grad_" + g])
+            assert_group(got[i * k:(i + 1) * k] if per else got[i], ref["grad_" + g], g)
+        assert_points(to_np(r["grad_points"])[i * n:(i + 1) * n], ref["grad_points"])
 
 
 @pytest.mark.parametrize("n,k,off", [(1, 1, 0), (127, 2, 0), (4_097, 33, 5), (30_001, 1_023, 128), (8_193, 1_025, 600)])
