@@ -1455,31 +1455,61 @@ __global__ void label_stats_kernel(const float4* __restrict__ pts, int64_t n, in
     }
 }
 
-// Batched: the instance of point i by binary search over the offsets.
+// Batched: each thread takes LS_PPT consecutive points (in Morton order within an instance,
+// so mostly of one label), the instance of the first by binary search over the offsets, and
+// sums runs as above.  (One binary64 atomic per point and statistic took 533 us on 1.4M
+// points of 48 clouds.)
 __global__ void label_stats_batched_kernel(const float4* __restrict__ pts, int64_t n, const int64_t* __restrict__ offsets,
                                            int batch, const KppInst* __restrict__ table,
                                            const int32_t* __restrict__ labels, const float4* __restrict__ shift4,
                                            double* stats64, DeviceState* states) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        int lo = 0, hi = batch;
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (offsets[mid] <= i) lo = mid; else hi = mid;
+    const int64_t step = (int64_t)gridDim.x * blockDim.x * LS_PPT;
+    for (int64_t i0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * LS_PPT; i0 < n; i0 += step) {
+        int inst = 0, hi = batch;
+        while (hi - inst > 1) {
+            const int mid = (inst + hi) >> 1;
+            if (offsets[mid] <= i0) inst = mid; else hi = mid;
         }
-        if (states[lo].error) continue;
-        if (!GIRA_IN(labels[i] >= 0 && labels[i] < table[lo].k, states + lo)) continue;
-        const int b = table[lo].comp_off + labels[i];
-        const float4 x = pts[i], s = shift4[b];
-        const double d[3] = {(double)x.x - (double)s.x, (double)x.y - (double)s.y, (double)x.z - (double)s.z};
-        double* S = stats64 + (size_t)b * NSTAT;
-        atomicAdd(&S[0], 1.0);
-        for (int t = 0; t < 3; ++t) atomicAdd(&S[1 + t], d[t]);
-        atomicAdd(&S[4], d[0] * d[0]);
-        atomicAdd(&S[5], d[0] * d[1]);
-        atomicAdd(&S[6], d[0] * d[2]);
-        atomicAdd(&S[7], d[1] * d[1]);
-        atomicAdd(&S[8], d[1] * d[2]);
-        atomicAdd(&S[9], d[2] * d[2]);
+        int64_t end = offsets[inst + 1];
+        int off = table[inst].comp_off, k = table[inst].k;
+        bool bad = states[inst].error != 0;
+        int key = -1;
+        float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+        double a[NSTAT];
+#pragma unroll
+        for (int t = 0; t < NSTAT; ++t) a[t] = 0.0;
+        for (int r = 0; r < LS_PPT; ++r) {
+            const int64_t i = i0 + r;
+            if (i >= n) break;
+            while (i >= end) {
+                end = offsets[++inst + 1];
+                off = table[inst].comp_off;
+                k = table[inst].k;
+                bad = states[inst].error != 0;
+            }
+            if (bad || !GIRA_IN(labels[i] >= 0 && labels[i] < k, states + inst)) continue;
+            const int b = off + labels[i];
+            if (b != key) {
+                if (key >= 0) label_stats_flush(stats64, key, a);
+#pragma unroll
+                for (int t = 0; t < NSTAT; ++t) a[t] = 0.0;
+                key = b;
+                s = shift4[b];
+            }
+            const float4 x = pts[i];
+            const double d0 = (double)x.x - (double)s.x, d1 = (double)x.y - (double)s.y, d2 = (double)x.z - (double)s.z;
+            a[0] += 1.0;
+            a[1] += d0;
+            a[2] += d1;
+            a[3] += d2;
+            a[4] += d0 * d0;
+            a[5] += d0 * d1;
+            a[6] += d0 * d2;
+            a[7] += d1 * d1;
+            a[8] += d1 * d2;
+            a[9] += d2 * d2;
+        }
+        if (key >= 0) label_stats_flush(stats64, key, a);
     }
 }
 
@@ -1724,7 +1754,7 @@ cudaError_t launch_label_stats_batched(const float4* pts4, int64_t n, const int6
     int dev = 0, sms = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int64_t want = (n + 255) / 256;
+    const int64_t want = (n + 256 * LS_PPT - 1) / (256 * LS_PPT);
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)sms * 8));
     label_stats_batched_kernel<<<grid, 256, 0, s>>>(pts4, n, offsets, batch, table, labels, shift4, stats64, states);
     return cudaGetLastError();
