@@ -374,7 +374,9 @@ __global__ void pack4_kernel(const float* __restrict__ p4in, int64_t n, float4* 
 // value twice (the operands of packed operations on two locations): slots 0 .. 14; then the
 // norms of P_xx's columns (15 .. 17) and a lower bound of sigma_min(P_xx)^2 (18), once each.
 constexpr int COND_SLOTS = 20;
-constexpr int COND_FLOATS = 2 * COND_SLOTS;
+constexpr int COND_FLOATS = 2 * COND_SLOTS;   // a component's slots in pairs, read by whole warps
+constexpr int COND_ALL = COND_FLOATS + COND_SLOTS;   // + the slots once more, slot i of component b at [i * k + b]:
+                                                     // the listing reads 32 components at a time
 
 __global__ void cond_prepare_kernel(const float* __restrict__ w, const float* __restrict__ mu,
                                     const float* __restrict__ cov, int k, float* prep, DeviceState* st) {
@@ -424,7 +426,11 @@ __global__ void cond_prepare_kernel(const float* __restrict__ w, const float* __
     if (!(pi > 0.0)) { set_error(st, GIRA_ERR_INVALID_ARG); return; }
     const double c = log(pi) - (log(L[0]) + log(L[4]) + log(L[8])) - 1.5 * log(2.0 * 3.14159265358979323846);
     float* o = prep + (size_t)b * COND_FLOATS;
-    auto put = [&](int slot, float x) { o[2 * slot] = o[2 * slot + 1] = x; };
+    float* t = prep + (size_t)k * COND_FLOATS + b;
+    auto put = [&](int slot, float x) {
+        o[2 * slot] = o[2 * slot + 1] = x;
+        t[(size_t)slot * k] = x;
+    };
     put(0, (float)P[0]); put(1, (float)P[3]); put(2, (float)P[4]); put(3, (float)P[6]); put(4, (float)P[7]);
     put(5, (float)P[8]);
     for (int i = 0; i < 3; ++i) put(6 + i, (float)g[i]);
@@ -442,41 +448,51 @@ __global__ void cond_prepare_kernel(const float* __restrict__ w, const float* __
     put(19, 0.f);
 }
 
-// One warp per 128 consecutive locations (four blocks of 32, a location of each per lane).
-// Pass 1 takes the maximum log-weight and, as a reference, the regression mean m_ref of that
-// component; pass 2 sums w_b = exp(lw_b - max), w_b (m_b - m_ref) and w_b (v_b + (m_b -
-// m_ref)^2) in binary32 (the shift keeps the variance free of cancellation), both over the
-// components in increasing order, two locations per packed operation.
+// Four warps per 256 locations, neighbours in `order`: a warp has 64 of them, a lane one of
+// each block of 32.  Pass 1 takes the maximum log-weight and, as a reference, the regression
+// mean m_ref of that component; pass 2 sums w_b = exp(lw_b - max), w_b (m_b - m_ref) and
+// w_b (v_b + (m_b - m_ref)^2) in binary32 (the shift keeps the variance free of
+// cancellation), both over the components in increasing order, two locations per packed
+// operation.
 // Only components that can matter are visited: exp of less than -104 is exactly 0 in
-// binary32, and a term of weight 0 changes no sum.  For each block of 32, the component of
-// largest log-weight at the centre of its box gives every location a log-weight; with L the
-// smallest of these, a component whose upper bound over the box (the two bounds of the
+// binary32, and a term of weight 0 changes no sum.  Over a set of locations, the component
+// of largest log-weight at the centre of their box gives every location a log-weight; with L
+// the smallest of these, a component whose upper bound over the box (the two bounds of the
 // E-step's reach test) is below L - 106 is neither a maximum nor of nonzero weight there.
-// What it costs is the listing (~3 % of the dense evaluation) and the listed evaluations.
-// Measured: 307,200 locations, K = 1163: 725 us for every component twice, XXX us now.
+// Listed first for the 256 locations, by all four warps, then from that list for each warp's
+// two blocks (a listing for each warp from all components was two thirds of the time).  The
+// listed components' slots go through shared memory, 16 at a time: a block across an edge
+// may list hundreds, and their loads one by one are that warp's (and so the kernel's) time.
+// Measured: 307,200 locations, K = 1163: 725 us for every component twice, 79 us now (485 us with one
+// listing per warp of locations in a depth image's rows).
 constexpr int COND_WARPS = 4;
 constexpr int COND_CAP = 2048;   // components listed at a time
-constexpr size_t cond_smem() { return (size_t)COND_WARPS * COND_CAP * (sizeof(uint16_t) + 1); }
+constexpr int COND_SEG = COND_CAP / COND_WARPS;
+constexpr int COND_LOCS = 64;    // locations per warp
+constexpr int COND_CHUNK = 16;   // components staged at a time
 
-__global__ void __launch_bounds__(32 * COND_WARPS) conditional4_kernel(const float* __restrict__ locs, int64_t m, int k,
+__global__ void __launch_bounds__(32 * COND_WARPS) conditional4_kernel(const float* __restrict__ locs,
+                                                                       const int* __restrict__ order, int64_t m, int k,
                                                                        const float* __restrict__ prep, float* cmean,
                                                                        float* cvar, DeviceState* st) {
-    extern __shared__ __align__(16) unsigned char cond_dsm[];
+    __shared__ __align__(16) float4 s_rec[COND_WARPS][COND_CHUNK][8];
+    __shared__ uint16_t s_seg[COND_WARPS][COND_SEG];
+    __shared__ uint16_t s_list[COND_WARPS][COND_CAP];
+    __shared__ float s_box[COND_WARPS][6], s_bv[COND_WARPS], s_L[COND_WARPS];
+    __shared__ int s_bb[COND_WARPS], s_n[COND_WARPS];
     __shared__ int s_err;
     if (threadIdx.x == 0) s_err = st->error;
     __syncthreads();
     if (s_err) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint16_t* list = reinterpret_cast<uint16_t*>(cond_dsm) + warp * COND_CAP;
-    uint8_t* need = cond_dsm + (size_t)COND_WARPS * COND_CAP * sizeof(uint16_t) + warp * COND_CAP;
-    const int64_t base = ((int64_t)blockIdx.x * COND_WARPS + warp) * 128;
-    if (base >= m) return;
-    float x[4][3];   // location base + 32 r + lane
-    float lo[4][3], hi[4][3];
+    uint16_t* list = s_list[warp];
+    const int64_t base = ((int64_t)blockIdx.x * COND_WARPS + warp) * COND_LOCS;
+    float x[2][3];   // location base + 32 r + lane
+    float lo[2][3], hi[2][3];
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        const int64_t i = base + 32 * r + lane;
-        const int64_t at = min(i, m - 1);   // an absent location: the last one, not written
+    for (int r = 0; r < 2; ++r) {
+        const int64_t i = min(base + 32 * r + lane, m - 1);   // an absent location: the last one, not written
+        const int64_t at = order ? order[i] : i;
         bool fin = true;
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
@@ -493,174 +509,278 @@ __global__ void __launch_bounds__(32 * COND_WARPS) conditional4_kernel(const flo
                 hi[r][j] = fmaxf(hi[r][j], __shfl_xor_sync(FULL, hi[r][j], o));
             }
     }
-    float2 X[2][3];   // locations of blocks 2q, 2q + 1
+    if (lane == 0)
 #pragma unroll
-    for (int q = 0; q < 2; ++q)
+        for (int j = 0; j < 3; ++j) {
+            s_box[warp][j] = fminf(lo[0][j], lo[1][j]);
+            s_box[warp][3 + j] = fmaxf(hi[0][j], hi[1][j]);
+        }
+    __syncthreads();
+    float wlo[3], whi[3];   // the box of all
 #pragma unroll
-        for (int j = 0; j < 3; ++j) X[q][j] = f2(x[2 * q][j], x[2 * q + 1][j]);
-    auto slot = [&](const float2* o, int i) { return __ldg(o + i); };
+    for (int j = 0; j < 3; ++j) {
+        wlo[j] = s_box[0][j];
+        whi[j] = s_box[0][3 + j];
+#pragma unroll
+        for (int w = 1; w < COND_WARPS; ++w) {
+            wlo[j] = fminf(wlo[j], s_box[w][j]);
+            whi[j] = fmaxf(whi[j], s_box[w][3 + j]);
+        }
+    }
+    const float* soa = prep + (size_t)k * COND_FLOATS;
+    auto slot = [&](int b, int i) { return __ldg(soa + (size_t)i * k + b); };
+    auto scan_slots = [&](int b, float (&P)[6], float (&nm)[3], float& c) {
+#pragma unroll
+        for (int i = 0; i < 6; ++i) P[i] = slot(b, i);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) nm[i] = slot(b, 11 + i);
+        c = slot(b, 10);
+    };
+    auto maha = [&](const float (&P)[6], const float (&d)[3]) {
+        const float y0 = P[0] * d[0], y1 = fmaf(P[2], d[1], P[1] * d[0]);
+        const float y2 = fmaf(P[5], d[2], fmaf(P[4], d[1], P[3] * d[0]));
+        return fmaf(y2, y2, fmaf(y1, y1, y0 * y0));
+    };
+    auto centre_lw = [&](const float (&P)[6], const float (&nm)[3], float c, const float (&l)[3], const float (&h)[3]) {
+        const float d[3] = {0.5f * (l[0] + h[0]) + nm[0], 0.5f * (l[1] + h[1]) + nm[1], 0.5f * (l[2] + h[2]) + nm[2]};
+        return fmaf(-0.5f, maha(P, d), c);
+    };
+    // the upper bound of component b's log-weight over the box
+    auto upper = [&](int b, const float (&P)[6], const float (&nm)[3], float c, const float (&l)[3],
+                     const float (&u)[3]) {
+        const float n0 = slot(b, 15), n1 = slot(b, 16), n2 = slot(b, 17), s2 = slot(b, 18);
+        float d[3], h[3], e2 = 0.f;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const float ctr = 0.5f * (l[j] + u[j]);
+            h[j] = fmaxf(u[j] - ctr, ctr - l[j]);
+            d[j] = ctr + nm[j];
+            const float e = fmaxf(fabsf(d[j]) - h[j], 0.f);
+            e2 = fmaf(e, e, e2);
+        }
+        const float reach = fmaf(h[0], n0, fmaf(h[1], n1, h[2] * n2));
+        const float t = fmaxf(sqrtf(maha(P, d)) * (1.f - 1.f / 256.f) - reach * (1.f + 1.f / 256.f), 0.f);
+        const float q = fmaxf(t * t, s2 * e2 * (1.f - 1.f / 128.f));   // <= |P (x - mu)|^2 over the box
+        return fmaf(-0.5f, q, c);
+    };
+    auto warp_best = [&](float& v, int& b) {   // the same choice in every lane
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const float v2 = __shfl_xor_sync(FULL, v, o);
+            const int b2 = __shfl_xor_sync(FULL, b, o);
+            if (v2 > v || (v2 == v && b2 < b)) {
+                v = v2;
+                b = b2;
+            }
+        }
+    };
+    auto warp_min = [&](float v) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(FULL, v, o));
+        return v;
+    };
+    auto at_mine = [&](int b, int r) {   // log-weight of component b at this lane's location r
+        float P[6], nm[3], c;
+        scan_slots(b, P, nm, c);
+        const float d[3] = {x[r][0] + nm[0], x[r][1] + nm[1], x[r][2] + nm[2]};
+        return fmaf(-0.5f, maha(P, d), c);
+    };
+    // ---- L of all
+    float L_all;
+    {
+        float v = -INFINITY;
+        int best = 0;
+        for (int b = threadIdx.x; b < k; b += 32 * COND_WARPS) {
+            float P[6], nm[3], c;
+            scan_slots(b, P, nm, c);
+            const float lw = centre_lw(P, nm, c, wlo, whi);
+            if (lw > v) { v = lw; best = b; }
+        }
+        warp_best(v, best);
+        if (lane == 0) {
+            s_bv[warp] = v;
+            s_bb[warp] = best;
+        }
+        __syncthreads();
+        v = s_bv[0];
+        best = s_bb[0];
+#pragma unroll
+        for (int w = 1; w < COND_WARPS; ++w)
+            if (s_bv[w] > v) { v = s_bv[w]; best = s_bb[w]; }
+        const float mine = warp_min(fminf(at_mine(best, 0), at_mine(best, 1)));
+        if (lane == 0) s_L[warp] = mine;
+        __syncthreads();
+        L_all = s_L[0];
+#pragma unroll
+        for (int w = 1; w < COND_WARPS; ++w) L_all = fminf(L_all, s_L[w]);
+    }
+    // ---- the components of [b0, b1) that this warp's blocks need, in order (called by all warps)
+    int nl = 0;
+    float known[2] = {-INFINITY, -INFINITY};   // a log-weight of some component at this lane's locations
+    auto make_list = [&](int b0, int b1) {
+        __syncthreads();   // the segments of the list before this one are read
+        const int per = ((b1 - b0 + 32 * COND_WARPS - 1) / (32 * COND_WARPS)) * 32;   // <= COND_SEG
+        const int e = min(b1, b0 + per * (warp + 1));
+        int n = 0;
+        for (int j0 = b0 + per * warp; j0 < e; j0 += 32) {
+            const int b = j0 + lane;
+            bool want = false;
+            if (b < e) {
+                float P[6], nm[3], c;
+                scan_slots(b, P, nm, c);
+                want = !(upper(b, P, nm, c, wlo, whi) < L_all - 106.f);
+            }
+            const unsigned mk = __ballot_sync(FULL, want);
+            if (want) s_seg[warp][n + __popc(mk & ((1u << lane) - 1u))] = (uint16_t)b;
+            n += __popc(mk);
+        }
+        if (lane == 0) s_n[warp] = n;
+        __syncthreads();
+        int off[COND_WARPS + 1];
+        off[0] = 0;
+#pragma unroll
+        for (int w = 0; w < COND_WARPS; ++w) off[w + 1] = off[w] + s_n[w];
+        auto listed = [&](int t) {
+            int w = 0, o = 0;
+#pragma unroll
+            for (int q = 1; q < COND_WARPS; ++q)
+                if (t >= off[q]) { w = q; o = off[q]; }
+            return (int)s_seg[w][t - o];
+        };
+        float v[2] = {-INFINITY, -INFINITY}, L[2];
+        int best[2] = {-1, -1};
+        for (int t = lane; t < off[COND_WARPS]; t += 32) {
+            const int b = listed(t);
+            float P[6], nm[3], c;
+            scan_slots(b, P, nm, c);
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                const float lw = centre_lw(P, nm, c, lo[r], hi[r]);
+                if (lw > v[r]) { v[r] = lw; best[r] = b; }
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            warp_best(v[r], best[r]);
+            known[r] = best[r] < 0 ? -INFINITY : at_mine(best[r], r);
+            L[r] = fmaxf(L_all, warp_min(known[r]));
+        }
+        nl = 0;
+        for (int t0 = 0; t0 < off[COND_WARPS]; t0 += 32) {
+            const int t = t0 + lane;
+            int b = 0;
+            bool want = false;
+            if (t < off[COND_WARPS]) {
+                b = listed(t);
+                float P[6], nm[3], c;
+                scan_slots(b, P, nm, c);
+#pragma unroll
+                for (int r = 0; r < 2; ++r) want = want || !(upper(b, P, nm, c, lo[r], hi[r]) < L[r] - 106.f);
+            }
+            const unsigned mk = __ballot_sync(FULL, want);
+            if (want) list[nl + __popc(mk & ((1u << lane) - 1u))] = (uint16_t)b;
+            nl += __popc(mk);
+        }
+        __syncwarp();
+    };
+    // the listed components through shared memory; each(o) gets one component's slots in pairs.
+    // A list of one chunk that is still there (`staged`) is not loaded again.
+    auto for_listed = [&](bool staged, auto&& each) {
+        float4 next[COND_CHUNK / 4];   // the chunk after the one in shared memory
+        auto fetch = [&](int t0) {
+#pragma unroll
+            for (int i = 0; i < COND_CHUNK / 4; ++i) {
+                const int t = t0 + 4 * i + (lane >> 3);
+                if (t < nl)
+                    next[i] = __ldg(reinterpret_cast<const float4*>(prep + (size_t)list[t] * COND_FLOATS) + (lane & 7));
+            }
+        };
+        const int total = nl;
+        if (!staged) fetch(0);
+        for (int t0 = 0; t0 < total; t0 += COND_CHUNK) {
+            const int cnt = min(COND_CHUNK, total - t0);
+            if (!staged) {
+                __syncwarp();
+#pragma unroll
+                for (int i = 0; i < COND_CHUNK / 4; ++i) s_rec[warp][4 * i + (lane >> 3)][lane & 7] = next[i];
+                fetch(t0 + COND_CHUNK);
+                __syncwarp();
+            }
+#pragma unroll 2
+            for (int t = 0; t < cnt; ++t) {
+                float2 o[16];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const float4 q = s_rec[warp][t][i];
+                    o[2 * i] = f2(q.x, q.y);
+                    o[2 * i + 1] = f2(q.z, q.w);
+                }
+                each(o, t0 + t);
+            }
+        }
+    };
+    float2 X[3];   // locations of blocks 0, 1
+#pragma unroll
+    for (int j = 0; j < 3; ++j) X[j] = f2(x[0][j], x[1][j]);
     // log-weights and regression means of component o at two locations (every operation rounds
     // as the scalar one)
-    auto eval = [&](const float2 (&o)[15], const float2 (&Xq)[3], float2& mb) {
-        const float2 d0 = add2(Xq[0], o[11]), d1 = add2(Xq[1], o[12]), d2 = add2(Xq[2], o[13]);
+    auto eval = [&](const float2 (&o)[16], float2& mb) {
+        const float2 d0 = add2(X[0], o[11]), d1 = add2(X[1], o[12]), d2 = add2(X[2], o[13]);
         const float2 y0 = mul2(o[0], d0);
         const float2 y1 = fma2(o[2], d1, mul2(o[1], d0));
         const float2 y2 = fma2(o[5], d2, fma2(o[4], d1, mul2(o[3], d0)));
         mb = fma2(o[8], d2, fma2(o[7], d1, fma2(o[6], d0, o[14])));
         return fma2(dup(-0.5f), fma2(y2, y2, fma2(y1, y1, mul2(y0, y0))), o[10]);
     };
-    auto load = [&](int b, float2 (&o)[15]) {
-        const float4* p = reinterpret_cast<const float4*>(prep + (size_t)b * COND_FLOATS);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const float4 v = __ldg(p + i);
-            o[2 * i < 15 ? 2 * i : 14] = f2(v.x, v.y);
-            if (2 * i + 1 < 15) o[2 * i + 1] = f2(v.z, v.w);
-        }
-    };
-    // ---- L of each block
-    float L[4];
-    {
-        float bestv[4];
-        int bestb[4];
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            bestv[r] = -INFINITY;
-            bestb[r] = 0;
-        }
-        for (int b = lane; b < k; b += 32) {
-            float2 o[15];
-            load(b, o);
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                float2 C[3], mb;
-#pragma unroll
-                for (int j = 0; j < 3; ++j)
-                    C[j] = f2(0.5f * (lo[2 * q][j] + hi[2 * q][j]), 0.5f * (lo[2 * q + 1][j] + hi[2 * q + 1][j]));
-                const float2 lw = eval(o, C, mb);
-                if (lw.x > bestv[2 * q]) { bestv[2 * q] = lw.x; bestb[2 * q] = b; }
-                if (lw.y > bestv[2 * q + 1]) { bestv[2 * q + 1] = lw.y; bestb[2 * q + 1] = b; }
-            }
-        }
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const float v = __shfl_xor_sync(FULL, bestv[r], o);
-                const int b = __shfl_xor_sync(FULL, bestb[r], o);
-                if (v > bestv[r] || (v == bestv[r] && b < bestb[r])) {   // the same choice in every lane
-                    bestv[r] = v;
-                    bestb[r] = b;
-                }
-            }
-            float2 o[15], mb;
-            load(bestb[r], o);
-            const float2 Xr[3] = {dup(x[r][0]), dup(x[r][1]), dup(x[r][2])};
-            float lw = eval(o, Xr, mb).x;
-#pragma unroll
-            for (int o2 = 16; o2 > 0; o2 >>= 1) lw = fminf(lw, __shfl_xor_sync(FULL, lw, o2));
-            L[r] = lw;
-        }
-    }
-    // ---- the components of [b0, b1) that some block needs, in order, with the blocks' bits
-    int nl = 0;
-    auto make_list = [&](int b0, int b1) {
-        nl = 0;
-        for (int j0 = b0; j0 < b1; j0 += 32) {
-            const int b = j0 + lane;
-            unsigned bits = 0u;
-            if (b < b1) {
-                const float2* o = reinterpret_cast<const float2*>(prep + (size_t)b * COND_FLOATS);
-                float P[6], nm[3];
-#pragma unroll
-                for (int i = 0; i < 6; ++i) P[i] = slot(o, i).x;
-#pragma unroll
-                for (int i = 0; i < 3; ++i) nm[i] = slot(o, 11 + i).x;
-                const float c = slot(o, 10).x, n0 = slot(o, 15).x, n1 = slot(o, 16).x, n2 = slot(o, 17).x,
-                            s2 = slot(o, 18).x;
-#pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    float d[3], h[3], e2 = 0.f;
-#pragma unroll
-                    for (int j = 0; j < 3; ++j) {
-                        const float ctr = 0.5f * (lo[r][j] + hi[r][j]);
-                        h[j] = fmaxf(hi[r][j] - ctr, ctr - lo[r][j]);
-                        d[j] = ctr + nm[j];
-                        const float e = fmaxf(fabsf(d[j]) - h[j], 0.f);
-                        e2 = fmaf(e, e, e2);
-                    }
-                    const float y0 = P[0] * d[0], y1 = fmaf(P[2], d[1], P[1] * d[0]);
-                    const float y2 = fmaf(P[5], d[2], fmaf(P[4], d[1], P[3] * d[0]));
-                    const float yc = sqrtf(fmaf(y2, y2, fmaf(y1, y1, y0 * y0)));
-                    const float reach = fmaf(h[0], n0, fmaf(h[1], n1, h[2] * n2));
-                    const float t = fmaxf(yc * (1.f - 1.f / 256.f) - reach * (1.f + 1.f / 256.f), 0.f);
-                    const float q = fmaxf(t * t, s2 * e2 * (1.f - 1.f / 128.f));   // <= |P (x - mu)|^2 over the box
-                    if (!(fmaf(-0.5f, q, c) < L[r] - 106.f)) bits |= 1u << r;
-                }
-            }
-            const unsigned mk = __ballot_sync(FULL, bits != 0u);
-            if (bits) {
-                const int at = nl + __popc(mk & ((1u << lane) - 1u));
-                list[at] = (uint16_t)b;
-                need[at] = (uint8_t)bits;
-            }
-            nl += __popc(mk);
-        }
-        __syncwarp();
-    };
     const bool once = k <= COND_CAP;   // one list serves both passes
     if (once) make_list(0, k);
-    float2 mx[2] = {dup(-INFINITY), dup(-INFINITY)}, mref[2] = {dup(0.f), dup(0.f)};
+    const bool cut = once && nl > COND_CHUNK;   // a long list: pass 2 only visits what some location
+                                                // needs (one far location makes L low for its block)
+    int kept = 0;
+    float2 mx = dup(-INFINITY), mref = dup(0.f);
     for (int b0 = 0; b0 < k; b0 += COND_CAP) {
         if (!once) make_list(b0, min(k, b0 + COND_CAP));
-        for (int t = 0; t < nl; ++t) {
-            const unsigned bits = need[t];
-            float2 o[15];
-            load(list[t], o);
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                if (!((bits >> (2 * q)) & 3u)) continue;
-                float2 mb;
-                const float2 lw = eval(o, X[q], mb);
-                if (lw.x > mx[q].x) { mx[q].x = lw.x; mref[q].x = mb.x; }
-                if (lw.y > mx[q].y) { mx[q].y = lw.y; mref[q].y = mb.y; }
+        for_listed(false, [&](const float2 (&o)[16], int t) {
+            float2 mb;
+            const float2 lw = eval(o, mb);
+            if (lw.x > mx.x) { mx.x = lw.x; mref.x = mb.x; }
+            if (lw.y > mx.y) { mx.y = lw.y; mref.y = mb.y; }
+            if (cut) {   // kept <= t: only entries already fetched are overwritten
+                const bool want = !(lw.x < fmaxf(mx.x, known[0]) - 106.f) || !(lw.y < fmaxf(mx.y, known[1]) - 106.f);
+                if (__any_sync(FULL, want)) {
+                    const uint16_t b = list[t];
+                    __syncwarp();
+                    list[kept++] = b;
+                }
             }
-        }
-        __syncwarp();
+        });
     }
-    float2 s[2] = {dup(0.f), dup(0.f)}, e1[2] = {dup(0.f), dup(0.f)}, e2[2] = {dup(0.f), dup(0.f)};
+    if (cut) nl = kept;
+    float2 s = dup(0.f), e1 = dup(0.f), e2 = dup(0.f);
     for (int b0 = 0; b0 < k; b0 += COND_CAP) {
         if (!once) make_list(b0, min(k, b0 + COND_CAP));
-        for (int t = 0; t < nl; ++t) {
-            const unsigned bits = need[t];
-            float2 o[15];
-            load(list[t], o);
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                if (!((bits >> (2 * q)) & 3u)) continue;
-                float2 mb;
-                const float2 lw = eval(o, X[q], mb);
-                const float2 w = f2(__expf(lw.x - mx[q].x), __expf(lw.y - mx[q].y));
-                const float2 dm = f2(mb.x - mref[q].x, mb.y - mref[q].y);
-                s[q] = add2(s[q], w);
-                e1[q] = fma2(w, dm, e1[q]);
-                e2[q] = fma2(w, fma2(dm, dm, o[9]), e2[q]);
-            }
-        }
-        __syncwarp();
+        for_listed(once && !cut, [&](const float2 (&o)[16], int) {
+            float2 mb;
+            const float2 lw = eval(o, mb);
+            const float2 w = f2(__expf(lw.x - mx.x), __expf(lw.y - mx.y));
+            const float2 dm = f2(mb.x - mref.x, mb.y - mref.y);
+            s = add2(s, w);
+            e1 = fma2(w, dm, e1);
+            e2 = fma2(w, fma2(dm, dm, o[9]), e2);
+        });
     }
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        const int64_t i = base + 32 * r + lane;
-        if (i >= m) continue;
-        const float sr = r & 1 ? s[r >> 1].y : s[r >> 1].x;
+    for (int r = 0; r < 2; ++r) {
+        if (base + 32 * r + lane >= m) continue;
+        const int64_t i = order ? order[base + 32 * r + lane] : base + 32 * r + lane;
+        const float sr = r ? s.y : s.x;
         if (!(sr > 0.f)) {
             set_error(st, GIRA_ERR_NUMERIC);
             continue;
         }
-        const float inv = 1.f / sr, a = (r & 1 ? e1[r >> 1].y : e1[r >> 1].x) * inv;
-        cmean[i] = (r & 1 ? mref[r >> 1].y : mref[r >> 1].x) + a;
-        if (cvar) cvar[i] = fmaf(-a, a, (r & 1 ? e2[r >> 1].y : e2[r >> 1].x) * inv);
+        const float inv = 1.f / sr, a = (r ? e1.y : e1.x) * inv;
+        cmean[i] = (r ? mref.y : mref.x) + a;
+        if (cvar) cvar[i] = fmaf(-a, a, (r ? e2.y : e2.x) * inv);
     }
 }
 
@@ -1119,14 +1239,14 @@ cudaError_t launch_pack4(const float* pts4in, int64_t n, float4* pts4, float4* p
     return cudaGetLastError();
 }
 
-int cond_floats() { return COND_FLOATS; }
+int cond_floats() { return COND_ALL; }
 
-cudaError_t launch_conditional4(const float* locs, int64_t m, int k, const float* w, const float* mu,
+cudaError_t launch_conditional4(const float* locs, const int* order, int64_t m, int k, const float* w, const float* mu,
                                 const float* cov, float* prep, float* cmean, float* cvar, DeviceState* st,
                                 cudaStream_t s) {
     cond_prepare_kernel<<<(k + 63) / 64, 64, 0, s>>>(w, mu, cov, k, prep, st);
-    conditional4_kernel<<<(unsigned)((m + 128 * COND_WARPS - 1) / (128 * COND_WARPS)), 32 * COND_WARPS, cond_smem(),
-                          s>>>(locs, m, k, prep, cmean, cvar, st);
+    conditional4_kernel<<<(unsigned)((m + COND_LOCS * COND_WARPS - 1) / (COND_LOCS * COND_WARPS)), 32 * COND_WARPS, 0,
+                          s>>>(locs, order, m, k, prep, cmean, cvar, st);
     return cudaGetLastError();
 }
 

@@ -474,6 +474,12 @@ int64_t point_order_max_n();          // larger inputs keep the caller's order
 cudaError_t launch_point_order(const float4* p8, int64_t n, const int64_t* offsets_d, const int2* units_d,
                                int nunits, int batch, void* scratch, float4* p8_out, float4* p4_out, int* order_out,
                                cudaStream_t s);
+// The points of an n x 3 array cell by cell (a 32^3 grid over their bounding box, cells in
+// Morton order, no fixed order inside a cell): order.  For kernels whose result per point
+// does not depend on the order.  scratch: cell_group_scratch_bytes(n) bytes, n < 2^31.
+size_t cell_group_scratch_bytes(int64_t n);
+int cell_group_launches();
+cudaError_t launch_cell_group(const float* p3, int64_t n, void* scratch, int* order, cudaStream_t s);
 cudaError_t launch_fill_padding(float* params, int k, int npairs_pad, cudaStream_t s);
 // Sum of the per-CTA log-likelihoods into st->ll_sum (fixed order).
 cudaError_t launch_ll_reduce(const double* ll_partials, int grid, DeviceState* st, cudaStream_t s);
@@ -722,7 +728,9 @@ cudaError_t launch_label_stats4(const float4* pts4, int64_t n, int k, const int3
                                 double* stats64, DeviceState* st, cudaStream_t s);
 // Gaussian-mixture regression of the 4th coordinate on the first three.
 int cond_floats();
-cudaError_t launch_conditional4(const float* locs, int64_t m, int k, const float* w, const float* mu,
+// order (nullable): the order in which the kernel takes the locations (any permutation gives
+// the same results; one that keeps neighbours together is faster).
+cudaError_t launch_conditional4(const float* locs, const int* order, int64_t m, int k, const float* w, const float* mu,
                                 const float* cov, float* prep, float* cmean, float* cvar, DeviceState* st,
                                 cudaStream_t s);
 // m draws from a d-dimensional mixture (d = 3 or 4); cum: k doubles, chol: 16 k doubles.

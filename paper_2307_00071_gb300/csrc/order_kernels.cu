@@ -299,6 +299,95 @@ __global__ void __launch_bounds__(256) gather_kernel(const int* __restrict__ ord
     if (p4_out) p4_out[j] = make_float4(a.x, a.z, b.x, b.z);   // b.z: the fourth coordinate (0 in 3-D)
 }
 
+// ---- grouping by cell, where the order inside a cell does not matter (each point's result
+// is its own): cell = 15-bit Morton code (5 bits per axis of the bounding box), a point's
+// place in its cell by an atomic counter, one scan of the 32,768 counts.  Four short
+// kernels; the stable two-pass sort below takes ~100 us on a frame.
+constexpr int CELL_BINS = 1 << 15;
+__device__ __forceinline__ unsigned key_of(float f) {   // order-preserving unsigned
+    return (unsigned)ord_of(f) ^ 0x80000000u;
+}
+// box: [0..2] the smallest key per axis, [3..5] the smallest complemented key; all ones at start
+__global__ void __launch_bounds__(256) cell_box_kernel(const float* __restrict__ p3, int64_t n, unsigned* box) {
+    float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const float v = p3[3 * i + j];
+            lo[j] = fminf(lo[j], v);
+            hi[j] = fmaxf(hi[j], v);
+        }
+    __shared__ unsigned s_box[8][6];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        const unsigned a = __reduce_min_sync(FULL, key_of(lo[j])), b = __reduce_min_sync(FULL, ~key_of(hi[j]));
+        if ((threadIdx.x & 31) == 0) {
+            s_box[threadIdx.x >> 5][j] = a;
+            s_box[threadIdx.x >> 5][3 + j] = b;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < 6) {
+        unsigned a = s_box[0][threadIdx.x];
+        for (int w = 1; w < 8; ++w) a = min(a, s_box[w][threadIdx.x]);
+        atomicMin(box + threadIdx.x, a);
+    }
+}
+__global__ void __launch_bounds__(256) cell_key_kernel(const float* __restrict__ p3, int64_t n,
+                                                       const unsigned* __restrict__ box, int* hist, int* cell,
+                                                       int* rank) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int lane = threadIdx.x & 31;
+    int code = -1;
+    if (i < n) {
+        code = 0;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {   // fmaxf / fminf map a NaN to the bound
+            const float lo = float_of((int)(box[j] ^ 0x80000000u));
+            const float ext = float_of((int)(~box[3 + j] ^ 0x80000000u)) - lo;
+            const float scale = ext > 0.f ? 32.f / ext : 0.f;
+            code |= (int)(spread6((uint32_t)fminf(31.f, fmaxf(0.f, floorf((p3[3 * i + j] - lo) * scale)))) << j);
+        }
+    }
+    const unsigned peers = __match_any_sync(FULL, code);
+    const int lead = __ffs(peers) - 1;
+    int base = 0;
+    if (code >= 0 && lane == lead) base = atomicAdd(hist + code, __popc(peers));
+    base = __shfl_sync(FULL, base, lead);
+    if (code >= 0) {
+        cell[i] = code;
+        rank[i] = base + __popc(peers & ((1u << lane) - 1u));
+    }
+}
+__global__ void __launch_bounds__(1024) cell_scan_kernel(int* hist) {   // exclusive, in place, one block
+    __shared__ int s_warp[32];
+    int4 v[8];
+    int t = 0;
+    int4* h = reinterpret_cast<int4*>(hist) + 8 * threadIdx.x;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        v[q] = h[q];
+        t += v[q].x + v[q].y + v[q].z + v[q].w;
+    }
+    int run = block_exclusive_scan(t, s_warp, nullptr);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        int4 o;
+        o.x = run;
+        o.y = o.x + v[q].x;
+        o.z = o.y + v[q].y;
+        o.w = o.z + v[q].z;
+        run = o.w + v[q].w;
+        h[q] = o;
+    }
+}
+__global__ void __launch_bounds__(256) cell_place_kernel(int64_t n, const int* __restrict__ base,
+                                                         const int* __restrict__ cell, const int* __restrict__ rank,
+                                                         int* order) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) order[base[cell[i]] + rank[i]] = (int)i;
+}
+
 int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
 int radix_passes(int batch) {
@@ -325,6 +414,25 @@ int point_order_launches(int batch) { return 4 + 5 * radix_passes(batch); }   //
 
 // the largest n the scan's two levels hold (every tile's 512 digit counts)
 int64_t point_order_max_n() { return (int64_t)SCAN_PER_BLOCK * SCAN_PER_BLOCK / RADIX * TILE; }
+
+size_t cell_group_scratch_bytes(int64_t n) { return sizeof(int) * (CELL_BINS + 64 + 2 * (size_t)n); }
+int cell_group_launches() { return 4; }
+
+cudaError_t launch_cell_group(const float* p3, int64_t n, void* scratch, int* order, cudaStream_t s) {
+    if (n > INT32_MAX) return cudaErrorInvalidValue;
+    int* hist = static_cast<int*>(scratch);
+    unsigned* box = reinterpret_cast<unsigned*>(hist + CELL_BINS);
+    int *cell = hist + CELL_BINS + 64, *rank = cell + n;
+    cudaError_t e = cudaMemsetAsync(hist, 0, sizeof(int) * CELL_BINS, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(box, 0xff, sizeof(unsigned) * 6, s);
+    if (e != cudaSuccess) return e;
+    const unsigned blocks = (unsigned)ceil_div(n, 256);
+    cell_box_kernel<<<(unsigned)std::min<int64_t>(ceil_div(n, 1024), 304), 256, 0, s>>>(p3, n, box);
+    cell_key_kernel<<<blocks, 256, 0, s>>>(p3, n, box, hist, cell, rank);
+    cell_scan_kernel<<<1, 1024, 0, s>>>(hist);
+    cell_place_kernel<<<blocks, 256, 0, s>>>(n, hist, cell, rank, order);
+    return cudaGetLastError();
+}
 
 size_t point_order_scratch_bytes(int64_t n, int batch) {
     const int64_t ntiles = ceil_div(n, TILE);

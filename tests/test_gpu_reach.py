@@ -118,3 +118,33 @@ def test_4d_reach(gira, frame, n, k, off):
     ref = oracle.em(pts, w, m, c, iters=1, tol=0.0, reg=1e-6)
     assert abs(r["trace"][0] - ref["trace"][0]) <= LL_ABS + 1e-7 * abs(ref["trace"][0])
     assert_model_close((r["weights"], r["means"], r["covs"]), (ref["weights"], ref["means"], ref["covs"]))
+
+
+@pytest.mark.parametrize("m,k", [(8191, 37), (8192, 1), (8193, 640), (8449, 2101)])
+def test_regression_does_not_depend_on_the_order_of_the_locations(gira, frame, m, k):
+    """The regression visits only the components that can have nonzero weight, listed for 256 and
+    64 locations at a time (grouped by cell from 8,192 locations on, in rounds of 2,048 components).
+    A location's result is that of its own components in increasing order, so it is the same bits
+    in any order and in a call of a few locations; far locations make their neighbours' lists long.
+    Against the oracle: locations at the surface (log-weights of size ~100, rounded to ~1e-5 of
+    each weight), with the tolerances of the regression's own test."""
+    rng = np.random.default_rng(m)
+    pts4 = np.concatenate([frame, np.sin(3 * frame[:, :1])], 1).astype(np.float32)
+    w, mu, cov = ball_model(pts4, k, rng, d=4, sigma=0.1)
+    locs = frame[rng.choice(len(frame), m, replace=len(frame) < m)].astype(np.float32)
+    far = rng.choice(m, 40, replace=False)
+    locs[far] += rng.uniform(-30, 30, size=(40, 3)).astype(np.float32)
+    e, v = (to_np(a) for a in gira.gira_gmm_conditional4(locs, w, mu, cov))
+    p = rng.permutation(m)
+    ep, vp = (to_np(a) for a in gira.gira_gmm_conditional4(locs[p], w, mu, cov))
+    np.testing.assert_array_equal(ep, e[p])
+    np.testing.assert_array_equal(vp, v[p])
+    for a in (far[:7], np.arange(m - 300, m)):
+        ea, va = (to_np(t) for t in gira.gira_gmm_conditional4(locs[a], w, mu, cov))
+        np.testing.assert_array_equal(ea, e[a])
+        np.testing.assert_array_equal(va, v[a])
+    near = np.setdiff1d(np.arange(m), far)[:500]
+    near = near[np.min(np.linalg.norm(locs[near, None] - mu[None, :, :3], axis=2), axis=1) < 0.5]
+    re, rv = oracle.conditional4(locs[near], w, mu, cov)
+    np.testing.assert_allclose(e[near], re, rtol=0, atol=2e-4)
+    np.testing.assert_allclose(v[near], rv, rtol=2e-3, atol=2e-5)
