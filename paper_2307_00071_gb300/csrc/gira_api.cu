@@ -2155,7 +2155,7 @@ gira_status gira_gbms(const float* points, int64_t n, int d, double bandwidth, i
         int *idx, *idx2, *ulen, *ustart, *ints, *mcount, *rcount, *midx, *midx2, *mulen, *mustart, *state, *flags,
             *pos, *cout;
         double4 *modes64, *rmodes;
-        longlong2 *qxy, *qzw;
+        ulonglong2* table;
         double* mout;
         void* temp;
     } b{};
@@ -2172,8 +2172,7 @@ gira_status gira_gbms(const float* points, int64_t n, int d, double bandwidth, i
         b.ints = cv.take<int>(4);   // cells, live modes, mode cells, undecided
         b.modes64 = cv.take<double4>(n);
         b.rmodes = cv.take<double4>(n);
-        b.qxy = cv.take<longlong2>(n);
-        b.qzw = cv.take<longlong2>(n);
+        b.table = cv.take<ulonglong2>(gbms_table_slots(n));   // of the cells, then of the modes' cells
         b.mout = cv.take<double>((modes && km == Kind::Host) ? (size_t)d * n : 0);
         b.cout = cv.take<int>((counts && kq == Kind::Host) ? n : 0);
         b.temp = cv.take<unsigned char>(tb);
@@ -2215,10 +2214,13 @@ gira_status gira_gbms(const float* points, int64_t n, int d, double bandwidth, i
     TRY(device_status(h));
     const int S = hints[0];
     prof.t_init = prof.mark();
-    COUNTED(prof, 1, launch_gbms_gather(b.p4, b.idx2, n, b.spts, b.qxy, b.qzw, c.s));
-    COUNTED(prof, 1, launch_gbms_shift(b.spts, b.qxy, b.qzw, b.ukeys, b.ustart, b.ulen, S, d, bandwidth, max_iter,
+    COUNTED(prof, 1, launch_gbms_gather(b.p4, b.idx2, n, b.spts, c.s));
+    COUNTED(prof, 1, launch_gbms_table(b.ukeys, b.ustart, b.ulen, ncells, S, b.table, c.s));
+    float4* boxes = b.p4;   // read for the last time by the gather
+    COUNTED(prof, 1, launch_gbms_boxes(b.spts, b.ustart, b.ulen, S, boxes, c.s));
+    COUNTED(prof, 1, launch_gbms_shift(b.spts, boxes, b.ukeys, b.table, n, S, d, bandwidth, max_iter,
                                        b.modes64, b.mcount, b.st, c.s));
-    COUNTED(prof, 2, launch_gbms_rank(b.temp, tb, b.mcount, S, b.rkeys, b.rkeys2, nlive, c.s));
+    COUNTED(prof, 2, launch_gbms_rank(b.temp, tb, b.mcount, n, S, b.rkeys, b.rkeys2, nlive, c.s));
     GIRA_CUDA(cudaMemcpyAsync(hints, b.ints, sizeof hints, cudaMemcpyDeviceToHost, c.s));
     GIRA_CUDA(cudaStreamSynchronize(c.s));
     const int L = hints[1];
@@ -2228,14 +2230,15 @@ gira_status gira_gbms(const float* points, int64_t n, int d, double bandwidth, i
                                                 b.rcount, b.mkeys, b.midx, b.state, b.st, c.s));
         COUNTED(prof, 3, gbms_sort_cells(b.temp, tb, b.mkeys, b.mkeys2, b.midx, b.midx2, L, d, b.mukeys, b.mulen,
                                          b.mustart, mncells, c.s));
+        COUNTED(prof, 1, launch_gbms_table(b.mukeys, b.mustart, b.mulen, mncells, L, b.table, c.s));
         // every round decides at least the lowest undecided rank: at most L rounds
         for (int round = 0; round < L; round += 2) {
             GIRA_CUDA(cudaMemsetAsync(undecided, 0, sizeof(int), c.s));
-            COUNTED(prof, 1, launch_gbms_merge_round(b.rmodes, nlive, L, b.mukeys, b.mustart, b.mulen, mncells,
-                                                     b.midx2, d, bandwidth, b.state, undecided, c.s));
+            COUNTED(prof, 1, launch_gbms_merge_round(b.rmodes, nlive, L, b.table, b.midx2, d, bandwidth,
+                                                     b.state, undecided, c.s));
             GIRA_CUDA(cudaMemsetAsync(undecided, 0, sizeof(int), c.s));
-            COUNTED(prof, 1, launch_gbms_merge_round(b.rmodes, nlive, L, b.mukeys, b.mustart, b.mulen, mncells,
-                                                     b.midx2, d, bandwidth, b.state, undecided, c.s));
+            COUNTED(prof, 1, launch_gbms_merge_round(b.rmodes, nlive, L, b.table, b.midx2, d, bandwidth,
+                                                     b.state, undecided, c.s));
             int open = 0;
             GIRA_CUDA(cudaMemcpyAsync(&open, undecided, sizeof(int), cudaMemcpyDeviceToHost, c.s));
             GIRA_CUDA(cudaStreamSynchronize(c.s));

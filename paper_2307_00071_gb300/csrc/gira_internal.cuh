@@ -749,16 +749,25 @@ cudaError_t launch_gbms_keys(const float* pts, int64_t n, int d, double h, float
 cudaError_t gbms_sort_cells(void* temp, size_t temp_bytes, const uint64_t* keys_in, uint64_t* keys_out,
                             const int* idx_in, int* idx_out, int64_t n, int d, uint64_t* ukeys, int* ulen,
                             int* ustart, int* ncells, cudaStream_t s);
-// Points in cell order, with their fixed-point coordinates (x, y) and (z, w).
-cudaError_t launch_gbms_gather(const float4* pts4, const int* idx, int64_t n, float4* spts, longlong2* qxy,
-                               longlong2* qzw, cudaStream_t s);
-// One CTA per seed (cell): the seed's moves; modes[s] and counts[s] (0: dropped).
-cudaError_t launch_gbms_shift(const float4* spts, const longlong2* qxy, const longlong2* qzw, const uint64_t* ukeys,
-                              const int* ustart, const int* ulen, int ncells, int d, double h, int max_iter,
+// Points in cell order.
+cudaError_t launch_gbms_gather(const float4* pts4, const int* idx, int64_t n, float4* spts, cudaStream_t s);
+// Hash table of the *ncells <= nmax cells (key, length << 32 | start): gbms_table_slots(nmax)
+// slots.
+unsigned gbms_table_slots(int64_t nmax);
+cudaError_t launch_gbms_table(const uint64_t* ukeys, const int* ustart, const int* ulen, const int* ncells, int nmax,
+                              ulonglong2* table, cudaStream_t s);
+// The box of each cell's points at boxes[start], boxes[start + 1] (n entries; cells of one
+// point have none).
+cudaError_t launch_gbms_boxes(const float4* spts, const int* ustart, const int* ulen, int ncells, float4* boxes,
+                              cudaStream_t s);
+// One CTA per seed (cell): the seed's moves; modes[s] and counts[s] (0: dropped).  table: of
+// nmax = ncells cells.
+cudaError_t launch_gbms_shift(const float4* spts, const float4* boxes, const uint64_t* ukeys,
+                              const ulonglong2* table, int64_t n, int ncells, int d, double h, int max_iter,
                               double4* modes, int* counts, const DeviceState* st, cudaStream_t s);
-// Rank keys of the ns seeds and their sort; *nlive (device, zeroed by the caller)
+// Rank keys of the ns seeds (of n points) and their sort; *nlive (device, zeroed by the caller)
 // receives the number of live modes.
-cudaError_t launch_gbms_rank(void* temp, size_t temp_bytes, const int* counts, int ns, uint64_t* rkeys,
+cudaError_t launch_gbms_rank(void* temp, size_t temp_bytes, const int* counts, int64_t n, int ns, uint64_t* rkeys,
                              uint64_t* rkeys_sorted, int* nlive, cudaStream_t s);
 // Live modes in rank order (rmodes, rcount), their cell keys and rank indices for
 // the merge grid, and the merge state (undecided).
@@ -766,9 +775,9 @@ cudaError_t launch_gbms_rank_modes(const uint64_t* rkeys_sorted, const int* nliv
                                    const int* counts, int d, double h, double4* rmodes, int* rcount, uint64_t* mkeys,
                                    int* midx, int* state, DeviceState* st, cudaStream_t s);
 // One merge round; *undecided (zeroed by the caller) counts ranks still open.
-cudaError_t launch_gbms_merge_round(const double4* rmodes, const int* nlive, int nmax, const uint64_t* mukeys,
-                                    const int* mustart, const int* mulen, const int* mncells, const int* midx_sorted,
-                                    int d, double h, int* state, int* undecided, cudaStream_t s);
+cudaError_t launch_gbms_merge_round(const double4* rmodes, const int* nlive, int nmax, const ulonglong2* table,
+                                    const int* midx_sorted, int d, double h, int* state, int* undecided,
+                                    cudaStream_t s);
 // Kept modes in rank order -> modes_out (k x d binary64) and counts_out (nullable);
 // pos[r] is the output slot of rank r (exclusive sum of the kept flags).
 cudaError_t launch_gbms_output(void* temp, size_t temp_bytes, const int* state, const int* nlive, int nmax,

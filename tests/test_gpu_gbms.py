@@ -103,3 +103,34 @@ def test_errors(gira):
     with pytest.raises(gira.GiraError) as e:
         gira.gira_gbms(far, 1.0)
     assert e.value.status == gira.ERR_INVALID_ARG
+
+
+def flat_patch(rng, n, d):
+    p = np.zeros((n, d))
+    p[:, :2] = rng.random((n, 2))
+    p[:, 2:] = 0.3 * p[:, :1] + rng.normal(scale=0.003, size=(n, d - 2))
+    return p
+
+
+@pytest.mark.parametrize("d,shape,offset", [
+    (3, "patch", 0.0),            # over 64 points per cell on average, thousands of candidates per seed
+    (4, "patch", -4090.0),        # coordinates at the limit of the cell grid's range
+    (3, "patch+sparse", 0.0),     # the same candidates, but fewer points per cell on average
+    (4, "patch+sparse", 63.5),    # across the power of two where binary32 changes its spacing
+    (3, "ring", 0.0),             # thousands of points as far as the bandwidth from the seeds between them
+])
+def test_dense_flat_parts_bit_exact(gira, d, shape, offset):
+    """Seeds among more candidate points than fit in shared memory, that move many times: the sums
+    of the points that stay in the ball are kept while the seed is near the place they were taken
+    at, and only the shell is swept.  All in exact integers: the oracle's bits."""
+    rng = np.random.default_rng(d)
+    h = 0.15
+    if shape == "ring":
+        a, r = rng.uniform(0, 2 * np.pi, 9000), rng.normal(1.0, 0.04, 9000) * h
+        pts = np.stack([r * np.cos(a), r * np.sin(a), rng.normal(scale=0.01, size=9000)], 1)
+        pts = np.concatenate([pts, [0.3 * h, 0, 0] + rng.normal(scale=0.3 * h, size=(400, 3))])
+    else:
+        pts = flat_patch(rng, 16_000, d)
+        if shape == "patch+sparse":
+            pts = np.concatenate([pts, rng.uniform(-2, 2, size=(3000, d))])
+    check_equal(gira, (pts + offset).astype(np.float32), h)
