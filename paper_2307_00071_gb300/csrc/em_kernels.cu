@@ -580,17 +580,28 @@ int estep_pt_blocks() { return PT_B; }
 
 // ------------------------------------------------------------------ pack + padding
 namespace {
-__global__ void pack_kernel(const float* __restrict__ p3, int64_t n, float4* __restrict__ p4,
-                            float4* __restrict__ p8, DeviceState* st) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    float x = p3[3 * i], y = p3[3 * i + 1], z = p3[3 * i + 2];
-    if (!(isfinite(x) && isfinite(y) && isfinite(z))) set_error(st, GIRA_ERR_NONFINITE_INPUT);
+// Point i, packed; returns whether it is finite.
+__device__ __forceinline__ bool pack_point(const float* __restrict__ p3, int64_t i, float4* __restrict__ p4,
+                                           float4* __restrict__ p8) {
+    const float x = p3[3 * i], y = p3[3 * i + 1], z = p3[3 * i + 2];
     if (p4) p4[i] = make_float4(x, y, z, 0.f);
     if (p8) {
         p8[2 * i] = make_float4(x, x, y, y);
         p8[2 * i + 1] = make_float4(z, z, 0.f, 0.f);
     }
+    return isfinite(x) && isfinite(y) && isfinite(z);
+}
+
+__global__ void pack_kernel(const float* __restrict__ p3, int64_t n, float4* __restrict__ p4,
+                            float4* __restrict__ p8, DeviceState* st) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n && !pack_point(p3, i, p4, p8)) set_error(st, GIRA_ERR_NONFINITE_INPUT);
+}
+
+__device__ __forceinline__ void pad_slot(float* params, int b) {
+    float* base = params + (size_t)(b >> 1) * PAIR_FLOATS + (b & 1);
+    for (int s = 0; s < PAIR_FLOATS / 2; ++s) base[2 * s] = 0.f;
+    base[2 * SLOT_C] = -INFINITY;
 }
 
 // One block per instance: the padding component slots k .. 2 * npairs - 1 of its block.
@@ -598,19 +609,13 @@ __global__ void fill_padding_batched_kernel(float* params, const BatchInst* __re
                                             const int* __restrict__ npairs_of) {
     const BatchInst I = insts[blockIdx.x];
     const int slots = 2 * npairs_of[blockIdx.x];
-    for (int b = I.k + threadIdx.x; b < slots; b += blockDim.x) {
-        float* base = params + I.par_off + (size_t)(b >> 1) * PAIR_FLOATS + (b & 1);
-        for (int s = 0; s < PAIR_FLOATS / 2; ++s) base[2 * s] = 0.f;
-        base[2 * SLOT_C] = -INFINITY;
-    }
+    for (int b = I.k + threadIdx.x; b < slots; b += blockDim.x) pad_slot(params + I.par_off, b);
 }
 
 __global__ void fill_padding_kernel(float* params, int k, int npairs_pad) {
     int b = blockIdx.x * blockDim.x + threadIdx.x;   // component slot
     if (b >= 2 * npairs_pad || b < k) return;
-    float* base = params + (size_t)(b >> 1) * PAIR_FLOATS + (b & 1);
-    for (int s = 0; s < PAIR_FLOATS / 2; ++s) base[2 * s] = 0.f;
-    base[2 * SLOT_C] = -INFINITY;
+    pad_slot(params, b);
 }
 }  // namespace
 
@@ -656,28 +661,41 @@ cudaError_t launch_fill_padding(float* params, int k, int npairs_pad, cudaStream
 
 // ------------------------------------------------------------------ log-likelihood reduce
 namespace {
-__global__ void ll_reduce_batched_kernel(const double* __restrict__ llp, const BatchInst* __restrict__ insts,
-                                         DeviceState* states) {
-    const BatchInst I = insts[blockIdx.x];
+// The sum of n partials by one block, in an order that depends on n alone (a fit and a batch
+// give the same bits); valid in thread 0.  1,080 partials: 6.2 us by one warp, 4.5 us by eight.
+constexpr int LLR_THREADS = 256;
+__device__ double ll_block_sum(const double* __restrict__ llp, int n) {
+    __shared__ double s_w[LLR_THREADS / 32];
     double v = 0.0;
-    for (int c = threadIdx.x; c < I.ctas; c += 32) v += llp[I.ll_off + c];
+    for (int c = threadIdx.x; c < n; c += LLR_THREADS) v += llp[c];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
+    if ((threadIdx.x & 31) == 0) s_w[threadIdx.x >> 5] = v;
+    __syncthreads();
+    v = s_w[0];
+    if (threadIdx.x == 0)
+        for (int w = 1; w < LLR_THREADS / 32; ++w) v += s_w[w];
+    return v;
+}
+
+__global__ void __launch_bounds__(LLR_THREADS) ll_reduce_batched_kernel(const double* __restrict__ llp,
+                                                                        const BatchInst* __restrict__ insts,
+                                                                        DeviceState* states) {
+    const BatchInst I = insts[blockIdx.x];
+    const double v = ll_block_sum(llp + I.ll_off, I.ctas);
     if (threadIdx.x == 0) states[blockIdx.x].ll_sum = v;
 }
 
-__global__ void ll_reduce_kernel(const double* __restrict__ llp, int grid, DeviceState* st) {
-    if (st->error) return;
-    double v = 0.0;
-    for (int c = threadIdx.x; c < grid; c += 32) v += llp[c];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
+__global__ void __launch_bounds__(LLR_THREADS) ll_reduce_kernel(const double* __restrict__ llp, int grid,
+                                                                DeviceState* st) {
+    if (st->error) return;   // uniform: nothing sets it now
+    const double v = ll_block_sum(llp, grid);
     if (threadIdx.x == 0) st->ll_sum = v;
 }
 }  // namespace
 
 cudaError_t launch_ll_reduce(const double* ll_partials, int grid, DeviceState* st, cudaStream_t s) {
-    ll_reduce_kernel<<<1, 32, 0, s>>>(ll_partials, grid, st);
+    ll_reduce_kernel<<<1, LLR_THREADS, 0, s>>>(ll_partials, grid, st);
     return cudaGetLastError();
 }
 
@@ -1273,10 +1291,30 @@ __global__ void __launch_bounds__(FIN_THREADS) reduce_finalize_batched_kernel(co
     reduce_finalize_body(f, bi.y);
 }
 
-__global__ void params_from_model_kernel(const float* __restrict__ w, const float* __restrict__ mu,
-                                         const float* __restrict__ cov, int k, double* model64, float* params,
-                                         float4* shift4, DeviceState* st) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
+// What a given model and its points need before the E-step, in one launch: the first nbuild
+// blocks build 32 components each (a binary64 chain per lane, the launch's time) and fill the
+// padding slots, the others pack the points meanwhile.  A non-finite point is reported before
+// anything wrong with the model, whichever block finds what first.
+// Measured: 276,347 points, K = 1023: 7.0 + 2.1 + 5.2 us in three launches, 8.2 us in one.
+constexpr int MP_THREADS = 256;
+__global__ void __launch_bounds__(MP_THREADS) model_points_kernel(const float* __restrict__ p3, int64_t n,
+                                                                  float4* __restrict__ p8,
+                                                                  const float* __restrict__ w,
+                                                                  const float* __restrict__ mu,
+                                                                  const float* __restrict__ cov, int k, int slots,
+                                                                  int nbuild, double* model64, float* params,
+                                                                  float4* shift4, DeviceState* st) {
+    if ((int)blockIdx.x >= nbuild) {
+        const int64_t i = (int64_t)(blockIdx.x - nbuild) * MP_THREADS + threadIdx.x;
+        if (i < n && !pack_point(p3, i, nullptr, p8)) atomicExch(&st->error, GIRA_ERR_NONFINITE_INPUT);
+        return;
+    }
+    if (threadIdx.x >= 32) {
+        for (int b = k + blockIdx.x * (MP_THREADS - 32) + threadIdx.x - 32; b < slots; b += nbuild * (MP_THREADS - 32))
+            pad_slot(params, b);
+        return;
+    }
+    const int b = blockIdx.x * 32 + threadIdx.x;
     if (b >= k) return;
     const double pi = w[b];
     const double m[3] = {mu[3 * b], mu[3 * b + 1], mu[3 * b + 2]};
@@ -1734,13 +1772,16 @@ cudaError_t launch_model_out_batched(const double* model64, const BatchInst* ins
 
 cudaError_t launch_ll_reduce_batched(const double* ll_partials, const BatchInst* insts, int batch,
                                      DeviceState* states, cudaStream_t s) {
-    ll_reduce_batched_kernel<<<batch, 32, 0, s>>>(ll_partials, insts, states);
+    ll_reduce_batched_kernel<<<batch, LLR_THREADS, 0, s>>>(ll_partials, insts, states);
     return cudaGetLastError();
 }
 
-cudaError_t launch_params_from_model(const float* w, const float* mu, const float* cov, int k, double* model64,
-                                     float* params, float4* shift4, DeviceState* st, cudaStream_t s) {
-    params_from_model_kernel<<<(k + 63) / 64, 64, 0, s>>>(w, mu, cov, k, model64, params, shift4, st);
+cudaError_t launch_model_points(const float* pts3, int64_t n, float4* pts8, const float* w, const float* mu,
+                                const float* cov, int k, int npairs_pad, double* model64, float* params,
+                                float4* shift4, DeviceState* st, cudaStream_t s) {
+    const int nbuild = (k + 31) / 32;
+    model_points_kernel<<<(unsigned)(nbuild + (n + MP_THREADS - 1) / MP_THREADS), MP_THREADS, 0, s>>>(
+        pts3, n, pts8, w, mu, cov, k, 2 * npairs_pad, nbuild, model64, params, shift4, st);
     return cudaGetLastError();
 }
 

@@ -664,15 +664,24 @@ gira_status gira_gmm_fit(const float* points, int64_t n, int k, const gira_fit_o
         GIRA_CUDA(cudaMemcpyAsync(b.pin, points, sizeof(float) * 3 * n, cudaMemcpyHostToDevice, c.s));
         pts = b.pin;
     }
-    COUNTED(prof, 1, launch_pack(pts, n, kinit ? b.p4 : nullptr, b.p8, b.st, c.s));
-    if (sorted)
-        COUNTED(prof, point_order_launches(1),
-                launch_point_order(b.p8, n, nullptr, nullptr, 0, 1, b.osc, b.p8s, kinit ? b.p4s : nullptr, nullptr, c.s));
-    COUNTED(prof, 1, launch_fill_padding(b.params, k, npairs, c.s));
-
     float* w_d = (kw == Kind::Device) ? weights : b.mw;
     float* mu_d = (km == Kind::Device) ? means : b.mmu;
     float* cov_d = (kc == Kind::Device) ? covs : b.mcov;
+    if (kinit) {
+        COUNTED(prof, 1, launch_pack(pts, n, b.p4, b.p8, b.st, c.s));
+        COUNTED(prof, 1, launch_fill_padding(b.params, k, npairs, c.s));
+    } else {
+        if (kw == Kind::Host) GIRA_CUDA(cudaMemcpyAsync(b.mw, weights, sizeof(float) * k, cudaMemcpyHostToDevice, c.s));
+        if (km == Kind::Host)
+            GIRA_CUDA(cudaMemcpyAsync(b.mmu, means, sizeof(float) * 3 * k, cudaMemcpyHostToDevice, c.s));
+        if (kc == Kind::Host)
+            GIRA_CUDA(cudaMemcpyAsync(b.mcov, covs, sizeof(float) * 9 * k, cudaMemcpyHostToDevice, c.s));
+        COUNTED(prof, 1, launch_model_points(pts, n, b.p8, w_d, mu_d, cov_d, k, npairs, b.model64, b.params, b.shift4,
+                                             b.st, c.s));
+    }
+    if (sorted)
+        COUNTED(prof, point_order_launches(1),
+                launch_point_order(b.p8, n, nullptr, nullptr, 0, 1, b.osc, b.p8s, kinit ? b.p4s : nullptr, nullptr, c.s));
     if (kinit) {
         TRY(seed_centres(prof, c, b.p4, n, 3, k, o.seed, b.c4, b.ch, b.d2, b.bs, b.ksync, b.ksums, kgrid, b.st));
         GIRA_CUDA(cudaMemsetAsync(b.sums, 0, sizeof(double) * 4 * k, c.s));
@@ -684,13 +693,6 @@ gira_status gira_gmm_fit(const float* points, int64_t n, int k, const gira_fit_o
         GIRA_CUDA(cudaMemcpyAsync(b.shift4, b.c4, sizeof(float4) * k, cudaMemcpyDeviceToDevice, c.s));
         COUNTED(prof, 1, launch_reduce_finalize(nullptr, 0, nullptr, b.stats64, b.shift4, k, n, o.reg_covar, o.tol,
                                                 b.model64, b.params, b.trace, b.st, 0, false, c.s));
-    } else {
-        if (kw == Kind::Host) GIRA_CUDA(cudaMemcpyAsync(b.mw, weights, sizeof(float) * k, cudaMemcpyHostToDevice, c.s));
-        if (km == Kind::Host)
-            GIRA_CUDA(cudaMemcpyAsync(b.mmu, means, sizeof(float) * 3 * k, cudaMemcpyHostToDevice, c.s));
-        if (kc == Kind::Host)
-            GIRA_CUDA(cudaMemcpyAsync(b.mcov, covs, sizeof(float) * 9 * k, cudaMemcpyHostToDevice, c.s));
-        COUNTED(prof, 1, launch_params_from_model(w_d, mu_d, cov_d, k, b.model64, b.params, b.shift4, b.st, c.s));
     }
     // the EM runs with the components along a space-filling curve of their means
     // (the E-step then skips the many point-component pairs out of reach);
@@ -838,10 +840,9 @@ gira_status gira_gmm_loglik(const float* points, int64_t n, int k, const float* 
         GIRA_CUDA(cudaMemcpyAsync(b.mcov, covs, sizeof(float) * 9 * k, cudaMemcpyHostToDevice, c.s));
         cov_d = b.mcov;
     }
-    COUNTED(prof, 1, launch_pack(pts, n, nullptr, b.p8, b.st, c.s));
     float* ppd = per_point ? ((kpp == Kind::Device) ? per_point : b.pp) : nullptr;
-    COUNTED(prof, 1, launch_fill_padding(b.params, k, npairs, c.s));
-    COUNTED(prof, 1, launch_params_from_model(w_d, mu_d, cov_d, k, b.model64, b.params, b.shift4, b.st, c.s));
+    COUNTED(prof, 1, launch_model_points(pts, n, b.p8, w_d, mu_d, cov_d, k, npairs, b.model64, b.params, b.shift4,
+                                         b.st, c.s));
     prof.t_init = prof.mark();
     prof.t_em = prof.t_init;
     if (large) {

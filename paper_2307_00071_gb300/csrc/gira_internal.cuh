@@ -506,8 +506,9 @@ cudaError_t launch_estep_pt(const EStepLaunch& a, bool stats, int grid, cudaStre
 cudaError_t launch_estep_pt_units(const EStepLaunch& a, bool stats, int nunits, int kmax, cudaStream_t s);
 int estep_pt_points();   // points per CTA
 int estep_pt_blocks();   // point blocks per CTA (partial and mask rows per CTA)
-cudaError_t launch_params_from_model(const float* w, const float* mu, const float* cov, int k, double* model64,
-                                     float* params, float4* shift4, DeviceState* st, cudaStream_t s);
+cudaError_t launch_model_points(const float* pts3, int64_t n, float4* pts8, const float* w, const float* mu,
+                                const float* cov, int k, int npairs_pad, double* model64, float* params,
+                                float4* shift4, DeviceState* st, cudaStream_t s);
 // perm (nullable): slot s of model64 is the caller's component perm[s].
 cudaError_t launch_model_out(const double* model64, int k, float* w, float* mu, float* cov, const DeviceState* st,
                              cudaStream_t s, const int* perm = nullptr);
