@@ -1132,9 +1132,87 @@ __device__ void finalize_update_warp(const FinArgs& f, int b0, int nb, float pre
     }
 }
 
+// The same for one component by one lane: every entry by the same sequence of operations, so
+// the same bits.  A lane's chain is longer (8 us), but a binary64 instruction serves 32
+// components where the half-warps above serve two.
+__device__ void finalize_update_lane(const FinArgs& f, int b, bool white, const double* __restrict__ stats) {
+    double S[NSTAT];
+#pragma unroll
+    for (int i = 0; i < NSTAT; ++i) S[i] = stats[i];
+    float* base = f.params + (size_t)(b >> 1) * PAIR_FLOATS + (b & 1);
+    const float4 sh = f.shift4[b];
+    const double s0[3] = {(double)sh.x, (double)sh.y, (double)sh.z};
+    const double nbw = __dadd_rn(S[0], 10.0 * DBL_EPSILON);
+    const double inv = __drcp_rn(nbw);
+    double M[3][3] = {{1.0, 0.0, 0.0}, {0.0, 1.0, 0.0}, {0.0, 0.0, 1.0}};
+    if (white) {
+        double q[6];
+#pragma unroll
+        for (int l = 0; l < 6; ++l) q[l] = (double)base[2 * (SLOT_P + l)];
+        const double r0 = __drcp_rn(q[0]), r1 = __drcp_rn(q[2]), r2 = __drcp_rn(q[5]);
+        M[0][0] = r0;
+        M[1][1] = r1;
+        M[2][2] = r2;
+        M[1][0] = __dmul_rn(__dmul_rn(dneg(q[1]), r0), r1);
+        M[2][1] = __dmul_rn(__dmul_rn(dneg(q[4]), r1), r2);
+        M[2][0] = __dmul_rn(__fma_rn(q[4], M[1][0], __dmul_rn(q[3], r0)), dneg(r2));
+    }
+    double vb[3], C[3][3], mu[3], MC[3][3], c[6];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) vb[i] = __dmul_rn(S[1 + i], inv);
+#pragma unroll
+    for (int l = 0; l < 6; ++l) {
+        const int i = l < 3 ? 0 : (l < 5 ? 1 : 2), j = l < 3 ? l : (l < 5 ? l - 2 : 2);
+        C[i][j] = C[j][i] = __fma_rn(dneg(vb[i]), vb[j], __dmul_rn(S[4 + l], inv));
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        mu[i] = __fma_rn(M[i][2], vb[2], __fma_rn(M[i][1], vb[1], __fma_rn(M[i][0], vb[0], s0[i])));
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+            MC[i][j] = __fma_rn(M[i][2], C[2][j], __fma_rn(M[i][1], C[1][j], __fma_rn(M[i][0], C[0][j], 0.0)));
+    }
+#pragma unroll
+    for (int l = 0; l < 6; ++l) {
+        const int i = l < 3 ? 0 : (l < 5 ? 1 : 2), j = l < 3 ? l : (l < 5 ? l - 2 : 2);
+        c[l] = __fma_rn(MC[i][2], M[j][2], __fma_rn(MC[i][1], M[j][1],
+                                                    __fma_rn(MC[i][0], M[j][0], i == j ? f.reg : 0.0)));
+    }
+    const CholInv k = chol_inv(c);
+    if (!k.pd) {
+        atomicMin(&f.st->bad_component, f.perm ? f.perm[b] : b);
+        set_error(f.st, GIRA_ERR_NOT_PD);
+        return;
+    }
+    double* m = f.model64 + (size_t)b * MODEL;
+    m[0] = nbw;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) m[1 + i] = mu[i];
+#pragma unroll
+    for (int l = 0; l < 6; ++l) m[4 + l] = c[l];
+    double q[6];
+#pragma unroll
+    for (int l = 0; l < 6; ++l) {
+        q[l] = chol_q(k, l);
+        base[2 * (SLOT_P + l)] = (float)q[l];
+    }
+    base[2 * SLOT_B] = (float)bias_row(q[0], 0.0, 0.0, mu);
+    base[2 * (SLOT_B + 1)] = (float)bias_row(q[1], q[2], 0.0, mu);
+    base[2 * (SLOT_B + 2)] = (float)bias_row(q[3], q[4], q[5], mu);
+    base[2 * SLOT_C] = log2_norm(nbw, k);
+    const float m32[3] = {(float)mu[0], (float)mu[1], (float)mu[2]};
+#pragma unroll
+    for (int i = 0; i < 3; ++i) base[2 * (SLOT_NMU + i)] = -m32[i];
+    base[2 * SLOT_W] = (float)nbw;
+    const float c32[6] = {(float)c[0], (float)c[1], (float)c[2], (float)c[3], (float)c[4], (float)c[5]};
+    base[2 * SLOT_S] = sigma_min_sq_bound(c32);
+    f.shift4[b] = make_float4(m32[0], m32[1], m32[2], 0.f);
+}
+
 // Components blk * FIN_CPB .. of one fit; block index blk == 0 also does the
 // log-likelihood, trace and convergence of an EM iteration.
-__device__ void reduce_finalize_body(const FinArgs& f, int blk) {
+// sums != nullptr: only the statistics' sums, to sums[component][NSTAT].
+__device__ void reduce_finalize_body(const FinArgs& f, int blk, double* sums = nullptr) {
     __shared__ double W[FIN_CPB][FW];
     __shared__ float F[FIN_CPB][FF];
     __shared__ int s_skip;
@@ -1165,7 +1243,9 @@ __device__ void reduce_finalize_body(const FinArgs& f, int blk) {
         if (t < nout) W[t / NSTAT][W_S + t % NSTAT] = f.stats64[(size_t)b0 * NSTAT + t];
     }
     __syncthreads();
-    if (t < 32) {
+    if (sums) {
+        if (t < nout) sums[(size_t)b0 * NSTAT + t] = W[t / NSTAT][W_S + t % NSTAT];
+    } else if (t < 32) {
         finalize_update_warp(f, b0, nb, pre, W, F);
         if (t == 0 && b0 == 0) f.st->w_raw = 1;
     }
@@ -1267,7 +1347,8 @@ __global__ void __launch_bounds__(FIN_THREADS) reduce_finalize_kernel(const FinA
 __global__ void __launch_bounds__(FIN_THREADS) reduce_finalize_batched_kernel(const FinArgs base,
                                                                               const BatchInst* __restrict__ insts,
                                                                               const int2* __restrict__ blocks,
-                                                                              DeviceState* states, int iters) {
+                                                                              DeviceState* states, int iters,
+                                                                              double* sums) {
     const int2 bi = blocks[blockIdx.x];
     const BatchInst I = insts[bi.x];
     FinArgs f = base;
@@ -1288,7 +1369,29 @@ __global__ void __launch_bounds__(FIN_THREADS) reduce_finalize_batched_kernel(co
     f.params = base.params + I.par_off;
     f.trace = base.trace + (size_t)bi.x * iters;
     f.st = states + bi.x;
-    reduce_finalize_body(f, bi.y);
+    reduce_finalize_body(f, bi.y, sums ? sums + (size_t)I.comp_off * NSTAT : nullptr);
+}
+
+// The update of every component of a batch, one lane each, from the sums in stats.
+__global__ void __launch_bounds__(32) finalize_lanes_batched_kernel(const FinArgs base,
+                                                                    const BatchInst* __restrict__ insts,
+                                                                    const int* __restrict__ comp_inst, int total_k,
+                                                                    DeviceState* states, bool white,
+                                                                    const double* __restrict__ stats) {
+    const int g = blockIdx.x * 32 + threadIdx.x;
+    if (g >= total_k) return;
+    const int inst = comp_inst[g];
+    const BatchInst I = insts[inst];
+    FinArgs f = base;
+    f.st = states + inst;
+    if ((f.em && f.iter > f.st->stop_after) || f.st->error != 0) return;
+    f.perm = base.perm ? base.perm + I.comp_off : nullptr;
+    f.shift4 = base.shift4 + I.comp_off;
+    f.model64 = base.model64 + (size_t)I.comp_off * MODEL;
+    f.params = base.params + I.par_off;
+    const int b = g - I.comp_off;
+    finalize_update_lane(f, b, white, stats + (size_t)g * NSTAT);
+    if (b == 0) f.st->w_raw = 1;
 }
 
 // What a given model and its points need before the E-step, in one launch: the first nbuild
@@ -1739,14 +1842,27 @@ cudaError_t launch_reduce_finalize(const float* partials, int grid, const double
 
 int fin_components_per_block() { return FIN_CPB; }
 
-cudaError_t launch_reduce_finalize_batched(const float* partials, const double* ll_partials, const double* stats64,
+// Where the binary64 update is the launch (two components of it at a time per block, about
+// 1.8 us of an SM's binary64 pipe each), the sums are one launch and the updates, a lane per
+// component, another; below eight blocks per SM the update's chain counts and one launch does both.
+// 48 segments, 9,488 components: 101 us in one launch, 58 + 11 us in two.
+bool finalize_batched_splits(int nblocks) { return nblocks >= 8 * 152; }
+
+cudaError_t launch_reduce_finalize_batched(const float* partials, const double* ll_partials, double* stats64,
                                            float4* shift4, const BatchInst* insts, const int2* blocks, int nblocks,
-                                           double reg, double tol, int iters, double* model64, float* params,
-                                           double* trace, DeviceState* states, int iter, bool em, cudaStream_t s,
-                                           const int* perm, const uint32_t* masks) {
-    const FinArgs f{partials, 0, ll_partials, stats64, shift4, 0, 0, reg, tol, model64, params, trace, nullptr,
-                    iter, em ? 1 : 0, 0, 1, perm, masks, 0};
-    reduce_finalize_batched_kernel<<<nblocks, FIN_THREADS, 0, s>>>(f, insts, blocks, states, std::max(iters, 1));
+                                           const int* comp_inst, int total_k, double reg, double tol, int iters,
+                                           double* model64, float* params, double* trace, DeviceState* states,
+                                           int iter, bool em, cudaStream_t s, const int* perm,
+                                           const uint32_t* masks) {
+    const bool split = finalize_batched_splits(nblocks);
+    const FinArgs f{partials, 0, ll_partials, partials ? nullptr : stats64, shift4, 0, 0, reg, tol, model64, params,
+                    trace, nullptr, iter, em ? 1 : 0, 0, 1, perm, masks, 0};
+    if (!split || partials)
+        reduce_finalize_batched_kernel<<<nblocks, FIN_THREADS, 0, s>>>(f, insts, blocks, states, std::max(iters, 1),
+                                                                       split ? stats64 : nullptr);
+    if (split)
+        finalize_lanes_batched_kernel<<<(total_k + 31) / 32, 32, 0, s>>>(f, insts, comp_inst, total_k, states,
+                                                                        partials != nullptr, stats64);
     return cudaGetLastError();
 }
 

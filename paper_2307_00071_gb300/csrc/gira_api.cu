@@ -1275,8 +1275,8 @@ gira_status gira_gmm_fit_batched(const float* points, const int64_t* offsets, in
                                                     b.st, c.s));
         GIRA_CUDA(cudaMemcpyAsync(b.shift4, b.c4, sizeof(float4) * total_k, cudaMemcpyDeviceToDevice, c.s));
         COUNTED(prof, 1, launch_reduce_finalize_batched(nullptr, nullptr, b.stats64, b.shift4, b.insts, b.blocks,
-                                                        (int)fin_blocks.size(), o.reg_covar, o.tol, o.iters, b.model64,
-                                                        b.params, b.trace, b.st, 0, false, c.s));
+                                                        (int)fin_blocks.size(), b.comp_inst, total_k, o.reg_covar, o.tol,
+                                                        o.iters, b.model64, b.params, b.trace, b.st, 0, false, c.s));
     } else {
         if (kw == Kind::Host)
             GIRA_CUDA(cudaMemcpyAsync(b.mw, weights, sizeof(float) * total_k, cudaMemcpyHostToDevice, c.s));
@@ -1327,10 +1327,10 @@ gira_status gira_gmm_fit_batched(const float* points, const int64_t* offsets, in
             for (int t = 1; t <= o.iters && e == cudaSuccess; ++t) {
                 e = estep_all(true, t, cs);
                 if (e == cudaSuccess)
-                    e = launch_reduce_finalize_batched(b.partials, b.llp, nullptr, b.shift4, b.insts, b.blocks,
-                                                       (int)fin_blocks.size(), o.reg_covar, o.tol, o.iters,
-                                                       b.model64, b.params, b.trace, b.st, t, true, cs, b.perm,
-                                                       b.masks);
+                    e = launch_reduce_finalize_batched(b.partials, b.llp, b.stats64, b.shift4, b.insts, b.blocks,
+                                                       (int)fin_blocks.size(), b.comp_inst, total_k, o.reg_covar,
+                                                       o.tol, o.iters, b.model64, b.params, b.trace, b.st, t, true,
+                                                       cs, b.perm, b.masks);
             }
             cudaGraph_t graph = nullptr;
             cudaError_t e2 = cudaStreamEndCapture(cs, &graph);
@@ -1350,7 +1350,7 @@ gira_status gira_gmm_fit_batched(const float* points, const int64_t* offsets, in
             ws->graph_exec = exec;
             ws->graph_key = key;
         }
-        prof.launches += (long long)o.iters * 2;
+        prof.launches += (long long)o.iters * (finalize_batched_splits((int)fin_blocks.size()) ? 3 : 2);
         GIRA_CUDA(cudaGraphLaunch(ws->graph_exec, c.s));
     }
     prof.t_em = prof.mark();

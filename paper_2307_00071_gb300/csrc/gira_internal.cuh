@@ -525,11 +525,16 @@ cudaError_t launch_pack_batched(const float* pts3, int64_t n, const int64_t* off
                                 float4* pts8, DeviceState* states, cudaStream_t s);
 // Finalize blocks: (instance, block index within the instance), FIN_CPB components each.
 int fin_components_per_block();
-cudaError_t launch_reduce_finalize_batched(const float* partials, const double* ll_partials, const double* stats64,
+// stats64: the one-hot statistics (partials == nullptr), or room for the sums; comp_inst: the
+// instance of each of the total_k components.  Large batches take two launches
+// (finalize_batched_splits) when there are partials.
+bool finalize_batched_splits(int nblocks);
+cudaError_t launch_reduce_finalize_batched(const float* partials, const double* ll_partials, double* stats64,
                                            float4* shift4, const BatchInst* insts, const int2* blocks, int nblocks,
-                                           double reg, double tol, int iters, double* model64, float* params,
-                                           double* trace, DeviceState* states, int iter, bool em, cudaStream_t s,
-                                           const int* perm = nullptr, const uint32_t* masks = nullptr);
+                                           const int* comp_inst, int total_k, double reg, double tol, int iters,
+                                           double* model64, float* params, double* trace, DeviceState* states,
+                                           int iter, bool em, cudaStream_t s, const int* perm = nullptr,
+                                           const uint32_t* masks = nullptr);
 // Padding slots of every instance's parameter block (one block per instance).
 cudaError_t launch_fill_padding_batched(float* params, const BatchInst* insts, int batch, int npairs_max,
                                         const int* npairs_of, cudaStream_t s);

@@ -158,3 +158,29 @@ def test_single_fit_equals_batch_of_one(gira):
     for key in ("weights", "means", "covs"):
         np.testing.assert_array_equal(to_np(one[key]), to_np(bat[key]))
     np.testing.assert_array_equal(np.asarray(one["trace"]), np.asarray(bat["trace"][0]))
+
+
+@pytest.mark.parametrize("kinit", [False, True])
+def test_large_batch_equals_small_batches(gira, kinit):
+    """From 1,216 finalize blocks of two components on, a batch's sums and its updates (a lane per
+    component) are two launches; below, one launch with a half-warp per component.  Every entry is
+    the same sequence of operations: the same bits, also for odd K and in the last warp."""
+    ks = [129, 1, 64, 255, 33] * 6
+    sizes = [900 + 13 * i for i in range(len(ks))]
+    assert sum((k + 1) // 2 for k in ks) >= 1216 and sum(ks) % 32 != 0
+    clouds, pts, offsets, kk = make_batch(sizes, ks, seed=11)
+    opts = dict(iters=4, tol=0.0, reg_covar=1e-4, seed=0, lloyd_iters=2)
+    init = None
+    if not kinit:
+        r = [oracle.kinit(c, k, seed=0, lloyd_iters=1, reg=1e-3) for c, k in zip(clouds, ks)]
+        init = tuple(np.concatenate([x[key] for x in r]).astype(np.float32) for key in ("weights", "means", "covs"))
+    big = gira.gira_gmm_fit_batched(pts, offsets, kk, init=init, **opts)
+    at = np.concatenate([[0], np.cumsum(ks)])
+    for lo in range(0, len(ks), 10):
+        hi = lo + 10
+        sub = None if init is None else tuple(a[at[lo]:at[hi]] for a in init)
+        part = gira.gira_gmm_fit_batched(pts[offsets[lo]:offsets[hi]], offsets[lo:hi + 1] - offsets[lo], kk[lo:hi],
+                                         init=sub, **opts)
+        for key in ("weights", "means", "covs"):
+            np.testing.assert_array_equal(to_np(part[key]), to_np(big[key])[at[lo]:at[hi]])
+        np.testing.assert_array_equal(np.asarray(part["trace"]), np.asarray(big["trace"])[lo:hi])
