@@ -916,8 +916,8 @@ __global__ void sample_kernel(int64_t m, int k, int d, const float* __restrict__
 // distance to the box of the points -- a centre farther than U from the box (with slack for
 // the binary32 rounding of both) is farther than that from every point.  The pairs are
 // scanned in increasing order, so the argmin and its ties are those of the full scan.  Runs
-// of equal labels over the lanes are summed before the atomics, as in 3-D.
-// Bound by the scan's packed arithmetic and the binary64 scan of the sums; one point per
+// of equal labels are summed before the atomics (add_runs).
+// Bound by the scan's packed arithmetic and the binary64 sums: 35 us per launch; one point per
 // thread over every centre with five binary64 atomics per point took 104 us per launch on
 // the 276,348-point frame, K = 512.
 constexpr int LL4_THREADS = 256, LL4_PPT = 4;
@@ -954,13 +954,13 @@ __global__ void __launch_bounds__(LL4_THREADS) lloyd4_assign_kernel(const float4
     unsigned long long cnt = 0;
     constexpr int64_t group = (int64_t)LL4_THREADS * LL4_PPT;
     for (int64_t g0 = (int64_t)blockIdx.x * group; g0 < n; g0 += (int64_t)gridDim.x * group) {
-        const int64_t wb = g0 + (int64_t)warp * 32 * LL4_PPT;   // point r of this lane: wb + 32 r + lane
+        const int64_t wb = g0 + (int64_t)warp * 32 * LL4_PPT;   // point r of this lane: wb + 4 lane + r
         float2 X[LL4_PPT][4];
         float bd[LL4_PPT];
         int best[LL4_PPT];
 #pragma unroll
         for (int r = 0; r < LL4_PPT; ++r) {
-            const float4 x = pts[min(wb + r * 32 + lane, n - 1)];
+            const float4 x = pts[min(wb + LL4_PPT * lane + r, n - 1)];
             X[r][0] = dup(x.x);
             X[r][1] = dup(x.y);
             X[r][2] = dup(x.z);
@@ -986,7 +986,7 @@ __global__ void __launch_bounds__(LL4_THREADS) lloyd4_assign_kernel(const float4
                 U = 0.f;
 #pragma unroll
                 for (int r = 0; r < LL4_PPT; ++r) {
-                    const int lp = labels[min(wb + r * 32 + lane, n - 1)];
+                    const int lp = labels[min(wb + LL4_PPT * lane + r, n - 1)];
                     const CPair4 c = sc4[lp >> 1];
                     float s = 0.f;
 #pragma unroll
@@ -1054,38 +1054,21 @@ __global__ void __launch_bounds__(LL4_THREADS) lloyd4_assign_kernel(const float4
                 if (s.y < bd[r]) { bd[r] = s.y; best[r] = 2 * p + 1; }
             }
         }
+        int key[LL4_PPT];
+        float x[LL4_PPT][4];
 #pragma unroll
         for (int r = 0; r < LL4_PPT; ++r) {
-            const int64_t i = wb + r * 32 + lane;
-            int key = -1;
-            double v[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+            const int64_t i = wb + LL4_PPT * lane + r;
+            key[r] = -1;
             if (i < n) {
                 if (it == 0 || labels[i] != best[r]) ++cnt;
                 labels[i] = best[r];
-                key = best[r];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) v[j] = (double)X[r][j].x;
-                v[4] = 1.0;
+                key[r] = best[r];
             }
-            // segmented inclusive scan over runs of equal keys (fixed order)
-            const int prev = __shfl_up_sync(FULL, key, 1);
-            const bool head = (lane == 0) || (prev != key);
-            const unsigned heads = __ballot_sync(FULL, head);
-            const int start = 31 - __clz(heads & (0xffffffffu >> (31 - lane)));
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                if (__all_sync(FULL, lane - o < start)) break;   // no run is longer
-#pragma unroll
-                for (int q = 0; q < 5; ++q) {
-                    const double u = __shfl_up_sync(FULL, v[q], o);
-                    if (lane - o >= start) v[q] += u;
-                }
-            }
-            const bool tail = (lane == 31) || ((heads >> (lane + 1)) & 1u);
-            if (tail && key >= 0)
-#pragma unroll
-                for (int q = 0; q < 5; ++q) atomicAdd(&sums[5 * (size_t)key + q], v[q]);
+            for (int j = 0; j < 4; ++j) x[r][j] = X[r][j].x;
         }
+        add_runs<4>(key, x, sums);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(FULL, cnt, o);

@@ -1179,8 +1179,10 @@ __global__ void __launch_bounds__(1024) kpp_coherence_kernel(const float4* __res
 // that moved (every label for it == 0).  Centres are processed two at a time
 // with packed FP32 (each lane of FADD2/FMUL2 rounds exactly like the scalar
 // operation, so the distances are those of dist2_f32).  Each thread owns
-// LL_PPT points; equal consecutive labels in a warp are summed before the
-// atomics (runs of raster-order points share labels).
+// LL_PPT consecutive points; runs of equal labels are summed before the
+// atomics (add_runs).  Bound by the scan of the listed centres and the binary64 sums.
+// Measured per launch: 48 segments, 1.41M points, K <= 512: 105 us with a scan of one point
+// per lane, 98 us now; 276,348 points, K = 512: 28.5 and 24 us; 1M points, K = 768: 75 and 41 us.
 constexpr int LL_PPT = 4;
 constexpr int LL_THREADS = 256;
 
@@ -1252,14 +1254,14 @@ __device__ void lloyd_assign_groups(const float4* __restrict__ pts, int64_t n, i
     uint16_t* slist = lists ? lists + (threadIdx.x >> 5) * npair : nullptr;
     unsigned long long cnt = 0;
     for (int64_t g0 = first; g0 < n; g0 += stride) {
-        // point r of this thread: g0 + warp_base + r * 32 + lane (coalesced per r)
+        // point r of this lane: wb + 4 lane + r
         const int64_t wb = g0 + (int64_t)(threadIdx.x >> 5) * 32 * LL_PPT;
         float2 X[LL_PPT], Y[LL_PPT], Z[LL_PPT];
         float bd[LL_PPT];
         int best[LL_PPT];
 #pragma unroll
         for (int r = 0; r < LL_PPT; ++r) {
-            const int64_t i = min(wb + r * 32 + lane, n - 1);
+            const int64_t i = min(wb + LL_PPT * lane + r, n - 1);
             const float4 x = pts[i];
             X[r] = dup(x.x);
             Y[r] = dup(x.y);
@@ -1267,23 +1269,25 @@ __device__ void lloyd_assign_groups(const float4* __restrict__ pts, int64_t n, i
             bd[r] = INFINITY;
             best[r] = 0;
         }
-        // After the first assignment: every point's previous centre bounds its nearest
-        // distance from above (U, the warp's largest), and a centre whose distance to the
-        // box of the warp's points exceeds U (with slack for the binary32 rounding of
-        // both) is farther than that from every point: only the other pairs are scanned,
-        // in increasing order, so the argmin and its ties are those of the full scan.
+        // Only the pairs that can hold a nearest centre are scanned, in increasing order, so the
+        // argmin and its ties are those of the full scan.  U bounds the nearest distance of every
+        // point from above: the largest distance to the previous centres, or in the first
+        // assignment the smallest over the centres of the largest distance to the box of the
+        // warp's points.  A centre whose distance to the box exceeds U (with slack for the
+        // binary32 rounding of both) is farther than that from every point.
         int nl = npair;
-        if (it > 0 && slist) {
+        if (slist) {
             float U = 0.f, lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
             for (int r = 0; r < LL_PPT; ++r) {
-                const int64_t i = min(wb + r * 32 + lane, n - 1);
-                const int lp = labels[i];
-                const CPair c = sc[lp >> 1];
-                const float cx = (lp & 1) ? c.x.y : c.x.x, cy = (lp & 1) ? c.y.y : c.y.x, cz = (lp & 1) ? c.z.y : c.z.x;
-                const float dx = __fadd_rn(X[r].x, cx), dy = __fadd_rn(Y[r].x, cy), dz = __fadd_rn(Z[r].x, cz);
-                const float d = __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
-                U = fmaxf(U, d);
+                if (it > 0) {
+                    const int lp = labels[min(wb + LL_PPT * lane + r, n - 1)];
+                    const CPair c = sc[lp >> 1];
+                    const float cx = (lp & 1) ? c.x.y : c.x.x, cy = (lp & 1) ? c.y.y : c.y.x,
+                                cz = (lp & 1) ? c.z.y : c.z.x;
+                    const float dx = __fadd_rn(X[r].x, cx), dy = __fadd_rn(Y[r].x, cy), dz = __fadd_rn(Z[r].x, cz);
+                    U = fmaxf(U, __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz)));
+                }
                 lo[0] = fminf(lo[0], X[r].x); lo[1] = fminf(lo[1], Y[r].x); lo[2] = fminf(lo[2], Z[r].x);
                 hi[0] = fmaxf(hi[0], X[r].x); hi[1] = fmaxf(hi[1], Y[r].x); hi[2] = fmaxf(hi[2], Z[r].x);
             }
@@ -1295,6 +1299,22 @@ __device__ void lloyd_assign_groups(const float4* __restrict__ pts, int64_t n, i
                     lo[j] = fminf(lo[j], __shfl_xor_sync(FULL, lo[j], o));
                     hi[j] = fmaxf(hi[j], __shfl_xor_sync(FULL, hi[j], o));
                 }
+            }
+            if (it == 0) {
+                U = INFINITY;
+                for (int p = lane; p < npair; p += 32) {
+                    const CPair c = sc[p];
+                    const float ncx[2] = {c.x.x, c.x.y}, ncy[2] = {c.y.x, c.y.y}, ncz[2] = {c.z.x, c.z.y};
+#pragma unroll
+                    for (int m = 0; m < 2; ++m) {
+                        const float fx = fmaxf(fabsf(lo[0] + ncx[m]), fabsf(hi[0] + ncx[m]));
+                        const float fy = fmaxf(fabsf(lo[1] + ncy[m]), fabsf(hi[1] + ncy[m]));
+                        const float fz = fmaxf(fabsf(lo[2] + ncz[m]), fabsf(hi[2] + ncz[m]));
+                        U = fminf(U, fmaf(fz, fz, fmaf(fy, fy, fx * fx)));
+                    }
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) U = fminf(U, __shfl_xor_sync(FULL, U, o));
             }
             nl = 0;
             for (int j0 = 0; j0 < npair; j0 += 32) {
@@ -1328,39 +1348,22 @@ __device__ void lloyd_assign_groups(const float4* __restrict__ pts, int64_t n, i
                 if (d.y < bd[r]) { bd[r] = d.y; best[r] = 2 * p + 1; }
             }
         }
+        int key[LL_PPT];
+        float x[LL_PPT][3];
 #pragma unroll
         for (int r = 0; r < LL_PPT; ++r) {
-            const int64_t i = wb + r * 32 + lane;
-            const bool valid = i < n;
-            int key = -1;
-            double v[4] = {0.0, 0.0, 0.0, 0.0};
-            if (valid) {
+            const int64_t i = wb + LL_PPT * lane + r;
+            key[r] = -1;
+            if (i < n) {
                 if (it == 0 || labels[i] != best[r]) ++cnt;
                 labels[i] = best[r];
-                key = best[r];
-                v[0] = (double)X[r].x;
-                v[1] = (double)Y[r].x;
-                v[2] = (double)Z[r].x;
-                v[3] = 1.0;
+                key[r] = best[r];
             }
-            // segmented inclusive scan over runs of equal keys (fixed order)
-            const int prev = __shfl_up_sync(FULL, key, 1);
-            const bool head = (lane == 0) || (prev != key);
-            const unsigned heads = __ballot_sync(FULL, head);
-            const int start = 31 - __clz(heads & (0xffffffffu >> (31 - lane)));
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const double u = __shfl_up_sync(FULL, v[q], o);
-                    if (lane - o >= start) v[q] += u;
-                }
-            }
-            const bool tail = (lane == 31) || ((heads >> (lane + 1)) & 1u);
-            if (tail && key >= 0)
-#pragma unroll
-                for (int q = 0; q < 4; ++q) atomicAdd(&sums[4 * key + q], v[q]);
+            x[r][0] = X[r].x;
+            x[r][1] = Y[r].x;
+            x[r][2] = Z[r].x;
         }
+        add_runs<3>(key, x, sums);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(FULL, cnt, o);
