@@ -9,9 +9,12 @@
 // bounding cube of their cloud, so that a warp holds a few neighbouring cells.
 //
 // The sort is a stable least-significant-digit radix sort on 9-bit digits,
-// deterministic (no order decided by atomics): per tile of 512 keys a
+// deterministic (no order decided by atomics): per tile of keys a
 // histogram, one exclusive scan over (digit, tile), and a scatter in which
-// one warp walks its tile in order and ranks equal digits with match_any.  A
+// one warp walks its tile in order and ranks equal digits with match_any.
+// Both walks are chains of one step per 32 keys: tiles hold 512 keys, which
+// keeps the scan short, but 128 up to 131,072 keys, where the GPU is far from
+// full (20,000 points: the kernels 78 -> 68 us with cold caches).  A
 // batch sorts by (instance, code), which keeps every instance in its own range.
 // Only the order of the per-point terms in the E-step's sums changes; the
 // fit's k-means++ and Lloyd steps run on the points in the caller's order.
@@ -27,8 +30,9 @@ namespace {
 constexpr unsigned FULL = 0xffffffffu;
 constexpr int RADIX_BITS = 9;
 constexpr int RADIX = 1 << RADIX_BITS;   // 512 digits
-constexpr int TILE = 512;                // keys per histogram / scatter tile (one warp)
-constexpr int BOX_CHUNK = 4096;          // points per bounding-box block
+constexpr int TILE = 512, TILE_SMALL = 128;   // keys per histogram / scatter tile (one warp)
+constexpr int64_t SMALL_N = 131072;           // keys up to which tiles are small
+constexpr int BOX_CHUNK = 1024;          // points per bounding-box block
 constexpr int SCAN_PER_BLOCK = 8192;     // scan: 1024 threads x 8
 constexpr int MORTON_BITS = 18;
 
@@ -142,6 +146,7 @@ __global__ void __launch_bounds__(256) key_kernel(const float4* __restrict__ p8,
 
 // Per tile (one warp, TILE keys): the count of every digit, stored digit-major
 // ([digit][tile]) so that one exclusive scan gives every tile's output offsets.
+template <int TILE>
 __global__ void __launch_bounds__(256) radix_hist_kernel(const uint32_t* __restrict__ keys, int64_t n, int shift,
                                                          int ntiles, int* counts) {
     __shared__ int hist[8][RADIX];
@@ -152,9 +157,12 @@ __global__ void __launch_bounds__(256) radix_hist_kernel(const uint32_t* __restr
     __syncwarp();
     if (tile < ntiles) {
         const int64_t b = (int64_t)tile * TILE, e = min(n, b + TILE);
-        for (int64_t i0 = b; i0 < e; i0 += 32) {   // equal digits of the 32 keys counted once
-            const int64_t i = i0 + lane;
-            const int d = i < e ? (int)((keys[i] >> shift) & (RADIX - 1)) : RADIX;
+        uint32_t key[TILE / 32];   // all loads in flight at once
+#pragma unroll
+        for (int r = 0; r < TILE / 32; ++r) key[r] = b + 32 * r + lane < e ? keys[b + 32 * r + lane] : 0u;
+#pragma unroll
+        for (int r = 0; r < TILE / 32; ++r) {   // equal digits of the 32 keys counted once
+            const int d = b + 32 * r + lane < e ? (int)((key[r] >> shift) & (RADIX - 1)) : RADIX;
             const uint32_t peers = __match_any_sync(FULL, d);
             if (d < RADIX && (peers & ((1u << lane) - 1u)) == 0u) h[d] += __popc(peers);
             __syncwarp();
@@ -163,8 +171,8 @@ __global__ void __launch_bounds__(256) radix_hist_kernel(const uint32_t* __restr
     }
 }
 
-// Exclusive scan of m ints in place: block sums, a scan of the block sums
-// (one block), then every block's local scan plus its offset.
+// Exclusive scan of m ints: block sums, then every block's local scan plus the sum of the
+// block sums before it.
 __device__ __forceinline__ int block_exclusive_scan(int v, int* s_warp, int* total) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int x = v;
@@ -203,24 +211,6 @@ __global__ void __launch_bounds__(1024) scan_sums_kernel(const int* __restrict__
     if (threadIdx.x == 0) bsum[blockIdx.x] = total;
 }
 
-__global__ void __launch_bounds__(1024) scan_bsum_kernel(int* bsum, int nb) {
-    __shared__ int s_warp[32];
-    int v[8], t = 0;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        const int i = 8 * threadIdx.x + j;
-        v[j] = i < nb ? bsum[i] : 0;
-        t += v[j];
-    }
-    int run = block_exclusive_scan(t, s_warp, nullptr);
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        const int i = 8 * threadIdx.x + j;
-        if (i < nb) bsum[i] = run;
-        run += v[j];
-    }
-}
-
 // (writes the offsets tile-major too, [tile][digit], for the scatter's coalesced loads)
 __global__ void __launch_bounds__(1024) scan_apply_kernel(const int* __restrict__ a, int64_t m,
                                                           const int* __restrict__ bsum, int ntiles, int* at) {
@@ -232,7 +222,10 @@ __global__ void __launch_bounds__(1024) scan_apply_kernel(const int* __restrict_
         v[j] = base + j < m ? a[base + j] : 0;
         t += v[j];
     }
-    int run = block_exclusive_scan(t, s_warp, nullptr) + bsum[blockIdx.x];
+    int before = 0, offset;   // the block sums before this block's, summed by all threads
+    for (int b = threadIdx.x; b < (int)blockIdx.x; b += 1024) before += bsum[b];
+    block_exclusive_scan(before, s_warp, &offset);
+    int run = block_exclusive_scan(t, s_warp, nullptr) + offset;
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
         if (base + j < m) {
@@ -247,11 +240,12 @@ __global__ void __launch_bounds__(1024) scan_apply_kernel(const int* __restrict_
 // equal digits rank among themselves (match_any) after the count of that digit so
 // far in the tile, which starts at the tile's scanned offset.  The tile's keys and
 // indices are loaded before the walk (all loads in flight at once).
-constexpr int SC_ROUNDS = TILE / 32;
+template <int TILE>
 __global__ void __launch_bounds__(256) radix_scatter_kernel(const uint32_t* __restrict__ keys_in,
                                                             const int* __restrict__ idx_in, int64_t n, int shift,
                                                             int ntiles, const int* __restrict__ offs,
                                                             uint32_t* keys_out, int* idx_out) {
+    constexpr int SC_ROUNDS = TILE / 32;
     __shared__ int cnt[8][RADIX];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int tile = blockIdx.x * 8 + warp;
@@ -410,9 +404,9 @@ void point_order_fill_units(const int64_t* offsets, int batch, int2* units) {
         for (int64_t c = 0; c * BOX_CHUNK < offsets[i + 1] - offsets[i]; ++c) units[u++] = make_int2(i, (int)c);
 }
 
-int point_order_launches(int batch) { return 4 + 5 * radix_passes(batch); }   // with the gather
+int point_order_launches(int batch) { return 4 + 4 * radix_passes(batch); }   // with the gather
 
-// the largest n the scan's two levels hold (every tile's 512 digit counts)
+// the largest n ordered (8,192 scan blocks over every tile's 512 digit counts)
 int64_t point_order_max_n() { return (int64_t)SCAN_PER_BLOCK * SCAN_PER_BLOCK / RADIX * TILE; }
 
 size_t cell_group_scratch_bytes(int64_t n) { return sizeof(int) * (CELL_BINS + 64 + 2 * (size_t)n); }
@@ -435,7 +429,7 @@ cudaError_t launch_cell_group(const float* p3, int64_t n, void* scratch, int* or
 }
 
 size_t point_order_scratch_bytes(int64_t n, int batch) {
-    const int64_t ntiles = ceil_div(n, TILE);
+    const int64_t ntiles = ceil_div(n, n <= SMALL_N ? TILE_SMALL : TILE);
     const int64_t m = ntiles * RADIX;
     size_t bytes = 0;
     auto add = [&](size_t b) { bytes += (b + 255) & ~size_t(255); };
@@ -453,7 +447,8 @@ size_t point_order_scratch_bytes(int64_t n, int batch) {
 cudaError_t launch_point_order(const float4* p8, int64_t n, const int64_t* offsets_d, const int2* units_d,
                                int nunits, int batch, void* scratch, float4* p8_out, float4* p4_out, int* order_out,
                                cudaStream_t s) {
-    const int64_t ntiles = ceil_div(n, TILE);
+    const bool small = n <= SMALL_N;
+    const int64_t ntiles = ceil_div(n, small ? TILE_SMALL : TILE);
     const int64_t m = ntiles * RADIX;
     const int64_t nb = ceil_div(m, SCAN_PER_BLOCK);
     if (nb > SCAN_PER_BLOCK || n > INT32_MAX) return cudaErrorInvalidValue;
@@ -482,12 +477,15 @@ cudaError_t launch_point_order(const float4* p8, int64_t n, const int64_t* offse
     for (int pass = 0; pass < passes; ++pass) {
         const int shift = pass * RADIX_BITS;
         const bool last = pass == passes - 1;
-        radix_hist_kernel<<<tblocks, 256, 0, s>>>(k0, n, shift, (int)ntiles, counts);
+        if (small) radix_hist_kernel<TILE_SMALL><<<tblocks, 256, 0, s>>>(k0, n, shift, (int)ntiles, counts);
+        else radix_hist_kernel<TILE><<<tblocks, 256, 0, s>>>(k0, n, shift, (int)ntiles, counts);
         scan_sums_kernel<<<(unsigned)nb, 1024, 0, s>>>(counts, m, bsum);
-        scan_bsum_kernel<<<1, 1024, 0, s>>>(bsum, (int)nb);
         scan_apply_kernel<<<(unsigned)nb, 1024, 0, s>>>(counts, m, bsum, (int)ntiles, toffs);
         int* io = (last && order_out) ? order_out : iout;
-        radix_scatter_kernel<<<tblocks, 256, 0, s>>>(k0, iin, n, shift, (int)ntiles, toffs, k1, io);
+        if (small)
+            radix_scatter_kernel<TILE_SMALL><<<tblocks, 256, 0, s>>>(k0, iin, n, shift, (int)ntiles, toffs, k1, io);
+        else
+            radix_scatter_kernel<TILE><<<tblocks, 256, 0, s>>>(k0, iin, n, shift, (int)ntiles, toffs, k1, io);
         std::swap(k0, k1);
         iout = iin;   // the input indices are free for the next pass's output
         iin = io;
