@@ -45,14 +45,20 @@ class GmmLogLik(torch.autograd.Function):
             if name in want:
                 g[name] = r["grad_" + name]
         ctx.grads = g
-        return torch.tensor(r["loglik"], dtype=torch.float64, device=points.device)
+        # a fill on the stream; torch.tensor would copy from the host and wait
+        return torch.full((), r["loglik"], dtype=torch.float64, device=points.device)
 
     @staticmethod
     def backward(ctx, gout):
         out = []
+        scale = {gout.dtype: gout}   # the incoming gradient in each gradient's type, converted once
         for name in _NAMES:
             v = ctx.grads[name]
-            out.append(None if v is None else v * gout.to(v.dtype))
+            if v is not None:
+                if v.dtype not in scale:
+                    scale[v.dtype] = gout.to(v.dtype)
+                v = v * scale[v.dtype]
+            out.append(v)
         return tuple(out)
 
 

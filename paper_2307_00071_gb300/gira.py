@@ -105,20 +105,27 @@ def _is_torch(x):
     return type(x).__module__.startswith("torch")
 
 
-def _ptr(x):
-    """(pointer, keepalive, stream) for a torch tensor or numpy array (contiguous float32/int32)."""
+def _arg(x):
+    """(pointer, keepalive) for a torch tensor or numpy array (contiguous float32/int32)."""
     if x is None:
-        return None, None, None
+        return None, None
     if _is_torch(x):
         if not x.is_contiguous():
             raise ValueError("tensor must be contiguous")
-        stream = None
-        if x.is_cuda:
-            import torch
-            stream = torch.cuda.current_stream(x.device).cuda_stream
-        return x.data_ptr(), x, stream
+        return x.data_ptr(), x
     a = np.ascontiguousarray(x)
-    return a.ctypes.data, a, None
+    return a.ctypes.data, a
+
+
+def _ptr(x):
+    """(pointer, keepalive, stream): _arg and the current stream of a CUDA tensor's device.  One argument
+    per call gives the stream (several microseconds); the others go through _arg."""
+    p, keep = _arg(x)
+    stream = None
+    if _is_torch(x) and x.is_cuda:
+        import torch
+        stream = torch.cuda.current_stream(x.device).cuda_stream
+    return p, keep, stream
 
 
 def _new(like, shape, dtype):
@@ -176,8 +183,8 @@ def gira_kmeans_init(points, k: int, seed: int = 0, lloyd_iters: int = 10, cente
     if labels is None and want_labels:
         labels = _new(points, (n,), np.int32)
     pp, kp, s = _ptr(points)
-    cp, kc, _ = _ptr(centers)
-    lp, kl, _ = _ptr(labels)
+    cp, kc = _arg(centers)
+    lp, kl = _arg(labels)
     done = C.c_int(0)
     _check(_lib.gira_kmeans_init(pp, n, k, seed, lloyd_iters, cp, lp, C.byref(done), s))
     return centers, labels, done.value
@@ -211,9 +218,9 @@ def gira_gmm_fit(points, k: int, iters: int = 100, tol: float = 1e-3, reg_covar:
                 dst[...] = np.asarray(src, dtype=np.float32)
     tr = np.full(max(iters, 1), np.nan) if trace else None
     pp, kp, s = _ptr(points)
-    wp, kw, _ = _ptr(weights)
-    mp, km, _ = _ptr(means)
-    cp, kc, _ = _ptr(covs)
+    wp, kw = _arg(weights)
+    mp, km = _arg(means)
+    cp, kc = _arg(covs)
     done, fll = C.c_int(0), C.c_double(np.nan)
     _check(_lib.gira_gmm_fit(pp, n, k, C.byref(o), wp, mp, cp,
                              tr.ctypes.data_as(C.POINTER(C.c_double)) if tr is not None else None,
@@ -229,10 +236,10 @@ def gira_gmm_loglik(points, weights, means, covs, per_point: bool = False, out=N
     if per_point and out is None:
         out = _new(points, (n,), np.float32)
     pp, kp, s = _ptr(points)
-    wp, kw, _ = _ptr(weights)
-    mp, km, _ = _ptr(means)
-    cp, kc, _ = _ptr(covs)
-    op, ko, _ = _ptr(out if per_point else None)
+    wp, kw = _arg(weights)
+    mp, km = _arg(means)
+    cp, kc = _arg(covs)
+    op, ko = _arg(out if per_point else None)
     mean = C.c_double(np.nan)
     _check(_lib.gira_gmm_loglik(pp, n, k, wp, mp, cp, C.byref(mean), op, s))
     return (mean.value, out) if per_point else mean.value
@@ -251,10 +258,10 @@ def gira_gmm_loglik_noalloc(points, weights, means, covs, per_point: bool = Fals
     if per_point and out is None:
         out = _new(points, (n,), np.float32)
     pp, kp, s = _ptr(points)
-    wp, kw, _ = _ptr(weights)
-    mp, km, _ = _ptr(means)
-    cp, kc, _ = _ptr(covs)
-    op, ko, _ = _ptr(out if per_point else None)
+    wp, kw = _arg(weights)
+    mp, km = _arg(means)
+    cp, kc = _arg(covs)
+    op, ko = _arg(out if per_point else None)
     mean = C.c_double(np.nan)
     _check(_lib.gira_gmm_loglik_noalloc(pp, n, k, wp, mp, cp, C.byref(mean), op, s))
     return (mean.value, out) if per_point else mean.value
@@ -304,10 +311,10 @@ def gira_gmm_loglik_grad(points, logits, means, chol, pose=None, want=GRADS):
     keep = [kp]
     ptrs = []
     for x in (po, lg, mu, ch):
-        p_, k_, _ = _ptr(x)
+        p_, k_ = _arg(x)
         ptrs.append(p_)
         keep.append(k_)
-    optr = [(_ptr(outs[g])[0] if g in outs else None) for g in GRADS]
+    optr = [(_arg(outs[g])[0] if g in outs else None) for g in GRADS]
     ll = C.c_double(np.nan)
     _check(_lib.gira_gmm_loglik_grad(pp, n, k, ptrs[0], ptrs[1], ptrs[2], ptrs[3], C.byref(ll), *optr, s))
     r = {"loglik": ll.value}
@@ -349,9 +356,9 @@ def gira_gmm_fit_batched(points, offsets, ks, iters: int = 100, tol: float = 1e-
     fll = np.full(B, np.nan)
     stat = np.zeros(B, np.int32)
     pp, kp, s = _ptr(points)
-    wp, kw, _ = _ptr(w)
-    mp, km, _ = _ptr(m)
-    cp, kc, _ = _ptr(c)
+    wp, kw = _arg(w)
+    mp, km = _arg(m)
+    cp, kc = _arg(c)
     st = _lib.gira_gmm_fit_batched(pp, offs.ctypes.data, B, kk.ctypes.data, C.byref(o), wp, mp, cp,
                                    trace.ctypes.data if iters > 0 else None, done.ctypes.data,
                                    fll.ctypes.data if final_loglik else None, stat.ctypes.data, s)
@@ -386,10 +393,10 @@ def gira_gmm_loglik_grad_batched(points, offsets, ks, logits, means, chol, poses
     keep = [kp]
     ptrs = []
     for x in (po, lg, mu, ch):
-        p_, k_, _ = _ptr(x)
+        p_, k_ = _arg(x)
         ptrs.append(p_)
         keep.append(k_)
-    optr = [(_ptr(outs[g])[0] if g in outs else None) for g in GRADS]
+    optr = [(_arg(outs[g])[0] if g in outs else None) for g in GRADS]
     st = _lib.gira_gmm_loglik_grad_batched(pp, offs.ctypes.data, B, kk.ctypes.data, ptrs[0], ptrs[1], ptrs[2],
                                            ptrs[3], ll.ctypes.data, *optr, stat.ctypes.data, s)
     if raise_on_error:
@@ -418,9 +425,9 @@ def gira_gmm_fit4(points, k: int, iters: int = 100, tol: float = 1e-3, reg_covar
         o.init_mode = INIT_PARAMS
     tr = np.full(max(iters, 1), np.nan)
     pp, kp, s = _ptr(points)
-    wp, kw, _ = _ptr(w)
-    mp, km, _ = _ptr(m)
-    cp, kc, _ = _ptr(c)
+    wp, kw = _arg(w)
+    mp, km = _arg(m)
+    cp, kc = _arg(c)
     done, fll = C.c_int(0), C.c_double(np.nan)
     _check(_lib.gira_gmm_fit4(pp, n, k, C.byref(o), wp, mp, cp, tr.ctypes.data_as(C.POINTER(C.c_double)),
                               C.byref(done), C.byref(fll) if final_loglik else None, s))
@@ -435,10 +442,10 @@ def gira_gmm_loglik4(points, weights, means, covs, per_point: bool = False):
     w, m, c = (_f32_like(a, points) for a in (weights, means, covs))
     out = _new(points, (n,), np.float32) if per_point else None
     pp, kp, s = _ptr(points)
-    wp, kw, _ = _ptr(w)
-    mp, km, _ = _ptr(m)
-    cp, kc, _ = _ptr(c)
-    op, ko, _ = _ptr(out)
+    wp, kw = _arg(w)
+    mp, km = _arg(m)
+    cp, kc = _arg(c)
+    op, ko = _arg(out)
     mean = C.c_double(np.nan)
     _check(_lib.gira_gmm_loglik4(pp, n, k, wp, mp, cp, C.byref(mean), op, s))
     return (mean.value, out) if per_point else mean.value
@@ -453,11 +460,11 @@ def gira_gmm_conditional4(locs, weights, means, covs, want_var: bool = True):
     e = _new(locs, (m_,), np.float32)
     v = _new(locs, (m_,), np.float32) if want_var else None
     lp, kl, s = _ptr(locs)
-    wp, kw, _ = _ptr(w)
-    mp, km, _ = _ptr(m)
-    cp, kc, _ = _ptr(c)
-    ep, ke, _ = _ptr(e)
-    vp_, kv, _ = _ptr(v)
+    wp, kw = _arg(w)
+    mp, km = _arg(m)
+    cp, kc = _arg(c)
+    ep, ke = _arg(e)
+    vp_, kv = _arg(v)
     _check(_lib.gira_gmm_conditional4(lp, m_, k, wp, mp, cp, ep, vp_, s))
     return e, v
 
@@ -479,11 +486,11 @@ def gira_gmm_sample(m: int, weights, means, covs, seed: int = 0, device=None, wa
     if _is_torch(like) and like.is_cuda:
         import torch
         s = torch.cuda.current_stream(like.device).cuda_stream
-    wp, kw, _ = _ptr(w)
-    mp, km, _ = _ptr(mu)
-    cp, kc, _ = _ptr(c)
-    op, ko, _ = _ptr(out)
-    qp, kq, _ = _ptr(comp)
+    wp, kw = _arg(w)
+    mp, km = _arg(mu)
+    cp, kc = _arg(c)
+    op, ko = _arg(out)
+    qp, kq = _arg(comp)
     _check(_lib.gira_gmm_sample(m, k, d, wp, mp, cp, seed, op, qp, s))
     return out, comp
 
@@ -500,8 +507,8 @@ def gira_gbms(points, bandwidth: float, max_iter: int = 300):
     modes = _new(points, (n, d), np.float64)
     counts = _new(points, (n,), np.int32)
     pp, kp, s = _ptr(points)
-    mp, km, _ = _ptr(modes)
-    cp, kc, _ = _ptr(counts)
+    mp, km = _arg(modes)
+    cp, kc = _arg(counts)
     k = C.c_int(0)
     _check(_lib.gira_gbms(pp, n, d, float(bandwidth), max_iter, C.byref(k), mp, cp, s))
     return modes[:k.value], counts[:k.value]
