@@ -330,6 +330,40 @@ constexpr int MAX_K_DIRECT = 1024;
 // ---------------------------------------------------------------- kernel entry points
 // (defined in em_kernels.cu / kmeans_kernels.cu, launched from gira_api.cu)
 
+// Runs of equal keys over a warp whose lanes hold consecutive elements: a lane has key_first ..
+// key_last with the sum and count of its last run and, unless it is `whole` (one run), of its
+// first.  Runs that go on over lanes are joined by a segmented scan of the lanes' last runs
+// (fixed order) and put(key, sum, count) is called once for each.  Called by whole warps.
+template <int NV, class Put>
+__device__ __forceinline__ void join_runs(int key_first, int key_last, bool whole, double (&first)[NV], int nfirst,
+                                          double (&run)[NV], int nrun, Put put) {
+    constexpr unsigned ALL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const int before = __shfl_up_sync(ALL, key_last, 1), after = __shfl_down_sync(ALL, key_first, 1);
+    const bool joins = lane > 0 && before == key_first;   // the lane's first run goes on from the lane before
+    const unsigned heads = __ballot_sync(ALL, !(whole && joins));
+    const int start = 31 - __clz(heads & (ALL >> (31 - lane)));
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        if (__all_sync(ALL, lane - o < start)) break;   // no run is longer
+        const int c = __shfl_up_sync(ALL, nrun, o);
+        if (lane - o >= start) nrun += c;
+#pragma unroll
+        for (int q = 0; q < NV; ++q) {
+            const double u = __shfl_up_sync(ALL, run[q], o);
+            if (lane - o >= start) run[q] += u;
+        }
+    }
+    const int nprev = __shfl_up_sync(ALL, nrun, 1);
+#pragma unroll
+    for (int q = 0; q < NV; ++q) {
+        const double u = __shfl_up_sync(ALL, run[q], 1);
+        if (!whole && joins) first[q] += u;
+    }
+    if (!whole) put(key_first, first, nfirst + (joins ? nprev : 0));
+    if (lane == 31 || after != key_last) put(key_last, run, nrun);
+}
+
 // sums[(D + 1) key + q] += the coordinates (binary64) and the count of a warp's 128 points, lane l
 // holding points 4 l .. 4 l + 3 with labels key[0 .. 3] (-1: none, only at the end).  Runs of equal
 // labels are summed first, inside the lane and then over the lanes (a segmented scan of the lanes'
@@ -338,8 +372,6 @@ constexpr int MAX_K_DIRECT = 1024;
 // and a scan for each of four rounds took 92.
 template <int D>
 __device__ __forceinline__ void add_runs(const int (&key)[4], const float (&x)[4][D], double* sums) {
-    constexpr unsigned ALL = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
     auto put = [&](int k, const double (&v)[D], int c) {
         if (k < 0) return;
         double* s = sums + (size_t)(D + 1) * k;
@@ -375,29 +407,7 @@ __device__ __forceinline__ void add_runs(const int (&key)[4], const float (&x)[4
             nrun = 1;
         }
     }
-    const int before = __shfl_up_sync(ALL, key[3], 1), after = __shfl_down_sync(ALL, key[0], 1);
-    const bool joins = lane > 0 && before == key[0];   // the lane's first run goes on from the lane before
-    const unsigned heads = __ballot_sync(ALL, !(whole && joins));
-    const int start = 31 - __clz(heads & (ALL >> (31 - lane)));
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        if (__all_sync(ALL, lane - o < start)) break;   // no run is longer
-        const int c = __shfl_up_sync(ALL, nrun, o);
-        if (lane - o >= start) nrun += c;
-#pragma unroll
-        for (int q = 0; q < D; ++q) {
-            const double u = __shfl_up_sync(ALL, run[q], o);
-            if (lane - o >= start) run[q] += u;
-        }
-    }
-    const int nprev = __shfl_up_sync(ALL, nrun, 1);
-#pragma unroll
-    for (int q = 0; q < D; ++q) {
-        const double u = __shfl_up_sync(ALL, run[q], 1);
-        if (!whole && joins) first[q] += u;
-    }
-    if (!whole) put(key[0], first, nfirst + (joins ? nprev : 0));
-    if (lane == 31 || after != key[3]) put(key[3], run, nrun);
+    join_runs(key[0], key[3], whole, first, nfirst, run, nrun, put);
 }
 
 // Batched fits: one entry per instance (device table).

@@ -10,21 +10,48 @@ import oracle
 pytestmark = pytest.mark.gpu
 
 
+def runs_of_points(n, longest):
+    rng = np.random.default_rng(n * 1000 + longest)
+    runs = []
+    while sum(map(len, runs)) < n:
+        runs.append(np.full(rng.integers(1, longest + 1), rng.integers(5)))
+    which = np.concatenate(runs)[:n]
+    corners = 16.0 * np.array([[0, 0, 0], [1, 0, 0], [0, 1, 0], [0, 0, 1], [1, 1, 1]])
+    return (corners[which] + rng.integers(-512, 513, size=(n, 3)) / 1024.0).astype(np.float32)
+
+
 @pytest.mark.parametrize("n", [7, 63, 127, 128, 129, 131, 1024, 1031, 5003])
 @pytest.mark.parametrize("longest", [1, 3, 9, 300])
 def test_runs_of_labels(n, longest):
     from paper_2307_00071_gb300 import gira
-    rng = np.random.default_rng(n * 1000 + longest)
     k = 5
-    runs = []
-    while sum(map(len, runs)) < n:
-        runs.append(np.full(rng.integers(1, longest + 1), rng.integers(k)))
-    which = np.concatenate(runs)[:n]
-    corners = 16.0 * np.array([[0, 0, 0], [1, 0, 0], [0, 1, 0], [0, 0, 1], [1, 1, 1]])
-    pts = (corners[which] + rng.integers(-512, 513, size=(n, 3)) / 1024.0).astype(np.float32)
+    pts = runs_of_points(n, longest)
     c0, _ = oracle.kmeanspp(pts, k, 1)
     ref_c, ref_lab, ref_done = oracle.lloyd(pts, c0, 6)
     c, lab, done = gira.gira_kmeans_init(pts, k, seed=1, lloyd_iters=6)
     assert done == ref_done
     np.testing.assert_array_equal(np.asarray(lab), ref_lab)
     np.testing.assert_array_equal(np.asarray(c), ref_c.astype(np.float32))
+
+
+@pytest.mark.parametrize("n", [255, 256, 513, 2051, 70001])
+@pytest.mark.parametrize("batched", [False, True])
+def test_one_hot_statistics_of_runs(n, batched):
+    """The statistics that start EM, summed over runs the same way (eight points per lane; small
+    blocks up to 65,536 points): the model of a fit without iterations.  Binary64 throughout, so
+    within two roundings of the binary32 outputs."""
+    from paper_2307_00071_gb300 import gira
+    pts = [runs_of_points(n, 9)] + ([runs_of_points(301, 3)] if batched else [])
+    for p in pts:
+        assert len(np.unique(np.round(p / 16.0), axis=0)) == 5
+    opts = dict(iters=0, tol=0.0, reg_covar=1e-3, seed=1, lloyd_iters=2)
+    if batched:
+        offs = np.cumsum([0] + [len(p) for p in pts]).astype(np.int64)
+        r = gira.gira_gmm_fit_batched(np.concatenate(pts), offs, np.array([5, 5], np.int32), **opts)
+    else:
+        r = gira.gira_gmm_fit(pts[0], 5, **opts)
+    for i, p in enumerate(pts):
+        ref = oracle.kinit(p, 5, 1, 2, 1e-3)
+        for key in ("weights", "means", "covs"):
+            got = np.asarray(r[key], np.float64)[5 * i:5 * i + 5]
+            np.testing.assert_allclose(got, ref[key], rtol=1.2e-7, atol=1e-8)
