@@ -231,7 +231,7 @@ gira_status gira_gmm_loglik_grad(const float *points, int64_t n, int k, const fl
  *   grad_pose, grad_twist [host|device] batch x 12, batch x 6 binary64, or NULL
  *   grad_logits, grad_means, grad_chol  [host|device] stacked, binary32, or NULL
  *   statuses              [host] batch gira_status values, or NULL
- * Every gradient is computed (NULL only skips its copy-out).  Returns the
+ * What only a NULL gradient needs is not computed.  Returns the
  * status of the first failing instance, else GIRA_OK.
  */
 gira_status gira_gmm_loglik_grad_batched(const float *points, const int64_t *offsets, int batch, const int *ks,
@@ -249,13 +249,13 @@ gira_status gira_gmm_loglik_grad_batched(const float *points, const int64_t *off
  * over all four coordinates, binary32 in the order ((d0^2 + d1^2) + d2^2) + d3^2),
  * the same E-step (Eq. estep / logestep with the log-density of
  * Eq. simplifiedGaussian for D = 4) and M-step, the same opts and stopping rule.
- * k <= GIRA_MAX_K4 (above 1024 the log-sum-exp runs in two levels, over chunks
- * of 512 components, with the exact per-point maximum for points whose total
- * underflows, as gira_gmm_fit does).
+ * k <= GIRA_MAX_K4.  Components whose terms are exactly 0 in binary32 for a block of
+ * points are skipped, and a point whose total underflows is summed about its block's
+ * own maximum, as gira_gmm_fit does.
  *   weights [host|device] K binary32, means K x 4, covs K x 4 x 4 (row-major;
  *   the lower triangle is read when GIRA_INIT_PARAMS), written on return.
  */
-#define GIRA_MAX_K4 8192   /* above 1024: the E-step runs over chunks of 512 components */
+#define GIRA_MAX_K4 8192
 gira_status gira_gmm_fit4(const float *points, int64_t n, int k, const gira_fit_opts *opts, float *weights,
                           float *means, float *covs, double *loglik_trace, int *iters_done, double *final_loglik,
                           void *stream);

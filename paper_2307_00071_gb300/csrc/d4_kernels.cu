@@ -94,7 +94,7 @@ __device__ bool build_component4(int b, double w, const double mu[4], const doub
 // shared memory: GB300 issues one binary64 warp instruction per 64 cycles per warp whatever
 // the number of active lanes, so a stage costs what one entry costs (~170 instructions in
 // all; one thread per component, one block each, ran ~500 in a row: 58 us per launch at
-// K = 512, 9 us now).  The statistics are about y = P'(x - s) with the binary32 P' of
+// K = 512, 16 us now under a profiler that empties the caches).  The statistics are about y = P'(x - s) with the binary32 P' of
 // the E-step (a component thin in one direction keeps that direction's digits): with M =
 // P'^{-1}, mu = (S0 / N_b) s + M ybar, Sigma = M (S2 / N_b - ybar ybar^T) M^T + reg I; one-hot
 // statistics are about shift4 with M = I.

@@ -5,24 +5,16 @@
 // (Eq. simplifiedGaussian); the M-step (standard full-covariance update, not
 // written in the paper) is fed by per-component sufficient statistics.
 //
-// Mapping (component-stationary): one CTA holds ALL K components, spread over
-// its G warps; lane (warp w, lane l) owns NP component pairs in registers, and
-// warp w the contiguous block of pairs [w NP 32, (w + 1) NP 32).  All lanes walk
-// the CTA's contiguous range of points together, Q_BATCH points at a time.
-// Pass 1 computes e_nb = 2^(l_nb - cmax) for the lane's components (kept in
-// registers), the per-point sums are combined across lanes (shuffle
-// transpose-reduce) and warps (shared memory), and pass 2 accumulates the
-// per-component statistics S0 = sum r, S1 = sum r d, S2 = sum r d d^T with
-// d = x - mu_old (binary32, per-CTA partials).  Pass 1 processes component
-// pairs with packed FP32 (FFMA2/FADD2); pass 2 uses scalar FP32.  The
-// responsibility matrix is never stored.
-//
-// Pass 2 skips a (point, pair of lanes' components) wherever e is exactly 0
-// for every lane of the warp (ex2.approx.ftz returns +0 below 2^-126, and a
-// zero responsibility adds exactly nothing to any accumulator, so the skip
-// changes no bit).  The fit orders the components along a space-filling curve
-// of their means (order_components_kernel), so a warp's 128 components are
-// close together and most of them are out of reach of any given point.
+// estep_pt_kernel (K <= 1024, 3-D; point-stationary): a block of 128 points stays in
+// the registers of two warps, which split the component pairs; every pair's parameters
+// come from shared memory as broadcasts, two components per packed operation
+// (FADD2/FMUL2/FFMA2).  Phase 1 takes e_nb = 2^(l_nb - cmax) and the per-point totals,
+// phase 2 the per-component statistics S0 = sum r, S1 = sum r y, S2 = sum r y y^T with
+// y = P'(x - mu_old), for the pairs that are live in the block.  The responsibility
+// matrix is never stored.  A pair out of reach of the block's box is skipped: its e is
+// exactly 0 for every point (ex2.approx.ftz returns +0 below 2^-126) and a zero term
+// changes no sum.  Points and components run in Morton order, so most pairs are out of
+// reach.  Larger K and 4-D: reach_kernels.cu; the gradient: adjoint_kernels.cu.
 #include <cxxabi.h>
 #include <float.h>
 #include <math.h>

@@ -1234,7 +1234,8 @@ gira_status gira_gmm_fit_batched(const float* points, const int64_t* offsets, in
                                   cudaMemcpyHostToDevice, c.s));
         // One launch per cluster size, side by side: each is a chain of K draws on a few SMs
         // (2 ms at K = 512), so one after another they left most of the chip idle (10.2 ms for
-        // 48 clouds of 2k .. 200k points in five sizes, 3.0 ms side by side).  The largest
+        // 48 clouds of 2k .. 200k points in five sizes; side by side the whole call without
+        // Lloyd and EM takes 3.0 ms).  The largest
         // clusters first: they need the most SMs of one GPC free.
         const int nclass = (int)seed_class.size();
         if (nclass > 1) {

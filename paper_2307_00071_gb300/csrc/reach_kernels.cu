@@ -27,7 +27,7 @@
 // The mode for gradients adds, in reach_estep_kernel, sum_b gamma Sigma_b^-1 (x' - mu_b)
 // per point from the live pairs, and the pose sums.
 //
-// Measured on GB300 (4M points of 16 posed frames, K = 8192): E-step 0.70 ms, statistics
+// Measured on GB300 (4M points of 16 posed frames, K = 8192): E-step 0.72 ms, statistics
 // 0.50 ms per iteration; the dense two-pass kernels over chunks of 512 components that
 // this replaced took 2 x 15.5 ms.  A call of two iterations with the final
 // log-likelihood: 79.2 -> 3.9 ms.

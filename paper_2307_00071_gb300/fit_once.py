@@ -5,7 +5,8 @@
 ``frame``: the 276k-point 640x480 depth frame, K=512, 30 iterations, tol 1e-4
 (the benchmark's step).  ``gmm20k``: 20k points from a K=8 GMM, 20 iterations.
 ``grad1024``: L and all gradients of a 100k-point scan under a K=1024 GMM of the
-frame (``--fits`` calls).  ``chunk2048``: the chunked E-step, K=2048 on the frame.
+frame (``--fits`` calls).  ``chunk2048``: the E-step above K=1024, K=2048 on the
+frame.
 ``frame4``: the frame with its intensity channel (N x 4), K=512, 30 iterations,
 tol 1e-4.  ``gbms``: mode seeking on the frame with intensity, bandwidth 0.05.
 Used under ncu, where a fixed, short launch sequence is wanted.
