@@ -1661,19 +1661,23 @@ __global__ void pack_pose_batched_kernel(const float* __restrict__ p3, int64_t n
 // instructions of 64 cycles; K exponentials on one SM take ~6 us), so every block takes
 // 32 components, one lane each, and repeats the softmax sums and the Morton ranks
 // (each component's rank is the count of smaller keys) instead of waiting for another
-// launch.  One block building all K = 1024 took 51 us.  blockIdx.y: instance.
+// launch.  One block building all K = 1024 took 51 us.  A batch that fills the GPU twice
+// that way takes 128 components per block, four warps' lanes: the repeated exponentials
+// were its binary64 work (16 models of K = 1024: 41 us with 32, 23 us with 128).
+// blockIdx.y: instance.
 constexpr int PFC_THREADS = 256;
-constexpr int PFC_COMPS = 32;   // components built per block
 __device__ __forceinline__ int ord_of(float f) {   // float -> int of the same order (atomicMax)
     const int b = __float_as_int(f);
     return b >= 0 ? b : b ^ 0x7fffffff;
 }
+template <int PFC_COMPS>   // components built per block
 __global__ void __launch_bounds__(PFC_THREADS) params_from_chol_kernel(
     const float* __restrict__ logits, const float* __restrict__ mu, const float* __restrict__ chol, int k,
     const BatchInst* __restrict__ insts, double* model64, float* params, float4* shift4, int* perm, float4* ctr,
     float2* aux, DeviceState* st) {
     __shared__ double s_red[PFC_THREADS / 32];
     __shared__ double s_max, s_lz;
+    __shared__ float s_max32[PFC_THREADS / 32];
     __shared__ float s_box[PFC_THREADS / 32][6];
     __shared__ unsigned long long s_key[MAX_K_DIRECT];
     __shared__ int s_slot[PFC_COMPS];
@@ -1699,11 +1703,11 @@ __global__ void __launch_bounds__(PFC_THREADS) params_from_chol_kernel(
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     // ---- softmax normaliser, bounding box of the means
     bool fin = true;
-    double m = -INFINITY;
+    float m = -INFINITY;   // of binary32 values: the binary64 pipe is not needed for it
     float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
     for (int b = t; b < k; b += PFC_THREADS) {
         fin = fin && isfinite(logits[b]);
-        m = fmax(m, (double)logits[b]);
+        m = fmaxf(m, logits[b]);
         for (int i = 0; i < 3; ++i) {
             lo[i] = fminf(lo[i], mu[3 * b + i]);
             hi[i] = fmaxf(hi[i], mu[3 * b + i]);
@@ -1712,7 +1716,7 @@ __global__ void __launch_bounds__(PFC_THREADS) params_from_chol_kernel(
     if (!fin) set_error(st, GIRA_ERR_NONFINITE_INPUT);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-        m = fmax(m, __shfl_xor_sync(FULL, m, o));
+        m = fmaxf(m, __shfl_xor_sync(FULL, m, o));
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
             lo[i] = fminf(lo[i], __shfl_xor_sync(FULL, lo[i], o));
@@ -1720,7 +1724,7 @@ __global__ void __launch_bounds__(PFC_THREADS) params_from_chol_kernel(
         }
     }
     if (lane == 0) {
-        s_red[warp] = m;
+        s_max32[warp] = m;
         for (int i = 0; i < 3; ++i) {
             s_box[warp][i] = lo[i];
             s_box[warp][3 + i] = hi[i];
@@ -1728,9 +1732,9 @@ __global__ void __launch_bounds__(PFC_THREADS) params_from_chol_kernel(
     }
     __syncthreads();
     if (t == 0) {
-        double v = s_red[0];
-        for (int w = 1; w < PFC_THREADS / 32; ++w) v = fmax(v, s_red[w]);
-        s_max = v;
+        float v = s_max32[0];
+        for (int w = 1; w < PFC_THREADS / 32; ++w) v = fmaxf(v, s_max32[w]);
+        s_max = (double)v;
     }
     float scale[3];
     for (int i = 0; i < 3; ++i) {
@@ -1761,8 +1765,9 @@ __global__ void __launch_bounds__(PFC_THREADS) params_from_chol_kernel(
         s_lz = amax + log(v);
     }
     // ---- the slots of this block's components: 8 lanes count the smaller keys of each
-    {
-        const int j = t >> 3, part = t & 7;
+#pragma unroll
+    for (int j0 = 0; j0 < PFC_COMPS; j0 += PFC_THREADS / 8) {
+        const int j = j0 + (t >> 3), part = t & 7;
         int cnt = 0;
         if (c0 + j < k) {
             const unsigned long long key = s_key[c0 + j];
@@ -1773,12 +1778,12 @@ __global__ void __launch_bounds__(PFC_THREADS) params_from_chol_kernel(
         if (part == 0) s_slot[j] = cnt;
     }
     __syncthreads();
-    if (warp != 0) return;
+    if (warp >= PFC_COMPS / 32) return;
     const double lz = s_lz;
-    const int b = c0 + lane;
+    const int b = c0 + t;
     float cc = -INFINITY;
     if (b < k) {
-        const int slot = perm ? s_slot[lane] : b;
+        const int slot = perm ? s_slot[t] : b;
         if (perm) perm[slot] = b;
         const float* L = chol + 9 * (size_t)b;
         const double m3[3] = {mu[3 * b], mu[3 * b + 1], mu[3 * b + 2]};
@@ -1807,7 +1812,7 @@ __global__ void __launch_bounds__(PFC_THREADS) params_from_chol_kernel(
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) cc = fmaxf(cc, __shfl_xor_sync(FULL, cc, o));
     if (lane == 0) atomicMax(&st->cmax_ord, ord_of(cc));
-    if (c0 == 0 && (k & 1) && lane < PAIR_FLOATS / 2) {   // the odd pair's padding component
+    if (c0 == 0 && (k & 1) && t < PAIR_FLOATS / 2) {   // the odd pair's padding component
         float* base = params + (size_t)(k >> 1) * PAIR_FLOATS + 1;
         base[2 * lane] = lane == SLOT_C ? -INFINITY : 0.f;
     }
@@ -1953,9 +1958,16 @@ cudaError_t launch_pack_pose(const float* pts3, int64_t n, const float* pose12, 
 cudaError_t launch_params_from_chol(const float* logits, const float* mu, const float* chol, int kmax,
                                     const BatchInst* insts, int batch, double* model64, float* params, float4* shift4,
                                     int* perm, float4* ctr, float2* aux, DeviceState* st, cudaStream_t s) {
-    const dim3 grid((kmax + PFC_COMPS - 1) / PFC_COMPS, insts ? batch : 1);
-    params_from_chol_kernel<<<grid, PFC_THREADS, 0, s>>>(logits, mu, chol, kmax, insts, model64, params, shift4, perm,
-                                                         ctr, aux, st);
+    const int nb = insts ? batch : 1;
+    if ((int64_t)((kmax + 31) / 32) * nb > 2 * 152) {
+        const dim3 grid((kmax + 127) / 128, nb);
+        params_from_chol_kernel<128><<<grid, PFC_THREADS, 0, s>>>(logits, mu, chol, kmax, insts, model64, params,
+                                                                  shift4, perm, ctr, aux, st);
+    } else {
+        const dim3 grid((kmax + 31) / 32, nb);
+        params_from_chol_kernel<32><<<grid, PFC_THREADS, 0, s>>>(logits, mu, chol, kmax, insts, model64, params,
+                                                                 shift4, perm, ctr, aux, st);
+    }
     return cudaGetLastError();
 }
 

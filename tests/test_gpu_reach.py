@@ -148,3 +148,33 @@ def test_regression_does_not_depend_on_the_order_of_the_locations(gira, frame, m
     re, rv = oracle.conditional4(locs[near], w, mu, cov)
     np.testing.assert_allclose(e[near], re, rtol=0, atol=2e-4)
     np.testing.assert_allclose(v[near], rv, rtol=2e-3, atol=2e-5)
+
+
+@pytest.mark.parametrize("ks", [[416] * 24, [33, 1024, 129, 512, 1, 128] * 10])
+def test_models_of_a_large_batch_equal_those_of_small_ones(gira, frame, ks):
+    """From 305 blocks of 32 components on (here K_max / 32 per instance) a batch of gradients builds
+    128 components per block: the same operations per component, so the same bits as in batches
+    below that, also for odd K and in the last warps."""
+    rng = np.random.default_rng(len(ks))
+    ns = [1100 + 7 * i for i in range(len(ks))]
+    assert (max(ks) + 31) // 32 * len(ks) > 304
+    pts = [frame[rng.choice(len(frame), n, replace=False)] for n in ns]
+    models = [ball_model(frame, k, rng) for k in ks]
+    lg = [np.log(w) for w, _, _ in models]
+    mu = [m for _, m, _ in models]
+    ch = [np.linalg.cholesky(c.astype(np.float64)).astype(np.float32) for _, _, c in models]
+    pose = np.tile(np.concatenate([np.eye(3).ravel(), [0.01, 0.0, 0.02]]).astype(np.float32), (len(ks), 1))
+
+    def call(a, b):
+        offs = np.concatenate([[0], np.cumsum(ns[a:b])]).astype(np.int64)
+        return gira.gira_gmm_loglik_grad_batched(
+            np.concatenate(pts[a:b]), offs, np.array(ks[a:b], np.int32), np.concatenate(lg[a:b]),
+            np.concatenate(mu[a:b]), np.concatenate(ch[a:b]), pose[a:b], want=("twist", "means"))
+
+    big = call(0, len(ks))
+    at = np.concatenate([[0], np.cumsum(ks)])
+    for a in range(0, len(ks), 6):
+        part = call(a, a + 6)
+        np.testing.assert_array_equal(np.asarray(part["loglik"]), np.asarray(big["loglik"])[a:a + 6])
+        np.testing.assert_array_equal(to_np(part["grad_twist"]), to_np(big["grad_twist"])[a:a + 6])
+        np.testing.assert_array_equal(to_np(part["grad_means"]), to_np(big["grad_means"])[at[a]:at[a + 6]])
