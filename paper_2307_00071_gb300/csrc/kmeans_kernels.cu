@@ -858,8 +858,11 @@ __global__ void __launch_bounds__(KC_THREADS, 1) kpp_cluster_kernel(const float4
 // holds the threshold scans its sub-block totals, then one sub-block's 32 weights.
 // What bounds it: the chain of one centre (an L2 round trip to update, the totals to every
 // CTA, the search, another round trip, the point to every CTA), not the points.  Measured
-// (GB300): 1M points of 4 frames, K = 768, 5.9 us per centre (two launches per centre:
-// 12.4); the 276,348-point frame with intensity, K = 512, 3.9 us (the persistent kernel: 8.3).
+// (GB300): 1M points of 4 frames, K = 768, 5.3 us per centre (two launches per centre:
+// 12.4; with one box test per lane in flight and the sub-block's warp by division: 5.9); the
+// 276,348-point frame with intensity, K = 512, 4.0 us (the persistent kernel: 8.3).  Of a centre's
+// 10,900 cycles at 1M points the tests take 1,050, the update 2,900, the totals of every CTA
+// 2,700, the search 1,300 and the point 2,900.
 template <int DIM>
 __device__ __forceinline__ float dist2_dim(float4 x, float4 c) {
     return DIM == 4 ? dist2_f32_4(x, c) : dist2_f32(x, c);
@@ -880,6 +883,7 @@ __device__ __forceinline__ void fx48_pieces(float d, unsigned& h, unsigned& m, u
 // shared memory per sub-block: box, total, largest D^2, list entry
 constexpr size_t kb_sub_bytes(int dim) { return (size_t)dim * 8 + sizeof(u128) + 4 + 2; }
 constexpr int KB_FLIGHT = 4;   // reached sub-blocks loaded at once
+constexpr int KB_Q_BITS = 12;  // list entry: warp << KB_Q_BITS | its sub-block
 
 template <int DIM>
 __global__ void __launch_bounds__(KC_THREADS, 1) kpp_blocks_kernel(const float4* __restrict__ pts, int64_t n, int k,
@@ -947,31 +951,44 @@ __global__ void __launch_bounds__(KC_THREADS, 1) kpp_blocks_kernel(const float4*
         const bool m64 = sh.m64 != 0;   // as in kpp_cluster_kernel
         // ---- 1. the sub-blocks within reach of the centre
         const float cv[4] = {cen.x, cen.y, cen.z, cen.w};
-        for (int r0 = 0; r0 < nsub; r0 += 32) {
-            const int q = r0 + lane;
-            bool in = false;
-            if (q < nsub) {
-                float e2 = 0.f;
+        for (int r0 = 0; r0 < nsub; r0 += 128) {   // four tests per lane in flight
+            unsigned m[4];
+            int found = 0;
 #pragma unroll
-                for (int c = 0; c < DIM; ++c) {
-                    const float e = fmaxf(fmaxf(box[c * ns + w0 + q] - cv[c], cv[c] - box[(DIM + c) * ns + w0 + q]), 0.f);
-                    e2 = fmaf(e, e, e2);
+            for (int u = 0; u < 4; ++u) {
+                const int q = r0 + 32 * u + lane;
+                bool in = false;
+                if (q < nsub) {
+                    float e2 = 0.f;
+#pragma unroll
+                    for (int c = 0; c < DIM; ++c) {
+                        const float e =
+                            fmaxf(fmaxf(box[c * ns + w0 + q] - cv[c], cv[c] - box[(DIM + c) * ns + w0 + q]), 0.f);
+                        e2 = fmaf(e, e, e2);
+                    }
+                    // (the slack covers the rounding of the box distance and of every D^2)
+                    in = e2 * (1.f - 1e-5f) <= dmax[w0 + q];
                 }
-                // (the slack covers the rounding of the box distance and of every D^2)
-                in = e2 * (1.f - 1e-5f) <= dmax[w0 + q];
+                m[u] = __ballot_sync(FULL, in);
+                found += __popc(m[u]);
             }
-            const unsigned m = __ballot_sync(FULL, in);
+            if (found == 0) continue;
             int base = 0;
-            if (lane == 0 && m) base = atomicAdd(&s_cnt[b], __popc(m));
+            if (lane == 0) base = atomicAdd(&s_cnt[b], found);
             base = __shfl_sync(FULL, base, 0);
-            if (in) list[base + __popc(m & ((1u << lane) - 1u))] = (uint16_t)(w0 + q);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (m[u] >> lane & 1u)
+                    list[base + __popc(m[u] & ((1u << lane) - 1u))] = (uint16_t)(warp << KB_Q_BITS | (r0 + 32 * u + lane));
+                base += __popc(m[u]);
+            }
         }
         __syncthreads();
         const int cnt = s_cnt[b];
         if (tid == 0) s_cnt[b ^ 1] = 0;   // free since the barrier: read before the previous centre's end
         if (cnt > 0) {
             for (int e0 = warp; e0 < cnt; e0 += KC_WARPS * KB_FLIGHT) {
-                int at[KB_FLIGHT];
+                int at[KB_FLIGHT], of[KB_FLIGHT];
                 float4 x[KB_FLIGHT];
                 float dn[KB_FLIGHT], dold[KB_FLIGHT];
                 int64_t i[KB_FLIGHT];
@@ -979,17 +996,17 @@ __global__ void __launch_bounds__(KC_THREADS, 1) kpp_blocks_kernel(const float4*
 #pragma unroll
                 for (int u = 0; u < KB_FLIGHT; ++u) {
                     const int e = e0 + u * KC_WARPS;
-                    at[u] = e < cnt ? (int)list[e] : -1;
-                    // sub-block at[u] % nsb of warp at[u] / nsb
-                    const int w = max(at[u], 0) / nsb;
-                    i[u] = ((int64_t)(w * cs + me) * nsb + (max(at[u], 0) - w * nsb)) * 32 + lane;
-                    ok[u] = at[u] >= 0 && i[u] < n;
+                    const int v = e < cnt ? (int)list[e] : -1, q = v & ((1 << KB_Q_BITS) - 1);
+                    of[u] = v >> KB_Q_BITS;   // the sub-block's warp, -1: none
+                    at[u] = of[u] * nsb + q;
+                    i[u] = ((int64_t)(of[u] * cs + me) * nsb + q) * 32 + lane;
+                    ok[u] = v >= 0 && i[u] < n;
                     x[u] = ok[u] ? __ldg(pts + i[u]) : make_float4(0.f, 0.f, 0.f, 0.f);
                     dold[u] = (ok[u] && j > 1) ? d2[i[u]] : INFINITY;
                 }
 #pragma unroll
                 for (int u = 0; u < KB_FLIGHT; ++u) {
-                    if (at[u] < 0) continue;
+                    if (of[u] < 0) continue;
                     dn[u] = ok[u] ? fminf(dold[u], dist2_dim<DIM>(x[u], cen)) : 0.f;
                     const bool low = ok[u] && dn[u] < dold[u];
                     if (low) d2[i[u]] = dn[u];
@@ -1008,7 +1025,7 @@ __global__ void __launch_bounds__(KC_THREADS, 1) kpp_blocks_kernel(const float4*
                     const unsigned mx = __reduce_max_sync(FULL, __float_as_uint(dn[u]));   // D^2 >= 0
                     if (lane == 0) {   // the block's total by the difference (mod 2^128: any order)
                         const u128 dt = u128_sub(t, tot[at[u]]);
-                        unsigned long long* wt = s_wtot[at[u] / nsb];
+                        unsigned long long* wt = s_wtot[of[u]];
                         const unsigned long long was = atomicAdd(&wt[0], dt.lo);
                         const unsigned long long up = dt.hi + (was + dt.lo < was ? 1ull : 0ull);
                         if (up) atomicAdd(&wt[1], up);
@@ -1676,6 +1693,8 @@ int kpp_blocks_per_warp(int64_t n, int dim) {
     }
     const int64_t nsb = ((n + 31) / 32 + KC_MAX_CS * KC_WARPS - 1) / (KC_MAX_CS * KC_WARPS);
     if (!ok || nsb > INT_MAX / 64 || kb_smem_bytes(dim, (int)nsb) > KB_SMEM_MAX) return 0;
+    static_assert(KC_WARPS <= 16 && KB_SMEM_MAX / (KC_WARPS * kb_sub_bytes(3)) < (1u << KB_Q_BITS),
+                  "a list entry holds the warp and its sub-block");
     return (int)nsb;
 }
 
