@@ -1434,7 +1434,12 @@ gira_status gira_gmm_loglik_grad_batched(const float* points, const int64_t* off
         if (a.p) TRY(check_ptr(a.p, a.name, c.dev, &a.k));
     for (auto& a : out)
         if (a.p) TRY(check_ptr(a.p, a.name, c.dev, &a.k));
-    const bool dense = grad_chol != nullptr;   // every component (adjoint_kernels.cu says why); else reach lists
+    // Every component (adjoint_kernels.cu) when the Cholesky factors' gradient is asked for (it
+    // says why), and for at most 64 components of up to 500,000 points together: the dense kernel
+    // holds 64 in one warp's lanes, and sorting the points for the reach lists costs more than the
+    // lists save (2 scans of 71,000 points together, K = 64: 234 us dense, 268 by lists; 16 of
+    // 468,000: 309 and 316; K = 128: 275 and 273, 484 and 332).
+    const bool dense = grad_chol || (*std::max_element(ks, ks + batch) <= 64 && total_n <= 500000);
     const bool gpar = !dense && (grad_logits || grad_means);
     const bool sorted = !dense && total_n <= point_order_max_n();
 

@@ -178,3 +178,24 @@ def test_models_of_a_large_batch_equal_those_of_small_ones(gira, frame, ks):
         np.testing.assert_array_equal(np.asarray(part["loglik"]), np.asarray(big["loglik"])[a:a + 6])
         np.testing.assert_array_equal(to_np(part["grad_twist"]), to_np(big["grad_twist"])[a:a + 6])
         np.testing.assert_array_equal(to_np(part["grad_means"]), to_np(big["grad_means"])[at[a]:at[a + 6]])
+
+
+@pytest.mark.parametrize("k,n", [(64, 3000), (65, 3000), (64, 260_000)])
+def test_batched_gradient_on_both_sides_of_the_dense_rule(gira, frame, k, n):
+    """Two scans of at most 64 components and 500,000 points together take the dense kernel, others
+    the reach lists; the same gradients as the single calls, which are dense: sums of n binary32
+    terms in another order (a few 1e-6 of the sum of magnitudes, bounded by 2e-5 of the largest)."""
+    rng = np.random.default_rng(k + n)
+    pts = frame[rng.choice(len(frame), n, replace=False)]
+    w, mu, cov = ball_model(frame, k, rng, sigma=0.2)
+    lg, ch = np.log(w), np.linalg.cholesky(cov.astype(np.float64)).astype(np.float32)
+    want = ("twist", "means", "points")
+    one = gira.gira_gmm_loglik_grad(pts, lg, mu, ch, None, want=want)
+    two = gira.gira_gmm_loglik_grad_batched(np.concatenate([pts, pts]), np.array([0, n, 2 * n], np.int64),
+                                            np.array([k, k], np.int32), np.concatenate([lg, lg]),
+                                            np.concatenate([mu, mu]), np.concatenate([ch, ch]), want=want)
+    assert two["loglik"][1] == pytest.approx(one["loglik"], rel=1e-6)
+    for key, rows in (("grad_twist", 1), ("grad_means", k), ("grad_points", n)):
+        a = to_np(one[key]).astype(np.float64)
+        b = to_np(two[key]).astype(np.float64).reshape(2, *a.shape)[1]
+        assert np.max(np.abs(a - b)) <= 2e-5 * np.max(np.abs(a)), key
