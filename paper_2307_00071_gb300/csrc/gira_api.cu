@@ -1435,11 +1435,13 @@ gira_status gira_gmm_loglik_grad_batched(const float* points, const int64_t* off
     for (auto& a : out)
         if (a.p) TRY(check_ptr(a.p, a.name, c.dev, &a.k));
     // Every component (adjoint_kernels.cu) when the Cholesky factors' gradient is asked for (it
-    // says why), and for at most 64 components of up to 500,000 points together: the dense kernel
-    // holds 64 in one warp's lanes, and sorting the points for the reach lists costs more than the
-    // lists save (2 scans of 71,000 points together, K = 64: 234 us dense, 268 by lists; 16 of
-    // 468,000: 309 and 316; K = 128: 275 and 273, 484 and 332).
-    const bool dense = grad_chol || (*std::max_element(ks, ks + batch) <= 64 && total_n <= 500000);
+    // says why), and for little dense work: sorting the points for the reach lists then costs more
+    // than the lists save.  The dense kernel holds 64 components in one warp's lanes; above 256 its
+    // batches of points wait longer.  Dense and by lists, us: 2 scans of 12,800 points together,
+    // K = 128: 195, 247; 2 of 71,000, K = 64: 219, 268; 4 of 57,000, K = 256: 249, 274; 8 of 90,000,
+    // K = 128: 254, 270; the other way, 8 of 260,000, K = 128: 380, 309; 2 of 12,800, K = 512: 324, 272.
+    const int kbig = *std::max_element(ks, ks + batch);
+    const bool dense = grad_chol || (kbig <= 256 && total_n <= (kbig <= 64 ? 500000 : 16000000 / kbig));
     const bool gpar = !dense && (grad_logits || grad_means);
     const bool sorted = !dense && total_n <= point_order_max_n();
 

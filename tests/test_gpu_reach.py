@@ -180,10 +180,10 @@ def test_models_of_a_large_batch_equal_those_of_small_ones(gira, frame, ks):
         np.testing.assert_array_equal(to_np(part["grad_means"]), to_np(big["grad_means"])[at[a]:at[a + 6]])
 
 
-@pytest.mark.parametrize("k,n", [(64, 3000), (65, 3000), (64, 260_000)])
+@pytest.mark.parametrize("k,n", [(64, 3000), (65, 200_000), (64, 260_000), (256, 3000), (257, 3000)])
 def test_batched_gradient_on_both_sides_of_the_dense_rule(gira, frame, k, n):
-    """Two scans of at most 64 components and 500,000 points together take the dense kernel, others
-    the reach lists; the same gradients as the single calls, which are dense: sums of n binary32
+    """Batches of little dense work (at most 64 components and 500,000 points together, or 256 and
+    16M pairs) take the dense kernel, others the reach lists; the same gradients as the single calls, which are dense: sums of n binary32
     terms in another order (a few 1e-6 of the sum of magnitudes, bounded by 2e-5 of the largest)."""
     rng = np.random.default_rng(k + n)
     pts = frame[rng.choice(len(frame), n, replace=False)]
