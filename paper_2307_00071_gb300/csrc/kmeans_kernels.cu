@@ -1009,7 +1009,7 @@ __global__ void __launch_bounds__(KC_THREADS, 1) kpp_blocks_kernel(const float4*
                     if (of[u] < 0) continue;
                     dn[u] = ok[u] ? fminf(dold[u], dist2_dim<DIM>(x[u], cen)) : 0.f;
                     const bool low = ok[u] && dn[u] < dold[u];
-                    if (low) d2[i[u]] = dn[u];
+                    if (low || (j == 1 && ok[u])) d2[i[u]] = dn[u];   // the first centre writes every point's, +inf too
                     if (!__any_sync(FULL, low) && j > 1) continue;   // no D^2 dropped
                     u128 t{0ull, 0ull};
                     if (__any_sync(FULL, !(dn[u] < 1024.f))) {   // a weight >= 2^10: sum in 128 bits

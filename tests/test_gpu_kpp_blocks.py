@@ -62,3 +62,25 @@ def test_lloyd_4d(gira, frames, n, k, lloyd):
     for key in ("means", "covs"):
         got, want = np.asarray(r[key], np.float64), np.asarray(ref[key], np.float64)
         assert np.all(np.abs(got - want) <= 2e-7 * np.abs(want).max() + 1e-12), key
+
+
+@pytest.mark.parametrize("dim,n,far", [(3, 300_001, [(7, 3e38)]), (3, 294_913, [(294_912, -1e20), (40, 1e20)]),
+                                       (4, 5_000, [(4_999, 2e19)]), (4, 70_001, [(33, 1e20), (69_000, -1e20), (1, 3e38)])])
+def test_overflowing_distances(gira, frames, dim, n, far):
+    """Points so far away that D^2 is +inf (weight 2^95 - 1): drawn first, whatever an earlier call left in
+    the workspace.  Bits in 3-D; in 4-D the counts, with every far point alone in its cluster."""
+    pts = frames[:n] if dim == 3 else np.concatenate([frames[:n], synth.frame_intensity(frames[:n])[:, None]], axis=1)
+    pts = pts.astype(np.float32)   # a copy
+    k = 6
+    other = np.repeat((np.arange(n, dtype=np.float32) % 977)[:, None], 4, axis=1)
+    gira.gira_gmm_fit4(other, 4, iters=0, reg_covar=1e-3, final_loglik=False)   # other D^2 in the workspace
+    for at, value in far:
+        pts[at, at % dim] = value
+    if dim == 3:
+        assert np.array_equal(seeds(gira, pts, k, 5), oracle.kmeanspp(pts, k, 5)[0].astype(np.float32))
+        return
+    r = gira.gira_gmm_fit4(pts, k, iters=0, seed=5, lloyd_iters=0, reg_covar=1e-3, final_loglik=False)
+    ref = oracle.kinit(pts, k, 5, 0, 1e-3)
+    want = np.bincount(ref["labels"], minlength=k)
+    assert sum(want == 1) >= len(far)
+    assert np.array_equal(np.rint(np.asarray(r["weights"], np.float64) * n), want)
