@@ -119,11 +119,12 @@ __device__ __forceinline__ uint32_t spread6(uint32_t v) {   // bit i -> bit 3 i
     return v;
 }
 
-// key = (instance << 18) | Morton code of the point in its instance's bounding
-// cube (cells of the largest extent / 64 on every axis); idx = the point
+// key = (instance << bits) | the upper `bits` bits (key_code_bits) of the Morton code of the
+// point in its instance's bounding cube (cells of the largest extent / 64 on every axis);
+// idx = the point
 __global__ void __launch_bounds__(256) key_kernel(const float4* __restrict__ p8, int64_t n,
                                                   const int64_t* __restrict__ offs, const int2* __restrict__ units,
-                                                  const int* __restrict__ box, uint32_t* keys, int* idx) {
+                                                  const int* __restrict__ box, int bits, uint32_t* keys, int* idx) {
     const Span s = span_of(offs, units, n);
     const int* bb = box + 6 * s.inst;
     const float lo[3] = {float_of(bb[0]), float_of(bb[1]), float_of(bb[2])};
@@ -139,7 +140,7 @@ __global__ void __launch_bounds__(256) key_kernel(const float4* __restrict__ p8,
             const float q = fminf(63.f, fmaxf(0.f, floorf((c[j] - lo[j]) * scale)));
             code |= spread6((uint32_t)q) << j;
         }
-        keys[i] = ((uint32_t)s.inst << MORTON_BITS) | code;
+        keys[i] = ((uint32_t)s.inst << bits) | (code >> (MORTON_BITS - bits));
         idx[i] = (int)i;
     }
 }
@@ -384,11 +385,15 @@ __global__ void __launch_bounds__(256) cell_place_kernel(int64_t n, const int* _
 
 int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
-int radix_passes(int batch) {
-    int bits = MORTON_BITS;
-    while (batch > 1 && (1 << (bits - MORTON_BITS)) < batch) ++bits;
-    return (int)ceil_div(bits, RADIX_BITS);
+int instance_bits(int batch) {
+    int bits = 0;
+    while ((int64_t(1) << bits) < batch) ++bits;
+    return bits;
 }
+// Bits of the Morton code in a 32-bit key: all 18 up to 16,384 instances, then what the
+// instance leaves (many instances have few points each, which need no finer order).
+int key_code_bits(int batch) { return std::min(MORTON_BITS, 32 - instance_bits(batch)); }
+int radix_passes(int batch) { return (int)ceil_div(instance_bits(batch) + key_code_bits(batch), RADIX_BITS); }
 
 }  // namespace
 
@@ -470,7 +475,7 @@ cudaError_t launch_point_order(const float4* p8, int64_t n, const int64_t* offse
     box_init_kernel<<<(unsigned)ceil_div(6 * (int64_t)batch, 256), 256, 0, s>>>(box, batch);
     const int blocks = units_d ? nunits : (int)ceil_div(n, BOX_CHUNK);
     box_kernel<<<blocks, 256, 0, s>>>(p8, n, offsets_d, units_d, box);
-    key_kernel<<<blocks, 256, 0, s>>>(p8, n, offsets_d, units_d, box, k0, i0);
+    key_kernel<<<blocks, 256, 0, s>>>(p8, n, offsets_d, units_d, box, key_code_bits(batch), k0, i0);
     const int passes = radix_passes(batch);
     const unsigned tblocks = (unsigned)ceil_div(ntiles, 8);
     int *iin = i0, *iout = i1;

@@ -74,3 +74,34 @@ def test_batch_keeps_instances_in_place():
              for i, n in enumerate(sizes)]
     offs = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
     run(np.concatenate(parts), offs)
+
+
+@pytest.mark.parametrize("batch", [16_384, 16_385, 70_000])
+def test_many_instances(batch):
+    """Above 16,384 instances the 32-bit keys hold the upper bits of the Morton code only: every point stays
+    in its instance, in the (stable) order of those."""
+    from paper_2307_00071_gb300 import gira
+    rng = np.random.default_rng(batch)
+    sizes = rng.integers(1, 6, size=batch)
+    offs = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    pts = rng.normal(size=(offs[-1], 3)).astype(np.float32)
+    got = gira.gira_test_point_order(torch.as_tensor(pts, device="cuda"), offs).cpu().numpy()
+    drop = 18 - min(18, 32 - int(np.ceil(np.log2(batch))))
+    want = [a + np.argsort(codes(pts[a:b]) >> drop, kind="stable") for a, b in zip(offs[:-1], offs[1:])]
+    np.testing.assert_array_equal(got, np.concatenate(want))
+
+
+def test_fits_of_many_instances():
+    """One component per cloud: the mean and covariance of each cloud's own points."""
+    from paper_2307_00071_gb300 import gira
+    batch, n = 20_000, 4
+    pts = np.random.default_rng(3).normal(size=(batch, n, 3)).astype(np.float32)
+    r = gira.gira_gmm_fit_batched(pts.reshape(-1, 3), (np.arange(batch + 1) * n).astype(np.int64),
+                                  np.ones(batch, np.int32), iters=1, tol=0.0, reg_covar=1e-2)
+    x = pts.astype(np.float64)
+    mean = x.mean(1)
+    d = x - mean[:, None]
+    cov = np.einsum("bni,bnj->bij", d, d) / n + 1e-2 * np.eye(3)
+    # whitened binary32 sums of four terms: ~10 roundings of values up to about 5 (25 squared)
+    assert np.abs(np.asarray(r["means"]).reshape(batch, 3) - mean).max() <= 10 * 5 * 2.0 ** -23
+    assert np.abs(np.asarray(r["covs"]).reshape(batch, 3, 3) - cov).max() <= 10 * 25 * 2.0 ** -23
