@@ -1664,7 +1664,7 @@ __global__ void pack_pose_batched_kernel(const float* __restrict__ p3, int64_t n
 // launch.  One block building all K = 1024 took 51 us.  A batch that fills the GPU twice
 // that way takes 128 components per block, four warps' lanes: the repeated exponentials
 // were its binary64 work (16 models of K = 1024: 41 us with 32, 23 us with 128).
-// blockIdx.y: instance.
+// blockIdx.x: instance (a grid's other dimensions end at 65,535).
 constexpr int PFC_THREADS = 256;
 __device__ __forceinline__ int ord_of(float f) {   // float -> int of the same order (atomicMax)
     const int b = __float_as_int(f);
@@ -1682,7 +1682,7 @@ __global__ void __launch_bounds__(PFC_THREADS) params_from_chol_kernel(
     __shared__ unsigned long long s_key[MAX_K_DIRECT];
     __shared__ int s_slot[PFC_COMPS];
     if (insts) {
-        const BatchInst I = insts[blockIdx.y];
+        const BatchInst I = insts[blockIdx.x];
         const size_t c = I.comp_off;
         k = I.k;
         logits += c;
@@ -1696,9 +1696,9 @@ __global__ void __launch_bounds__(PFC_THREADS) params_from_chol_kernel(
             ctr += c;
             aux += c;
         }
-        st += blockIdx.y;
+        st += blockIdx.x;
     }
-    const int c0 = blockIdx.x * PFC_COMPS;
+    const int c0 = blockIdx.y * PFC_COMPS;
     if (c0 >= k) return;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     // ---- softmax normaliser, bounding box of the means
@@ -1960,11 +1960,11 @@ cudaError_t launch_params_from_chol(const float* logits, const float* mu, const 
                                     int* perm, float4* ctr, float2* aux, DeviceState* st, cudaStream_t s) {
     const int nb = insts ? batch : 1;
     if ((int64_t)((kmax + 31) / 32) * nb > 2 * 152) {
-        const dim3 grid((kmax + 127) / 128, nb);
+        const dim3 grid(nb, (kmax + 127) / 128);
         params_from_chol_kernel<128><<<grid, PFC_THREADS, 0, s>>>(logits, mu, chol, kmax, insts, model64, params,
                                                                   shift4, perm, ctr, aux, st);
     } else {
-        const dim3 grid((kmax + 31) / 32, nb);
+        const dim3 grid(nb, (kmax + 31) / 32);
         params_from_chol_kernel<32><<<grid, PFC_THREADS, 0, s>>>(logits, mu, chol, kmax, insts, model64, params,
                                                                  shift4, perm, ctr, aux, st);
     }

@@ -921,7 +921,7 @@ __global__ void __launch_bounds__(RG_THREADS) reach_grad_finalize_kernel(const R
     int k = f_in.k, slices = f_in.slices, ctas = f_in.grid;
     int64_t n = f_in.n;
     size_t c_off = 0, part_off = 0, live_off = 0, ll_off = 0, par_off = 0;
-    const int inst = blockIdx.y;
+    const int inst = blockIdx.x;   // (a grid's other dimensions end at 65,535)
     if (insts) {
         const BatchInst I = insts[inst];
         int sl;
@@ -937,7 +937,7 @@ __global__ void __launch_bounds__(RG_THREADS) reach_grad_finalize_kernel(const R
     }
     DeviceState* const st = f_in.st + inst;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const int npairs = (k + 1) >> 1, pair0 = blockIdx.x * RG_PAIRS;
+    const int npairs = (k + 1) >> 1, pair0 = blockIdx.y * RG_PAIRS;
     if (pair0 >= npairs || st->error) return;
     if (f_in.partials) {
         const int pp = pair0 + t / (2 * NSTAT), v = t % (2 * NSTAT);
@@ -977,7 +977,7 @@ __global__ void __launch_bounds__(RG_THREADS) reach_grad_finalize_kernel(const R
             if (f_in.g_logits) f_in.g_logits[c_off + src_b] = (float)(S[0] - (double)n * f_in.model64[(c_off + b) * MODEL]);
         }
     }
-    if (blockIdx.x != 0 || warp != 1) return;
+    if (blockIdx.y != 0 || warp != 1) return;
     // log-likelihood and pose sums, fixed order
     double v[13] = {};
     for (int c = lane; c < ctas; c += 32) {
@@ -1024,7 +1024,7 @@ __global__ void __launch_bounds__(RG_THREADS) reach_grad_finalize_kernel(const R
 // f.k: the largest k of a batch.  Without parameter gradients one block per instance.
 cudaError_t launch_reach_grad_finalize(const ReachGradArgs& f, const BatchInst* insts, int batch, cudaStream_t s) {
     const int blocks = f.partials ? ((f.k + 1) / 2 + RG_PAIRS - 1) / RG_PAIRS : 1;
-    reach_grad_finalize_kernel<<<dim3(blocks, insts ? batch : 1), RG_THREADS, 0, s>>>(f, insts);
+    reach_grad_finalize_kernel<<<dim3(insts ? batch : 1, blocks), RG_THREADS, 0, s>>>(f, insts);
     return cudaGetLastError();
 }
 

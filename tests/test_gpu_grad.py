@@ -334,3 +334,28 @@ def test_registration_k1024_second_scan_of_the_scene(gira, offset_seed):
     ang = math.degrees(math.acos(np.clip((np.trace(dR) - 1) / 2, -1, 1)))
     dt = np.linalg.norm(t + R_off.T @ t_off)
     assert ang < 0.5 and dt < 0.02, (ang, dt, ll)
+
+
+@pytest.mark.parametrize("points", [2, 8])
+def test_batch_beyond_65535_instances(gira, points):
+    """More instances than a grid's second dimension holds, over both evaluations (every component up to
+    500,000 points, reach lists above): value and twist of every instance by the definition."""
+    batch = 65_700
+    rng = np.random.default_rng(points)
+    pts = rng.normal(size=(batch * points, 3)).astype(np.float32)
+    mu = rng.normal(size=(batch, 3)).astype(np.float32)
+    chol = np.zeros((batch, 3, 3), np.float32)
+    chol[:, [0, 1, 2], [0, 1, 2]] = rng.uniform(0.5, 2.0, size=(batch, 3)).astype(np.float32)
+    offs = (np.arange(batch + 1) * points).astype(np.int64)
+    r = gira.gira_gmm_loglik_grad_batched(pts, offs, np.ones(batch, np.int32), np.zeros(batch, np.float32), mu, chol,
+                                          want=("twist",))
+    x = pts.reshape(batch, points, 3).astype(np.float64)
+    s = chol[:, [0, 1, 2], [0, 1, 2]].astype(np.float64)[:, None]
+    y = (x - mu[:, None]) / s
+    ll = (-0.5 * (y ** 2).sum(2) - np.log(s).sum(2) - 1.5 * np.log(2 * np.pi)).sum(1)
+    g = -y / s
+    twist = np.concatenate([np.cross(x, g).sum(1), g.sum(1)], axis=1)
+    # per point ~20 roundings of values up to |q| (y to 10): 2^-24 * 20 * 100 * points
+    tol = 20 * 100 * points * 2.0 ** -24
+    assert np.abs(np.asarray(r["loglik"]) - ll).max() <= tol
+    assert np.abs(np.asarray(r["grad_twist"]).reshape(batch, 6) - twist).max() <= 4 * tol
