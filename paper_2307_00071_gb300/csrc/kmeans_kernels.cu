@@ -1574,13 +1574,32 @@ cudaError_t launch_kpp_persistent(const float4* pts4, int64_t n, int k, uint64_t
     return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(KPPP_THREADS), args, 0, s);
 }
 
+namespace {
+// What find() gives on the current device, asked once on each: function attributes and what
+// fits belong to a device.  (Racing first calls find the same.)
+constexpr int DEVICES = 64;
+template <class F>
+int per_device(std::atomic<int> (&found)[DEVICES], F find) {   // found: 0 not asked, else find() + 1
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= DEVICES) {
+        cudaGetLastError();
+        return find();
+    }
+    int v = found[dev].load();
+    if (v == 0) {
+        v = find() + 1;
+        found[dev].store(v);
+    }
+    return v - 1;
+}
+}  // namespace
+
 // Cluster size for the one-cluster seeding of n points, or 0 when it does not
 // apply (too many points, or no cluster of that size fits on this GPU).
 int kpp_cluster_size(int64_t n) {
-    static std::atomic<int> cached_size{-1};   // largest usable cluster size (one GPU model per process)
-    int cached = cached_size.load();
-    if (cached < 0) {
-        cached = 0;
+    static std::atomic<int> found[DEVICES];   // largest usable cluster size
+    const int largest = per_device(found, [] {
+        int best = 0;
         const size_t smem = kc_smem_bytes();
         if (cudaFuncSetAttribute(kpp_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) ==
                 cudaSuccess &&
@@ -1601,16 +1620,16 @@ int kpp_cluster_size(int64_t n) {
                 int nclusters = 0;
                 if (cudaOccupancyMaxActiveClusters(&nclusters, kpp_cluster_kernel, &cfg) == cudaSuccess &&
                     nclusters >= 1) {
-                    cached = cs;
+                    best = cs;
                     break;
                 }
             }
         }
         cudaGetLastError();
-        cached_size.store(cached);   // racing first calls compute the same value
-    }
-    if (cached == 0 || n > (int64_t)cached * KC_THREADS * KC_LMAX) return 0;
-    return cached;
+        return best;
+    });
+    if (largest == 0 || n > (int64_t)largest * KC_THREADS * KC_LMAX) return 0;
+    return largest;
 }
 
 cudaError_t launch_kpp_cluster_batched(const float4* pts4, const KppInst* table, int clusters, uint64_t seed,
@@ -1675,22 +1694,21 @@ constexpr size_t KB_SMEM_MAX = 224 * 1024;
 // Sub-blocks per warp for the one-cluster seeding of n points in L2, or 0 when it does not
 // apply (too many points, or a cluster of 16 does not fit on this GPU).
 int kpp_blocks_per_warp(int64_t n, int dim) {
-    static std::atomic<int> usable{-1};
-    int ok = usable.load();
-    if (ok < 0) {
-        ok = 1;
-        for (int d = 3; d <= 4 && ok; ++d) {
+    static std::atomic<int> found[DEVICES];
+    const int ok = per_device(found, [] {
+        int usable = 1;
+        for (int d = 3; d <= 4 && usable; ++d) {
             const void* fn = d == 3 ? (const void*)kpp_blocks_kernel<3> : (const void*)kpp_blocks_kernel<4>;
             cudaLaunchAttribute at[1];
             const cudaLaunchConfig_t cfg = kb_config(KC_MAX_CS, KB_SMEM_MAX, at, nullptr);
             int nclusters = 0;
-            ok = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)KB_SMEM_MAX) == cudaSuccess &&
-                 cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-                 cudaOccupancyMaxActiveClusters(&nclusters, fn, &cfg) == cudaSuccess && nclusters >= 1;
+            usable = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)KB_SMEM_MAX) == cudaSuccess &&
+                     cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+                     cudaOccupancyMaxActiveClusters(&nclusters, fn, &cfg) == cudaSuccess && nclusters >= 1;
         }
         cudaGetLastError();
-        usable.store(ok);   // racing first calls compute the same value
-    }
+        return usable;
+    });
     const int64_t nsb = ((n + 31) / 32 + KC_MAX_CS * KC_WARPS - 1) / (KC_MAX_CS * KC_WARPS);
     if (!ok || nsb > INT_MAX / 64 || kb_smem_bytes(dim, (int)nsb) > KB_SMEM_MAX) return 0;
     static_assert(KC_WARPS <= 16 && KB_SMEM_MAX / (KC_WARPS * kb_sub_bytes(3)) < (1u << KB_Q_BITS),
