@@ -303,11 +303,10 @@ __global__ void rebuild_components4_kernel(const double* __restrict__ old, const
     build_component4(slot, r[0], r + 1, S, params, model64, st, b);
 }
 
-__global__ void params_from_model4_kernel(const float* __restrict__ w, const float* __restrict__ mu,
-                                          const float* __restrict__ cov, int k, double* model64, float* params,
-                                          DeviceState* st) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= k) return;
+// Component b of a given model; whether it was built.
+__device__ bool build_from_model4(const float* __restrict__ w, const float* __restrict__ mu,
+                                  const float* __restrict__ cov, int b, double* model64, float* params,
+                                  DeviceState* st) {
     const double pi = w[b];
     double m[4], S[16];
     bool fin = isfinite(pi);
@@ -322,9 +321,23 @@ __global__ void params_from_model4_kernel(const float* __restrict__ w, const flo
             fin = fin && isfinite(v);
             S[4 * i + j] = S[4 * j + i] = v;
         }
-    if (!fin) { set_error(st, GIRA_ERR_NONFINITE_INPUT); return; }
-    if (!(pi > 0.0)) { set_error(st, GIRA_ERR_INVALID_ARG); return; }
-    build_component4(b, pi, m, S, params, model64, st, b);
+    if (!fin) { set_error(st, GIRA_ERR_NONFINITE_INPUT); return false; }
+    if (!(pi > 0.0)) { set_error(st, GIRA_ERR_INVALID_ARG); return false; }
+    return build_component4(b, pi, m, S, params, model64, st, b);
+}
+
+__global__ void params_from_model4_kernel(const float* __restrict__ w, const float* __restrict__ mu,
+                                          const float* __restrict__ cov, int k, double* model64, float* params,
+                                          float4* ctr, float2* aux, DeviceState* st) {
+    const int b = blockIdx.x * blockDim.x + threadIdx.x;
+    float c = -INFINITY;
+    if (b < k && build_from_model4(w, mu, cov, b, model64, params, st) && ctr) {
+        const float* m = mu + 4 * (size_t)b;
+        c = params[slot4(b, SLOT4_C)];
+        ctr[b] = make_float4(m[0], m[1], m[2], m[3]);
+        aux[b] = f2(c, params[slot4(b, SLOT4_S)]);
+    }
+    if (ctr) raise_cmax(st, c);
 }
 
 __global__ void model_out4_kernel(const double* __restrict__ model64, int k, float* w, float* mu, float* cov,
@@ -1197,8 +1210,8 @@ cudaError_t launch_order_components4(double* model64, double* scratch, int k, in
 }
 
 cudaError_t launch_params_from_model4(const float* w, const float* mu, const float* cov, int k, double* model64,
-                                      float* params, DeviceState* st, cudaStream_t s) {
-    params_from_model4_kernel<<<(k + 63) / 64, 64, 0, s>>>(w, mu, cov, k, model64, params, st);
+                                      float* params, float4* ctr, float2* aux, DeviceState* st, cudaStream_t s) {
+    params_from_model4_kernel<<<(k + 63) / 64, 64, 0, s>>>(w, mu, cov, k, model64, params, ctr, aux, st);
     return cudaGetLastError();
 }
 

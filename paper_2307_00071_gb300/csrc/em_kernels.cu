@@ -1398,7 +1398,8 @@ __global__ void __launch_bounds__(MP_THREADS) model_points_kernel(const float* _
                                                                   const float* __restrict__ mu,
                                                                   const float* __restrict__ cov, int k, int slots,
                                                                   int nbuild, double* model64, float* params,
-                                                                  float4* shift4, DeviceState* st) {
+                                                                  float4* shift4, float4* ctr, float2* aux,
+                                                                  DeviceState* st) {
     if ((int)blockIdx.x >= nbuild) {
         const int64_t i = (int64_t)(blockIdx.x - nbuild) * MP_THREADS + threadIdx.x;
         if (i < n && !pack_point(p3, i, nullptr, p8)) atomicExch(&st->error, GIRA_ERR_NONFINITE_INPUT);
@@ -1410,16 +1411,27 @@ __global__ void __launch_bounds__(MP_THREADS) model_points_kernel(const float* _
         return;
     }
     const int b = blockIdx.x * 32 + threadIdx.x;
-    if (b >= k) return;
-    const double pi = w[b];
-    const double m[3] = {mu[3 * b], mu[3 * b + 1], mu[3 * b + 2]};
-    const float* S = cov + 9 * (size_t)b;
-    const double c[6] = {S[0], S[3], S[6], S[4], S[7], S[8]};   // lower triangle, as the oracle reads it
-    bool fin = isfinite(pi) && isfinite(m[0]) && isfinite(m[1]) && isfinite(m[2]);
-    for (int i = 0; i < 9; ++i) fin = fin && isfinite(S[i]);
-    if (!fin) { set_error(st, GIRA_ERR_NONFINITE_INPUT); return; }
-    if (!(pi > 0.0)) { set_error(st, GIRA_ERR_INVALID_ARG); return; }
-    build_component(b, pi, m, c, params, shift4, model64, st, b);
+    float cc = -INFINITY;
+    if (b < k) {
+        const double pi = w[b];
+        const double m[3] = {mu[3 * b], mu[3 * b + 1], mu[3 * b + 2]};
+        const float* S = cov + 9 * (size_t)b;
+        const double c[6] = {S[0], S[3], S[6], S[4], S[7], S[8]};   // lower triangle, as the oracle reads it
+        bool fin = isfinite(pi) && isfinite(m[0]) && isfinite(m[1]) && isfinite(m[2]);
+        for (int i = 0; i < 9; ++i) fin = fin && isfinite(S[i]);
+        if (!fin) {
+            set_error(st, GIRA_ERR_NONFINITE_INPUT);
+        } else if (!(pi > 0.0)) {
+            set_error(st, GIRA_ERR_INVALID_ARG);
+        } else if (build_component(b, pi, m, c, params, shift4, model64, st, b) && ctr) {
+            const float* base = params + (size_t)(b >> 1) * PAIR_FLOATS + (b & 1);
+            const float s2 = base[2 * SLOT_S];
+            cc = base[2 * SLOT_C];
+            ctr[b] = make_float4((float)m[0], (float)m[1], (float)m[2], s2);
+            aux[b] = f2(cc, s2);
+        }
+    }
+    if (ctr) raise_cmax(st, cc);
 }
 
 // ------------------------------------------------------------------ batched helpers
@@ -1666,10 +1678,6 @@ __global__ void pack_pose_batched_kernel(const float* __restrict__ p3, int64_t n
 // were its binary64 work (16 models of K = 1024: 41 us with 32, 23 us with 128).
 // blockIdx.x: instance (a grid's other dimensions end at 65,535).
 constexpr int PFC_THREADS = 256;
-__device__ __forceinline__ int ord_of(float f) {   // float -> int of the same order (atomicMax)
-    const int b = __float_as_int(f);
-    return b >= 0 ? b : b ^ 0x7fffffff;
-}
 template <int PFC_COMPS>   // components built per block
 __global__ void __launch_bounds__(PFC_THREADS) params_from_chol_kernel(
     const float* __restrict__ logits, const float* __restrict__ mu, const float* __restrict__ chol, int k,
@@ -1809,9 +1817,7 @@ __global__ void __launch_bounds__(PFC_THREADS) params_from_chol_kernel(
             }
         }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) cc = fmaxf(cc, __shfl_xor_sync(FULL, cc, o));
-    if (lane == 0) atomicMax(&st->cmax_ord, ord_of(cc));
+    raise_cmax(st, cc);
     if (c0 == 0 && (k & 1) && t < PAIR_FLOATS / 2) {   // the odd pair's padding component
         float* base = params + (size_t)(k >> 1) * PAIR_FLOATS + 1;
         base[2 * lane] = lane == SLOT_C ? -INFINITY : 0.f;
@@ -1891,10 +1897,10 @@ cudaError_t launch_ll_reduce_batched(const double* ll_partials, const BatchInst*
 
 cudaError_t launch_model_points(const float* pts3, int64_t n, float4* pts8, const float* w, const float* mu,
                                 const float* cov, int k, int npairs_pad, double* model64, float* params,
-                                float4* shift4, DeviceState* st, cudaStream_t s) {
+                                float4* shift4, float4* ctr, float2* aux, DeviceState* st, cudaStream_t s) {
     const int nbuild = (k + 31) / 32;
     model_points_kernel<<<(unsigned)(nbuild + (n + MP_THREADS - 1) / MP_THREADS), MP_THREADS, 0, s>>>(
-        pts3, n, pts8, w, mu, cov, k, 2 * npairs_pad, nbuild, model64, params, shift4, st);
+        pts3, n, pts8, w, mu, cov, k, 2 * npairs_pad, nbuild, model64, params, shift4, ctr, aux, st);
     return cudaGetLastError();
 }
 

@@ -404,12 +404,15 @@ cudaError_t reach_estep_stats(int d, const ReachBufs& b, ReachLaunch a, long lon
     return e;
 }
 
-// The log-likelihood alone: a.per_point (nullable) and st->ll_sum.
-cudaError_t reach_loglik(int d, const ReachBufs& b, const ReachLaunch& a, long long* launches, cudaStream_t s) {
-    cudaError_t e = launch_reach_prepare(d, a.params, a.k, a.st, a.iter, b.ctr, b.aux, b.gref, s);
+// The log-likelihood alone: a.per_point (nullable) and st->ll_sum.  given: the launch that built
+// the model wrote the compact arrays and st->cmax_ord.
+cudaError_t reach_loglik(int d, const ReachBufs& b, ReachLaunch a, bool given, long long* launches, cudaStream_t s) {
+    cudaError_t e = cudaSuccess;
+    if (given) a.gref = nullptr;
+    else e = launch_reach_prepare(d, a.params, a.k, a.st, a.iter, b.ctr, b.aux, b.gref, s);
     if (e == cudaSuccess) e = launch_estep_reach(d, a, 0, b.grid, b.h, a.k, s);
     if (e == cudaSuccess) e = launch_ll_reduce(b.llp, b.grid, a.st, s);
-    *launches += 3;
+    *launches += given ? 2 : 3;
     return e;
 }
 
@@ -677,7 +680,7 @@ gira_status gira_gmm_fit(const float* points, int64_t n, int k, const gira_fit_o
         if (kc == Kind::Host)
             GIRA_CUDA(cudaMemcpyAsync(b.mcov, covs, sizeof(float) * 9 * k, cudaMemcpyHostToDevice, c.s));
         COUNTED(prof, 1, launch_model_points(pts, n, b.p8, w_d, mu_d, cov_d, k, npairs, b.model64, b.params, b.shift4,
-                                             b.st, c.s));
+                                             nullptr, nullptr, b.st, c.s));
     }
     if (sorted)
         COUNTED(prof, point_order_launches(1),
@@ -711,7 +714,7 @@ gira_status gira_gmm_fit(const float* points, int64_t n, int k, const gira_fit_o
         }
         prof.t_em = prof.mark();
         if (final_loglik)
-            GIRA_CUDA(reach_loglik(3, rb, reach_launch(rb, pe, n, k, b.params, b.st, 0), &prof.launches, c.s));
+            GIRA_CUDA(reach_loglik(3, rb, reach_launch(rb, pe, n, k, b.params, b.st, 0), false, &prof.launches, c.s));
     }
     EStepLaunch a{sorted ? b.p8s : b.p8, n, k, b.params, b.partials, b.llp, nullptr, b.st, 0};
     a.n_buf = n;
@@ -819,6 +822,7 @@ gira_status gira_gmm_loglik(const float* points, int64_t n, int k, const float* 
     DeviceState h{};
     h.stop_after = 0;
     h.bad_component = INT_MAX;
+    h.cmax_ord = CMAX_ORD_NONE;
     GIRA_CUDA(cudaMemcpyAsync(b.st, &h, sizeof h, cudaMemcpyHostToDevice, c.s));
     const float* pts = points;
     if (kp == Kind::Host) {
@@ -842,13 +846,13 @@ gira_status gira_gmm_loglik(const float* points, int64_t n, int k, const float* 
     }
     float* ppd = per_point ? ((kpp == Kind::Device) ? per_point : b.pp) : nullptr;
     COUNTED(prof, 1, launch_model_points(pts, n, b.p8, w_d, mu_d, cov_d, k, npairs, b.model64, b.params, b.shift4,
-                                         b.st, c.s));
+                                         large ? rb.ctr : nullptr, rb.aux, b.st, c.s));
     prof.t_init = prof.mark();
     prof.t_em = prof.t_init;
     if (large) {
         ReachLaunch a = reach_launch(rb, b.p8, n, k, b.params, b.st, 0);
         a.per_point = ppd;
-        GIRA_CUDA(reach_loglik(3, rb, a, &prof.launches, c.s));
+        GIRA_CUDA(reach_loglik(3, rb, a, true, &prof.launches, c.s));
     } else {
         EStepLaunch a{b.p8, n, k, b.params, nullptr, b.llp, ppd, b.st, 0};
         a.n_buf = n;
@@ -1852,7 +1856,7 @@ gira_status gira_gmm_fit4(const float* points, int64_t n, int k, const gira_fit_
             GIRA_CUDA(cudaMemcpyAsync(b.mmu, means, sizeof(float) * 4 * k, cudaMemcpyHostToDevice, c.s));
         if (kc == Kind::Host)
             GIRA_CUDA(cudaMemcpyAsync(b.mcov, covs, sizeof(float) * 16 * k, cudaMemcpyHostToDevice, c.s));
-        COUNTED(prof, 1, launch_params_from_model4(w_d, mu_d, cov_d, k, b.model64, b.params, b.st, c.s));
+        COUNTED(prof, 1, launch_params_from_model4(w_d, mu_d, cov_d, k, b.model64, b.params, nullptr, nullptr, b.st, c.s));
     }
     // components in Morton order of their means, as in the 3-D fit
     COUNTED(prof, 2, launch_order_components4(b.model64, b.stats64, k, b.perm, b.params, b.st, c.s));
@@ -1870,7 +1874,7 @@ gira_status gira_gmm_fit4(const float* points, int64_t n, int k, const gira_fit_
     }
     prof.t_em = prof.mark();
     if (final_loglik)
-        GIRA_CUDA(reach_loglik(4, rb, reach_launch(rb, pe, n, k, b.params, b.st, 0), &prof.launches, c.s));
+        GIRA_CUDA(reach_loglik(4, rb, reach_launch(rb, pe, n, k, b.params, b.st, 0), false, &prof.launches, c.s));
     COUNTED(prof, 1, launch_model_out4(b.model64, k, w_d, mu_d, cov_d, b.perm, b.st, c.s));
     if (kw == Kind::Host) GIRA_CUDA(cudaMemcpyAsync(weights, b.mw, sizeof(float) * k, cudaMemcpyDeviceToHost, c.s));
     if (km == Kind::Host) GIRA_CUDA(cudaMemcpyAsync(means, b.mmu, sizeof(float) * 4 * k, cudaMemcpyDeviceToHost, c.s));
@@ -1938,6 +1942,7 @@ gira_status gira_gmm_loglik4(const float* points, int64_t n, int k, const float*
     DeviceState h{};
     h.stop_after = 0;
     h.bad_component = INT_MAX;
+    h.cmax_ord = CMAX_ORD_NONE;
     GIRA_CUDA(cudaMemcpyAsync(b.st, &h, sizeof h, cudaMemcpyHostToDevice, c.s));
     const float* pts = points;
     if (kp == Kind::Host) {
@@ -1961,13 +1966,13 @@ gira_status gira_gmm_loglik4(const float* points, int64_t n, int k, const float*
     }
     COUNTED(prof, 1, launch_pack4(pts, n, nullptr, b.p8, b.st, c.s));
     COUNTED(prof, 1, launch_fill_padding4(b.params, k, c.s));
-    COUNTED(prof, 1, launch_params_from_model4(w_d, mu_d, cov_d, k, b.model64, b.params, b.st, c.s));
+    COUNTED(prof, 1, launch_params_from_model4(w_d, mu_d, cov_d, k, b.model64, b.params, rb.ctr, rb.aux, b.st, c.s));
     prof.t_init = prof.mark();
     prof.t_em = prof.t_init;
     float* ppd = per_point ? ((kpp == Kind::Device) ? per_point : b.pp) : nullptr;
     ReachLaunch a = reach_launch(rb, b.p8, n, k, b.params, b.st, 0);
     a.per_point = ppd;
-    GIRA_CUDA(reach_loglik(4, rb, a, &prof.launches, c.s));
+    GIRA_CUDA(reach_loglik(4, rb, a, true, &prof.launches, c.s));
     if (per_point && kpp == Kind::Host)
         GIRA_CUDA(cudaMemcpyAsync(per_point, b.pp, sizeof(float) * n, cudaMemcpyDeviceToHost, c.s));
     GIRA_CUDA(cudaMemcpyAsync(&h, b.st, sizeof h, cudaMemcpyDeviceToHost, c.s));

@@ -47,11 +47,19 @@ struct DeviceState {
     // evaluations made (pairs within reach of the warp's box) and with statistics
     unsigned long long pairs_near, pairs_live;
     int coherent;          // k-means++: the points' order keeps neighbours together (launch_kpp_coherence)
-    int cmax_ord;          // gradient: max_b c_b as an order-preserving int (host: that of -inf)
+    int cmax_ord;          // given models: max_b c_b as an order-preserving int (host: that of -inf)
 };
 constexpr int CMAX_ORD_NONE = (int)0x807fffff;   // -inf
 
 __device__ __forceinline__ void set_error(DeviceState* st, int code) { atomicCAS(&st->error, 0, code); }
+
+// Raise st->cmax_ord to the largest c of a warp's lanes (-inf: none).  Called by whole warps.
+__device__ __forceinline__ void raise_cmax(DeviceState* st, float c) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) c = fmaxf(c, __shfl_xor_sync(0xffffffffu, c, o));
+    const int b = __float_as_int(c);
+    if ((threadIdx.x & 31) == 0) atomicMax(&st->cmax_ord, b >= 0 ? b : b ^ 0x7fffffff);
+}
 
 // Index checks of the debug build (-DGIRA_DEBUG): GIRA_IN(cond, st) is cond, and a
 // false cond records GIRA_ERR_BOUNDS in st (the caller skips the access).  In
@@ -448,9 +456,10 @@ struct ReachLaunch {
     int64_t n;
     int k;
     const float* params;     // pair-interleaved
-    const float4* ctr;       // compact per-component arrays and references of launch_reach_prepare
+    const float4* ctr;       // compact per-component arrays and references of launch_reach_prepare,
+                             // or the arrays of the launch that built a given model
     const float2* aux;
-    const float* gref;       // nullptr (gradient): max_b c_b from st->cmax_ord
+    const float* gref;       // nullptr (given models): max_b c_b from st->cmax_ord
     double* llp;             // [grid] log-likelihood partials
     float* per_point;        // mode 0: [n] natural-log lse, or nullptr
     DeviceState* st;
@@ -586,9 +595,10 @@ cudaError_t launch_estep_pt(const EStepLaunch& a, bool stats, int grid, cudaStre
 cudaError_t launch_estep_pt_units(const EStepLaunch& a, bool stats, int nunits, int kmax, cudaStream_t s);
 int estep_pt_points();   // points per CTA
 int estep_pt_blocks();   // point blocks per CTA (partial and mask rows per CTA)
+// ctr, aux (nullable): the compact arrays of the reach tests, and max_b c_b in st->cmax_ord.
 cudaError_t launch_model_points(const float* pts3, int64_t n, float4* pts8, const float* w, const float* mu,
                                 const float* cov, int k, int npairs_pad, double* model64, float* params,
-                                float4* shift4, DeviceState* st, cudaStream_t s);
+                                float4* shift4, float4* ctr, float2* aux, DeviceState* st, cudaStream_t s);
 // perm (nullable): slot s of model64 is the caller's component perm[s].
 cudaError_t launch_model_out(const double* model64, int k, float* w, float* mu, float* cov, const DeviceState* st,
                              cudaStream_t s, const int* perm = nullptr);
@@ -803,8 +813,9 @@ cudaError_t launch_reduce_finalize4(const float* partials, const uint32_t* live2
 // Components in Morton order of their means, as launch_order_components (scratch: k * MODEL4 doubles).
 cudaError_t launch_order_components4(double* model64, double* scratch, int k, int* perm, float* params,
                                      DeviceState* st, cudaStream_t s);
+// ctr, aux (nullable): as launch_model_points.
 cudaError_t launch_params_from_model4(const float* w, const float* mu, const float* cov, int k, double* model64,
-                                      float* params, DeviceState* st, cudaStream_t s);
+                                      float* params, float4* ctr, float2* aux, DeviceState* st, cudaStream_t s);
 cudaError_t launch_model_out4(const double* model64, int k, float* w, float* mu, float* cov, const int* perm,
                               const DeviceState* st, cudaStream_t s);
 // Lloyd in four dimensions and the one-hot statistics about the final centres.

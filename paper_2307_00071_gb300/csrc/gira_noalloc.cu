@@ -140,7 +140,8 @@ extern "C" gira_status gira_gmm_loglik_noalloc(const float* points, int64_t n, i
     h.stop_after = 0;
     h.bad_component = INT_MAX;
     NA_CUDA(cudaMemcpyAsync(st, &h, sizeof h, cudaMemcpyHostToDevice, s));
-    NA_CUDA(launch_model_points(points, n, p8, weights, means, covs, k, npairs, model64, params, shift4, st, s));
+    NA_CUDA(launch_model_points(points, n, p8, weights, means, covs, k, npairs, model64, params, shift4,
+                                nullptr, nullptr, st, s));
     EStepLaunch a{p8, n, k, params, nullptr, llp, per_point, st, 0};
     a.n_buf = n;
     NA_CUDA(launch_estep_pt(a, false, grid, s));

@@ -27,6 +27,11 @@
 // The mode for gradients adds, in reach_estep_kernel, sum_b gamma Sigma_b^-1 (x' - mu_b)
 // per point from the live pairs, and the pose sums.
 //
+// The lists want neighbours in a block: fits and gradients sort the points, the log-likelihood
+// takes them as they come (a sensor's order keeps neighbours together; sorting is 60-100 us).
+// In no order every pair is listed and the lists are overhead; per call (276,348 points) in
+// sensor order and shuffled: K = 2048 199 and 387 us, K = 8192 501 and 1,443; 4-D, K = 512 149
+// and 199, K = 2048 282 and 538.  Dense kernels took 465, 1,477, 214 and 550 us in any order.
 // Measured on GB300 (4M points of 16 posed frames, K = 8192): E-step 0.72 ms, statistics
 // 0.50 ms per iteration; the dense two-pass kernels over chunks of 512 components that
 // this replaced took 2 x 15.5 ms.  A call of two iterations with the final
@@ -46,7 +51,8 @@ constexpr float LN2F = 0.693147180559945309f;
 constexpr double LN2 = 0.693147180559945309417232121458;
 constexpr int RB_P = 4;                    // points per lane
 constexpr int RB_PTS = 32 * RB_P;          // points per block (a row of the masks)
-constexpr int RB_W = 4;                    // warps per CTA
+constexpr int RB_W = 4;                    // warps per CTA, or those of one block where they are more
+__host__ __device__ constexpr int cta_warps(int h) { return h > RB_W ? h : RB_W; }
 constexpr float REACH = 128.f;             // q' above which a component is out of reach (e = 0 from q' > 126)
 
 template <int D>
@@ -228,18 +234,22 @@ __device__ __forceinline__ bool pair_reaches(const float2 (&s)[Lay<D>::PF / 2], 
 }
 
 // ------------------------------------------------------------------ the E-step
-// Shared memory: the CTA's surviving pairs by warp quarter and class (pp % H), every
+// Shared memory: the CTA's surviving pairs by warp and class (pp % H), every
 // warp's listed pairs, every warp's live-mask words.
-__host__ __device__ constexpr int reach_pairs(int k) { return (((k + 1) / 2) + 127) & ~127; }   // quarters of whole warps
+__host__ __device__ constexpr int reach_pairs(int k, int h) {   // as many whole warps of pairs as the CTA has warps
+    const int step = 32 * cta_warps(h);
+    return ((k + 1) / 2 + step - 1) / step * step;
+}
 __host__ __device__ constexpr int reach_words(int k) { return (((k + 1) / 2) + 31) / 32; }
 __host__ __device__ constexpr size_t reach_smem(int k, int h) {
-    return (size_t)reach_pairs(k) * 2 + (size_t)RB_W * (reach_pairs(k) / h) * 2 + (size_t)RB_W * reach_words(k) * 4;
+    return (size_t)reach_pairs(k, h) * 2 + (size_t)cta_warps(h) * (reach_pairs(k, h) / h) * 2 +
+           (size_t)cta_warps(h) * reach_words(k) * 4;
 }
 
 // The barrier of block blk's H warps.
 template <int H>
 __device__ __forceinline__ void block_sync(int blk) {
-    if (H == RB_W) {
+    if (H >= RB_W) {
         __syncthreads();
     } else if (blk == 0) {
         asm volatile("bar.sync 1, %0;" ::"n"(32 * H) : "memory");
@@ -253,16 +263,18 @@ __device__ __forceinline__ void block_sync(int blk) {
 // 16 registrations 763 against 698 us).
 // MODE 0: log-likelihood; 1: also (shift, 1 / total) and the masks for reach_stats_kernel;
 // 2: the gradient (the masks only when a.masks).  H warps share a block's pairs (pp % H):
-// 2 for large inputs, 4 where 256-point CTAs would leave SMs idle.
+// 2 for large inputs, 4 where 256-point CTAs would leave SMs idle, 8 or 16 for the
+// log-likelihood of few blocks (launch_estep_reach).
 template <int D, int H, int MODE>
-__global__ void __launch_bounds__(32 * RB_W, D == 3 && MODE != 2 ? 5 : 4) estep_reach_kernel(const ReachLaunch a_in) {
+__global__ void __launch_bounds__(32 * cta_warps(H), H > RB_W ? 16 / H : D == 3 && MODE != 2 ? 5 : 4)
+    estep_reach_kernel(const ReachLaunch a_in) {
     extern __shared__ __align__(16) unsigned char dsm[];
-    constexpr int B = RB_W / H;   // blocks per CTA
-    static_assert(B * H == RB_W && B <= 2, "one named barrier per block");
-    __shared__ float s_box[RB_W][2 * D];
-    __shared__ float2 s_tot[RB_W][RB_P][32];
-    __shared__ float s_ub[RB_W];
-    __shared__ int s_cnt[RB_W][H];
+    constexpr int W = cta_warps(H), B = W / H;   // warps and blocks per CTA
+    static_assert(B * H == W && B <= 2 && (32 % H) == 0, "one named barrier per block, lanes in classes");
+    __shared__ float s_box[W][2 * D];
+    __shared__ float2 s_tot[W][RB_P][32];
+    __shared__ float s_ub[W];
+    __shared__ int s_cnt[W][H];
     __shared__ double s_ll[B];
     __shared__ int s_skip;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -293,10 +305,10 @@ __global__ void __launch_bounds__(32 * RB_W, D == 3 && MODE != 2 ? 5 : 4) estep_
     const float4* const ctr4 = a_in.ctr + comp_off;
     const float2* const aux = a_in.aux + comp_off;
     const int npairs = (k + 1) >> 1;
-    const int nquarter = reach_pairs(k) / RB_W, ncap = reach_pairs(k) / H, nwords = reach_words(k);
-    uint16_t* slist0 = reinterpret_cast<uint16_t*>(dsm);                        // [RB_W][H][nquarter / H]
-    uint16_t* slist = slist0 + reach_pairs(k) + (size_t)warp * ncap;          // this warp's listed pairs
-    uint32_t* smask_all = reinterpret_cast<uint32_t*>(slist0 + reach_pairs(k) + (size_t)RB_W * ncap);
+    const int nall = reach_pairs(k, H), nshare = nall / W, ncap = nall / H, nwords = reach_words(k);
+    uint16_t* slist0 = reinterpret_cast<uint16_t*>(dsm);          // [W][H][nshare / H]
+    uint16_t* slist = slist0 + nall + (size_t)warp * ncap;        // this warp's listed pairs
+    uint32_t* smask_all = reinterpret_cast<uint32_t*>(slist0 + nall + (size_t)W * ncap);
     uint32_t* smask = smask_all + warp * nwords;
     // a slot beyond n holds a point 1e18 m away, where every q' is +inf and e exactly 0
     const int64_t row = (int64_t)cta * B + blk;
@@ -362,10 +374,10 @@ __global__ void __launch_bounds__(32 * RB_W, D == 3 && MODE != 2 ? 5 : 4) estep_
             }
         }
         int cnt = 0;   // lanes of class c keep the count of their class: lane % H == pp % H
-        const uint32_t cls = H == 2 ? 0x55555555u << (lane & 1) : 0x11111111u << (lane & 3);
-        uint16_t* dst = slist0 + warp * nquarter + (lane % H) * (nquarter / H);
-        for (int j0 = 0; j0 < nquarter; j0 += 32) {
-            const int pp = warp * nquarter + j0 + lane;
+        const uint32_t cls = (H == 2 ? 0x55555555u : H == 4 ? 0x11111111u : H == 8 ? 0x01010101u : 0x00010001u) << (lane % H);
+        uint16_t* dst = slist0 + warp * nshare + (lane % H) * (nshare / H);
+        for (int j0 = 0; j0 < nshare; j0 += 32) {
+            const int pp = warp * nshare + j0 + lane;
             bool live = false;
 #pragma unroll
             for (int m = 0; m < 2; ++m) {
@@ -409,8 +421,8 @@ __global__ void __launch_bounds__(32 * RB_W, D == 3 && MODE != 2 ? 5 : 4) estep_
         nlive += __popc(m);
     };
     if (lo[0] <= hi[0]) {
-        for (int w = 0; w < RB_W; ++w) {
-            const uint16_t* src = slist0 + w * nquarter + half * (nquarter / H);
+        for (int w = 0; w < W; ++w) {
+            const uint16_t* src = slist0 + w * nshare + half * (nshare / H);
             const int cnt = s_cnt[w][half];
             for (int i0 = 0; i0 < cnt; i0 += 32) {
                 const int pp = i0 + lane < cnt ? (int)src[i0 + lane] : -1;
@@ -846,12 +858,19 @@ __global__ void __launch_bounds__(32 * ST_W) reach_stats_kernel(const ReachLaunc
     }
 }
 
+static_assert(reach_smem(GIRA_MAX_K, 2) <= 40 * 1024 && reach_smem(GIRA_MAX_K, 4) <= 40 * 1024 &&
+                  reach_smem(GIRA_MAX_K, 8) <= 36 * 1024 && reach_smem(GIRA_MAX_K, 16) <= 28 * 1024 &&
+                  GIRA_MAX_K4 <= GIRA_MAX_K,
+              "with the static arrays (5, 5, 10 and 19 KB) within the 48 KB a launch has unasked");
+
 template <int D, int H>
 const void* reach_fn(int mode) {
-    if (mode == 0) return (const void*)estep_reach_kernel<D, H, 0>;
-    if constexpr (D == 3)   // the gradient is 3-D
-        if (mode == 2) return (const void*)estep_reach_kernel<D, H, 2>;
-    return (const void*)estep_reach_kernel<D, H, 1>;
+    if constexpr (H <= RB_W) {
+        if constexpr (D == 3)   // the gradient is 3-D
+            if (mode == 2) return (const void*)estep_reach_kernel<D, H, 2>;
+        if (mode == 1) return (const void*)estep_reach_kernel<D, H, 1>;
+    }
+    return (const void*)estep_reach_kernel<D, H, 0>;
 }
 
 }  // namespace
@@ -860,6 +879,11 @@ const void* reach_fn(int mode) {
 // pairs in parallel, twice the CTAs) up to 8 blocks per SM.  Measured, two against four:
 // the gradient of 100k points at K = 1024 924 / 905 us per call, a map of 4M points at
 // K = 8192 6.1 / 7.0 ms, its first test then being made twice as often.
+// The log-likelihood alone of few blocks under many components takes as many warps as an SM's
+// registers hold, sixteen for one block or eight for each of two: four warps walk a block's
+// thousands of pairs alone.  Per call, shuffled points: 8,192 at K = 8192 337 us with four warps,
+// 152 with sixteen; 20,000 at K = 8192 350 and (eight) 263; up to K = 1024 no difference.
+constexpr int RB_FEW_BLOCKS = 152, RB_FEW_K = 1024;
 int reach_h(int64_t n) { return n > 152 * 8 * RB_PTS ? 2 : 4; }
 int reach_points(int h) { return RB_W / h * RB_PTS; }
 int reach_grid(int64_t n) {
@@ -880,12 +904,13 @@ cudaError_t launch_reach_prepare(int d, const float* params, int k, const Device
 cudaError_t launch_estep_reach(int d, const ReachLaunch& a, int mode, int grid, int h, int kmax, cudaStream_t s) {
     const void* fn = d == 3 ? (h == 2 ? reach_fn<3, 2>(mode) : reach_fn<3, 4>(mode))
                             : (h == 2 ? reach_fn<4, 2>(mode) : reach_fn<4, 4>(mode));
+    if (mode == 0 && h == 4 && grid <= 2 * RB_FEW_BLOCKS && kmax > RB_FEW_K) {   // one block per CTA, as with four
+        h = grid <= RB_FEW_BLOCKS ? 16 : 8;
+        fn = d == 3 ? (h == 8 ? reach_fn<3, 8>(0) : reach_fn<3, 16>(0)) : (h == 8 ? reach_fn<4, 8>(0) : reach_fn<4, 16>(0));
+    }
     note_estep_kernel(fn);
-    const size_t smem = reach_smem(kmax, h);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
     void* args[] = {(void*)&a};
-    return cudaLaunchKernel(fn, dim3(grid), dim3(32 * RB_W), args, smem, s);
+    return cudaLaunchKernel(fn, dim3(grid), dim3(32 * cta_warps(h)), args, reach_smem(kmax, h), s);
 }
 
 cudaError_t launch_reach_stats(int d, const ReachLaunch& a, float* partials, cudaStream_t s) {

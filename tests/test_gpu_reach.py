@@ -199,3 +199,26 @@ def test_batched_gradient_on_both_sides_of_the_dense_rule(gira, frame, k, n):
         a = to_np(one[key]).astype(np.float64)
         b = to_np(two[key]).astype(np.float64).reshape(2, *a.shape)[1]
         assert np.max(np.abs(a - b)) <= 2e-5 * np.max(np.abs(a)), key
+
+
+@pytest.mark.parametrize("d", [3, 4])
+@pytest.mark.parametrize("n,k,off", [(1_025, 1_025, 0), (8_193, 8_192, 40), (38_912, 1_101, 300), (38_913, 1_101, 300),
+                                     (2_000, 511, 7), (2_000, 512, 7), (2_000, 1_537, 1_999)])
+def test_shuffled_scores(gira, frame, d, n, k, off):
+    """The log-likelihood of points in no order, where a block's box is the whole scene: sixteen warps share
+    a block up to 304 blocks (from 512 components), four above.  Points off the model take the exact maximum."""
+    rng = np.random.default_rng(n + k)
+    full = np.concatenate([frame, synth.frame_intensity(frame)[:, None]], axis=1)[:, :d]
+    pts, at = off_model(np.ascontiguousarray(full[rng.integers(0, len(full) - n) + np.arange(n)]), off, rng) if off else (
+        np.ascontiguousarray(full[:n]), np.zeros(0, np.int64))
+    w, m, c = ball_model(full, k, rng, d=d)
+    order = rng.permutation(n)
+    call = gira.gira_gmm_loglik if d == 3 else gira.gira_gmm_loglik4
+    mean, pp = call(np.ascontiguousarray(pts[order]), w, m, c, per_point=True)
+    back = np.empty(n)
+    back[order] = to_np(pp)
+    assert mean == pytest.approx(back.mean(), rel=1e-6)
+    sample = np.unique(np.concatenate([at[:100], [0, n - 1], rng.choice(n, min(n, 200), replace=False)]))
+    _, _, lse = oracle.estep(pts[sample], w, m, c, want_resp=False, want_lse=True)
+    err, bound = np.abs(back[sample] - lse), per_point_bound(pts[sample], w, m, c, form="d" if d == 4 else "b")
+    assert np.all(err <= bound), np.max(err / bound)
