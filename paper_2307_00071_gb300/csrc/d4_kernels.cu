@@ -10,8 +10,9 @@
 // the joint distribution.
 //
 // The E-step and its statistics are reach_kernels.cu with D = 4 (logits from d = x - mu_b:
-// intensity and metre-scale coordinates share a point); here are the M-step, KInit's
-// Lloyd iterations and one-hot statistics, the regression and the sampling.
+// intensity and metre-scale coordinates share a point), or, for little work, the dense
+// kernel here; also the M-step, KInit's Lloyd iterations and one-hot statistics, the
+// regression and the sampling.
 #include <float.h>
 #include <math.h>
 
@@ -39,6 +40,210 @@ constexpr double LOG2_2PI4 = 2.6514961294723187980;   // log2(2 pi)
 // squared entries: lambda_max <= ||Sigma||_F (and >= half of it).
 __device__ __forceinline__ float sigma_min_sq_bound4(double fro2) {
     return (float)(ALPHA4 * ALPHA4) / (sqrtf((float)fro2) * (1.f + 1e-4f)) * (1.f - 1e-4f);
+}
+
+// ------------------------------------------------------------------ the E-step of little work
+// Every component at every point, statistics in the same pass: the lists of reach_kernels.cu
+// (prepare, E-step, statistics over them, one launch each) save nothing where the dense work
+// is a few microseconds.  One CTA holds all K <= 1024 components, one pair per lane; all lanes
+// walk the CTA's points (staged by one TMA bulk copy) together, eight at a time: pass 1
+// forms e and the per-point sums over lanes and warps, pass 2 the statistics about y = P'(x - mu)
+// of both components, packed.  Rows [cta][pairs][2 NSTAT4], every one written.
+// Bound by the chain of a batch (the sums cross the warps) and, per launch, by latency.
+// Measured: 6 us an iteration for 2,000 points at K = 64, where the lists' prepare, E-step and
+// statistics take 5, 10 and 16; a call of 20 iterations 1,168 -> 546 us (both sides of the rule
+// at estep4_dense).
+constexpr int Q4 = 8;                             // points per batch
+constexpr int PPC4_MAX = 1024;                    // points staged per CTA (32 KB)
+constexpr long long MBAR_LIMIT4 = 2000000000ll;   // bound on the TMA wait: 2 s of wall time
+constexpr float LN2F4 = 0.693147180559945309f;
+constexpr double LN2_4 = 0.693147180559945309417232121458;
+
+template <bool STATS>
+__global__ void __launch_bounds__(512, 1) estep4_dense_kernel(const EStep4Launch a) {
+    extern __shared__ __align__(128) unsigned char dsm4[];
+    __shared__ __align__(8) uint64_t bar_tma;
+    __shared__ float red_sum[2][16][Q4];   // by parity of the batch: one barrier per batch
+    __shared__ float red_aux[2][16][Q4];
+    __shared__ float s_cmax[16], s_wsum[16];
+    __shared__ int s_skip, s_norm, s_dead;
+    constexpr int LPQ = 32 / Q4;
+    const int G = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int pr = threadIdx.x, npairs = (a.k + 1) >> 1;   // this lane's pair
+    const int64_t begin = (int64_t)blockIdx.x * a.pts_per_cta;
+    const int npts = (int)(min(a.n, begin + a.pts_per_cta) - begin);
+    const float4* spts = reinterpret_cast<const float4*>(dsm4);   // (x,x,y,y)(z,z,w,w) per point
+    if (threadIdx.x == 0) {
+        // the points are never written by the kernel this one may overlap
+        // (dependent launch), so their copy starts before the wait below
+        mbar_init(&bar_tma, 1);
+        mbar_fence_init();
+        mbar_expect_tx(&bar_tma, (uint32_t)npts * 32u);
+        tma_load_1d(reinterpret_cast<void*>(dsm4), a.pts8 + 2 * begin, (uint32_t)npts * 32u, &bar_tma);
+    }
+    pdl_wait();   // the parameters and the state written by the previous kernel
+    if (threadIdx.x == 0) {
+        s_skip = (a.iter > a.st->stop_after) || (a.st->error != 0);
+        s_norm = a.st->w_raw;
+        s_dead = 0;
+    }
+    __syncthreads();
+    if (s_skip) {   // let the copy land before leaving
+        if (threadIdx.x == 0) mbar_wait_bounded(&bar_tma, 0u, MBAR_LIMIT4);
+        return;
+    }
+    pdl_allow_next();
+    // ---- this lane's pair (lanes beyond the last: c = -inf, never contribute)
+    float2 P[10], nmu[4], c = dup(-INFINITY), w = dup(0.f);
+#pragma unroll
+    for (int i = 0; i < 10; ++i) P[i] = dup(0.f);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) nmu[i] = dup(0.f);
+    if (pr < npairs) {
+        const float4* src = reinterpret_cast<const float4*>(a.params + (size_t)pr * PAIR4_FLOATS);
+        float4 v[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = src[i];
+        const float2* f = reinterpret_cast<const float2*>(v);
+#pragma unroll
+        for (int i = 0; i < 10; ++i) P[i] = f[SLOT4_P + i];
+        c = f[SLOT4_C];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) nmu[i] = f[SLOT4_NMU + i];
+        w = f[SLOT4_W];
+    }
+    float cm = fmaxf(c.x, c.y), ws = w.x + w.y;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        cm = fmaxf(cm, __shfl_xor_sync(FULL, cm, o));
+        ws += __shfl_xor_sync(FULL, ws, o);
+    }
+    if (lane == 0) {
+        s_cmax[warp] = cm;
+        s_wsum[warp] = ws;
+    }
+    if (!mbar_wait_bounded(&bar_tma, 0u, MBAR_LIMIT4)) s_dead = 1;
+    __syncthreads();
+    if (s_dead) {   // the points never arrived: report, let the copy land, leave
+        if (threadIdx.x == 0) {
+            set_error(a.st, GIRA_ERR_TIMEOUT);
+            mbar_wait_bounded(&bar_tma, 0u, MBAR_LIMIT4);
+        }
+        return;
+    }
+    float cmax = s_cmax[0], wsum = s_wsum[0];
+    for (int i = 1; i < G; ++i) {
+        cmax = fmaxf(cmax, s_cmax[i]);
+        wsum += s_wsum[i];
+    }
+    const float2 cc = f2(cmax - c.x, cmax - c.y);   // >= 0; +inf for padding
+    const float ref0 = s_norm ? cmax - __log2f(wsum) : cmax;
+    float2 S[NSTAT4];
+#pragma unroll
+    for (int i = 0; i < NSTAT4; ++i) S[i] = f2(0.f, 0.f);
+    double ll_acc = 0.0;
+    const int myq = q_of_lane<Q4>(lane);
+    const bool owner = warp == 0 && (lane & (LPQ - 1)) == 0;
+    // y = P'(x - mu) at point li, and q' = |y|^2 + (cmax - c): minus the logit relative to cmax
+    auto whiten = [&](int li, float2 (&y)[4]) {
+        const float4 xy = spts[2 * li], zw = spts[2 * li + 1];
+        const float2 d0 = add2(f2(xy.x, xy.y), nmu[0]), d1 = add2(f2(xy.z, xy.w), nmu[1]);
+        const float2 d2 = add2(f2(zw.x, zw.y), nmu[2]), d3 = add2(f2(zw.z, zw.w), nmu[3]);
+        y[0] = mul2(P[0], d0);
+        y[1] = fma2(P[2], d1, mul2(P[1], d0));
+        y[2] = fma2(P[5], d2, fma2(P[4], d1, mul2(P[3], d0)));
+        y[3] = fma2(P[9], d3, fma2(P[8], d2, fma2(P[7], d1, mul2(P[6], d0))));
+    };
+    auto qform = [&](int li) {
+        float2 y[4];
+        whiten(li, y);
+        return fma2(y[3], y[3], fma2(y[2], y[2], fma2(y[1], y[1], fma2(y[0], y[0], cc))));
+    };
+    float2 E[Q4];
+    for (int t = 0, lb = 0; lb < npts; ++t, lb += Q4) {
+        const int nvalid = min(Q4, npts - lb);
+        float part[Q4];
+#pragma unroll
+        for (int q = 0; q < Q4; ++q) {
+            const float2 nq = qform(q < nvalid ? lb + q : lb);
+            E[q] = f2(ex2_approx(-nq.x), ex2_approx(-nq.y));
+            part[q] = E[q].x + E[q].y;
+        }
+        const float wt = warp_transpose_reduce<Q4>(part, lane, AddOp());
+        if ((lane & (LPQ - 1)) == 0) red_sum[t & 1][warp][myq] = wt;
+        __syncthreads();
+        float tot = red_sum[t & 1][0][myq];
+        for (int i = 1; i < G; ++i) tot += red_sum[t & 1][i][myq];
+        const bool myvalid = myq < nvalid;
+        float ref = ref0;
+        if (__any_sync(FULL, myvalid && !(tot >= 0x1p-100f))) {
+            // rare, the same in every warp: a point > 100 binades below cmax everywhere; the exact
+            // per-point maximum
+            float m[Q4];
+#pragma unroll
+            for (int q = 0; q < Q4; ++q) {
+                const float2 nq = qform(q < nvalid ? lb + q : lb);
+                E[q] = f2(-nq.x, -nq.y);
+                m[q] = fmaxf(E[q].x, E[q].y);
+            }
+            float mt = warp_transpose_reduce<Q4>(m, lane, MaxOp());
+            if ((lane & (LPQ - 1)) == 0) red_aux[0][warp][myq] = mt;
+            __syncthreads();
+            mt = red_aux[0][0][myq];
+            for (int i = 1; i < G; ++i) mt = fmaxf(mt, red_aux[0][i][myq]);
+            float p2[Q4];
+#pragma unroll
+            for (int q = 0; q < Q4; ++q) {
+                float mq = __shfl_sync(FULL, mt, q * LPQ);
+                mq = mq > -INFINITY ? mq : 0.f;
+                E[q] = f2(ex2_approx(E[q].x - mq), ex2_approx(E[q].y - mq));
+                p2[q] = E[q].x + E[q].y;
+            }
+            const float w2 = warp_transpose_reduce<Q4>(p2, lane, AddOp());
+            if ((lane & (LPQ - 1)) == 0) red_aux[1][warp][myq] = w2;
+            __syncthreads();
+            tot = red_aux[1][0][myq];
+            for (int i = 1; i < G; ++i) tot += red_aux[1][i][myq];
+            if (myvalid && !(mt > -INFINITY)) set_error(a.st, GIRA_ERR_NUMERIC);
+            ref = ref0 + (mt > -INFINITY ? mt : 0.f);
+        }
+        const bool ok = myvalid && tot > 0.f;
+        const float lse2 = lg2_approx(tot) + ref;
+        if (owner && ok) {
+            ll_acc += (double)lse2;
+            if (!STATS && a.per_point) a.per_point[begin + lb + myq] = lse2 * LN2F4;
+        }
+        if (STATS) {
+            const float r = ok ? __frcp_rn(tot) : 0.f;
+#pragma unroll
+            for (int q = 0; q < Q4; ++q) {
+                const float2 g = mul2(E[q], dup(__shfl_sync(FULL, r, q * LPQ)));
+                float2 y[4];
+                whiten(q < nvalid ? lb + q : lb, y);
+                S[0] = add2(S[0], g);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float2 gy = mul2(g, y[i]);
+                    S[1 + i] = add2(S[1 + i], gy);
+#pragma unroll
+                    for (int j = i; j < 4; ++j) S[5 + sym4(i, j)] = fma2(gy, y[j], S[5 + sym4(i, j)]);
+                }
+            }
+        }
+    }
+    if (STATS && pr < npairs) {
+        float* dst = a.partials + ((size_t)blockIdx.x * npairs + pr) * (2 * NSTAT4);
+#pragma unroll
+        for (int i = 0; i < NSTAT4; ++i) {
+            dst[i] = S[i].x;
+            dst[NSTAT4 + i] = S[i].y;
+        }
+    }
+    if (warp == 0) {   // the owner lanes hold the per-point sums; fixed order
+#pragma unroll
+        for (int o = LPQ; o < 32; o <<= 1) ll_acc += __shfl_xor_sync(FULL, ll_acc, o);
+        if (lane == 0) a.ll_partials[blockIdx.x] = ll_acc * LN2_4;
+    }
 }
 
 // From (w, mu, Sigma) in binary64: Cholesky, P = L^{-1}, the base-2 constants.
@@ -130,7 +335,7 @@ __global__ void __launch_bounds__(32 * FIN4_WARPS) reduce_finalize4_kernel(const
     const bool white = f.partials != nullptr;
     if (white) {
         const int npairs = (f.k + 1) >> 1;
-        const uint32_t* lw = f.live2 + (size_t)(pp >> 5) * f.slices;
+        const uint32_t* lw = f.live2 ? f.live2 + (size_t)(pp >> 5) * f.slices : nullptr;   // nullptr: every row
         const float* src = f.partials + (size_t)pp * 2 * NSTAT4 + lane;
         const size_t stride = (size_t)npairs * 2 * NSTAT4;
         const int c0 = warp * f.slices / FIN4_WARPS, c1 = (warp + 1) * f.slices / FIN4_WARPS;
@@ -144,8 +349,9 @@ __global__ void __launch_bounds__(32 * FIN4_WARPS) reduce_finalize4_kernel(const
             float x[8];
 #pragma unroll
             for (int u = 0; u < 8; ++u)
-                x[u] = (c + u < c1 && lane < 2 * NSTAT4 && ((lw[c + u] >> (pp & 31)) & 1u)) ? src[(size_t)(c + u) * stride]
-                                                                                           : 0.f;
+                x[u] = c + u < c1 && lane < 2 * NSTAT4 && (!lw || ((lw[c + u] >> (pp & 31)) & 1u))
+                           ? src[(size_t)(c + u) * stride]
+                           : 0.f;
 #pragma unroll
             for (int u = 0; u < 8; ++u) add(x[u]);
         }
@@ -1190,14 +1396,56 @@ cudaError_t launch_label_stats4(const float4* pts4, int64_t n, int k, const int3
     return cudaGetLastError();
 }
 
+// Where the dense E-step is used: up to 10M (point, component)s an iteration of a fit is its two
+// launches against five over the lists, and up to 2^24 a log-likelihood's is the shorter chain.
+// (More points than 131,072 under few components leave its small CTAs long chains.)  Dense
+// and by lists, us: 12 iterations from a given model, 17,000 points, K = 64: 499, 892; 60,000,
+// K = 128: 756, 968; 30,000, K = 300: 886, 993; 30,000, K = 550: 1,104, 1,070; 60,000, K = 280:
+// 1,176, 1,005; log-likelihood, 17,000, K = 1000: 97, 114; 60,000, K = 280: 95, 101; 250,000,
+// K = 64: 95, 101; 276,348, K = 30: 103, 94.  (Models whose components all overlap gain nothing
+// from the lists: 100,000 normal points, K = 512, 186 us an iteration dense, 255 by lists.)
+bool estep4_dense(int64_t n, int k, bool stats) {
+    return k <= MAX_K_DIRECT && n <= 131072 && n * k <= (stats ? 10000000 : 1 << 24);
+}
+
+namespace {
+int dense4_threads(int k) { return 32 * ((k + 63) / 64); }
+}  // namespace
+
+// One wave of CTAs over the points, at most four per SM, and those of one or two warps with 64
+// points each (fewer below 8,192 points, where some SMs would be idle): the finalize sums a row
+// of every CTA (12 iterations of 17,000 points, K = 64: 475 us with 304 CTAs, 529 with 608,
+// 791 with 2,432; 120,000 points: 900, 844, 933).
+int estep4_dense_grid(int64_t n, int k, int num_sms, int64_t* ppc) {
+    const int threads = dense4_threads(k);
+    int occ = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, estep4_dense_kernel<true>, threads, 0) != cudaSuccess ||
+        occ < 1) {
+        cudaGetLastError();
+        occ = 1;
+    }
+    const int64_t least = threads <= 64 ? std::min<int64_t>(64, std::max<int64_t>(Q4, n / 128)) : Q4;
+    const int64_t grid = std::min<int64_t>((n + least - 1) / least, (int64_t)num_sms * std::min(occ, 4));
+    *ppc = std::min<int64_t>(((n + grid - 1) / grid + Q4 - 1) / Q4 * Q4, PPC4_MAX);
+    return (int)((n + *ppc - 1) / *ppc);
+}
+
+cudaError_t launch_estep4_dense(const EStep4Launch& a, bool stats, int grid, cudaStream_t s, bool pdl) {
+    const void* fn = stats ? (const void*)estep4_dense_kernel<true> : (const void*)estep4_dense_kernel<false>;
+    note_estep_kernel(fn);
+    void* args[] = {(void*)&a};
+    PdlConfig c(dim3(grid), dim3(dense4_threads(a.k)), (size_t)a.pts_per_cta * 32, s, pdl);
+    return cudaLaunchKernelExC(&c.cfg, fn, args);
+}
+
 cudaError_t launch_reduce_finalize4(const float* partials, const uint32_t* live2, int slices, const double* llp,
                                     int ll_count, const double* stats64, const float4* shift4, int k, int64_t n,
                                     double reg, double tol, double* model64, float* params, double* trace,
-                                    const int* perm, DeviceState* st, int iter, bool em, cudaStream_t s) {
+                                    const int* perm, DeviceState* st, int iter, bool em, cudaStream_t s, bool pdl) {
     const Fin4Args f{partials, live2, slices, llp, ll_count, stats64, shift4, k, n, reg, tol, model64, params, trace,
                      perm, st, iter, em ? 1 : 0};
-    reduce_finalize4_kernel<<<(k + 1) / 2, 32 * FIN4_WARPS, 0, s>>>(f);
-    return cudaGetLastError();
+    PdlConfig c(dim3((k + 1) / 2), dim3(32 * FIN4_WARPS), 0, s, pdl);
+    return cudaLaunchKernelEx(&c.cfg, reduce_finalize4_kernel, f);
 }
 
 cudaError_t launch_order_components4(double* model64, double* scratch, int k, int* perm, float* params,

@@ -533,6 +533,7 @@ void note_estep_kernel(const void* fn) {
     size_t at = name.find("estep_pt_kernel<");
     if (at == std::string::npos) at = name.find("estep_adjoint_kernel<");
     if (at == std::string::npos) at = name.find("estep_reach_kernel<");
+    if (at == std::string::npos) at = name.find("estep4_dense_kernel<");
     if (at != std::string::npos) name = name.substr(at);
     const size_t par = name.rfind(">(");
     if (par != std::string::npos) name = name.substr(0, par + 1);

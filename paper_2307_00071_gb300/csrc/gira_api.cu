@@ -1762,16 +1762,22 @@ gira_status gira_gmm_fit4(const float* points, int64_t n, int k, const gira_fit_
     TRY(check_ptr(covs, "covs", c.dev, &kc));
     const bool kinit = o.init_mode == GIRA_INIT_KMEANS;
     const int kpad = params4_pairs(k);
-    const bool sorted = n <= point_order_max_n();   // the E-steps visit the points in Morton order of (x, y, z)
+    const bool dense = estep4_dense(n, k, true);   // little work: every component at every point
+    // the E-steps over lists visit the points in Morton order of (x, y, z), which saves nothing for
+    // the few pairs of 32 components; the dense one needs no order.  Lloyd's and the one-hot sums
+    // want runs of labels, where there are many points.
+    const bool sorted = n <= point_order_max_n() && (kinit ? !dense || n > 8192 : !dense && k > 32);
+    int64_t ppc = 0;
+    const int dgrid = dense ? estep4_dense_grid(n, k, c.sms, &ppc) : 0;
     const int nblk = kpp_num_blocks(n);
     int kgrid = kinit ? kpp_persistent_grid() : 0;
     if (kgrid > 0 && n > kpp_persistent_max_n(kgrid)) kgrid = 0;
     ReachBufs rb;
     struct Bufs {
         DeviceState* st;
-        float *pin, *params, *d2, *mw, *mmu, *mcov;
+        float *pin, *params, *partials, *d2, *mw, *mmu, *mcov;
         float4 *p4, *p8, *p8s, *p4s, *c4;
-        double *model64, *stats64, *trace, *sums;
+        double *model64, *stats64, *llp, *trace, *sums;
         u128 *bs, *ksums;
         int64_t* ch;
         int32_t* lab;
@@ -1791,7 +1797,9 @@ gira_status gira_gmm_fit4(const float* points, int64_t n, int k, const gira_fit_
         b.params = cv.take<float>((size_t)kpad * PAIR4_FLOATS);
         b.model64 = cv.take<double>((size_t)k * MODEL4);
         b.stats64 = cv.take<double>((size_t)k * NSTAT4);
-        carve_reach(cv, n, k, NSTAT4, true, &rb);
+        if (!dense) carve_reach(cv, n, k, NSTAT4, true, &rb);
+        b.partials = cv.take<float>((size_t)dgrid * ((k + 1) / 2) * 2 * NSTAT4);
+        b.llp = cv.take<double>(dgrid);
         b.trace = cv.take<double>(std::max(o.iters, 1));
         b.mw = cv.take<float>(kw == Kind::Host ? k : 0);
         b.mmu = cv.take<float>(km == Kind::Host ? 4 * (size_t)k : 0);
@@ -1859,23 +1867,39 @@ gira_status gira_gmm_fit4(const float* points, int64_t n, int k, const gira_fit_
         COUNTED(prof, 1, launch_params_from_model4(w_d, mu_d, cov_d, k, b.model64, b.params, nullptr, nullptr, b.st, c.s));
     }
     // components in Morton order of their means, as in the 3-D fit
-    COUNTED(prof, 2, launch_order_components4(b.model64, b.stats64, k, b.perm, b.params, b.st, c.s));
+    const int* perm = dense ? nullptr : b.perm;
+    if (!dense) COUNTED(prof, 2, launch_order_components4(b.model64, b.stats64, k, b.perm, b.params, b.st, c.s));
     prof.t_init = prof.mark();
     const float4* pe = sorted ? b.p8s : b.p8;
-    for (int t = 1; t <= o.iters; ++t) {
+    EStep4Launch da{pe, n, k, b.params, ppc, b.partials, b.llp, nullptr, b.st, 0};
+    for (int t = 1; t <= o.iters && dense; ++t) {
+        const bool pdl = !prof.per_launch;   // dependent launches, as in the 3-D loop
+        da.iter = t;
+        cudaEvent_t e0 = prof.mark_launch();
+        COUNTED(prof, 1, launch_estep4_dense(da, true, dgrid, c.s, pdl));
+        cudaEvent_t e1 = prof.mark_launch();
+        if (prof.per_launch) prof.timed(e0, e1);
+        COUNTED(prof, 1, launch_reduce_finalize4(b.partials, nullptr, dgrid, b.llp, dgrid, nullptr, nullptr, k, n, o.reg_covar,
+                                                 o.tol, b.model64, b.params, b.trace, perm, b.st, t, true, c.s, pdl));
+    }
+    for (int t = 1; t <= o.iters && !dense; ++t) {
         const ReachLaunch a = reach_launch(rb, pe, n, k, b.params, b.st, t);
         cudaEvent_t e0 = prof.mark_launch();
         GIRA_CUDA(reach_estep_stats(4, rb, a, &prof.launches, c.s));
         cudaEvent_t e1 = prof.mark_launch();
         if (prof.per_launch) prof.timed(e0, e1);
         COUNTED(prof, 1, launch_reduce_finalize4(rb.partials, rb.live2, rb.slices, rb.llp, rb.grid, nullptr, nullptr, k,
-                                                 n, o.reg_covar, o.tol, b.model64, b.params, b.trace, b.perm, b.st, t,
+                                                 n, o.reg_covar, o.tol, b.model64, b.params, b.trace, perm, b.st, t,
                                                  true, c.s));
     }
     prof.t_em = prof.mark();
-    if (final_loglik)
+    if (final_loglik && dense) {
+        da.iter = 0;
+        COUNTED(prof, 1, launch_estep4_dense(da, false, dgrid, c.s));
+        COUNTED(prof, 1, launch_ll_reduce(b.llp, dgrid, b.st, c.s));
+    } else if (final_loglik)
         GIRA_CUDA(reach_loglik(4, rb, reach_launch(rb, pe, n, k, b.params, b.st, 0), false, &prof.launches, c.s));
-    COUNTED(prof, 1, launch_model_out4(b.model64, k, w_d, mu_d, cov_d, b.perm, b.st, c.s));
+    COUNTED(prof, 1, launch_model_out4(b.model64, k, w_d, mu_d, cov_d, perm, b.st, c.s));
     if (kw == Kind::Host) GIRA_CUDA(cudaMemcpyAsync(weights, b.mw, sizeof(float) * k, cudaMemcpyDeviceToHost, c.s));
     if (km == Kind::Host) GIRA_CUDA(cudaMemcpyAsync(means, b.mmu, sizeof(float) * 4 * k, cudaMemcpyDeviceToHost, c.s));
     if (kc == Kind::Host) GIRA_CUDA(cudaMemcpyAsync(covs, b.mcov, sizeof(float) * 16 * k, cudaMemcpyDeviceToHost, c.s));
@@ -1906,12 +1930,15 @@ gira_status gira_gmm_loglik4(const float* points, int64_t n, int k, const float*
     TRY(check_ptr(covs, "covs", c.dev, &kc));
     if (per_point) TRY(check_ptr(per_point, "per_point", c.dev, &kpp));
     const int kpad = params4_pairs(k);
+    const bool dense = estep4_dense(n, k, false);
+    int64_t ppc = 0;
+    const int dgrid = dense ? estep4_dense_grid(n, k, c.sms, &ppc) : 0;
     ReachBufs rb;
     struct Bufs {
         DeviceState* st;
         float *pin, *params, *mw, *mmu, *mcov, *pp;
         float4* p8;
-        double* model64;
+        double *model64, *llp;
     } b{};
     auto layout = [&](Carver& cv) {
         b.st = cv.take<DeviceState>(1);
@@ -1919,7 +1946,8 @@ gira_status gira_gmm_loglik4(const float* points, int64_t n, int k, const float*
         b.p8 = cv.take<float4>(2 * (size_t)n);
         b.params = cv.take<float>((size_t)kpad * PAIR4_FLOATS);
         b.model64 = cv.take<double>((size_t)k * MODEL4);
-        carve_reach(cv, n, k, NSTAT4, false, &rb);
+        if (!dense) carve_reach(cv, n, k, NSTAT4, false, &rb);
+        b.llp = cv.take<double>(dgrid);
         b.mw = cv.take<float>(kw == Kind::Host ? k : 0);
         b.mmu = cv.take<float>(km == Kind::Host ? 4 * (size_t)k : 0);
         b.mcov = cv.take<float>(kc == Kind::Host ? 16 * (size_t)k : 0);
@@ -1966,13 +1994,20 @@ gira_status gira_gmm_loglik4(const float* points, int64_t n, int k, const float*
     }
     COUNTED(prof, 1, launch_pack4(pts, n, nullptr, b.p8, b.st, c.s));
     COUNTED(prof, 1, launch_fill_padding4(b.params, k, c.s));
-    COUNTED(prof, 1, launch_params_from_model4(w_d, mu_d, cov_d, k, b.model64, b.params, rb.ctr, rb.aux, b.st, c.s));
+    COUNTED(prof, 1, launch_params_from_model4(w_d, mu_d, cov_d, k, b.model64, b.params, dense ? nullptr : rb.ctr, rb.aux,
+                                               b.st, c.s));
     prof.t_init = prof.mark();
     prof.t_em = prof.t_init;
     float* ppd = per_point ? ((kpp == Kind::Device) ? per_point : b.pp) : nullptr;
-    ReachLaunch a = reach_launch(rb, b.p8, n, k, b.params, b.st, 0);
-    a.per_point = ppd;
-    GIRA_CUDA(reach_loglik(4, rb, a, true, &prof.launches, c.s));
+    if (dense) {
+        const EStep4Launch a{b.p8, n, k, b.params, ppc, nullptr, b.llp, ppd, b.st, 0};
+        COUNTED(prof, 1, launch_estep4_dense(a, false, dgrid, c.s));
+        COUNTED(prof, 1, launch_ll_reduce(b.llp, dgrid, b.st, c.s));
+    } else {
+        ReachLaunch a = reach_launch(rb, b.p8, n, k, b.params, b.st, 0);
+        a.per_point = ppd;
+        GIRA_CUDA(reach_loglik(4, rb, a, true, &prof.launches, c.s));
+    }
     if (per_point && kpp == Kind::Host)
         GIRA_CUDA(cudaMemcpyAsync(per_point, b.pp, sizeof(float) * n, cudaMemcpyDeviceToHost, c.s));
     GIRA_CUDA(cudaMemcpyAsync(&h, b.st, sizeof h, cudaMemcpyDeviceToHost, c.s));

@@ -802,14 +802,31 @@ int params4_pairs(int k);
 cudaError_t launch_pack4(const float* pts4in, int64_t n, float4* pts4, float4* pts8, DeviceState* st,
                          cudaStream_t s);
 cudaError_t launch_fill_padding4(float* params, int k, cudaStream_t s);
-// M-step from the slices' partials of launch_reach_stats ([slices][pairs][2 NSTAT4], live
-// where live2 says) or, when partials is nullptr, from binary64 one-hot statistics stats64
+// The dense E-step of little work (estep4_dense says for which n and k).
+struct EStep4Launch {
+    const float4* pts8;    // 2 float4 per point: (x,x,y,y) (z,z,I,I)
+    int64_t n;
+    int k;
+    const float* params;
+    int64_t pts_per_cta;   // multiple of 8
+    float* partials;       // [grid][pairs][2 NSTAT4] (stats launches)
+    double* ll_partials;   // [grid]
+    float* per_point;      // [n] natural-log lse, or nullptr
+    DeviceState* st;
+    int iter;              // 1-based EM iteration; skipped when iter > st->stop_after
+};
+bool estep4_dense(int64_t n, int k, bool stats);
+int estep4_dense_grid(int64_t n, int k, int num_sms, int64_t* pts_per_cta);
+cudaError_t launch_estep4_dense(const EStep4Launch& a, bool stats, int grid, cudaStream_t s, bool pdl = false);
+// M-step from the partials of launch_reach_stats or launch_estep4_dense ([slices][pairs][2 NSTAT4],
+// live where live2 says; nullptr: all) or, when partials is nullptr, from binary64 one-hot statistics stats64
 // about shift4; em as in launch_reduce_finalize, the log-likelihood being the sum of
 // llp[0 .. ll_count).  Slot b holds the caller's component perm[b] (nullptr: b).
 cudaError_t launch_reduce_finalize4(const float* partials, const uint32_t* live2, int slices, const double* llp,
                                     int ll_count, const double* stats64, const float4* shift4, int k, int64_t n,
                                     double reg, double tol, double* model64, float* params, double* trace,
-                                    const int* perm, DeviceState* st, int iter, bool em, cudaStream_t s);
+                                    const int* perm, DeviceState* st, int iter, bool em, cudaStream_t s,
+                                    bool pdl = false);
 // Components in Morton order of their means, as launch_order_components (scratch: k * MODEL4 doubles).
 cudaError_t launch_order_components4(double* model64, double* scratch, int k, int* perm, float* params,
                                      DeviceState* st, cudaStream_t s);

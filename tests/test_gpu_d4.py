@@ -244,3 +244,32 @@ def test_fit4_dependent_launches_give_the_same_fit(gira):
     for key in ("weights", "means", "covs"):
         np.testing.assert_array_equal(to_np(runs[0][key]), to_np(runs[1][key]))
     assert runs[0]["final_loglik"] == runs[1]["final_loglik"]
+
+
+# ----------------------------------------------------------------------------- little work: the dense E-step
+@pytest.mark.parametrize("n,k", [(1, 1), (7, 3), (64, 33), (1_025, 64), (1_025, 65), (9_765, 1_024), (9_766, 1_024),
+                                 (16_384, 1_024), (131_072, 9), (131_073, 9)])
+def test_little_work(gira, frame4, n, k):
+    """Both sides of the rule (10M point-component pairs in a fit, 2^24 in a log-likelihood, 131,072 points,
+    K = 1024), ragged batches of eight points and odd K: one EM iteration, and per-point log-likelihoods
+    within the derived bound (which covers the order of the sums), some points off the model."""
+    rng = np.random.default_rng(n + k)
+    pts = np.ascontiguousarray(frame4[rng.integers(0, len(frame4) - n) + np.arange(n)])
+    means = frame4[rng.choice(len(frame4), k, replace=False)].astype(np.float64)
+    means[:min(n, k)] = pts[rng.choice(n, min(n, k), replace=False)]
+    a = rng.normal(scale=0.2, size=(k, 4, 4))
+    c = (0.3 ** 2 * (np.eye(4) + a @ np.transpose(a, (0, 2, 1)))).astype(np.float32)
+    w, m = rng.dirichlet(np.ones(k) * 5).astype(np.float32), means.astype(np.float32)
+    r = gira.gira_gmm_fit4(pts, k, iters=1, tol=0.0, init=(w, m, c), reg_covar=1e-4)
+    ref = oracle.em_par(pts, w, m, c, iters=1, tol=0.0, reg=1e-4)
+    assert abs(r["trace"][0] - ref["trace"][0]) <= LL_ABS + 1e-7 * abs(ref["trace"][0])
+    assert_model_close((r["weights"], r["means"], r["covs"]), (ref["weights"], ref["means"], ref["covs"]))
+    far = np.arange(0, n, 97)
+    pts[far, :3] += np.float32(30.0)   # every component more than 100 binades below the reference
+    mean, pp = gira.gira_gmm_loglik4(pts, w, m, c, per_point=True)
+    pp = to_np(pp).astype(np.float64)
+    assert mean == pytest.approx(pp.mean(), rel=1e-6)
+    sample = np.unique(np.concatenate([far[:50], [0, n - 1], rng.choice(n, min(n, 150), replace=False)]))
+    _, _, lse = oracle.estep(pts[sample], w, m, c, want_resp=False, want_lse=True)
+    err, bound = np.abs(pp[sample] - lse), per_point_bound(pts[sample], w, m, c, form="d")
+    assert np.all(err <= bound), np.max(err / bound)
