@@ -667,12 +667,89 @@ __global__ void cond_prepare_kernel(const float* __restrict__ w, const float* __
     put(19, 0.f);
 }
 
-// Four warps per 256 locations, neighbours in `order`: a warp has 64 of them, a lane one of
-// each block of 32.  Pass 1 takes the maximum log-weight and, as a reference, the regression
-// mean m_ref of that component; pass 2 sums w_b = exp(lw_b - max), w_b (m_b - m_ref) and
+// Pass 1 takes the maximum log-weight and, as a reference, the regression mean m_ref of that
+// component; pass 2 sums w_b = exp(lw_b - max), w_b (m_b - m_ref) and
 // w_b (v_b + (m_b - m_ref)^2) in binary32 (the shift keeps the variance free of
-// cancellation), both over the components in increasing order, two locations per packed
-// operation.
+// cancellation), both over the components in increasing order.  Two kernels, the same bits.
+
+// Little work: one location per thread, every component, staged through shared memory.  Bound by
+// a thread's chain of 2 K components, the same for any order of the locations: up to 38,912
+// of them 55 us of kernel for K = 512, where the lists' kernel and the grouping take 85.
+constexpr int CD_THREADS = 128;
+constexpr int CD_TILE = 64;   // components staged at a time
+__global__ void __launch_bounds__(CD_THREADS) conditional4_dense_kernel(const float* __restrict__ locs, int64_t m, int k,
+                                                                        const float* __restrict__ prep, float* cmean,
+                                                                        float* cvar, DeviceState* st) {
+    __shared__ __align__(16) float4 s_rec[CD_TILE][4];   // slots 0 .. 15
+    __shared__ int s_err;
+    if (threadIdx.x == 0) s_err = st->error;
+    __syncthreads();
+    if (s_err) return;
+    const int64_t i = (int64_t)blockIdx.x * CD_THREADS + threadIdx.x;
+    float x[3] = {0.f, 0.f, 0.f};
+    if (i < m) {
+#pragma unroll
+        for (int j = 0; j < 3; ++j) x[j] = locs[3 * i + j];
+        if (!(isfinite(x[0]) && isfinite(x[1]) && isfinite(x[2]))) set_error(st, GIRA_ERR_NONFINITE_INPUT);
+    }
+    // each(o) gets the slots of components 0 .. k - 1
+    auto for_all = [&](auto&& each) {
+        for (int b0 = 0; b0 < k; b0 += CD_TILE) {
+            const int nb = min(CD_TILE, k - b0);
+            __syncthreads();
+            for (int t = threadIdx.x; t < 16 * nb; t += CD_THREADS)
+                reinterpret_cast<float*>(s_rec)[t] = prep[(size_t)(b0 + (t >> 4)) * COND_FLOATS + 2 * (t & 15)];
+            __syncthreads();
+#pragma unroll 4
+            for (int b = 0; b < nb; ++b) {
+                float o[16];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const float4 v = s_rec[b][q];
+                    o[4 * q] = v.x;
+                    o[4 * q + 1] = v.y;
+                    o[4 * q + 2] = v.z;
+                    o[4 * q + 3] = v.w;
+                }
+                each(o);
+            }
+        }
+    };
+    auto eval = [&](const float (&o)[16], float& mb) {   // log-weight and regression mean
+        const float d0 = x[0] + o[11], d1 = x[1] + o[12], d2 = x[2] + o[13];
+        const float y0 = o[0] * d0, y1 = fmaf(o[2], d1, o[1] * d0), y2 = fmaf(o[5], d2, fmaf(o[4], d1, o[3] * d0));
+        mb = fmaf(o[8], d2, fmaf(o[7], d1, fmaf(o[6], d0, o[14])));
+        return fmaf(-0.5f, fmaf(y2, y2, fmaf(y1, y1, y0 * y0)), o[10]);
+    };
+    float mx = -INFINITY, mref = 0.f;
+    for_all([&](const float (&o)[16]) {
+        float mb;
+        const float lw = eval(o, mb);
+        if (lw > mx) {
+            mx = lw;
+            mref = mb;
+        }
+    });
+    float s = 0.f, e1 = 0.f, e2 = 0.f;
+    for_all([&](const float (&o)[16]) {
+        float mb;
+        const float w = __expf(eval(o, mb) - mx), dm = mb - mref;
+        s += w;
+        e1 = fmaf(w, dm, e1);
+        e2 = fmaf(w, fmaf(dm, dm, o[9]), e2);
+    });
+    if (i >= m) return;
+    if (!(s > 0.f)) {
+        set_error(st, GIRA_ERR_NUMERIC);
+        return;
+    }
+    const float inv = 1.f / s, a = e1 * inv;
+    cmean[i] = mref + a;
+    if (cvar) cvar[i] = fmaf(-a, a, e2 * inv);
+}
+
+// More: four warps per 256 locations, neighbours in `order`: a warp has 64 of them, a lane one of
+// each block of 32, two locations per packed operation.
 // Only components that can matter are visited: exp of less than -104 is exactly 0 in
 // binary32, and a term of weight 0 changes no sum.  Over a set of locations, the component
 // of largest log-weight at the centre of their box gives every location a log-weight; with L
@@ -690,6 +767,7 @@ constexpr int COND_SEG = COND_CAP / COND_WARPS;
 constexpr int COND_LOCS = 64;    // locations per warp
 constexpr int COND_CHUNK = 16;   // components staged at a time
 
+template <int PER>   // locations per CTA: 256, or one
 __global__ void __launch_bounds__(32 * COND_WARPS) conditional4_kernel(const float* __restrict__ locs,
                                                                        const int* __restrict__ order, int64_t m, int k,
                                                                        const float* __restrict__ prep, float* cmean,
@@ -705,12 +783,13 @@ __global__ void __launch_bounds__(32 * COND_WARPS) conditional4_kernel(const flo
     if (s_err) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint16_t* list = s_list[warp];
-    const int64_t base = ((int64_t)blockIdx.x * COND_WARPS + warp) * COND_LOCS;
+    const int64_t base = (int64_t)blockIdx.x * PER + warp * COND_LOCS;
+    const int64_t end = PER == 1 ? (int64_t)blockIdx.x + 1 : m;
     float x[2][3];   // location base + 32 r + lane
     float lo[2][3], hi[2][3];
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
-        const int64_t i = min(base + 32 * r + lane, m - 1);   // an absent location: the last one, not written
+        const int64_t i = min(base + 32 * r + lane, end - 1);   // an absent location: the last one, not written
         const int64_t at = order ? order[i] : i;
         bool fin = true;
 #pragma unroll
@@ -990,7 +1069,7 @@ __global__ void __launch_bounds__(32 * COND_WARPS) conditional4_kernel(const flo
     }
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
-        if (base + 32 * r + lane >= m) continue;
+        if (base + 32 * r + lane >= end) continue;
         const int64_t i = order ? order[base + 32 * r + lane] : base + 32 * r + lane;
         const float sr = r ? s.y : s.x;
         if (!(sr > 0.f)) {
@@ -1485,12 +1564,33 @@ cudaError_t launch_pack4(const float* pts4in, int64_t n, float4* pts4, float4* p
 
 int cond_floats() { return COND_ALL; }
 
+// Whether the lists are taken, over 256 neighbouring locations (grouped by cell, 25 us): from 24M
+// (location, component)s, with an SM's worth of locations (above 2,048 components, listed in
+// rounds, two).  Dense and by lists, us per call (locations of a depth frame): 276,348, K = 8:
+// 75, 121; 100,000, K = 100: 91, 120; 30,000, K = 512: 126, 156; 17,000, K = 1163: 190, 211;
+// 100,000, K = 300: 139, 142; 60,000, K = 800: 203, 175; 100,000, K = 1163: 353, 220; 30,000,
+// K = 3000: 416, 509; 60,000: 580, 511.
+bool conditional4_grouped(int64_t m, int k) { return m * k > 24000000 && m > (k <= COND_CAP ? 16384 : 40000); }
+
 cudaError_t launch_conditional4(const float* locs, const int* order, int64_t m, int k, const float* w, const float* mu,
                                 const float* cov, float* prep, float* cmean, float* cvar, DeviceState* st,
                                 cudaStream_t s) {
     cond_prepare_kernel<<<(k + 63) / 64, 64, 0, s>>>(w, mu, cov, k, prep, st);
-    conditional4_kernel<<<(unsigned)((m + COND_LOCS * COND_WARPS - 1) / (COND_LOCS * COND_WARPS)), 32 * COND_WARPS, 0,
-                          s>>>(locs, order, m, k, prep, cmean, cvar, st);
+    // Few locations under many components: the lists of one location each, a CTA for each, wherever
+    // they lie (100 locations all over the frame, K = 1163: 96 us a call, 200 dense, 241 with the
+    // lists of 256; 608, K = 128: 83, 87, 88; 2,000, K = 1163: 157, 199, 190).
+    if (k >= 64 && m <= std::max(608, std::min(2 * k, 2048))) {
+        conditional4_kernel<1><<<(unsigned)m, 32 * COND_WARPS, 0, s>>>(locs, nullptr, m, k, prep, cmean, cvar, st);
+        return cudaGetLastError();
+    }
+    if (!conditional4_grouped(m, k)) {
+        conditional4_dense_kernel<<<(unsigned)((m + CD_THREADS - 1) / CD_THREADS), CD_THREADS, 0, s>>>(locs, m, k, prep,
+                                                                                                       cmean, cvar, st);
+        return cudaGetLastError();
+    }
+    constexpr int PER = COND_LOCS * COND_WARPS;
+    conditional4_kernel<PER><<<(unsigned)((m + PER - 1) / PER), 32 * COND_WARPS, 0, s>>>(locs, order, m, k, prep, cmean,
+                                                                                         cvar, st);
     return cudaGetLastError();
 }
 

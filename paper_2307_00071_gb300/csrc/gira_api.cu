@@ -2043,9 +2043,8 @@ gira_status gira_gmm_conditional4(const float* locs, int64_t m, int k, const flo
         void* osc;
     } b{};
     // locations taken cell by cell: a depth image's rows jump between surfaces at every edge
-    // (the grouping is 25 us for 307,200 locations); the few launches are not worth it for
-    // small inputs
-    const bool grouped = m >= 8192 && m <= INT32_MAX;
+    // (the grouping is 25 us for 307,200 locations)
+    const bool grouped = conditional4_grouped(m, k) && m <= INT32_MAX;
     auto layout = [&](Carver& cv) {
         b.st = cv.take<DeviceState>(1);
         b.lin = cv.take<float>(kl == Kind::Host ? 3 * m : 0);

@@ -842,6 +842,7 @@ cudaError_t launch_label_stats4(const float4* pts4, int64_t n, int k, const int3
                                 double* stats64, DeviceState* st, cudaStream_t s);
 // Gaussian-mixture regression of the 4th coordinate on the first three.
 int cond_floats();
+bool conditional4_grouped(int64_t m, int k);   // whether it takes neighbours together (wants an order)
 // order (nullable): the order in which the kernel takes the locations (any permutation gives
 // the same results; one that keeps neighbours together is faster).
 cudaError_t launch_conditional4(const float* locs, const int* order, int64_t m, int k, const float* w, const float* mu,

@@ -273,3 +273,22 @@ def test_little_work(gira, frame4, n, k):
     _, _, lse = oracle.estep(pts[sample], w, m, c, want_resp=False, want_lse=True)
     err, bound = np.abs(pp[sample] - lse), per_point_bound(pts[sample], w, m, c, form="d")
     assert np.all(err <= bound), np.max(err / bound)
+
+
+@pytest.mark.parametrize("k", [511, 512, 1_500, 2_049])
+def test_regression_forms_give_the_same_bits(gira, frame4, k):
+    """One location per CTA (few locations), every component (little work) and the lists of 256 neighbours:
+    a location's mean and variance are the same bits in each, whatever the others are."""
+    rng = np.random.default_rng(k)
+    means = frame4[rng.choice(len(frame4), k, replace=False)].astype(np.float32)
+    a = rng.normal(scale=0.2, size=(k, 4, 4))
+    covs = (0.1 ** 2 * (np.eye(4) + a @ np.transpose(a, (0, 2, 1)))).astype(np.float32)
+    w = rng.dirichlet(np.ones(k) * 5).astype(np.float32)
+    locs = np.ascontiguousarray(frame4[:50_000, :3])
+    locs[::501] += rng.normal(scale=5.0, size=locs[::501].shape).astype(np.float32)   # some far from the others
+    e, v = (to_np(x) for x in gira.gira_gmm_conditional4(locs, w, means, covs))       # by lists
+    assert np.all(np.isfinite(e)) and np.all(np.isfinite(v))
+    for at in (slice(0, 1), slice(7, 7 + 511), slice(9, 9 + 609), slice(0, 50_000, 99), slice(3, 3 + 2_049), slice(0, 16_384)):
+        part = gira.gira_gmm_conditional4(np.ascontiguousarray(locs[at]), w, means, covs)
+        np.testing.assert_array_equal(to_np(part[0]), e[at])
+        np.testing.assert_array_equal(to_np(part[1]), v[at])
