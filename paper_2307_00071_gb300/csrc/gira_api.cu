@@ -1404,6 +1404,39 @@ gira_status gira_gmm_fit_batched(const float* points, const int64_t* offsets, in
 }
 
 // ================================================================ gmm_loglik_grad_batched
+}  // extern "C"
+namespace {
+// Whether a batch of gradients evaluates every component at every point (adjoint_kernels.cu; it does
+// when the Cholesky factors' gradient is asked for, which that file explains) rather than sort the
+// points for the reach lists, which then costs more than the lists save.  The dense kernel
+// holds 64 components in one warp's lanes; up to 256 16M pairs, up to 64 500,000 points.  Above
+// 256 components, where the instances are few or hardly any point is one of a large
+// model's: if the dense work costs less than the lists do beyond it, both in us, fitted to measured
+// calls: 4.1 per million pairs (components padded to 128, or 64) and 0.017 per component for the
+// dense sums; 50 for the lists' launches, 0.17 per thousand points for the sort, 0.045 per
+// component of the largest model for the listing, 0.7 per instance.
+// Dense and by lists, us a call (twists): 2 scans of 12,800 points, K = 128: 176, 241; 60,000, K = 256:
+// 230, 237; 4 of 57,000, K = 256: 354, 304; 8 of 60,000, K = 16: 256, 316; 8 of 100,000, K = 64: 381,
+// 358; 5,000, K = 512: 175, 235; 10,000, K = 1024: 221, 283; 50,000, K = 300: 236, 238; 47 of 5,000, K =
+// 32, with one of 5,000, K = 1024: 325, 416; 16 of 1,000, K = 512: 324, 278.
+bool gradient_dense(const int64_t* offsets, int batch, const int* ks) {
+    const int kbig = *std::max_element(ks, ks + batch);
+    const int64_t total_n = offsets[batch];
+    if (kbig <= 256) return total_n <= (kbig <= 64 ? 500000 : 16000000 / kbig);
+    double pairs = 0.0, comps = 0.0;
+    int64_t large = 0;
+    for (int i = 0; i < batch; ++i) {
+        const int64_t n = offsets[i + 1] - offsets[i];
+        pairs += (double)n * (ks[i] <= 64 ? 64 : (ks[i] + 127) / 128 * 128);
+        comps += ks[i];
+        if (ks[i] > 256) large += n;
+    }
+    if (batch > 4 && 10 * large > total_n) return false;
+    return 4.1e-6 * pairs + 0.017 * comps < 50.0 + 0.17e-3 * (double)total_n + 0.045 * kbig + 0.7 * batch;
+}
+}  // namespace
+extern "C" {
+
 gira_status gira_gmm_loglik_grad_batched(const float* points, const int64_t* offsets, int batch, const int* ks,
                                          const float* poses, const float* logits, const float* means,
                                          const float* chol, double* logliks, float* grad_points, double* grad_pose,
@@ -1438,14 +1471,7 @@ gira_status gira_gmm_loglik_grad_batched(const float* points, const int64_t* off
         if (a.p) TRY(check_ptr(a.p, a.name, c.dev, &a.k));
     for (auto& a : out)
         if (a.p) TRY(check_ptr(a.p, a.name, c.dev, &a.k));
-    // Every component (adjoint_kernels.cu) when the Cholesky factors' gradient is asked for (it
-    // says why), and for little dense work: sorting the points for the reach lists then costs more
-    // than the lists save.  The dense kernel holds 64 components in one warp's lanes; above 256 its
-    // batches of points wait longer.  Dense and by lists, us: 2 scans of 12,800 points together,
-    // K = 128: 195, 247; 2 of 71,000, K = 64: 219, 268; 4 of 57,000, K = 256: 249, 274; 8 of 90,000,
-    // K = 128: 254, 270; the other way, 8 of 260,000, K = 128: 380, 309; 2 of 12,800, K = 512: 324, 272.
-    const int kbig = *std::max_element(ks, ks + batch);
-    const bool dense = grad_chol || (kbig <= 256 && total_n <= (kbig <= 64 ? 500000 : 16000000 / kbig));
+    const bool dense = grad_chol || gradient_dense(offsets, batch, ks);
     const bool gpar = !dense && (grad_logits || grad_means);
     const bool sorted = !dense && total_n <= point_order_max_n();
 

@@ -222,3 +222,32 @@ def test_shuffled_scores(gira, frame, d, n, k, off):
     _, _, lse = oracle.estep(pts[sample], w, m, c, want_resp=False, want_lse=True)
     err, bound = np.abs(back[sample] - lse), per_point_bound(pts[sample], w, m, c, form="d" if d == 4 else "b")
     assert np.all(err <= bound), np.max(err / bound)
+
+
+@pytest.mark.parametrize("ns,ks", [([5_000], [512]), ([5_000], [1_024]), ([300], [300]), ([2_500] * 4, [1_024] * 4),
+                                   ([2_500] * 5, [1_024] * 5), ([30_001, 2_000], [300, 1_023]),
+                                   ([5_000] * 9 + [1_500], [32] * 9 + [1_024])])
+def test_batched_gradient_of_few_scans_with_large_models(gira, frame, ns, ks):
+    """Above 256 components a few small scans, and batches with hardly a point under a large model, take the
+    dense kernel, others the reach lists: the same gradients as the single calls, within the rounding of
+    sums of n binary32 terms in another order (2e-5 of the largest)."""
+    rng = np.random.default_rng(sum(ns) + sum(ks))
+    pts = [frame[rng.choice(len(frame), n, replace=False)] for n in ns]
+    models = [ball_model(frame, k, rng, sigma=0.2) for k in ks]
+    lg, mu = [np.log(w) for w, _, _ in models], [m for _, m, _ in models]
+    ch = [np.linalg.cholesky(c.astype(np.float64)).astype(np.float32) for _, _, c in models]
+    want = ("twist", "logits", "means", "points")
+    r = gira.gira_gmm_loglik_grad_batched(np.concatenate(pts), np.concatenate([[0], np.cumsum(ns)]).astype(np.int64),
+                                          np.array(ks, np.int32), np.concatenate(lg), np.concatenate(mu),
+                                          np.concatenate(ch), want=want)
+    at = {"grad_points": np.concatenate([[0], np.cumsum(ns)]), "grad_twist": np.arange(len(ns) + 1)}
+    comps = np.concatenate([[0], np.cumsum(ks)])
+    for i, n in enumerate(ns):
+        one = gira.gira_gmm_loglik_grad(pts[i], lg[i], mu[i], ch[i], None, want=want)
+        assert r["loglik"][i] == pytest.approx(one["loglik"], rel=1e-6)
+        for key in ("grad_twist", "grad_logits", "grad_means", "grad_points"):
+            a = to_np(one[key]).astype(np.float64)
+            b = to_np(r[key]).astype(np.float64)
+            lo, hi = at.get(key, comps)[i:i + 2]
+            b = b.reshape(-1, 6)[i] if key == "grad_twist" else b[lo:hi]
+            assert np.max(np.abs(a - b.reshape(a.shape))) <= 2e-5 * np.max(np.abs(a)), key
