@@ -1366,7 +1366,7 @@ __global__ void __launch_bounds__(LL4_THREADS) lloyd4_assign_kernel(const float4
 #pragma unroll
             for (int j = 0; j < 4; ++j) x[r][j] = X[r][j].x;
         }
-        add_runs<4>(key, x, sums);
+        add_runs<4>(key, x, n > 4096, sums);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(FULL, cnt, o);

@@ -1380,7 +1380,7 @@ __device__ void lloyd_assign_groups(const float4* __restrict__ pts, int64_t n, i
             x[r][1] = Y[r].x;
             x[r][2] = Z[r].x;
         }
-        add_runs<3>(key, x, sums);
+        add_runs<3>(key, x, n > 4096, sums);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(FULL, cnt, o);

@@ -55,3 +55,25 @@ def test_one_hot_statistics_of_runs(n, batched):
         for key in ("weights", "means", "covs"):
             got = np.asarray(r[key], np.float64)[5 * i:5 * i + 5]
             np.testing.assert_allclose(got, ref[key], rtol=1.2e-7, atol=1e-8)
+
+
+@pytest.mark.parametrize("clusters", [2, 3, 4, 5])
+@pytest.mark.parametrize("n", [130, 1031, 40_007])
+def test_labels_in_no_order(n, clusters):
+    """Dozens of runs a warp: up to four labels are summed over the warp, more by runs; exact sums, so the
+    oracle's bits, in three and (the one-hot model) four dimensions."""
+    from paper_2307_00071_gb300 import gira
+    rng = np.random.default_rng(n + clusters)
+    corners = 16.0 * np.array([[0, 0, 0], [1, 0, 0], [0, 1, 0], [0, 0, 1], [1, 1, 1]])[:clusters]
+    pts = (corners[rng.integers(clusters, size=n)] + rng.integers(-512, 513, size=(n, 3)) / 1024.0).astype(np.float32)
+    c0, _ = oracle.kmeanspp(pts, clusters, 1)
+    ref_c, ref_lab, ref_done = oracle.lloyd(pts, c0, 6)
+    c, lab, done = gira.gira_kmeans_init(pts, clusters, seed=1, lloyd_iters=6)
+    assert done == ref_done
+    np.testing.assert_array_equal(np.asarray(lab), ref_lab)
+    np.testing.assert_array_equal(np.asarray(c), ref_c.astype(np.float32))
+    full = np.concatenate([pts, rng.integers(0, 1025, size=(n, 1)) / 1024.0], axis=1).astype(np.float32)
+    r = gira.gira_gmm_fit4(full, clusters, iters=0, seed=1, lloyd_iters=3, reg_covar=1e-3, final_loglik=False)
+    ref = oracle.kinit(full, clusters, 1, 3, 1e-3)
+    for key in ("weights", "means", "covs"):
+        np.testing.assert_allclose(np.asarray(r[key], np.float64), ref[key], rtol=1.2e-7, atol=1e-7)
