@@ -1700,8 +1700,8 @@ gira_status gira_gmm_loglik_grad_batched(const float* points, const int64_t* off
             }
             if (e == cudaSuccess) e = launch_estep_reach(3, a, 2, (int)units.size(), rh, kmax, cs);
             if (e == cudaSuccess && gpar) e = launch_reach_stats(3, a, b.partials, cs);
-            const ReachGradArgs f{gpar ? b.partials : nullptr, b.live2, 0, b.llp, b.ppart, 0, b.poses, b.params, b.model64,
-                                  b.perm, kmax, 0, gpar ? b.gl : nullptr, gpar ? b.gm : nullptr, b.gpose, b.gtwist, b.st};
+            const ReachGradArgs f{gpar ? b.partials : nullptr, b.live2, b.llp, b.ppart, b.poses, b.params, b.model64, b.perm,
+                                  kmax, b.gl, b.gm, b.gpose, b.gtwist, b.st};
             if (e == cudaSuccess) e = launch_reach_grad_finalize(f, b.insts, batch, cs);
         }
         cudaGraph_t graph = nullptr;

@@ -80,7 +80,6 @@ __device__ __forceinline__ float2 dup(float a) { return make_float2(a, a); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
 
 // a * b rounded on its own: ptxas contracts a packed multiplication whose result is added
 // (__fmul2_rn, and mul.rn.f32x2 too: a probe against the scalar _rn form differed in 21 % of
@@ -179,9 +178,6 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
         : "memory");
     return ok != 0;
 }
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
 // Programmatic dependent launch (PTX griddepcontrol).  In a kernel launched with
 // programmatic stream serialisation, pdl_wait() returns once the previous kernel
 // of the stream has completed and its writes are visible, and pdl_allow_next()
@@ -189,9 +185,6 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
 // launch both have no effect.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_allow_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void named_bar_sync(int id, int nthreads) {
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
-}
 __device__ __forceinline__ uint64_t globaltimer_ns() {
     uint64_t t;
     asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
@@ -521,7 +514,7 @@ struct ReachLaunch {
     // gradient (mode 2)
     float* grad_pts = nullptr;        // [n][3], at order[i] (or i) for the i-th point, or nullptr
     const int* order = nullptr;
-    const float* rot = nullptr;       // R of x' = R x + t, or nullptr
+    const float* rot = nullptr;       // batch x 12: R (row-major) of x' = R x + t, then t
     double* pose_partials = nullptr;  // [grid][12]
     // batched gradient launches: as EStepLaunch
     const BatchInst* insts = nullptr;
@@ -747,23 +740,21 @@ cudaError_t launch_params_from_chol(const float* logits, const float* mu, const 
                                     int* perm, float4* ctr, float2* aux, DeviceState* st, cudaStream_t s);
 // Sums of a gradient launch (fixed order): dL/dlogits (k), dL/dmeans (k x 3) in binary32
 // from the statistics, in the caller's order; in binary64 dL/dpose (dL/dR row-major, dL/dt) and dL/dtwist (omega, v); the log-likelihood in
-// st->ll_sum.  Outputs nullable; partials nullptr: no parameter gradients.
+// st->ll_sum, for every instance of a batch (bases offset by its table entry).
+// partials nullptr: no parameter gradients.
 struct ReachGradArgs {
     const float* partials;    // [slices][pairs][2 NSTAT], live where live2 says
     const uint32_t* live2;    // [words][slices]
-    int slices;
-    const double* llp;        // [grid]
-    const double* pp;         // [grid][12]
-    int grid;
-    const float* pose;
+    const double* llp;        // per CTA
+    const double* pp;         // per CTA, 12 each
+    const float* poses;       // batch x 12
     const float* params;
     const double* model64;
     const int* perm;
-    int k;
-    int64_t n;
+    int kmax;                 // the largest k
     float *g_logits, *g_means;
     double *g_pose, *g_twist;
-    DeviceState* st;
+    DeviceState* states;
 };
 cudaError_t launch_reach_grad_finalize(const ReachGradArgs& f, const BatchInst* insts, int batch, cudaStream_t s);
 

@@ -724,16 +724,10 @@ __global__ void __launch_bounds__(32 * cta_warps(H), H > RB_W ? 16 / H : D == 3 
                 if (a_in.grad_pts) {
                     const int64_t at = pt0 + base + 32 * p;
                     float* gp = a_in.grad_pts + 3 * (a_in.order ? (int64_t)a_in.order[at] : at);
-                    if (a_in.rot) {
-                        const float* Rm = a_in.rot + 12 * (size_t)inst;
-                        gp[0] = fmaf(Rm[6], g3[p][2], fmaf(Rm[3], g3[p][1], Rm[0] * g3[p][0]));
-                        gp[1] = fmaf(Rm[7], g3[p][2], fmaf(Rm[4], g3[p][1], Rm[1] * g3[p][0]));
-                        gp[2] = fmaf(Rm[8], g3[p][2], fmaf(Rm[5], g3[p][1], Rm[2] * g3[p][0]));
-                    } else {
-                        gp[0] = g3[p][0];
-                        gp[1] = g3[p][1];
-                        gp[2] = g3[p][2];
-                    }
+                    const float* Rm = a_in.rot + 12 * (size_t)inst;
+                    gp[0] = fmaf(Rm[6], g3[p][2], fmaf(Rm[3], g3[p][1], Rm[0] * g3[p][0]));
+                    gp[1] = fmaf(Rm[7], g3[p][2], fmaf(Rm[4], g3[p][1], Rm[1] * g3[p][0]));
+                    gp[2] = fmaf(Rm[8], g3[p][2], fmaf(Rm[5], g3[p][1], Rm[2] * g3[p][0]));
                 }
             }
 #pragma unroll
@@ -942,25 +936,14 @@ static_assert(RG_THREADS % 32 == 0, "whole warps");
 __global__ void __launch_bounds__(RG_THREADS) reach_grad_finalize_kernel(const ReachGradArgs f_in,
                                                                          const BatchInst* __restrict__ insts) {
     __shared__ double s_stat[2 * RG_PAIRS][NSTAT];
-    // an instance's offsets into the launch's arrays (as in estep_reach_kernel)
-    int k = f_in.k, slices = f_in.slices, ctas = f_in.grid;
-    int64_t n = f_in.n;
-    size_t c_off = 0, part_off = 0, live_off = 0, ll_off = 0, par_off = 0;
+    // the instance's offsets into the launch's arrays (as in estep_reach_kernel)
     const int inst = blockIdx.x;   // (a grid's other dimensions end at 65,535)
-    if (insts) {
-        const BatchInst I = insts[inst];
-        int sl;
-        slices = reach_slices(I.n, &sl);
-        c_off = I.comp_off;
-        part_off = I.part_off;
-        live_off = I.live_off;
-        ll_off = I.ll_off;
-        par_off = I.par_off;
-        ctas = I.ctas;
-        k = I.k;
-        n = I.n;
-    }
-    DeviceState* const st = f_in.st + inst;
+    const BatchInst I = insts[inst];
+    int sl;
+    const int k = I.k, slices = reach_slices(I.n, &sl), ctas = I.ctas;
+    const int64_t n = I.n;
+    const size_t c_off = I.comp_off, part_off = I.part_off, live_off = I.live_off, ll_off = I.ll_off, par_off = I.par_off;
+    DeviceState* const st = f_in.states + inst;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int npairs = (k + 1) >> 1, pair0 = blockIdx.y * RG_PAIRS;
     if (pair0 >= npairs || st->error) return;
@@ -991,15 +974,14 @@ __global__ void __launch_bounds__(RG_THREADS) reach_grad_finalize_kernel(const R
             const double* S = s_stat[lane];
             const int src_b = f_in.perm[c_off + b];
             const float* q = f_in.params + par_off + (size_t)(b >> 1) * PAIR_FLOATS + (b & 1);
-            if (f_in.g_means)
 #pragma unroll
-                for (int i = 0; i < 3; ++i) {
-                    double gm = 0.0;
+            for (int i = 0; i < 3; ++i) {
+                double gm = 0.0;
 #pragma unroll
-                    for (int m = i; m < 3; ++m) gm += (double)q[2 * (SLOT_P + m * (m + 1) / 2 + i)] * S[1 + m];
-                    f_in.g_means[3 * (c_off + src_b) + i] = (float)(1.3862943611198906 * gm);
-                }
-            if (f_in.g_logits) f_in.g_logits[c_off + src_b] = (float)(S[0] - (double)n * f_in.model64[(c_off + b) * MODEL]);
+                for (int m = i; m < 3; ++m) gm += (double)q[2 * (SLOT_P + m * (m + 1) / 2 + i)] * S[1 + m];
+                f_in.g_means[3 * (c_off + src_b) + i] = (float)(1.3862943611198906 * gm);
+            }
+            f_in.g_logits[c_off + src_b] = (float)(S[0] - (double)n * f_in.model64[(c_off + b) * MODEL]);
         }
     }
     if (blockIdx.y != 0 || warp != 1) return;
@@ -1019,24 +1001,21 @@ __global__ void __launch_bounds__(RG_THREADS) reach_grad_finalize_kernel(const R
         st->ll_sum = v[0];
         const double* M = v + 1;    // sum g x'^T
         const double* G = v + 10;   // sum g
-        if (f_in.g_twist) {
+        {
             double* const g_twist = f_in.g_twist + 6 * (size_t)inst;   // omega = sum x' x g, v = sum g
             g_twist[0] = M[3 * 2 + 1] - M[3 * 1 + 2];
             g_twist[1] = M[3 * 0 + 2] - M[3 * 2 + 0];
             g_twist[2] = M[3 * 1 + 0] - M[3 * 0 + 1];
             for (int i = 0; i < 3; ++i) g_twist[3 + i] = G[i];
         }
-        if (f_in.g_pose) {    // x = R^T (x' - t): dL/dR = (sum g x'^T - G t^T) R, dL/dt = G
-            const float* const pose = f_in.pose ? f_in.pose + 12 * (size_t)inst : nullptr;
+        {   // x = R^T (x' - t): dL/dR = (sum g x'^T - G t^T) R, dL/dt = G
+            const float* const pose = f_in.poses + 12 * (size_t)inst;
             double* const g_pose = f_in.g_pose + 12 * (size_t)inst;
-            const double tt[3] = {pose ? pose[9] : 0.0, pose ? pose[10] : 0.0, pose ? pose[11] : 0.0};
+            const double tt[3] = {pose[9], pose[10], pose[11]};
             for (int i = 0; i < 3; ++i)
                 for (int j = 0; j < 3; ++j) {
                     double acc = 0.0;
-                    for (int m = 0; m < 3; ++m) {
-                        const double Rmj = pose ? (double)pose[3 * m + j] : (m == j ? 1.0 : 0.0);
-                        acc += (M[3 * i + m] - G[i] * tt[m]) * Rmj;
-                    }
+                    for (int m = 0; m < 3; ++m) acc += (M[3 * i + m] - G[i] * tt[m]) * (double)pose[3 * m + j];
                     g_pose[3 * i + j] = acc;
                 }
             for (int i = 0; i < 3; ++i) g_pose[9 + i] = G[i];
@@ -1046,10 +1025,10 @@ __global__ void __launch_bounds__(RG_THREADS) reach_grad_finalize_kernel(const R
 
 }  // namespace
 
-// f.k: the largest k of a batch.  Without parameter gradients one block per instance.
+// Without parameter gradients one block per instance.
 cudaError_t launch_reach_grad_finalize(const ReachGradArgs& f, const BatchInst* insts, int batch, cudaStream_t s) {
-    const int blocks = f.partials ? ((f.k + 1) / 2 + RG_PAIRS - 1) / RG_PAIRS : 1;
-    reach_grad_finalize_kernel<<<dim3(insts ? batch : 1, blocks), RG_THREADS, 0, s>>>(f, insts);
+    const int blocks = f.partials ? ((f.kmax + 1) / 2 + RG_PAIRS - 1) / RG_PAIRS : 1;
+    reach_grad_finalize_kernel<<<dim3(batch, blocks), RG_THREADS, 0, s>>>(f, insts);
     return cudaGetLastError();
 }
 
