@@ -1229,6 +1229,7 @@ __host__ __device__ constexpr size_t lloyd4_smem(int npair) {
     return sizeof(CPair4) * (size_t)npair + (npair <= LL4_LIST_MAX ? (LL4_THREADS / 32) * (size_t)npair * 2 : 0);
 }
 
+template <bool CROWDED>
 __global__ void __launch_bounds__(LL4_THREADS) lloyd4_assign_kernel(const float4* __restrict__ pts, int64_t n, int k,
                                                                     const float4* __restrict__ centers,
                                                                     int32_t* labels, double* sums,
@@ -1366,7 +1367,7 @@ __global__ void __launch_bounds__(LL4_THREADS) lloyd4_assign_kernel(const float4
 #pragma unroll
             for (int j = 0; j < 4; ++j) x[r][j] = X[r][j].x;
         }
-        add_runs<4>(key, x, n > 4096, sums);
+        add_runs<4, CROWDED>(key, x, sums);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(FULL, cnt, o);
@@ -1453,15 +1454,15 @@ cudaError_t launch_lloyd4(const float4* pts4, int64_t n, int k, int lloyd_iters,
     const size_t smem = lloyd4_smem((k + 1) / 2);
     const int64_t want = (n + (int64_t)LL4_THREADS * LL4_PPT - 1) / ((int64_t)LL4_THREADS * LL4_PPT);
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)num_sms_now() * 8));
+    auto* const assign = k <= CROWDED_LABELS && n > CROWDED_POINTS ? lloyd4_assign_kernel<true> : lloyd4_assign_kernel<false>;
     if (smem > 48 * 1024) {
-        const cudaError_t e =
-            cudaFuncSetAttribute(lloyd4_assign_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = cudaFuncSetAttribute(assign, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    lloyd4_assign_kernel<<<grid, LL4_THREADS, smem, s>>>(pts4, n, k, centers, labels, sums, changed, 0, nz, st);
+    assign<<<grid, LL4_THREADS, smem, s>>>(pts4, n, k, centers, labels, sums, changed, 0, nz, st);
     for (int it = 1; it <= lloyd_iters; ++it) {
         lloyd4_update_kernel<<<(k + 127) / 128, 128, 0, s>>>(k, sums, centers, changed, it, st);
-        lloyd4_assign_kernel<<<grid, LL4_THREADS, smem, s>>>(pts4, n, k, centers, labels, sums, changed, it, nz, st);
+        assign<<<grid, LL4_THREADS, smem, s>>>(pts4, n, k, centers, labels, sums, changed, it, nz, st);
     }
     return cudaGetLastError();
 }

@@ -372,11 +372,13 @@ __device__ __forceinline__ void join_runs(int key_first, int key_last, bool whol
 // which bound this (64 cycles each per warp): 39 for 128 points in 3-D, where one point per lane
 // and a scan for each of four rounds took 92.
 // Points in no order under two to four labels have dozens of runs a warp and all their atomics
-// on a few addresses: there (`crowded`, more than 4,096 points) each label's points are summed over
-// the warp instead, in a fixed order, for one set of atomics each.  KInit with five Lloyd iterations of
-// shuffled points, K = 2: 300,000 2,750 us by runs, 335 so; 20,000 341 and 170; but 1,000 139 and 169.
-template <int D>
-__device__ __forceinline__ void add_runs(const int (&key)[4], const float (&x)[4][D], bool crowded, double* sums) {
+// on a few addresses: there (CROWDED: up to four labels in all, more than 4,096 points) each label's
+// points are summed over the warp instead, in a fixed order, for one set of atomics each.  KInit with
+// five Lloyd iterations of shuffled points, K = 2: 300,000 2,750 us by runs, 335 so; 20,000 341 and 170;
+// but 1,000 139 and 169.
+constexpr int CROWDED_LABELS = 4, CROWDED_POINTS = 4096;
+template <int D, bool CROWDED>
+__device__ __forceinline__ void add_runs(const int (&key)[4], const float (&x)[4][D], double* sums) {
     auto put = [&](int k, const double (&v)[D], int c) {
         if (k < 0) return;
         double* s = sums + (size_t)(D + 1) * k;
@@ -385,8 +387,8 @@ __device__ __forceinline__ void add_runs(const int (&key)[4], const float (&x)[4
         atomicAdd(s + D, (double)c);
     };
     constexpr unsigned ALL = 0xffffffffu;
-    constexpr int MANY = 24, LABELS = 4;
-    if (crowded && __reduce_add_sync(ALL, (key[1] != key[0]) + (key[2] != key[1]) + (key[3] != key[2])) >= MANY) {
+    constexpr int MANY = 24, LABELS = CROWDED_LABELS + 1;   // and -1
+    if (CROWDED && __reduce_add_sync(ALL, (key[1] != key[0]) + (key[2] != key[1]) + (key[3] != key[2])) >= MANY) {
         int label[LABELS], found = 0;
         unsigned open = 0xfu;   // this lane's points whose label is not found yet
 #pragma unroll

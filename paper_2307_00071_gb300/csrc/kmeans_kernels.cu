@@ -1209,6 +1209,7 @@ struct CPair {
 
 // The points of groups g0 = first, first + stride, ... (LL_THREADS * LL_PPT points
 // each) against the k centres in shared memory.
+template <bool CROWDED>
 __device__ void lloyd_assign_groups(const float4* __restrict__ pts, int64_t n, int npair, const CPair* sc,
                                     int32_t* labels, double* sums, unsigned long long* changed, int it,
                                     int64_t first, int64_t stride, uint16_t* lists);
@@ -1220,6 +1221,7 @@ __host__ __device__ inline size_t lloyd_smem_bytes(int npair) {
     return sizeof(CPair) * (size_t)npair + (npair <= LL_LIST_MAX ? (LL_THREADS / 32) * (size_t)npair * 2 : 0);
 }
 
+template <bool CROWDED>
 __global__ void __launch_bounds__(LL_THREADS) lloyd_assign_kernel(
     const float4* __restrict__ pts, int64_t n, int k, const float4* __restrict__ centers, int32_t* labels,
     double* sums, unsigned long long* changed, int it, DeviceState* st) {
@@ -1235,7 +1237,7 @@ __global__ void __launch_bounds__(LL_THREADS) lloyd_assign_kernel(
     __syncthreads();
     const int64_t group = (int64_t)LL_THREADS * LL_PPT;
     uint16_t* lists = npair <= LL_LIST_MAX ? reinterpret_cast<uint16_t*>(sc + npair) : nullptr;
-    lloyd_assign_groups(pts, n, npair, sc, labels, sums, changed, it, (int64_t)blockIdx.x * group,
+    lloyd_assign_groups<CROWDED>(pts, n, npair, sc, labels, sums, changed, it, (int64_t)blockIdx.x * group,
                         (int64_t)gridDim.x * group, lists);
 }
 
@@ -1260,10 +1262,11 @@ __global__ void __launch_bounds__(LL_THREADS) lloyd_assign_batched_kernel(
     __syncthreads();
     const int64_t group = (int64_t)LL_THREADS * LL_PPT;
     uint16_t* lists = npair <= LL_LIST_MAX ? reinterpret_cast<uint16_t*>(sc + npair) : nullptr;
-    lloyd_assign_groups(pts + e.pt_off, e.n, npair, sc, labels + e.pt_off, sums + 4 * (size_t)e.comp_off, chg, it,
+    lloyd_assign_groups<false>(pts + e.pt_off, e.n, npair, sc, labels + e.pt_off, sums + 4 * (size_t)e.comp_off, chg, it,
                         (int64_t)u.cta * group, INT64_MAX / 2, lists);
 }
 
+template <bool CROWDED>
 __device__ void lloyd_assign_groups(const float4* __restrict__ pts, int64_t n, int npair, const CPair* sc,
                                     int32_t* labels, double* sums, unsigned long long* changed, int it,
                                     int64_t first, int64_t stride, uint16_t* lists) {
@@ -1380,7 +1383,7 @@ __device__ void lloyd_assign_groups(const float4* __restrict__ pts, int64_t n, i
             x[r][1] = Y[r].x;
             x[r][2] = Z[r].x;
         }
-        add_runs<3>(key, x, n > 4096, sums);
+        add_runs<3, CROWDED>(key, x, sums);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(FULL, cnt, o);
@@ -1752,14 +1755,15 @@ cudaError_t launch_lloyd(const float4* pts4, int64_t n, int k, int lloyd_iters, 
     const int threads = LL_THREADS;
     const int64_t want = (n + (int64_t)threads * LL_PPT - 1) / ((int64_t)threads * LL_PPT);
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)sms * 4));
+    auto* const assign = k <= CROWDED_LABELS && n > CROWDED_POINTS ? lloyd_assign_kernel<true> : lloyd_assign_kernel<false>;
     cudaError_t e = cudaSuccess;
     if (smem > 48 * 1024)
-        e = cudaFuncSetAttribute(lloyd_assign_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = cudaFuncSetAttribute(assign, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    lloyd_assign_kernel<<<grid, threads, smem, s>>>(pts4, n, k, centers, labels, sums, changed, 0, st);
+    assign<<<grid, threads, smem, s>>>(pts4, n, k, centers, labels, sums, changed, 0, st);
     for (int it = 1; it <= lloyd_iters; ++it) {
         lloyd_update_kernel<<<(k + 127) / 128, 128, 0, s>>>(k, sums, centers, changed, it, st);
-        lloyd_assign_kernel<<<grid, threads, smem, s>>>(pts4, n, k, centers, labels, sums, changed, it, st);
+        assign<<<grid, threads, smem, s>>>(pts4, n, k, centers, labels, sums, changed, it, st);
     }
     return cudaGetLastError();
 }
