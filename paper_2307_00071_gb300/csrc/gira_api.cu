@@ -83,6 +83,21 @@ gira_status side_streams(DeviceWs* ws) {
     return GIRA_OK;
 }
 
+// Back to the driver (the workspace's device is current; nothing of them is in flight after a
+// call); the next batched call makes them again.
+void drop_streams(DeviceWs* ws) {
+    for (int i = 0; i < 4; ++i) {
+        if (ws->side[i]) cudaStreamDestroy(ws->side[i]);
+        if (ws->join[i]) cudaEventDestroy(ws->join[i]);
+        ws->side[i] = nullptr;
+        ws->join[i] = nullptr;
+    }
+    if (ws->fork) cudaEventDestroy(ws->fork);
+    if (ws->capture_stream) cudaStreamDestroy(ws->capture_stream);
+    ws->fork = nullptr;
+    ws->capture_stream = nullptr;
+}
+
 void drop_graph(DeviceWs* ws) {
     if (ws->graph_exec) cudaGraphExecDestroy(ws->graph_exec);
     ws->graph_exec = nullptr;
@@ -277,7 +292,8 @@ struct CallProfile {
 };
 
 // k-means++ of one cloud (pts4 in the caller's order, which defines the draws), by the
-// first form that applies; every form draws the same points.
+// first form that applies; every form draws the same points (but for the last bit of D^2 in
+// the first: see dist2_f32).
 //  - 3-D up to 294,912 points: one cluster with the points in shared memory;
 //  - 4-D, or more points: one cluster with the points in L2, when each of its warps has at
 //    most 8 sub-blocks of 32 points or the points' order is coherent (one kernel and one
@@ -452,8 +468,9 @@ gira_status gira_release_workspace(void) {
         if (!g_ws[d]) continue;
         std::lock_guard<std::mutex> l2(g_ws[d]->mu);
         drop_graph(g_ws[d]);
+        cudaSetDevice((int)d);
+        drop_streams(g_ws[d]);
         if (g_ws[d]->ptr) {
-            cudaSetDevice((int)d);
             cudaError_t e = cudaFree(g_ws[d]->ptr);
             g_ws[d]->ptr = nullptr;
             g_ws[d]->bytes = 0;

@@ -184,3 +184,38 @@ def test_large_batch_equals_small_batches(gira, kinit):
         for key in ("weights", "means", "covs"):
             np.testing.assert_array_equal(to_np(part[key]), to_np(big[key])[at[lo]:at[hi]])
         np.testing.assert_array_equal(np.asarray(part["trace"]), np.asarray(big["trace"])[lo:hi])
+
+
+def test_on_a_stream_of_the_callers_beside_another(gira):
+    """The seeding's side streams fork from and join the caller's stream: on a stream of its own, with another
+    stream busy and inputs written there just before the call, the fit is that of the default stream (the
+    one-hot sums' atomics may end in another last bit: binary32 outputs to 1e-5)."""
+    import torch
+    rng = np.random.default_rng(4)
+    ns, ks = [2_500, 19_000, 45_000, 90_000, 150_000], [16, 16, 32, 32, 32]   # five cluster sizes
+    offs = np.concatenate([[0], np.cumsum(ns)]).astype(np.int64)
+    pts = torch.as_tensor(rng.normal(size=(offs[-1], 3)).astype(np.float32), device="cuda")
+    opts = dict(iters=3, tol=0.0, reg_covar=1e-4, seed=2)
+    ref = gira.gira_gmm_fit_batched(pts, offs, ks, **opts)
+    torch.cuda.synchronize()
+    busy, own = torch.cuda.Stream(), torch.cuda.Stream()
+    a = torch.ones(2048, 2048, device="cuda")
+    torch.cuda.synchronize()
+    with torch.cuda.stream(busy):
+        for _ in range(200):
+            a = (a @ a) * 1e-4
+    with torch.cuda.stream(own):
+        late = pts * 0.0
+        for _ in range(20):
+            late = late + 0.05 * pts
+        late.copy_(pts)
+        got = gira.gira_gmm_fit_batched(late, offs, ks, **opts)
+    torch.cuda.synchronize()
+    for key in ("weights", "means", "covs"):
+        x, y = to_np(got[key]).astype(np.float64), to_np(ref[key]).astype(np.float64)
+        assert np.abs(x - y).max() <= 1e-5 * np.abs(y).max(), key
+    gira.gira_release_workspace()   # with the side streams and events: made again by the next call
+    again = gira.gira_gmm_fit_batched(pts, offs, ks, **opts)
+    for key in ("weights", "means", "covs"):
+        x, y = to_np(again[key]).astype(np.float64), to_np(ref[key]).astype(np.float64)
+        assert np.abs(x - y).max() <= 1e-5 * np.abs(y).max(), key
