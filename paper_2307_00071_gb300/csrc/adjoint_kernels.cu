@@ -1,16 +1,15 @@
 // adjoint_kernels.cu -- the gradient of the log-likelihood with every component at every
 // point and the statistics about mu_b in world axes: every call on one scan, and batched calls
-// that ask for dL/dL_b (Cholesky factors).
+// that ask for dL/dL_b (Cholesky factors) or have little work (gradient_dense in gira_api.cu has
+// the rule and both sides measured).  Other batched calls take the reach lists.
 //
 // dL/dL_b = lower(P^T (P S2 P^T)) - S0 diag(1/L_ii) multiplies S2 = sum gamma d d^T four
 // times by P = L_b^{-1}: for a component thin in one direction (a wall, millimetres against
 // decimetres) the binary32 rounding of S2's sums is amplified by the square of its aspect
-// ratio, and the value carries up to 1e-4 of it.  The statistics over reach lists
-// (reach_kernels.cu, in whitened coordinates) are an order of magnitude closer to 64-bit
-// results there, but differ from these values by that rounding; callers that compare or
-// resume Cholesky gradients get the same bits as ever from this kernel, and a call on one
-// scan gives the same bits whichever gradients it asks for.  Batched calls for the other
-// gradients (registrations: the twists) take the reach lists.
+// ratio, and the value carries up to 1e-4 of it.  Statistics in whitened coordinates, as the
+// reach lists keep them, are an order of magnitude closer to 64-bit results there, but no
+// finish of dL/dL_b from them exists, and its values would move by that rounding.  A call on one
+// scan gives the same bits whichever gradients it asks for.
 //
 // Mapping (component-stationary): one CTA holds all K <= 1024 components, spread over its
 // warps; lane l of warp w owns NP component pairs in registers.  All lanes walk the CTA's
@@ -68,7 +67,8 @@ constexpr int QB = 8;                                 // points per batch
 // gamma P'^T P' d.  The per-point sums are double-buffered by batch parity: a warp can only
 // overwrite a buffer after the next barrier, which every warp reaches after reading it.  The
 // owner lanes write dL/dx = R^T dL/dx' and accumulate the pose sums (dL/dx' x'^T, dL/dx').
-// Measured: 336 us for 100k points at K = 1024.
+// Measured: 100k points, K = 1024: 266 to 274 us for a scan on its model, 313 to 339 us for one 0.1 to
+// 0.5 m off it (points more than 100 binades below the reference take the exact maximum).
 template <int NP, int Q, int MAXT, int MINB, bool GRAD>
 __global__ void __launch_bounds__(MAXT, MINB) estep_adjoint_kernel(const AdjointLaunch a_in) {
     extern __shared__ __align__(128) unsigned char dsm[];

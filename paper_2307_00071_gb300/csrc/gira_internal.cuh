@@ -84,7 +84,8 @@ __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a
 // a * b rounded on its own: ptxas contracts a packed multiplication whose result is added
 // (__fmul2_rn, and mul.rn.f32x2 too: a probe against the scalar _rn form differed in 21 % of
 // random squared distances) and folds an fma with a literal -0; with a -0 it cannot see
-// (nz = (-0, -0), a kernel argument) the product stays one rounded operation.
+// (nz = (-0, -0), a kernel argument) the product stays one rounded operation.  4-D Lloyd uses it;
+// the packed 3-D kernels do not (dist2_f32 says what that means).
 __device__ __forceinline__ float2 mul2_alone(float2 a, float2 b, float2 nz) { return fma2(a, b, nz); }
 
 __device__ __forceinline__ float ex2_approx(float x) {
@@ -229,8 +230,15 @@ __device__ __forceinline__ bool wait_counter_bounded(const int* counter, int tar
 }
 
 // binary32 squared distance in the fixed order d_i = x_i - c_i; (d0^2 + d1^2) + d2^2,
-// every operation rounded separately (no contraction): k-means decisions are taken
-// in exactly this arithmetic.
+// every operation rounded separately (no contraction): the D^2 of the seeding kernels over
+// sub-blocks, of the persistent one and of two launches per centre, and (dist2_f32_4) every
+// distance in four dimensions.  The packed 3-D kernels (kpp_cluster_kernel and Lloyd's
+// assignment) write the same order, but the compiler fuses the additions with the products: they
+// compute fma(d2, d2, fma(d0, d0, d1^2)) (the labels of 156,000 near ties are that form's, every
+// one), within 1.5 units in the last place of it.  Labels then differ from this arithmetic's only
+// between centres whose distances agree to 2^-22 (about one point in a few frames), draws only
+// where the running sum meets the threshold within that rounding (none in 26 seedings of 100 to
+// 512 centres compared).
 __device__ __forceinline__ float dist2_f32(float4 x, float4 c) {
     float d0 = __fsub_rn(x.x, c.x), d1 = __fsub_rn(x.y, c.y), d2 = __fsub_rn(x.z, c.z);
     float s = __fadd_rn(__fmul_rn(d0, d0), __fmul_rn(d1, d1));

@@ -676,7 +676,7 @@ __global__ void __launch_bounds__(KC_THREADS, 1) kpp_cluster_kernel(const float4
         // 64-bit totals: set by this CTA's warp 0 at centre j - 1 or before, from the same
         // totals in every CTA; every warp reads it before warp 0 can change it again
         const bool m64 = sh.m64 != 0;
-        // ---- 1. D^2 (packed: each lane of FADD2/FMUL2 rounds like dist2_f32) and,
+        // ---- 1. D^2 (packed; the order of dist2_f32, fused by the compiler as told there) and,
         //         where any D^2 dropped, the lane's exact sum from scratch (raster-
         //         order lanes see their points' D^2 drop together, so one pass over
         //         the lane beats per-point differences)
@@ -1194,8 +1194,8 @@ __global__ void __launch_bounds__(1024) kpp_coherence_kernel(const float4* __res
 // labels = argmin_b ||x - c_b||^2 (binary32, ties to the lowest b); binary64
 // sums of the raw coordinates and counts per label; changed[it] counts labels
 // that moved (every label for it == 0).  Centres are processed two at a time
-// with packed FP32 (each lane of FADD2/FMUL2 rounds exactly like the scalar
-// operation, so the distances are those of dist2_f32).  Each thread owns
+// with packed FP32 (in the order of dist2_f32, the additions fused with the
+// products, as told there).  Each thread owns
 // LL_PPT consecutive points; runs of equal labels are summed before the
 // atomics (add_runs).  Bound by the scan of the listed centres and the binary64 sums.
 // Measured per launch: 48 segments, 1.41M points, K <= 512: 105 us with a scan of one point

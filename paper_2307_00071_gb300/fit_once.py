@@ -5,7 +5,7 @@
 ``frame``: the 276k-point 640x480 depth frame, K=512, 30 iterations, tol 1e-4
 (the benchmark's step).  ``gmm20k``: 20k points from a K=8 GMM, 20 iterations.
 ``grad1024``: L and all gradients of a 100k-point scan under a K=1024 GMM of the
-frame (``--fits`` calls).  ``chunk2048``: the E-step above K=1024, K=2048 on the
+frame (``--fits`` calls).  ``large2048``: the E-step above K=1024, K=2048 on the
 frame.
 ``frame4``: the frame with its intensity channel (N x 4), K=512, 30 iterations,
 tol 1e-4.  ``gbms``: mode seeking on the frame with intensity, bandwidth 0.05.
@@ -23,15 +23,15 @@ from . import gira, synth
 
 def main():
     p = argparse.ArgumentParser()
-    p.add_argument("--workload", choices=["frame", "gmm20k", "grad1024", "chunk2048", "frame4", "gbms"],
+    p.add_argument("--workload", choices=["frame", "gmm20k", "grad1024", "large2048", "frame4", "gbms"],
                    default="frame")
     p.add_argument("--fits", type=int, default=1)
     a = p.parse_args()
     if a.workload == "grad1024":
         grad_workload(a.fits)
         return
-    if a.workload == "chunk2048":
-        chunk_workload(a.fits)
+    if a.workload == "large2048":
+        large_workload(a.fits)
         return
     if a.workload in ("frame4", "gbms"):
         x4 = torch.as_tensor(synth.depth_frame4(seed=1), device="cuda")
@@ -73,8 +73,8 @@ def grad_workload(calls):
     print(f"grad1024: loglik={r['loglik']:.3f}")
 
 
-def chunk_workload(fits):
-    """Chunked E-step: K=2048 on the frame from means at random points, 3 EM iterations."""
+def large_workload(fits):
+    """The E-step above K=1024: K=2048 on the frame from means at random points, 3 EM iterations."""
     frame = synth.depth_frame(seed=1).points
     x = torch.as_tensor(frame, device="cuda")
     rng = np.random.default_rng(3)
@@ -84,7 +84,7 @@ def chunk_workload(fits):
         c0 = (torch.eye(3, device="cuda") * 0.05 ** 2).expand(2048, 3, 3).contiguous()
         r = gira.gira_gmm_fit(x, 2048, iters=3, tol=0.0, init=(w0, x[idx].clone(), c0), final_loglik=False)
     torch.cuda.synchronize()
-    print(f"chunk2048: trace={list(r['trace'])}")
+    print(f"large2048: trace={list(r['trace'])}")
 
 
 if __name__ == "__main__":

@@ -77,3 +77,22 @@ def test_labels_in_no_order(n, clusters):
     ref = oracle.kinit(full, clusters, 1, 3, 1e-3)
     for key in ("weights", "means", "covs"):
         np.testing.assert_allclose(np.asarray(r[key], np.float64), ref[key], rtol=1.2e-7, atol=1e-7)
+
+
+def test_near_ties():
+    """Points around the plane half way between two centres: a label is the nearer centre, or one whose
+    distance agrees with it to 2^-21 (D^2 in binary32: four roundings, fused or not, on both sides)."""
+    from paper_2307_00071_gb300 import gira
+    rng = np.random.default_rng(7)
+    m = 50_000
+    a, b = rng.uniform(-1, 1, size=(2, 3)).astype(np.float32)
+    u = b.astype(np.float64) - a
+    u /= np.linalg.norm(u)
+    t = rng.normal(size=(m, 3))
+    t -= (t @ u)[:, None] * u
+    probes = (a.astype(np.float64) + b) / 2 + t + rng.normal(scale=1e-7, size=(m, 1)) * u
+    pts = np.concatenate([np.tile(a, (m, 1)), np.tile(b, (m, 1)), probes]).astype(np.float32)
+    c, lab, _ = gira.gira_kmeans_init(pts, 2, seed=0, lloyd_iters=0)
+    d = ((pts.astype(np.float64)[:, None] - np.asarray(c, np.float64)[None]) ** 2).sum(2)
+    mine = np.take_along_axis(d, np.asarray(lab, np.int64)[:, None], 1)[:, 0]
+    assert np.all(mine <= d.min(1) * (1 + 2.0 ** -21))
