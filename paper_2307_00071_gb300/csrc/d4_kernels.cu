@@ -59,7 +59,7 @@ constexpr long long MBAR_LIMIT4 = 2000000000ll;   // bound on the TMA wait: 2 s 
 constexpr float LN2F4 = 0.693147180559945309f;
 constexpr double LN2_4 = 0.693147180559945309417232121458;
 
-template <bool STATS>
+template <bool STATS, bool WORLD = false>   // WORLD: the statistics about x - mu, as in reach_stats_kernel
 __global__ void __launch_bounds__(512, 1) estep4_dense_kernel(const EStep4Launch a) {
     extern __shared__ __align__(128) unsigned char dsm4[];
     __shared__ __align__(8) uint64_t bar_tma;
@@ -219,7 +219,16 @@ __global__ void __launch_bounds__(512, 1) estep4_dense_kernel(const EStep4Launch
             for (int q = 0; q < Q4; ++q) {
                 const float2 g = mul2(E[q], dup(__shfl_sync(FULL, r, q * LPQ)));
                 float2 y[4];
-                whiten(q < nvalid ? lb + q : lb, y);
+                if (WORLD) {
+                    const int li = q < nvalid ? lb + q : lb;
+                    const float4 xy = spts[2 * li], zw = spts[2 * li + 1];
+                    y[0] = add2(f2(xy.x, xy.y), nmu[0]);
+                    y[1] = add2(f2(xy.z, xy.w), nmu[1]);
+                    y[2] = add2(f2(zw.x, zw.y), nmu[2]);
+                    y[3] = add2(f2(zw.z, zw.w), nmu[3]);
+                } else {
+                    whiten(q < nvalid ? lb + q : lb, y);
+                }
                 S[0] = add2(S[0], g);
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
@@ -320,6 +329,7 @@ struct Fin4Args {
     const int* perm;
     DeviceState* st;
     int iter, em;
+    bool world;   // the partials are about x - s: M = I
 };
 constexpr int FIN4_WARPS = 8;
 __global__ void __launch_bounds__(32 * FIN4_WARPS) reduce_finalize4_kernel(const Fin4Args f) {
@@ -332,8 +342,8 @@ __global__ void __launch_bounds__(32 * FIN4_WARPS) reduce_finalize4_kernel(const
     if ((f.em && f.iter > st->stop_after) || st->error) return;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int pp = blockIdx.x;
-    const bool white = f.partials != nullptr;
-    if (white) {
+    const bool white = f.partials != nullptr && !f.world;
+    if (f.partials) {
         const int npairs = (f.k + 1) >> 1;
         const uint32_t* lw = f.live2 ? f.live2 + (size_t)(pp >> 5) * f.slices : nullptr;   // nullptr: every row
         const float* src = f.partials + (size_t)pp * 2 * NSTAT4 + lane;
@@ -404,7 +414,7 @@ __global__ void __launch_bounds__(32 * FIN4_WARPS) reduce_finalize4_kernel(const
         // mu = (S0 / N_b) s + M ybar (lanes 0 .. 3), A = M C
         if (on && l < 4) {
             double s;
-            if (white) s = -(double)f.params[slot4(b, SLOT4_NMU + l)];
+            if (f.partials) s = -(double)f.params[slot4(b, SLOT4_NMU + l)];
             else s = l == 0 ? f.shift4[b].x : l == 1 ? f.shift4[b].y : l == 2 ? f.shift4[b].z : f.shift4[b].w;
             s *= S[0] * inv;   // sum_n r x / N_b: 0 for a component without support
             for (int m = 0; m <= l; ++m) s = __fma_rn(M[4 * l + m], S[1 + m] * inv, s);
@@ -548,6 +558,7 @@ __global__ void params_from_model4_kernel(const float* __restrict__ w, const flo
 
 __global__ void model_out4_kernel(const double* __restrict__ model64, int k, float* w, float* mu, float* cov,
                                   const int* __restrict__ perm, const DeviceState* st) {
+    if (st->error) return;         // the given model stays what it was (outputs of a failed call are unspecified)
     __shared__ double s_part[2];   // (the same sum in every block)
     double part = 0.0;
     for (int a2 = threadIdx.x; a2 < k; a2 += blockDim.x) part += model64[(size_t)a2 * MODEL4];
@@ -1511,7 +1522,9 @@ int estep4_dense_grid(int64_t n, int k, int num_sms, int64_t* ppc) {
 }
 
 cudaError_t launch_estep4_dense(const EStep4Launch& a, bool stats, int grid, cudaStream_t s, bool pdl) {
-    const void* fn = stats ? (const void*)estep4_dense_kernel<true> : (const void*)estep4_dense_kernel<false>;
+    const void* fn = !stats    ? (const void*)estep4_dense_kernel<false>
+                     : a.world ? (const void*)estep4_dense_kernel<true, true>
+                               : (const void*)estep4_dense_kernel<true>;
     note_estep_kernel(fn);
     void* args[] = {(void*)&a};
     PdlConfig c(dim3(grid), dim3(dense4_threads(a.k)), (size_t)a.pts_per_cta * 32, s, pdl);
@@ -1521,9 +1534,10 @@ cudaError_t launch_estep4_dense(const EStep4Launch& a, bool stats, int grid, cud
 cudaError_t launch_reduce_finalize4(const float* partials, const uint32_t* live2, int slices, const double* llp,
                                     int ll_count, const double* stats64, const float4* shift4, int k, int64_t n,
                                     double reg, double tol, double* model64, float* params, double* trace,
-                                    const int* perm, DeviceState* st, int iter, bool em, cudaStream_t s, bool pdl) {
+                                    const int* perm, DeviceState* st, int iter, bool em, cudaStream_t s, bool pdl,
+                                    bool world) {
     const Fin4Args f{partials, live2, slices, llp, ll_count, stats64, shift4, k, n, reg, tol, model64, params, trace,
-                     perm, st, iter, em ? 1 : 0};
+                     perm, st, iter, em ? 1 : 0, world};
     PdlConfig c(dim3((k + 1) / 2), dim3(32 * FIN4_WARPS), 0, s, pdl);
     return cudaLaunchKernelEx(&c.cfg, reduce_finalize4_kernel, f);
 }

@@ -410,12 +410,13 @@ cudaError_t reach_zero_live(const ReachBufs& b, cudaStream_t s) {
 }
 
 // One E-step with statistics: b.partials rows and b.live2 masks for the finalize.
-cudaError_t reach_estep_stats(int d, const ReachBufs& b, ReachLaunch a, long long* launches, cudaStream_t s) {
+cudaError_t reach_estep_stats(int d, const ReachBufs& b, ReachLaunch a, bool world, long long* launches,
+                              cudaStream_t s) {
     reach_with_stats(b, &a);
     cudaError_t e = launch_reach_prepare(d, a.params, a.k, a.st, a.iter, b.ctr, b.aux, b.gref, s);
     if (e == cudaSuccess) e = reach_zero_live(b, s);
     if (e == cudaSuccess) e = launch_estep_reach(d, a, 1, b.grid, b.h, a.k, s);
-    if (e == cudaSuccess) e = launch_reach_stats(d, a, b.partials, s);
+    if (e == cudaSuccess) e = launch_reach_stats(d, a, world, b.partials, s);
     *launches += 3;
     return e;
 }
@@ -724,7 +725,8 @@ gira_status gira_gmm_fit(const float* points, int64_t n, int k, const gira_fit_o
     if (large) {
         const float4* pe = sorted ? b.p8s : b.p8;
         for (int t = 1; t <= o.iters; ++t) {
-            GIRA_CUDA(reach_estep_stats(3, rb, reach_launch(rb, pe, n, k, b.params, b.st, t), &prof.launches, c.s));
+            GIRA_CUDA(reach_estep_stats(3, rb, reach_launch(rb, pe, n, k, b.params, b.st, t), false, &prof.launches,
+                                        c.s));
             COUNTED(prof, 1, launch_reduce_finalize(rb.partials, rb.slices, rb.llp, nullptr, b.shift4, k, n,
                                                     o.reg_covar, o.tol, b.model64, b.params, b.trace, b.st, t, true,
                                                     c.s, false, perm, rb.live2, rb.words, rb.grid));
@@ -1716,7 +1718,7 @@ gira_status gira_gmm_loglik_grad_batched(const float* points, const int64_t* off
                 if (e == cudaSuccess) e = cudaMemsetAsync(b.live2, 0, sizeof(uint32_t) * (live_words + 2), cs);
             }
             if (e == cudaSuccess) e = launch_estep_reach(3, a, 2, (int)units.size(), rh, kmax, cs);
-            if (e == cudaSuccess && gpar) e = launch_reach_stats(3, a, b.partials, cs);
+            if (e == cudaSuccess && gpar) e = launch_reach_stats(3, a, false, b.partials, cs);
             const ReachGradArgs f{gpar ? b.partials : nullptr, b.live2, b.llp, b.ppart, b.poses, b.params, b.model64, b.perm,
                                   kmax, b.gl, b.gm, b.gpose, b.gtwist, b.st};
             if (e == cudaSuccess) e = launch_reach_grad_finalize(f, b.insts, batch, cs);
@@ -1873,84 +1875,93 @@ gira_status gira_gmm_fit4(const float* points, int64_t n, int k, const gira_fit_
     prof.per_launch = g_prof_on.load() == 1;
     prof.s = c.s;
     prof.t0 = prof.mark();
+    // The statistics are whitened.  A point far off in one coordinate (1e5 m and more in a cloud of
+    // metres) then fills every later row of a component's sums, and binary32 loses the
+    // covariance, which sums about x - mu keep: such a fit, and one that truly ends
+    // there, is made once more with those.
     DeviceState h{};
-    h.stop_after = o.iters;
-    h.bad_component = INT_MAX;
-    GIRA_CUDA(cudaMemcpyAsync(b.st, &h, sizeof h, cudaMemcpyHostToDevice, c.s));
-    GIRA_CUDA(cudaMemsetAsync(b.trace, 0xff, sizeof(double) * std::max(o.iters, 1), c.s));   // NaN
-    const float* pts = points;
-    if (kp == Kind::Host) {
-        GIRA_CUDA(cudaMemcpyAsync(b.pin, points, sizeof(float) * 4 * n, cudaMemcpyHostToDevice, c.s));
-        pts = b.pin;
+    for (int world = 0; world < 2; ++world) {
+        h = DeviceState{};
+        h.stop_after = o.iters;
+        h.bad_component = INT_MAX;
+        GIRA_CUDA(cudaMemcpyAsync(b.st, &h, sizeof h, cudaMemcpyHostToDevice, c.s));
+        GIRA_CUDA(cudaMemsetAsync(b.trace, 0xff, sizeof(double) * std::max(o.iters, 1), c.s));   // NaN
+        const float* pts = points;
+        if (kp == Kind::Host) {
+            GIRA_CUDA(cudaMemcpyAsync(b.pin, points, sizeof(float) * 4 * n, cudaMemcpyHostToDevice, c.s));
+            pts = b.pin;
+        }
+        COUNTED(prof, 1, launch_pack4(pts, n, kinit ? b.p4 : nullptr, b.p8, b.st, c.s));
+        if (sorted)
+            COUNTED(prof, point_order_launches(1),
+                    launch_point_order(b.p8, n, nullptr, nullptr, 0, 1, b.osc, b.p8s, kinit ? b.p4s : nullptr, nullptr, c.s));
+        COUNTED(prof, 1, launch_fill_padding4(b.params, k, c.s));
+        float* w_d = (kw == Kind::Device) ? weights : b.mw;
+        float* mu_d = (km == Kind::Device) ? means : b.mmu;
+        float* cov_d = (kc == Kind::Device) ? covs : b.mcov;
+        if (kinit) {
+            TRY(seed_centres(prof, c, b.p4, n, 4, k, o.seed, b.c4, b.ch, b.d2, b.bs, b.ksync, b.ksums, kgrid, b.st));
+            GIRA_CUDA(cudaMemsetAsync(b.sums, 0, sizeof(double) * 5 * k, c.s));
+            GIRA_CUDA(cudaMemsetAsync(b.chg, 0, sizeof(unsigned long long) * (o.lloyd_iters + 1), c.s));
+            COUNTED(prof, 1 + 2 * o.lloyd_iters, launch_lloyd4(sorted ? b.p4s : b.p4, n, k, o.lloyd_iters, b.c4, b.lab, b.sums, b.chg,
+                                                              b.st, c.s));
+            GIRA_CUDA(cudaMemsetAsync(b.stats64, 0, sizeof(double) * NSTAT4 * k, c.s));
+            COUNTED(prof, 1, launch_label_stats4(sorted ? b.p4s : b.p4, n, k, b.lab, b.c4, b.stats64, b.st, c.s));
+            COUNTED(prof, 1, launch_reduce_finalize4(nullptr, nullptr, 0, nullptr, 0, b.stats64, b.c4, k, n, o.reg_covar,
+                                                     o.tol, b.model64, b.params, b.trace, nullptr, b.st, 0, false, c.s));
+        } else {
+            if (kw == Kind::Host) GIRA_CUDA(cudaMemcpyAsync(b.mw, weights, sizeof(float) * k, cudaMemcpyHostToDevice, c.s));
+            if (km == Kind::Host)
+                GIRA_CUDA(cudaMemcpyAsync(b.mmu, means, sizeof(float) * 4 * k, cudaMemcpyHostToDevice, c.s));
+            if (kc == Kind::Host)
+                GIRA_CUDA(cudaMemcpyAsync(b.mcov, covs, sizeof(float) * 16 * k, cudaMemcpyHostToDevice, c.s));
+            COUNTED(prof, 1, launch_params_from_model4(w_d, mu_d, cov_d, k, b.model64, b.params, nullptr, nullptr, b.st, c.s));
+        }
+        // components in Morton order of their means, as in the 3-D fit
+        const int* perm = dense ? nullptr : b.perm;
+        if (!dense) COUNTED(prof, 2, launch_order_components4(b.model64, b.stats64, k, b.perm, b.params, b.st, c.s));
+        prof.t_init = prof.mark();
+        const float4* pe = sorted ? b.p8s : b.p8;
+        EStep4Launch da{pe, n, k, b.params, ppc, b.partials, b.llp, nullptr, b.st, 0, world != 0};
+        for (int t = 1; t <= o.iters && dense; ++t) {
+            const bool pdl = !prof.per_launch;   // dependent launches, as in the 3-D loop
+            da.iter = t;
+            cudaEvent_t e0 = prof.mark_launch();
+            COUNTED(prof, 1, launch_estep4_dense(da, true, dgrid, c.s, pdl));
+            cudaEvent_t e1 = prof.mark_launch();
+            if (prof.per_launch) prof.timed(e0, e1);
+            COUNTED(prof, 1, launch_reduce_finalize4(b.partials, nullptr, dgrid, b.llp, dgrid, nullptr, nullptr, k, n, o.reg_covar,
+                                                     o.tol, b.model64, b.params, b.trace, perm, b.st, t, true, c.s, pdl,
+                                                     world != 0));
+        }
+        for (int t = 1; t <= o.iters && !dense; ++t) {
+            const ReachLaunch a = reach_launch(rb, pe, n, k, b.params, b.st, t);
+            cudaEvent_t e0 = prof.mark_launch();
+            GIRA_CUDA(reach_estep_stats(4, rb, a, world != 0, &prof.launches, c.s));
+            cudaEvent_t e1 = prof.mark_launch();
+            if (prof.per_launch) prof.timed(e0, e1);
+            COUNTED(prof, 1, launch_reduce_finalize4(rb.partials, rb.live2, rb.slices, rb.llp, rb.grid, nullptr, nullptr, k,
+                                                     n, o.reg_covar, o.tol, b.model64, b.params, b.trace, perm, b.st, t,
+                                                     true, c.s, false, world != 0));
+        }
+        prof.t_em = prof.mark();
+        if (final_loglik && dense) {
+            da.iter = 0;
+            COUNTED(prof, 1, launch_estep4_dense(da, false, dgrid, c.s));
+            COUNTED(prof, 1, launch_ll_reduce(b.llp, dgrid, b.st, c.s));
+        } else if (final_loglik)
+            GIRA_CUDA(reach_loglik(4, rb, reach_launch(rb, pe, n, k, b.params, b.st, 0), false, &prof.launches, c.s));
+        COUNTED(prof, 1, launch_model_out4(b.model64, k, w_d, mu_d, cov_d, perm, b.st, c.s));
+        if (kw == Kind::Host) GIRA_CUDA(cudaMemcpyAsync(weights, b.mw, sizeof(float) * k, cudaMemcpyDeviceToHost, c.s));
+        if (km == Kind::Host) GIRA_CUDA(cudaMemcpyAsync(means, b.mmu, sizeof(float) * 4 * k, cudaMemcpyDeviceToHost, c.s));
+        if (kc == Kind::Host) GIRA_CUDA(cudaMemcpyAsync(covs, b.mcov, sizeof(float) * 16 * k, cudaMemcpyDeviceToHost, c.s));
+        if (loglik_trace && o.iters > 0)
+            GIRA_CUDA(cudaMemcpyAsync(loglik_trace, b.trace, sizeof(double) * o.iters, cudaMemcpyDeviceToHost, c.s));
+        GIRA_CUDA(cudaMemcpyAsync(&h, b.st, sizeof h, cudaMemcpyDeviceToHost, c.s));
+        prof.t_end = prof.mark();
+        GIRA_CUDA(cudaStreamSynchronize(c.s));
+        if (h.error != GIRA_ERR_NOT_PD || h.iters_done == 0) break;   // 0: the start itself was not sound
     }
-    COUNTED(prof, 1, launch_pack4(pts, n, kinit ? b.p4 : nullptr, b.p8, b.st, c.s));
-    if (sorted)
-        COUNTED(prof, point_order_launches(1),
-                launch_point_order(b.p8, n, nullptr, nullptr, 0, 1, b.osc, b.p8s, kinit ? b.p4s : nullptr, nullptr, c.s));
-    COUNTED(prof, 1, launch_fill_padding4(b.params, k, c.s));
-    float* w_d = (kw == Kind::Device) ? weights : b.mw;
-    float* mu_d = (km == Kind::Device) ? means : b.mmu;
-    float* cov_d = (kc == Kind::Device) ? covs : b.mcov;
-    if (kinit) {
-        TRY(seed_centres(prof, c, b.p4, n, 4, k, o.seed, b.c4, b.ch, b.d2, b.bs, b.ksync, b.ksums, kgrid, b.st));
-        GIRA_CUDA(cudaMemsetAsync(b.sums, 0, sizeof(double) * 5 * k, c.s));
-        GIRA_CUDA(cudaMemsetAsync(b.chg, 0, sizeof(unsigned long long) * (o.lloyd_iters + 1), c.s));
-        COUNTED(prof, 1 + 2 * o.lloyd_iters, launch_lloyd4(sorted ? b.p4s : b.p4, n, k, o.lloyd_iters, b.c4, b.lab, b.sums, b.chg,
-                                                          b.st, c.s));
-        GIRA_CUDA(cudaMemsetAsync(b.stats64, 0, sizeof(double) * NSTAT4 * k, c.s));
-        COUNTED(prof, 1, launch_label_stats4(sorted ? b.p4s : b.p4, n, k, b.lab, b.c4, b.stats64, b.st, c.s));
-        COUNTED(prof, 1, launch_reduce_finalize4(nullptr, nullptr, 0, nullptr, 0, b.stats64, b.c4, k, n, o.reg_covar,
-                                                 o.tol, b.model64, b.params, b.trace, nullptr, b.st, 0, false, c.s));
-    } else {
-        if (kw == Kind::Host) GIRA_CUDA(cudaMemcpyAsync(b.mw, weights, sizeof(float) * k, cudaMemcpyHostToDevice, c.s));
-        if (km == Kind::Host)
-            GIRA_CUDA(cudaMemcpyAsync(b.mmu, means, sizeof(float) * 4 * k, cudaMemcpyHostToDevice, c.s));
-        if (kc == Kind::Host)
-            GIRA_CUDA(cudaMemcpyAsync(b.mcov, covs, sizeof(float) * 16 * k, cudaMemcpyHostToDevice, c.s));
-        COUNTED(prof, 1, launch_params_from_model4(w_d, mu_d, cov_d, k, b.model64, b.params, nullptr, nullptr, b.st, c.s));
-    }
-    // components in Morton order of their means, as in the 3-D fit
-    const int* perm = dense ? nullptr : b.perm;
-    if (!dense) COUNTED(prof, 2, launch_order_components4(b.model64, b.stats64, k, b.perm, b.params, b.st, c.s));
-    prof.t_init = prof.mark();
-    const float4* pe = sorted ? b.p8s : b.p8;
-    EStep4Launch da{pe, n, k, b.params, ppc, b.partials, b.llp, nullptr, b.st, 0};
-    for (int t = 1; t <= o.iters && dense; ++t) {
-        const bool pdl = !prof.per_launch;   // dependent launches, as in the 3-D loop
-        da.iter = t;
-        cudaEvent_t e0 = prof.mark_launch();
-        COUNTED(prof, 1, launch_estep4_dense(da, true, dgrid, c.s, pdl));
-        cudaEvent_t e1 = prof.mark_launch();
-        if (prof.per_launch) prof.timed(e0, e1);
-        COUNTED(prof, 1, launch_reduce_finalize4(b.partials, nullptr, dgrid, b.llp, dgrid, nullptr, nullptr, k, n, o.reg_covar,
-                                                 o.tol, b.model64, b.params, b.trace, perm, b.st, t, true, c.s, pdl));
-    }
-    for (int t = 1; t <= o.iters && !dense; ++t) {
-        const ReachLaunch a = reach_launch(rb, pe, n, k, b.params, b.st, t);
-        cudaEvent_t e0 = prof.mark_launch();
-        GIRA_CUDA(reach_estep_stats(4, rb, a, &prof.launches, c.s));
-        cudaEvent_t e1 = prof.mark_launch();
-        if (prof.per_launch) prof.timed(e0, e1);
-        COUNTED(prof, 1, launch_reduce_finalize4(rb.partials, rb.live2, rb.slices, rb.llp, rb.grid, nullptr, nullptr, k,
-                                                 n, o.reg_covar, o.tol, b.model64, b.params, b.trace, perm, b.st, t,
-                                                 true, c.s));
-    }
-    prof.t_em = prof.mark();
-    if (final_loglik && dense) {
-        da.iter = 0;
-        COUNTED(prof, 1, launch_estep4_dense(da, false, dgrid, c.s));
-        COUNTED(prof, 1, launch_ll_reduce(b.llp, dgrid, b.st, c.s));
-    } else if (final_loglik)
-        GIRA_CUDA(reach_loglik(4, rb, reach_launch(rb, pe, n, k, b.params, b.st, 0), false, &prof.launches, c.s));
-    COUNTED(prof, 1, launch_model_out4(b.model64, k, w_d, mu_d, cov_d, perm, b.st, c.s));
-    if (kw == Kind::Host) GIRA_CUDA(cudaMemcpyAsync(weights, b.mw, sizeof(float) * k, cudaMemcpyDeviceToHost, c.s));
-    if (km == Kind::Host) GIRA_CUDA(cudaMemcpyAsync(means, b.mmu, sizeof(float) * 4 * k, cudaMemcpyDeviceToHost, c.s));
-    if (kc == Kind::Host) GIRA_CUDA(cudaMemcpyAsync(covs, b.mcov, sizeof(float) * 16 * k, cudaMemcpyDeviceToHost, c.s));
-    if (loglik_trace && o.iters > 0)
-        GIRA_CUDA(cudaMemcpyAsync(loglik_trace, b.trace, sizeof(double) * o.iters, cudaMemcpyDeviceToHost, c.s));
-    GIRA_CUDA(cudaMemcpyAsync(&h, b.st, sizeof h, cudaMemcpyDeviceToHost, c.s));
-    prof.t_end = prof.mark();
-    GIRA_CUDA(cudaStreamSynchronize(c.s));
     prof.commit(h.iters_done, h.iters_done);
     TRY(device_status(h));
     if (iters_done) *iters_done = h.iters_done;

@@ -541,8 +541,8 @@ cudaError_t launch_reach_prepare(int d, const float* params, int k, const Device
 // d: 3 or 4 dimensions.  mode 0 log-likelihood, 1 with masks and pref, 2 gradient (3-D); h: reach_h of the launch; kmax: the largest k.
 cudaError_t launch_estep_reach(int d, const ReachLaunch& a, int mode, int grid, int h, int kmax, cudaStream_t s);
 // partials [slices][pairs][2 NSTAT (4-D: NSTAT4)], written where a.live2 has the bit:
-// launch_reduce_finalize takes the two as rows and masks.
-cudaError_t launch_reach_stats(int d, const ReachLaunch& a, float* partials, cudaStream_t s);
+// launch_reduce_finalize takes the two as rows and masks.  world (4-D): about x - mu, not whitened.
+cudaError_t launch_reach_stats(int d, const ReachLaunch& a, bool world, float* partials, cudaStream_t s);
 
 struct EStepLaunch {
     const float4* pts8;      // 2 float4 per point: (x,x,y,y) (z,z,0,0)
@@ -859,19 +859,20 @@ struct EStep4Launch {
     float* per_point;      // [n] natural-log lse, or nullptr
     DeviceState* st;
     int iter;              // 1-based EM iteration; skipped when iter > st->stop_after
+    bool world = false;    // statistics about x - mu, not whitened
 };
 bool estep4_dense(int64_t n, int k, bool stats);
 int estep4_dense_grid(int64_t n, int k, int num_sms, int64_t* pts_per_cta);
 cudaError_t launch_estep4_dense(const EStep4Launch& a, bool stats, int grid, cudaStream_t s, bool pdl = false);
 // M-step from the partials of launch_reach_stats or launch_estep4_dense ([slices][pairs][2 NSTAT4],
-// live where live2 says; nullptr: all) or, when partials is nullptr, from binary64 one-hot statistics stats64
+// live where live2 says; nullptr: all; world as there) or, when partials is nullptr, from binary64 one-hot statistics stats64
 // about shift4; em as in launch_reduce_finalize, the log-likelihood being the sum of
 // llp[0 .. ll_count).  Slot b holds the caller's component perm[b] (nullptr: b).
 cudaError_t launch_reduce_finalize4(const float* partials, const uint32_t* live2, int slices, const double* llp,
                                     int ll_count, const double* stats64, const float4* shift4, int k, int64_t n,
                                     double reg, double tol, double* model64, float* params, double* trace,
                                     const int* perm, DeviceState* st, int iter, bool em, cudaStream_t s,
-                                    bool pdl = false);
+                                    bool pdl = false, bool world = false);
 // Components in Morton order of their means, as launch_order_components (scratch: k * MODEL4 doubles).
 cudaError_t launch_order_components4(double* model64, double* scratch, int k, int* perm, float* params,
                                      DeviceState* st, cudaStream_t s);

@@ -764,8 +764,10 @@ __global__ void __launch_bounds__(32 * cta_warps(H), H > RB_W ? 16 / H : D == 3 
 // launch on the 276,348-point frame in 4-D at K = 512 and 1.33 ms on the 4M-point map at
 // K = 8192, with 9 of 16 resident warps active (CTAs of 8 such warps); 38 us and 0.50 ms now.
 // Copying a unit's next block to shared memory meanwhile (cp.async) changed nothing.
+// WORLD: about d = x - mu_old instead (a fit repeated after whitened sums lost a covariance to
+// binary32: see gira_gmm_fit4).
 constexpr int ST_W = 4;   // warps per CTA
-template <int D>
+template <int D, bool WORLD>
 __global__ void __launch_bounds__(32 * ST_W) reach_stats_kernel(const ReachLaunch a_in, float* partials) {
     constexpr int NS = Lay<D>::NS;
     const int lane = threadIdx.x & 31;
@@ -818,6 +820,9 @@ __global__ void __launch_bounds__(32 * ST_W) reach_stats_kernel(const ReachLaunc
                     const float2 nq = nlogit<D>(P, X, y);
                     const float2 e = f2(ex2_approx(pr.x - nq.x), ex2_approx(pr.x - nq.y));
                     const float2 g = mul2(e, dup(ok ? pr.y : 0.f));
+                    if (WORLD)
+#pragma unroll
+                        for (int j = 0; j < D; ++j) y[j] = add2(X[j], P.nmu[j]);
                     S[0] = add2(S[0], g);
 #pragma unroll
                     for (int i2 = 0, q = 1 + D; i2 < D; ++i2) {
@@ -907,13 +912,14 @@ cudaError_t launch_estep_reach(int d, const ReachLaunch& a, int mode, int grid, 
     return cudaLaunchKernel(fn, dim3(grid), dim3(32 * cta_warps(h)), args, reach_smem(kmax, h), s);
 }
 
-cudaError_t launch_reach_stats(int d, const ReachLaunch& a, float* partials, cudaStream_t s) {
+cudaError_t launch_reach_stats(int d, const ReachLaunch& a, bool world, float* partials, cudaStream_t s) {
     int dev = 0, sms = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int grid = sms * (d == 3 ? 7 : 5);   // as many warps as fit (72 and 96 registers a thread)
-    if (d == 3) reach_stats_kernel<3><<<grid, 32 * ST_W, 0, s>>>(a, partials);
-    else reach_stats_kernel<4><<<grid, 32 * ST_W, 0, s>>>(a, partials);
+    if (d == 3) reach_stats_kernel<3, false><<<grid, 32 * ST_W, 0, s>>>(a, partials);
+    else if (!world) reach_stats_kernel<4, false><<<grid, 32 * ST_W, 0, s>>>(a, partials);
+    else reach_stats_kernel<4, true><<<grid, 32 * ST_W, 0, s>>>(a, partials);
     return cudaGetLastError();
 }
 

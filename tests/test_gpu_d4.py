@@ -292,3 +292,20 @@ def test_regression_forms_give_the_same_bits(gira, frame4, k):
         part = gira.gira_gmm_conditional4(np.ascontiguousarray(locs[at]), w, means, covs)
         np.testing.assert_array_equal(to_np(part[0]), e[at])
         np.testing.assert_array_equal(to_np(part[1]), v[at])
+
+
+@pytest.mark.parametrize("n,k", [(3_000, 7), (40_000, 700)])
+@pytest.mark.parametrize("axis,far", [(0, 1e6), (0, 1e8), (1, 1e5), (1, 1e10), (2, 1e10), (3, 1e8)])
+def test_point_far_off_in_one_coordinate(gira, n, k, axis, far):
+    """A finite garbage value in one coordinate: the component that takes it keeps its covariance (statistics
+    about x - mu where the whitened ones lose it), by the dense E-step and over the lists."""
+    rng = np.random.default_rng(0)
+    a = rng.normal(size=(k, 4, 4)) * 0.2
+    w = rng.dirichlet(np.ones(k)).astype(np.float32)
+    m = rng.normal(size=(k, 4)).astype(np.float32)
+    c = (a @ np.transpose(a, (0, 2, 1)) + 0.05 * np.eye(4)).astype(np.float32)
+    pts = np.random.default_rng(1).normal(size=(n, 4)).astype(np.float32)
+    pts[n // 3, axis] = far
+    r = gira.gira_gmm_fit4(pts, k, iters=1, tol=0.0, reg_covar=1e-3, init=(w, m, c))
+    ref = oracle.em_par(pts, w, m, c, iters=1, tol=0.0, reg=1e-3)
+    assert_model_close((r["weights"], r["means"], r["covs"]), (ref["weights"], ref["means"], ref["covs"]))
