@@ -1176,7 +1176,8 @@ __global__ void __launch_bounds__(SP_THREADS) sample_prepare_kernel(const float*
             tot += (double)w[b];
             cum[b] = tot;
         }
-        if (!(tot > 0.0)) set_error(st, GIRA_ERR_INVALID_ARG);
+        // (a sum that is not finite has a weight that is not: the components' blocks report it)
+        if (!(tot > 0.0) && isfinite(tot)) set_error(st, GIRA_ERR_INVALID_ARG);
     }
 }
 

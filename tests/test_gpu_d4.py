@@ -309,3 +309,16 @@ def test_point_far_off_in_one_coordinate(gira, n, k, axis, far):
     r = gira.gira_gmm_fit4(pts, k, iters=1, tol=0.0, reg_covar=1e-3, init=(w, m, c))
     ref = oracle.em_par(pts, w, m, c, iters=1, tol=0.0, reg=1e-3)
     assert_model_close((r["weights"], r["means"], r["covs"]), (ref["weights"], ref["means"], ref["covs"]))
+
+
+@pytest.mark.parametrize("k", [5, 300, 1_500])
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
+def test_sampling_reports_a_weight_that_is_not_finite(gira, k, bad):
+    """Not as one that is not positive, whichever check comes first."""
+    w, m = np.full(k, 1.0 / k, np.float32), np.zeros((k, 4), np.float32)
+    c = np.tile(np.eye(4, dtype=np.float32), (k, 1, 1))
+    w[k - 2] = bad
+    for _ in range(3):
+        with pytest.raises(gira.GiraError) as e:
+            gira.gira_gmm_sample(100, w, m, c, seed=1)
+        assert e.value.status == 2   # GIRA_ERR_NONFINITE_INPUT
