@@ -329,8 +329,14 @@ struct Fin4Args {
     const int* perm;
     DeviceState* st;
     int iter, em;
-    bool world;   // the partials are about x - s: M = I
+    Sums4 sums;
 };
+// Binary32 sums whitened by the old components lose part of Sigma = M C M^T on the way back: of Sigma_ii up to
+// 2^-24 root_i^2, root_i = sum_m |M_im| (S2_mm / N_b)^(1/2).  One point 1e2 .. 1e6 off in one coordinate of a cloud
+// of unit extent: normalised errors of 0.1 .. 2.5 times 2^-24 root_i^2 / Sigma_ii (from 1e-5 to above 1), sums about
+// x - mu 2e-6.  From root_i = 16 sqrt(Sigma_ii) on (1.5e-5) the fit goes over to those;
+// 256 fits of depth frames (2 .. 15,000 points a component) stayed below 8.1.
+constexpr float MAX_LOSS4 = 16.f;
 constexpr int FIN4_WARPS = 8;
 __global__ void __launch_bounds__(32 * FIN4_WARPS) reduce_finalize4_kernel(const Fin4Args f) {
     __shared__ float s_hi[FIN4_WARPS][2][32];
@@ -342,7 +348,7 @@ __global__ void __launch_bounds__(32 * FIN4_WARPS) reduce_finalize4_kernel(const
     if ((f.em && f.iter > st->stop_after) || st->error) return;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int pp = blockIdx.x;
-    const bool white = f.partials != nullptr && !f.world;
+    const bool white = f.partials != nullptr && f.sums != Sums4::About;
     if (f.partials) {
         const int npairs = (f.k + 1) >> 1;
         const uint32_t* lw = f.live2 ? f.live2 + (size_t)(pp >> 5) * f.slices : nullptr;   // nullptr: every row
@@ -436,6 +442,11 @@ __global__ void __launch_bounds__(32 * FIN4_WARPS) reduce_finalize4_kernel(const
         }
         __syncwarp();
         const double sig = on ? C[l] : 0.0;
+        if (on && white && i == j && f.sums == Sums4::Checked) {
+            float root = 0.f;
+            for (int m = 0; m <= i; ++m) root += fabsf((float)M[4 * i + m]) * sqrtf((float)(S[5 + sym4(m, m)] * inv));
+            if (root * rsqrtf((float)sig) > MAX_LOSS4) set_error(st, LOST_SUMS4);
+        }
         double fro2 = sig * sig;
 #pragma unroll
         for (int o = 8; o > 0; o >>= 1) fro2 += __shfl_xor_sync(FULL, fro2, o);
@@ -1536,9 +1547,9 @@ cudaError_t launch_reduce_finalize4(const float* partials, const uint32_t* live2
                                     int ll_count, const double* stats64, const float4* shift4, int k, int64_t n,
                                     double reg, double tol, double* model64, float* params, double* trace,
                                     const int* perm, DeviceState* st, int iter, bool em, cudaStream_t s, bool pdl,
-                                    bool world) {
+                                    Sums4 sums) {
     const Fin4Args f{partials, live2, slices, llp, ll_count, stats64, shift4, k, n, reg, tol, model64, params, trace,
-                     perm, st, iter, em ? 1 : 0, world};
+                     perm, st, iter, em ? 1 : 0, sums};
     PdlConfig c(dim3((k + 1) / 2), dim3(32 * FIN4_WARPS), 0, s, pdl);
     return cudaLaunchKernelEx(&c.cfg, reduce_finalize4_kernel, f);
 }

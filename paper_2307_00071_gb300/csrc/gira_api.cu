@@ -1875,24 +1875,26 @@ gira_status gira_gmm_fit4(const float* points, int64_t n, int k, const gira_fit_
     prof.per_launch = g_prof_on.load() == 1;
     prof.s = c.s;
     prof.t0 = prof.mark();
-    // The statistics are whitened.  A point far off in one coordinate (1e5 m and more in a cloud of
-    // metres) then fills every later row of a component's sums, and binary32 loses the
-    // covariance, which sums about x - mu keep: such a fit, and one that truly ends
-    // there, is made once more with those.
+    // The statistics are whitened.  A point far off in one coordinate (1e3 m and more in a cloud of
+    // metres) fills every later row of a component's sums, and binary32 loses the covariance
+    // on the way back, which sums about x - mu keep.  The finalize reports that, or a covariance that is no
+    // longer positive definite, and the EM is made again with those sums (the seeding is
+    // not).  Where they end the fit themselves, the whitened sums are taken as they come.
     DeviceState h{};
-    for (int world = 0; world < 2; ++world) {
+    for (const Sums4 sums : {Sums4::Checked, Sums4::About, Sums4::Whitened}) {
+        const bool first = sums == Sums4::Checked, world = sums == Sums4::About;
         h = DeviceState{};
         h.stop_after = o.iters;
         h.bad_component = INT_MAX;
         GIRA_CUDA(cudaMemcpyAsync(b.st, &h, sizeof h, cudaMemcpyHostToDevice, c.s));
         GIRA_CUDA(cudaMemsetAsync(b.trace, 0xff, sizeof(double) * std::max(o.iters, 1), c.s));   // NaN
         const float* pts = points;
-        if (kp == Kind::Host) {
+        if (kp == Kind::Host && first) {
             GIRA_CUDA(cudaMemcpyAsync(b.pin, points, sizeof(float) * 4 * n, cudaMemcpyHostToDevice, c.s));
             pts = b.pin;
         }
-        COUNTED(prof, 1, launch_pack4(pts, n, kinit ? b.p4 : nullptr, b.p8, b.st, c.s));
-        if (sorted)
+        if (first) COUNTED(prof, 1, launch_pack4(pts, n, kinit ? b.p4 : nullptr, b.p8, b.st, c.s));
+        if (sorted && first)
             COUNTED(prof, point_order_launches(1),
                     launch_point_order(b.p8, n, nullptr, nullptr, 0, 1, b.osc, b.p8s, kinit ? b.p4s : nullptr, nullptr, c.s));
         COUNTED(prof, 1, launch_fill_padding4(b.params, k, c.s));
@@ -1900,11 +1902,13 @@ gira_status gira_gmm_fit4(const float* points, int64_t n, int k, const gira_fit_
         float* mu_d = (km == Kind::Device) ? means : b.mmu;
         float* cov_d = (kc == Kind::Device) ? covs : b.mcov;
         if (kinit) {
-            TRY(seed_centres(prof, c, b.p4, n, 4, k, o.seed, b.c4, b.ch, b.d2, b.bs, b.ksync, b.ksums, kgrid, b.st));
-            GIRA_CUDA(cudaMemsetAsync(b.sums, 0, sizeof(double) * 5 * k, c.s));
-            GIRA_CUDA(cudaMemsetAsync(b.chg, 0, sizeof(unsigned long long) * (o.lloyd_iters + 1), c.s));
-            COUNTED(prof, 1 + 2 * o.lloyd_iters, launch_lloyd4(sorted ? b.p4s : b.p4, n, k, o.lloyd_iters, b.c4, b.lab, b.sums, b.chg,
-                                                              b.st, c.s));
+            if (first) {
+                TRY(seed_centres(prof, c, b.p4, n, 4, k, o.seed, b.c4, b.ch, b.d2, b.bs, b.ksync, b.ksums, kgrid, b.st));
+                GIRA_CUDA(cudaMemsetAsync(b.sums, 0, sizeof(double) * 5 * k, c.s));
+                GIRA_CUDA(cudaMemsetAsync(b.chg, 0, sizeof(unsigned long long) * (o.lloyd_iters + 1), c.s));
+                COUNTED(prof, 1 + 2 * o.lloyd_iters, launch_lloyd4(sorted ? b.p4s : b.p4, n, k, o.lloyd_iters, b.c4, b.lab, b.sums, b.chg,
+                                                                  b.st, c.s));
+            }
             GIRA_CUDA(cudaMemsetAsync(b.stats64, 0, sizeof(double) * NSTAT4 * k, c.s));
             COUNTED(prof, 1, launch_label_stats4(sorted ? b.p4s : b.p4, n, k, b.lab, b.c4, b.stats64, b.st, c.s));
             COUNTED(prof, 1, launch_reduce_finalize4(nullptr, nullptr, 0, nullptr, 0, b.stats64, b.c4, k, n, o.reg_covar,
@@ -1922,7 +1926,7 @@ gira_status gira_gmm_fit4(const float* points, int64_t n, int k, const gira_fit_
         if (!dense) COUNTED(prof, 2, launch_order_components4(b.model64, b.stats64, k, b.perm, b.params, b.st, c.s));
         prof.t_init = prof.mark();
         const float4* pe = sorted ? b.p8s : b.p8;
-        EStep4Launch da{pe, n, k, b.params, ppc, b.partials, b.llp, nullptr, b.st, 0, world != 0};
+        EStep4Launch da{pe, n, k, b.params, ppc, b.partials, b.llp, nullptr, b.st, 0, world};
         for (int t = 1; t <= o.iters && dense; ++t) {
             const bool pdl = !prof.per_launch;   // dependent launches, as in the 3-D loop
             da.iter = t;
@@ -1932,17 +1936,17 @@ gira_status gira_gmm_fit4(const float* points, int64_t n, int k, const gira_fit_
             if (prof.per_launch) prof.timed(e0, e1);
             COUNTED(prof, 1, launch_reduce_finalize4(b.partials, nullptr, dgrid, b.llp, dgrid, nullptr, nullptr, k, n, o.reg_covar,
                                                      o.tol, b.model64, b.params, b.trace, perm, b.st, t, true, c.s, pdl,
-                                                     world != 0));
+                                                     sums));
         }
         for (int t = 1; t <= o.iters && !dense; ++t) {
             const ReachLaunch a = reach_launch(rb, pe, n, k, b.params, b.st, t);
             cudaEvent_t e0 = prof.mark_launch();
-            GIRA_CUDA(reach_estep_stats(4, rb, a, world != 0, &prof.launches, c.s));
+            GIRA_CUDA(reach_estep_stats(4, rb, a, world, &prof.launches, c.s));
             cudaEvent_t e1 = prof.mark_launch();
             if (prof.per_launch) prof.timed(e0, e1);
             COUNTED(prof, 1, launch_reduce_finalize4(rb.partials, rb.live2, rb.slices, rb.llp, rb.grid, nullptr, nullptr, k,
                                                      n, o.reg_covar, o.tol, b.model64, b.params, b.trace, perm, b.st, t,
-                                                     true, c.s, false, world != 0));
+                                                     true, c.s, false, sums));
         }
         prof.t_em = prof.mark();
         if (final_loglik && dense) {
@@ -1960,7 +1964,7 @@ gira_status gira_gmm_fit4(const float* points, int64_t n, int k, const gira_fit_
         GIRA_CUDA(cudaMemcpyAsync(&h, b.st, sizeof h, cudaMemcpyDeviceToHost, c.s));
         prof.t_end = prof.mark();
         GIRA_CUDA(cudaStreamSynchronize(c.s));
-        if (h.error != GIRA_ERR_NOT_PD || h.iters_done == 0) break;   // 0: the start itself was not sound
+        if (h.error != GIRA_ERR_NOT_PD && h.error != LOST_SUMS4) break;
     }
     prof.commit(h.iters_done, h.iters_done);
     TRY(device_status(h));

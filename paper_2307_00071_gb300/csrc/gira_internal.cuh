@@ -841,6 +841,11 @@ constexpr int MODEL4 = 15;
 // index of (i, j), i <= j, in the upper-triangle order 00,01,02,03,11,12,13,22,23,33
 __host__ __device__ constexpr int sym4(int i, int j) { return i * (7 - i) / 2 + j; }
 
+// A 4-D fit's sums: whitened, with LOST_SUMS4 in DeviceState::error (no gira_status) where binary32 lost part
+// of a covariance in them; about x - mu; whitened and not checked.
+enum class Sums4 { Checked, About, Whitened };
+constexpr int LOST_SUMS4 = -1;
+
 // Component pairs the parameter buffer holds for k.
 int params4_pairs(int k);
 // N x 4 -> pts4 (x,y,z,I) (nullable) and pts8 (x,x,y,y)(z,z,I,I); flags non-finite input.
@@ -865,14 +870,14 @@ bool estep4_dense(int64_t n, int k, bool stats);
 int estep4_dense_grid(int64_t n, int k, int num_sms, int64_t* pts_per_cta);
 cudaError_t launch_estep4_dense(const EStep4Launch& a, bool stats, int grid, cudaStream_t s, bool pdl = false);
 // M-step from the partials of launch_reach_stats or launch_estep4_dense ([slices][pairs][2 NSTAT4],
-// live where live2 says; nullptr: all; world as there) or, when partials is nullptr, from binary64 one-hot statistics stats64
-// about shift4; em as in launch_reduce_finalize, the log-likelihood being the sum of
+// live where live2 says; nullptr: all) or, when partials is nullptr, from binary64 one-hot statistics stats64
+// about shift4; sums as the partials are; em as in launch_reduce_finalize, the log-likelihood being the sum of
 // llp[0 .. ll_count).  Slot b holds the caller's component perm[b] (nullptr: b).
 cudaError_t launch_reduce_finalize4(const float* partials, const uint32_t* live2, int slices, const double* llp,
                                     int ll_count, const double* stats64, const float4* shift4, int k, int64_t n,
                                     double reg, double tol, double* model64, float* params, double* trace,
                                     const int* perm, DeviceState* st, int iter, bool em, cudaStream_t s,
-                                    bool pdl = false, bool world = false);
+                                    bool pdl = false, Sums4 sums = Sums4::Whitened);
 // Components in Morton order of their means, as launch_order_components (scratch: k * MODEL4 doubles).
 cudaError_t launch_order_components4(double* model64, double* scratch, int k, int* perm, float* params,
                                      DeviceState* st, cudaStream_t s);

@@ -322,3 +322,24 @@ def test_sampling_reports_a_weight_that_is_not_finite(gira, k, bad):
         with pytest.raises(gira.GiraError) as e:
             gira.gira_gmm_sample(100, w, m, c, seed=1)
         assert e.value.status == 2   # GIRA_ERR_NONFINITE_INPUT
+
+
+@pytest.mark.parametrize("n,k", [(3_000, 7), (40_000, 700), (20_000, 1_500)])
+@pytest.mark.parametrize("far", [0.0, 1e2, 1e3, 1e4, 1e5, 1e6])
+def test_covariances_keep_their_digits_beside_a_far_point(gira, n, k, far):
+    """A far point in each coordinate in turn: every covariance within 1e-4 of the oracle's in units of its own
+    standard deviations.  Whitened binary32 sums are kept while they lose less than 16^2 2^-24 = 1.5e-5, sums about
+    x - mu lose 2e-6; the rest is the responsibilities' rounding."""
+    rng = np.random.default_rng(0)
+    a = rng.normal(size=(k, 4, 4)) * 0.2
+    w = rng.dirichlet(np.ones(k)).astype(np.float32)
+    m = rng.normal(size=(k, 4)).astype(np.float32)
+    c = (a @ np.transpose(a, (0, 2, 1)) + 0.05 * np.eye(4)).astype(np.float32)
+    for axis in range(4):
+        pts = np.random.default_rng(5 + n).normal(size=(n, 4)).astype(np.float32)
+        pts[n // 3, axis] += far
+        r = gira.gira_gmm_fit4(pts, k, iters=1, tol=0.0, reg_covar=1e-3, init=(w, m, c))
+        want = oracle.em_par(pts, w, m, c, iters=1, tol=0.0, reg=1e-3)["covs"].reshape(k, 4, 4)
+        sd = np.sqrt(np.einsum("kii->ki", want))
+        err = np.abs(to_np(r["covs"]).reshape(k, 4, 4) - want) / (sd[:, :, None] * sd[:, None, :])
+        assert err.max() < 1e-4, (axis, err.max())
